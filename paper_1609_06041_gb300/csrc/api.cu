@@ -138,10 +138,10 @@ Layout layout(const Geometry *g, const ct_pdtv_params *prm)
     L.scal = o;     o += align256(sizeof(double) * S_COUNT);
     L.partials = o; o += align256(sizeof(double) * 2 * dot_partials_doubles());   // two concurrent reductions
     L.taps = o;     o += align256(sizeof(float) * (2 * (size_t)g->n_bins - 1));
-    L.hhat = o;     o += align256(sizeof(float2) * (size_t)g->n_fft);
+    L.hhat = o;     o += align256(sizeof(float2) * (size_t)g->p_fft);
     // the shift-variant D: its high band's taps and response, and s
     L.taps2 = o;    o += align256(sizeof(float) * (2 * (size_t)g->n_bins - 1));
-    L.hhat2 = o;    o += align256(sizeof(float2) * (size_t)g->n_fft);
+    L.hhat2 = o;    o += align256(sizeof(float2) * (size_t)g->p_fft);
     L.sv = o;       o += align256(sizeof(float) * I);
     L.winv = o;     o += align256(sizeof(float) * I);
     L.mu = o;       o += align256(sizeof(float) * I);
@@ -453,6 +453,7 @@ ct_status ct_geometry_create(int n, int n_views, int n_bins, const double *angle
     g->n_bins = n_bins;
     g->n_fft = 1;
     while (g->n_fft < 2 * n_bins) g->n_fft <<= 1;
+    g->p_fft = fft_length(n_bins);
     g->orbit = !angles && (n_views % 2 == 0) && (n % 2 == 0);   // V <= 8192, so a slice has <= 1024 base views
     cudaGetDevice(&g->device);
     g->n_sm = 0;
@@ -516,14 +517,13 @@ ct_status ct_geometry_create(int n, int n_views, int n_bins, const double *angle
             else if (2 * v == n_views) hci[g->n_col_items++] = make_int2(v, -1);
         }
     }
-    float2 *htw = new float2[g->n_fft];
-    for (int k = 0; k < g->n_fft; ++k) {
-        const double ang = -2.0 * M_PI * (double)k / (double)g->n_fft;
-        htw[k] = make_float2((float)cos(ang), (float)sin(ang));
-    }
+    // twiddles of the frequency-domain D (none above its longest transform)
+    const size_t ntw = fft_supported(g) ? fft_table_elems(g->p_fft) : 1;
+    float2 *htw = new float2[ntw]();
+    if (fft_supported(g)) fft_table(g->p_fft, htw);
     cudaError_t e = cudaMalloc(&g->d_views, sizeof(ViewP) * n_views);
-    if (e == cudaSuccess) e = cudaMalloc(&g->d_tw, sizeof(float2) * g->n_fft);
-    if (e == cudaSuccess) e = cudaMemcpy(g->d_tw, htw, sizeof(float2) * g->n_fft, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&g->d_tw, sizeof(float2) * ntw);
+    if (e == cudaSuccess) e = cudaMemcpy(g->d_tw, htw, sizeof(float2) * ntw, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMalloc(&g->d_row_list, sizeof(int) * (n_views + 1));
     if (e == cudaSuccess) e = cudaMalloc(&g->d_col_list, sizeof(int) * (n_views + 1));
     if (e == cudaSuccess) e = cudaMalloc(&g->d_trig, sizeof(float4) * n_views);
@@ -650,13 +650,13 @@ ct_status ct_ramp_filter_split(const ct_geometry *g, const float *taps_lo, const
         return fail(CT_ERR_ARG, "ct_ramp_filter_split: bad pointer");
     // the bands' frequency responses: stream-ordered scratch, freed after use
     float2 *hs = nullptr;
-    cudaError_t e = cudaMallocAsync((void **)&hs, sizeof(float2) * 2 * g->n_fft, S(stream));
+    cudaError_t e = cudaMallocAsync((void **)&hs, sizeof(float2) * 2 * g->p_fft, S(stream));
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(CT_ERR_OOM, "ct_ramp_filter_split: scratch allocation failed");
     }
-    launch_sv_hhat(g, taps_lo, taps_hi, half_len, hs, hs + g->n_fft, S(stream));
-    launch_filter_sv(g, hs, hs + g->n_fft, sv, in, out, nullptr, nullptr, 0, nullptr, batch, S(stream));
+    launch_sv_hhat(g, taps_lo, taps_hi, half_len, hs, hs + g->p_fft, S(stream));
+    launch_filter_sv(g, hs, hs + g->p_fft, sv, in, out, nullptr, nullptr, 0, nullptr, batch, S(stream));
     cudaFreeAsync(hs, S(stream));
     return cuda_check("ct_ramp_filter_split");
 }
@@ -675,13 +675,13 @@ ct_status ct_ramp_filter(const ct_geometry *g, const float *taps, int half_len, 
     }
     // frequency response of the taps: stream-ordered scratch, freed after use
     float2 *hhat = nullptr;
-    cudaError_t e = cudaMallocAsync((void **)&hhat, sizeof(float2) * g->n_fft, S(stream));
+    cudaError_t e = cudaMallocAsync((void **)&hhat, sizeof(float2) * g->p_fft, S(stream));
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(CT_ERR_OOM, "ct_ramp_filter: scratch allocation failed");
     }
     launch_hhat(g, taps, half_len, hhat, S(stream));
-    launch_filter_fft(g, hhat, in, out, nullptr, nullptr, 0, nullptr, batch, S(stream));
+    launch_filter_fft(g, hhat, in, out, nullptr, nullptr, 0, nullptr, batch, S(stream), true);
     cudaFreeAsync(hhat, S(stream));
     return cuda_check("ct_ramp_filter");
 }

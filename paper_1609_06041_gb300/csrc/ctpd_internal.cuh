@@ -32,14 +32,15 @@ struct ViewP {
 
 struct Geometry {
     int n, n_views, n_bins, device;
-    int n_fft;            // P = 2^ceil(log2(2B))
+    int n_fft;            // P = 2^ceil(log2(2B)), the period of the taps
+    int p_fft;            // transform length of D's convolution: n_fft, at least 64
     int n_row, n_col;     // views stepping along rows / columns
     float win_eps;        // candidate-window margin (bins) of the backprojector
     ViewP *d_views;       // device, n_views entries
     int *d_row_list;      // device, the n_row row-stepping view indices
     int *d_col_list;      // device, the n_col column-stepping view indices
     float4 *d_trig;       // device, per view (cos t, sin t, |a|, 1 - |a|/2) for A^T
-    float2 *d_tw;         // device, n_fft twiddles e^{-2 pi i k / P} (from double precision)
+    float2 *d_tw;         // device, twiddles of a p_fft-point transform (fft_table, from double precision)
     int orbit;            // default angles with V and N even: A^T by rotation orbits
     int vpair;            // default angles: A by view pairs (v, V-v)
     int n_row_items, n_col_items;
@@ -265,6 +266,10 @@ inline void counted(unsigned n = 1)
 // blocks of a kernel still run were measured slower in replayed graphs.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Lets the next kernel, launched with the attribute, start now (it still
+// waits at its pdl_wait() for this kernel to complete).
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Launches made through launch_kernel while a PdlScope is open on the
 // calling thread carry the programmatic-serialization attribute (the solve
 // loop, whose kernels each begin with pdl_wait()); otherwise launch_kernel
@@ -342,7 +347,7 @@ size_t orbit_smem_bytes();                      // shared memory of one orbit bl
 bool quad_ok(const Geometry *g);                // the view-pair projector serves this geometry
 // TV prox tiles of one image spread over n_sm blocks (k_tv.cu's rule)
 void tv_tile_shape(int n, int steps, int n_sm, int min_rows, int *tc, int *tr, int *ncb, int *nrb, int rows = 0);
-size_t dual_fft_smem(const Geometry *g);
+size_t dual_fft_smem(const Geometry *g);       // one exchange buffer of the dual update's transform
 // Device pointers into a solve workspace (api.cu's layout).
 struct SolveBuffers {
     double *scal;
@@ -402,12 +407,17 @@ void launch_taps(const Geometry *g, int mode, const double *scal, double tau, do
 // Frequency-domain D (k_fft.cu), for n_fft <= FFT_MAX_P.
 constexpr int FFT_MAX_P = 8192;
 bool fft_supported(const Geometry *g);
-// hhat (n_fft complex) = DFT of the taps placed circularly
+int fft_length(int n_bins);          // p_fft
+size_t fft_table_elems(int p);       // host twiddle table of a p-point transform
+void fft_table(int p, float2 *tw);
+// hhat (p_fft complex) = DFT of the taps placed circularly
 void launch_hhat(const Geometry *g, const float *taps, int half, float2 *hhat, cudaStream_t st);
-// out = post .* D(pre .* in) * (mode 1 ? -sigma : 1)
+// out = post .* D(pre .* in) * (mode 1 ? -sigma : 1).  early: the launch just
+// before it on st is launch_hhat, itself an ordinary launch, so in, pre and
+// post are complete when the kernel starts and only hhat is waited for
 void launch_filter_fft(const Geometry *g, const float2 *hhat, const float *in, float *out,
                        const float *pre, const float *post, int mode, const double *scal, int batch,
-                       cudaStream_t st);
+                       cudaStream_t st, bool early = false);
 // out = D (A x) with A x given as the projector's band partial sums
 void launch_filter_fft_bands(const Geometry *g, const float2 *hhat, const float *partial, float *out, int batch,
                              cudaStream_t st);
@@ -415,7 +425,7 @@ void launch_filter_fft_bands(const Geometry *g, const float2 *hhat, const float 
 void launch_dual_fft(const Geometry *g, const float2 *hhat, const float *partial, const float *b, float *mu,
                      float *mu_bar, const float *winv, int lowdose, const double *scal, cudaStream_t st);
 // The shift-variant preconditioner D = T_lo + S T_hi S (k_fft.cu; low-dose,
-// FFT path).  hs, hd (n_fft complex each) = (H_lo +- H_hi) / 2 from the band
+// FFT path).  hs, hd (p_fft complex each) = (H_lo +- H_hi) / 2 from the band
 // taps; sv = s (V x B), s_i = sqrt(kappa w_i).
 void launch_sv_hhat(const Geometry *g, const float *taps_lo, const float *taps_hi, int half, float2 *hs, float2 *hd,
                     cudaStream_t st);

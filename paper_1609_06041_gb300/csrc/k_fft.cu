@@ -8,127 +8,273 @@
 // P-point DFT of the circularly placed taps.  The taps are real, so two
 // views travel as the real and imaginary parts of one complex sequence.
 //
-// FFTs run in shared memory as Stockham autosort stages (radix 8, then a
-// radix-4 or radix-2 stage for the remaining factor), twiddles from a
-// table built in double precision on the host.
+// P / 8 threads run one transform with its elements in registers
+// (body_fft.cuh); the kernels are instantiated per length, so that all
+// index arithmetic is constant, and a block holds one transform (more for
+// P < 256, to fill a warp).
+#include <math.h>
+
+#include <algorithm>
+
 #include "body_fft.cuh"
 
 namespace ctpd {
 
+// Convolution length: the period n_fft of the taps, at least the shortest
+// transform.
+int fft_length(int n_bins)
+{
+    int p = 64;
+    while (p < 2 * n_bins) p <<= 1;
+    return p;
+}
+
+size_t fft_table_elems(int p) { return fft_tw_elems(p); }
+
+// tw: fft_table_elems(p) twiddles of a p-point transform (see fft_tw_elems)
+void fft_table(int p, float2 *tw)
+{
+    const int half = fft_tw_half(p), last = fft_last_radix(p);
+    for (int ns = 8; ns < p; ns *= 8) {
+        const int R = p / ns >= 8 ? 8 : last;
+        for (int r = 0; r < R; ++r)
+            for (int k = 0; k < ns; ++k) {
+                const double ang = -2.0 * M_PI * (double)((long)r * k * (p / (ns * R))) / (double)p;
+                const float2 w = make_float2((float)cos(ang), (float)sin(ang));
+                tw[fft_tw_off(ns) + r * ns + k] = w;
+                tw[half + fft_tw_off(ns) + r * ns + k] = make_float2(w.x, -w.y);
+            }
+    }
+}
+
+namespace {
+
+constexpr int block_threads(int P) { return fft_threads(P) < 32 ? 32 : fft_threads(P); }
+constexpr int block_transforms(int P) { return block_threads(P) / fft_threads(P); }
+constexpr size_t buf_bytes(int P) { return sizeof(float2) * fft_elems(P); }
+// dynamic shared memory: two exchange buffers per transform
+constexpr size_t block_smem(int P) { return 2 * buf_bytes(P) * block_transforms(P); }
+// three blocks of 256 threads an SM (85 registers): 360 view pairs on 152 SMs are one wave
+constexpr int min_blocks(int P) { return block_threads(P) >= 768 ? 1 : 768 / block_threads(P); }
+
+// Threads of a block that reads band sums.  A grid with a block or more for
+// every SM takes the transforms' threads only.  A smaller one (few views,
+// small images) is bound by the latency of its 16 loads an element, so there
+// 512 threads stage the residual and the transforms' threads go on alone
+// (measured on a form with 16 elements a thread: 512^2 / 32 views 19.6 us a
+// step without the extra threads, 10.7 with them; 64^2 / 90: 14.0 and 10.7).
+constexpr int wide_threads(int P) { return block_threads(P) < 512 ? 512 : block_threads(P); }
+bool wide_grid(const Geometry *g, int batch)
+{
+    const int per = std::max(1, 32 / fft_threads(g->p_fft));   // transforms a block
+    return wide_threads(g->p_fft) > block_threads(g->p_fft) &&
+           (long long)((g->n_views + 1) / 2) * batch < (long long)g->n_sm * per;
+}
+
+// Calls f(IntC<P>) for the transform length p.
+template <class F>
+void with_length(int p, F f)
+{
+    switch (p) {
+    case 64: f(IntC<64>{}); break;
+    case 128: f(IntC<128>{}); break;
+    case 256: f(IntC<256>{}); break;
+    case 512: f(IntC<512>{}); break;
+    case 1024: f(IntC<1024>{}); break;
+    case 2048: f(IntC<2048>{}); break;
+    case 4096: f(IntC<4096>{}); break;
+    case 8192: f(IntC<8192>{}); break;
+    default: break;
+    }
+}
+
+// This thread's place: element offset t, transform number, exchange buffers.
+template <int P>
+struct Place {
+    int t, which;
+    float2 *buf;
+    __device__ __forceinline__ Place(float2 *sm)
+    {
+        constexpr int T = fft_threads(P);
+        t = threadIdx.x % T;
+        const int sub = threadIdx.x / T;
+        which = blockIdx.x * block_transforms(P) + sub;
+        buf = sm + (size_t)sub * 2 * fft_elems(P);
+    }
+};
+
+}  // namespace
+
 // Hhat = DFT_P of the taps placed circularly (t[k] at k mod P).
-__global__ void __launch_bounds__(FFT_T)
-k_hhat(const float *__restrict__ taps, int half, int P, const float2 *__restrict__ tw, float2 *__restrict__ hhat)
+template <int P>
+__global__ void __launch_bounds__(block_threads(P), min_blocks(P))
+k_hhat(const float *__restrict__ taps, int half, const float2 *__restrict__ tw, float2 *__restrict__ hhat)
 {
     extern __shared__ float2 fsm[];
-    float2 *a = fsm, *b = fsm + fft_elems(P);
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
+    pdl_wait();
+    pdl_launch();   // a filter launched after this one stages its input meanwhile
+    const Place<P> pl(fsm);
+    float2 v[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
         // index i holds t[k] with k = i (i < half) or k = i - P (i > P - half)
-        float v = 0.0f;
-        if (i < half) v = taps[half - 1 + i];
-        else if (i > P - half) v = taps[half - 1 + (i - P)];
-        a[fp(i)] = make_float2(v, 0.0f);
+        const int i = pl.t + r * fft_threads(P);
+        float x = 0.0f;
+        if (i < half) x = taps[half - 1 + i];
+        else if (i > P - half) x = taps[half - 1 + (i - P)];
+        v[r] = make_float2(x, 0.0f);
     }
-    const float2 *res = fft_block(whole_block(), a, b, P, tw, false);
-    for (int i = threadIdx.x; i < P; i += blockDim.x) hhat[i] = res[fp(i)];
+    int ph = 0;
+    fft_regs<P, false, true>(whole_block(), pl.t, v, pl.buf, ph, tw, 1.0f);
+    if (pl.which != 0) return;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) hhat[pl.t + r * fft_threads(P)] = v[r];
 }
 
 void launch_hhat(const Geometry *g, const float *taps, int half, float2 *hhat, cudaStream_t st)
 {
-    const int P = g->n_fft;
     counted();
-    k_hhat<<<1, FFT_T, sizeof(float2) * 2 * fft_elems(P), st>>>(taps, half, P, g->d_tw, hhat);
+    with_length(g->p_fft, [&](auto L) {
+        constexpr int P = decltype(L)::value;
+        launch_kernel(k_hhat<P>, dim3(1), dim3(block_threads(P)), block_smem(P), st, taps, half, g->d_tw, hhat);
+    });
 }
 
 // out = post .* D(pre .* in) * sc, sc = 1 (mode 0) or -sigma (mode 1);
-// one block per pair of views (v, v+1) of image `blockIdx.y`.  BANDS: the
+// one transform per pair of views (v, v+1) of image `blockIdx.y`.  BANDS: the
 // input is A x given as band partial sums (in = partial, nb bands), added
-// in band order and scaled by the views' path lengths.
-template <bool BANDS>
-__global__ void __launch_bounds__(FFT_T)
+// in band order and scaled by the views' path lengths.  early: the kernel's
+// predecessor wrote hhat only, so the input is staged before the wait for it.
+// The plain form keeps no state, so it runs at 64 registers, four 256-thread
+// blocks an SM: 4 x 720 views x 736 bins 39.0 -> 22.3 us (issue 58 %; 23.8 us
+// at three blocks), the transform of the taps before it 12 -> 5.3 us.
+template <int P, bool BANDS, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? wide_threads(P) : block_threads(P),
+                                  WIDE ? 1 : BANDS ? min_blocks(P) : 4 * min_blocks(P) / 3)
 k_filter_fft(const float2 *__restrict__ hhat, const float *__restrict__ in, float *__restrict__ out,
              const float *__restrict__ pre, const float *__restrict__ post, int mode,
-             const double *__restrict__ scal, int V, int B, int P, const float2 *__restrict__ tw, int nb,
-             const ViewP *__restrict__ views)
+             const double *__restrict__ scal, int V, int B, const float2 *__restrict__ tw, int nb,
+             const ViewP *__restrict__ views, int early)
 {
     extern __shared__ float2 fsm[];
-    float2 *a = fsm, *b = fsm + fft_elems(P);
-    const int v0 = 2 * blockIdx.x, v1 = v0 + 1;
-    const bool has1 = v1 < V;
-    const size_t base = (size_t)blockIdx.y * V * B;
-    const size_t o0 = base + (size_t)v0 * B, o1 = base + (size_t)v1 * B;
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        float x0 = 0.0f, x1 = 0.0f;
-        if (i < B) {
-            if (BANDS) {
-                const size_t VB = (size_t)V * B;
-                const float *p0 = in + (size_t)blockIdx.y * nb * VB + (size_t)v0 * B + i;
-                const float *p1 = in + (size_t)blockIdx.y * nb * VB + (size_t)(has1 ? v1 : v0) * B + i;
-                float s0, s1;
-                band_sum2(p0, p1, VB, nb, s0, s1);
-                x0 = s0 * views[v0].scale;
-                x1 = has1 ? s1 * views[v1].scale : 0.0f;
-            } else {
-                x0 = in[o0 + i];
-                if (pre) x0 *= pre[o0 + i];
-                if (has1) {
-                    x1 = in[o1 + i];
-                    if (pre) x1 *= pre[o1 + i];
-                }
-            }
+    if (!early) pdl_wait();
+    constexpr int T = fft_threads(P);
+    const Place<P> pl(fsm);
+    const int v0 = 2 * pl.which, v1 = v0 + 1;
+    const bool has0 = v0 < V, has1 = v1 < V;
+    const size_t VB = (size_t)V * B, base = (size_t)blockIdx.y * VB;
+    const size_t o0 = base + (size_t)(has0 ? v0 : 0) * B, o1 = base + (size_t)(has1 ? v1 : 0) * B;
+    if constexpr (BANDS) {
+        // every thread stages elements of the block's transforms, in the second buffer (the exchanges write it
+        // after a barrier)
+        for (int q = 0; q < block_transforms(P); ++q) {
+            const int w0 = 2 * (blockIdx.x * block_transforms(P) + q), w1 = w0 + 1 < V ? w0 + 1 : w0;
+            if (w0 >= V) break;
+            const float *p = in + (size_t)blockIdx.y * nb * VB;
+            const float c0 = views[w0].scale, c1 = w1 > w0 ? views[w1].scale : 0.0f;
+            stage_bands(threadIdx.x, blockDim.x, B, p + (size_t)w0 * B, p + (size_t)w1 * B, VB, nb,
+                        fsm + (2 * q + 1) * fft_elems(P),
+                        [&](int, float s0, float s1) { return make_float2(s0 * c0, s1 * c1); });
         }
-        a[fp(i)] = make_float2(x0, x1);
+        __syncthreads();
+        if (WIDE && threadIdx.x >= block_threads(P)) return;
+    } else {
+#pragma unroll 1
+        for (int i = pl.t; i < B; i += T) {
+            float x0 = has0 ? in[o0 + i] : 0.0f, x1 = has1 ? in[o1 + i] : 0.0f;
+            if (pre) {
+                if (has0) x0 *= pre[o0 + i];
+                if (has1) x1 *= pre[o1 + i];
+            }
+            pl.buf[fft_elems(P) + fp(i)] = make_float2(x0, x1);
+        }
     }
-    // the response and the output scaling fused into the transforms' last stages
-    auto mul_h = [&](int d, float2 v, float2 *dst) { dst[fp(d)] = cmul(v, hhat[d]); };
-    float2 *f = fft_block_out(whole_block(), a, b, P, tw, false, mul_h);
+    if (early) pdl_wait();
+    const float2 *stage = pl.buf + fft_elems(P);
+    float2 v[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        const int i = pl.t + r * T;
+        v[r] = r < 4 && i < B && has0 ? stage[fp(i)] : make_float2(0.0f, 0.0f);
+    }
+    int ph = 0;
+    const GroupCtx ctx{(int)threadIdx.x, block_threads(P), 1};
+    fft_apply<P, false, true>(ctx, pl.t, v, pl.buf, ph, hhat, tw);
     const float sc = ((mode == 1) ? -fscal(scal, F_SIGMA) : 1.0f) / (float)P;
-    auto outp = [&](int d, float2 v, float2 *) {
-        if (d < B) {
-            float y0 = v.x * sc, y1 = v.y * sc;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = pl.t + r * T;
+        if (i < B && has0) {
+            float y0 = v[r].x * sc, y1 = v[r].y * sc;
             if (post) {
-                y0 *= post[o0 + d];
-                if (has1) y1 *= post[o1 + d];
+                y0 *= post[o0 + i];
+                if (has1) y1 *= post[o1 + i];
             }
-            out[o0 + d] = y0;
-            if (has1) out[o1 + d] = y1;
+            out[o0 + i] = y0;
+            if (has1) out[o1 + i] = y1;
         }
-    };
-    fft_block_out(whole_block(), f, f == a ? b : a, P, tw, true, outp);
+    }
+}
+
+// grid of one transform per view pair (views: per view) and image
+template <int P>
+static dim3 fft_grid(int transforms, int batch)
+{
+    return dim3((transforms + block_transforms(P) - 1) / block_transforms(P), batch);
 }
 
 // out = D (A x) from the projector's band partial sums
 void launch_filter_fft_bands(const Geometry *g, const float2 *hhat, const float *partial, float *out, int batch,
                              cudaStream_t st)
 {
-    const int P = g->n_fft;
-    dim3 grd((g->n_views + 1) / 2, batch);
     counted();
-    k_filter_fft<true><<<grd, FFT_T, sizeof(float2) * 2 * fft_elems(P), st>>>(hhat, partial, out, nullptr, nullptr, 0, nullptr,
-                                                                   g->n_views, g->n_bins, P, g->d_tw,
-                                                                   proj_bands(g->n), g->d_views);
+    with_length(g->p_fft, [&](auto L) {
+        constexpr int P = decltype(L)::value;
+        const bool wide = wide_grid(g, batch);
+        launch_kernel(wide ? k_filter_fft<P, true, true> : k_filter_fft<P, true, false>,
+                      fft_grid<P>((g->n_views + 1) / 2, batch), dim3(wide ? wide_threads(P) : block_threads(P)),
+                      block_smem(P), st, hhat, partial, out, nullptr, nullptr, 0, nullptr, g->n_views, g->n_bins,
+                      g->d_tw, proj_bands(g->n), g->d_views, 0);
+    });
 }
 
 void launch_filter_fft(const Geometry *g, const float2 *hhat, const float *in, float *out,
                        const float *pre, const float *post, int mode, const double *scal, int batch,
-                       cudaStream_t st)
+                       cudaStream_t st, bool early)
 {
-    const int P = g->n_fft;
-    dim3 grd((g->n_views + 1) / 2, batch);
     counted();
-    k_filter_fft<false><<<grd, FFT_T, sizeof(float2) * 2 * fft_elems(P), st>>>(hhat, in, out, pre, post, mode, scal,
-                                                                    g->n_views, g->n_bins, P, g->d_tw, 0, nullptr);
+    PdlScope pdl(early || t_pdl);
+    with_length(g->p_fft, [&](auto L) {
+        constexpr int P = decltype(L)::value;
+        launch_kernel(k_filter_fft<P, false, false>, fft_grid<P>((g->n_views + 1) / 2, batch), dim3(block_threads(P)),
+                      block_smem(P), st, hhat, in, out, pre, post, mode, scal, g->n_views, g->n_bins, g->d_tw, 0,
+                      nullptr, early ? 1 : 0);
+    });
 }
 
-__global__ void __launch_bounds__(FFT_T, 4)
-k_dual_fft(const float2 *__restrict__ hhat, const float *__restrict__ partial, int nb,
-           const float *b, const float *mu_in, float *mu, float *mu_bar,
-           const float *winv, int lowdose, const ViewP *__restrict__ views,
-           const double *__restrict__ scal, int V, int B, int P, const float2 *__restrict__ tw)
+// The fused dual step.  Bound: the latency of the 16 band loads an element
+// and of the exchanges between stages (issue 46 %, 29 % of the warp slots).
+// 512^2 / 720 views / 736 bins (360 view pairs, one wave of three 256-thread
+// blocks an SM): 35.3 -> 22.7 us; 32 views (16 pairs, the wide form): 16.6 ->
+// 10.9 us; 64^2 / 90 / 95: 14.6 -> 7.7 us (cold cache).
+template <int P, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? wide_threads(P) : block_threads(P), WIDE ? 1 : min_blocks(P))
+k_dual_fft(const DualArgs a)
 {
     extern __shared__ float2 fsm[];
     pdl_wait();
-    dual_fft_body(whole_block(), blockIdx.x, blockIdx.y, fsm, hhat, partial, nb, b, mu_in, mu, mu_bar, winv, lowdose,
-                  views, scal, V, B, P, tw);
+    const Place<P> pl(fsm);
+    if (WIDE) {
+        for (int q = 0; q < block_transforms(P); ++q)
+            dual_stage<P, true>(threadIdx.x, blockDim.x, blockIdx.x * block_transforms(P) + q, blockIdx.y,
+                                fsm + 2 * q * fft_elems(P), a);
+        __syncthreads();
+        if (threadIdx.x >= block_threads(P)) return;
+    } else {
+        dual_stage<P, true>(pl.t, fft_threads(P), pl.which, blockIdx.y, pl.buf, a);
+    }
+    const GroupCtx ctx{(int)threadIdx.x, block_threads(P), 1};
+    dual_update<P, true, true>(ctx, pl.t, pl.which, blockIdx.y, pl.buf, a);
 }
 
 // =====================================================================
@@ -159,65 +305,94 @@ void launch_sv_hhat(const Geometry *g, const float *taps_lo, const float *taps_h
     launch_hhat(g, taps_lo, half, hs, st);
     launch_hhat(g, taps_hi, half, hd, st);
     counted();
-    k_sv_combine<<<(g->n_fft + 255) / 256, 256, 0, st>>>(hs, hd, g->n_fft);
+    k_sv_combine<<<(g->p_fft + 255) / 256, 256, 0, st>>>(hs, hd, g->p_fft);
 }
 
-// Y(k) = hs(k) Z(k) + hd(k) conj Z(P-k), in place: each thread takes the pair (k, P-k)
-__device__ __forceinline__ void sv_spectrum(float2 *f, const float2 *__restrict__ hs, const float2 *__restrict__ hd,
-                                            int P)
+// v <- the shift-variant D's (u, v) pair (up to the factor P) of the
+// sequence (y, S y) in v: forward transform, Y(k) = hs(k) Z(k) + hd(k) conj
+// Z(P-k) with the mirrored elements taken through an exchange buffer, inverse.
+template <int P>
+__device__ __forceinline__ void sv_apply(int t, float2 (&v)[8], float2 *buf, int &ph, const float2 *__restrict__ hs,
+                                         const float2 *__restrict__ hd, const float2 *__restrict__ tw)
 {
-    for (int k = threadIdx.x; k <= P / 2; k += blockDim.x) {
-        const int k2 = (P - k) & (P - 1);
-        const float2 z1 = f[fp(k)], z2 = f[fp(k2)];
-        const float2 c1 = make_float2(z1.x, -z1.y), c2 = make_float2(z2.x, -z2.y);
-        f[fp(k)] = cadd(cmul(hs[k], z1), cmul(hd[k], c2));
-        if (k2 != k) f[fp(k2)] = cadd(cmul(hs[k2], z2), cmul(hd[k2], c1));
+    constexpr int T = fft_threads(P);
+    float s = 1.0f;
+#pragma unroll 1
+    for (int inv = 0; inv < 2; ++inv) {
+        fft_regs<P, true, true>(whole_block(), t, v, buf, ph, tw + inv * fft_tw_half(P), s);
+        s = -1.0f;
+        if (inv == 0) {
+            float2 *m = buf + ph * fft_elems(P);
+            ph ^= 1;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) m[fp(t + r * T)] = v[r];
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const int k = t + r * T;
+                const float2 z = m[fp((P - k) & (P - 1))];
+                v[r] = cadd(cmul(hs[k], v[r]), cmul(hd[k], make_float2(z.x, -z.y)));
+            }
+        }
     }
 }
 
+// sum of the nb band partial sums of one ray, in band order
+__device__ __forceinline__ float band_sum(const float *__restrict__ p, size_t VB, int nb)
+{
+    float acc = 0.0f;
+    for (int q = 0; q < nb; ++q) acc += p[q * VB];
+    return acc;
+}
+
 // out = post .* D(pre .* in) * sc, sc = 1 (mode 0) or -sigma (mode 1), D the
-// shift-variant form; one block per view v = blockIdx.x of image blockIdx.y.
+// shift-variant form; one transform per view of image blockIdx.y.
 // BANDS: the input is A x as the projector's nb band partial sums.
-template <bool BANDS>
-__global__ void __launch_bounds__(FFT_T)
+template <int P, bool BANDS>
+__global__ void __launch_bounds__(block_threads(P), min_blocks(P))
 k_filter_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const float *__restrict__ sv,
             const float *__restrict__ in, float *__restrict__ out, const float *__restrict__ pre,
-            const float *__restrict__ post, int mode, const double *__restrict__ scal, int V, int B, int P,
+            const float *__restrict__ post, int mode, const double *__restrict__ scal, int V, int B,
             const float2 *__restrict__ tw, int nb, const ViewP *__restrict__ views)
 {
     extern __shared__ float2 fsm[];
-    float2 *a = fsm, *b = fsm + fft_elems(P);
-    const int v = blockIdx.x;
+    pdl_wait();
+    constexpr int T = fft_threads(P);
+    const Place<P> pl(fsm);
+    const bool has = pl.which < V;
+    const int vw = has ? pl.which : 0;
     const size_t VB = (size_t)V * B;
-    const size_t o = (size_t)blockIdx.y * VB + (size_t)v * B;
-    const float *s = sv + (size_t)v * B;   // the weights, so S, are one slice's
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
+    const size_t o = (size_t)blockIdx.y * VB + (size_t)vw * B;
+    const float *s = sv + (size_t)vw * B;   // the weights, so S, are one slice's
+    float2 v[8];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = pl.t + r * T;
         float y = 0.0f, sy = 0.0f;
-        if (i < B) {
+        if (i < B && has) {
             if (BANDS) {
-                const float *pp = in + (size_t)blockIdx.y * nb * VB + (size_t)v * B + i;
-                float acc = 0.0f;
-                for (int q = 0; q < nb; ++q) acc += pp[q * VB];
-                y = acc * views[v].scale;
+                y = band_sum(in + (size_t)blockIdx.y * nb * VB + (size_t)vw * B + i, VB, nb) * views[vw].scale;
             } else {
                 y = in[o + i];
                 if (pre) y *= pre[o + i];
             }
             sy = s[i] * y;
         }
-        a[fp(i)] = make_float2(y, sy);
+        v[r] = make_float2(y, sy);
+        v[r + 4] = make_float2(0.0f, 0.0f);
     }
-    float2 *f = fft_block(whole_block(), a, b, P, tw, false);
-    sv_spectrum(f, hs, hd, P);
+    int ph = 0;
+    sv_apply<P>(pl.t, v, pl.buf, ph, hs, hd, tw);
     const float sc = ((mode == 1) ? -fscal(scal, F_SIGMA) : 1.0f) / (float)P;
-    auto outp = [&](int d, float2 uv, float2 *) {   // fused into the inverse transform's last stage
-        if (d < B) {
-            float y = fmaf(s[d], uv.y, uv.x) * sc;
-            if (post) y *= post[o + d];
-            out[o + d] = y;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = pl.t + r * T;
+        if (i < B && has) {
+            float y = fmaf(s[i], v[r].y, v[r].x) * sc;
+            if (post) y *= post[o + i];
+            out[o + i] = y;
         }
-    };
-    fft_block_out(whole_block(), f, f == a ? b : a, P, tw, true, outp);
+    }
 }
 
 void launch_filter_sv(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv, const float *in,
@@ -225,78 +400,88 @@ void launch_filter_sv(const Geometry *g, const float2 *hs, const float2 *hd, con
                       cudaStream_t st)
 {
     counted();
-    k_filter_sv<false><<<dim3(g->n_views, batch), FFT_T, sizeof(float2) * 2 * fft_elems(g->n_fft), st>>>(
-        hs, hd, sv, in, out, pre, post, mode, scal, g->n_views, g->n_bins, g->n_fft, g->d_tw, 0, nullptr);
+    with_length(g->p_fft, [&](auto L) {
+        constexpr int P = decltype(L)::value;
+        launch_kernel(k_filter_sv<P, false>, fft_grid<P>(g->n_views, batch), dim3(block_threads(P)), block_smem(P), st,
+                      hs, hd, sv, in, out, pre, post, mode, scal, g->n_views, g->n_bins, g->d_tw, 0, nullptr);
+    });
 }
 
 void launch_filter_sv_bands(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv,
                             const float *partial, float *out, int batch, cudaStream_t st)
 {
     counted();
-    k_filter_sv<true><<<dim3(g->n_views, batch), FFT_T, sizeof(float2) * 2 * fft_elems(g->n_fft), st>>>(
-        hs, hd, sv, partial, out, nullptr, nullptr, 0, nullptr, g->n_views, g->n_bins, g->n_fft, g->d_tw,
-        proj_bands(g->n), g->d_views);
+    with_length(g->p_fft, [&](auto L) {
+        constexpr int P = decltype(L)::value;
+        launch_kernel(k_filter_sv<P, true>, fft_grid<P>(g->n_views, batch), dim3(block_threads(P)), block_smem(P), st,
+                      hs, hd, sv, partial, out, nullptr, nullptr, 0, nullptr, g->n_views, g->n_bins, g->d_tw,
+                      proj_bands(g->n), g->d_views);
+    });
 }
 
 // Fused Step 3 and next Step 1 of Algorithm 1 with the shift-variant D, one
-// view per block (the form of k_dual_fft):
+// view per transform (the form of k_dual_fft):
 //   r = scale_v sum_b partial[b] - b - winv mu;  mu' = mu + sigma D r;
 //   mubar = 2 mu' - mu - sigma D (winv .* (mu' - mu)).
-__global__ void __launch_bounds__(FFT_T)
+template <int P>
+__global__ void __launch_bounds__(block_threads(P), min_blocks(P))
 k_dual_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const float *__restrict__ sv,
           const float *__restrict__ partial, int nb, const float *__restrict__ b, float *mu,
           float *__restrict__ mu_bar, const float *__restrict__ winv, const ViewP *__restrict__ views,
-          const double *__restrict__ scal, int V, int B, int P, const float2 *__restrict__ tw)
+          const double *__restrict__ scal, int V, int B, const float2 *__restrict__ tw)
 {
     extern __shared__ float2 fsm[];
-    float2 *a = fsm, *bb = fsm + fft_elems(P);
-    float *m_old = reinterpret_cast<float *>(fsm + 2 * fft_elems(P));   // B
-    float *m_new = m_old + B;                                          // B
-    const int v = blockIdx.x;
-    const size_t VB = (size_t)V * B, o = (size_t)v * B;
+    pdl_wait();
+    constexpr int T = fft_threads(P);
+    const Place<P> pl(fsm);
+    const bool has = pl.which < V;
+    const int vw = has ? pl.which : 0;
+    const size_t VB = (size_t)V * B, o = (size_t)vw * B;
     const float *s = sv + o;
-    const float sc = views[v].scale;
-    const float sigma = fscal(scal, F_SIGMA);
-    const float invP = 1.0f / (float)P;
-
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        float r = 0.0f, sr = 0.0f;
-        if (i < B) {
-            const float *pp = partial + o + i;
-            float acc = 0.0f;
-            for (int q = 0; q < nb; ++q) acc += pp[q * VB];
-            const float m0 = mu[o + i];
-            m_old[i] = m0;
-            r = acc * sc - b[o + i] - winv[o + i] * m0;
-            sr = s[i] * r;
+    const float sc = views[vw].scale;
+    const float sp = fscal(scal, F_SIGMA) * (1.0f / (float)P);
+    float2 v[8];
+    float mo[4], mn[4];   // mu, then 2 mu' - mu, and mu'
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = pl.t + r * T;
+        float res = 0.0f, sr = 0.0f;
+        mo[r] = 0.0f;
+        if (i < B && has) {
+            mo[r] = mu[o + i];
+            res = band_sum(partial + o + i, VB, nb) * sc - b[o + i] - winv[o + i] * mo[r];
+            sr = s[i] * res;
         }
-        a[fp(i)] = make_float2(r, sr);
+        v[r] = make_float2(res, sr);
+        v[r + 4] = make_float2(0.0f, 0.0f);
     }
-    float2 *f = fft_block(whole_block(), a, bb, P, tw, false);
-    sv_spectrum(f, hs, hd, P);
-    // the dual update fused into the inverse transform's last stage, which
-    // also stages the second filter's input (d, s d) in the buffer it writes
-    auto upd = [&](int i, float2 uv, float2 *dst) {
-        float d = 0.0f, sd = 0.0f;
-        if (i < B) {
-            const float n0 = m_old[i] + sigma * (fmaf(s[i], uv.y, uv.x) * invP);
-            m_new[i] = n0;
-            d = winv[o + i] * (n0 - m_old[i]);
-            sd = s[i] * d;
+    int ph = 0;
+#pragma unroll 1
+    for (int pass = 0;; ++pass) {
+        sv_apply<P>(pl.t, v, pl.buf, ph, hs, hd, tw);
+        if (pass) break;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int i = pl.t + r * T;
+            float d = 0.0f, sd = 0.0f;
+            if (i < B && has) {
+                mn[r] = fmaf(sp, fmaf(s[i], v[r].y, v[r].x), mo[r]);
+                d = winv[o + i] * (mn[r] - mo[r]);
+                sd = s[i] * d;
+                mo[r] = fmaf(2.0f, mn[r], -mo[r]);
+            }
+            v[r] = make_float2(d, sd);
+            v[r + 4] = make_float2(0.0f, 0.0f);
         }
-        dst[fp(i)] = make_float2(d, sd);
-    };
-    f = fft_block_out(whole_block(), f, f == a ? bb : a, P, tw, true, upd);
-    f = fft_block(whole_block(), f, f == a ? bb : a, P, tw, false);
-    sv_spectrum(f, hs, hd, P);
-    auto fin = [&](int i, float2 uv, float2 *) {
-        if (i < B) {
-            const float n0 = m_new[i];
-            mu[o + i] = n0;
-            mu_bar[o + i] = 2.0f * n0 - m_old[i] - sigma * (fmaf(s[i], uv.y, uv.x) * invP);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = pl.t + r * T;
+        if (i < B && has) {
+            mu[o + i] = mn[r];
+            mu_bar[o + i] = fmaf(-sp, fmaf(s[i], v[r].y, v[r].x), mo[r]);
         }
-    };
-    fft_block_out(whole_block(), f, f == a ? bb : a, P, tw, true, fin);
+    }
 }
 
 void launch_dual_sv(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv, const float *partial,
@@ -304,12 +489,16 @@ void launch_dual_sv(const Geometry *g, const float2 *hs, const float2 *hd, const
                     cudaStream_t st)
 {
     counted();
-    const size_t smem = sizeof(float2) * 2 * fft_elems(g->n_fft) + sizeof(float) * 2 * g->n_bins;
-    k_dual_sv<<<g->n_views, FFT_T, smem, st>>>(hs, hd, sv, partial, proj_bands(g->n), b, mu, mu_bar, winv,
-                                               g->d_views, scal, g->n_views, g->n_bins, g->n_fft, g->d_tw);
+    with_length(g->p_fft, [&](auto L) {
+        constexpr int P = decltype(L)::value;
+        launch_kernel(k_dual_sv<P>, fft_grid<P>(g->n_views, 1), dim3(block_threads(P)), block_smem(P), st, hs, hd, sv,
+                      partial, proj_bands(g->n), b, mu, mu_bar, winv, g->d_views, scal, g->n_views, g->n_bins,
+                      g->d_tw);
+    });
 }
 
-size_t dual_fft_smem(const Geometry *g) { return sizeof(float2) * 2 * fft_elems(g->n_fft) + sizeof(float) * 4 * g->n_bins; }
+// one exchange buffer, per thread group of a transform (the persistent kernel)
+size_t dual_fft_smem(const Geometry *g) { return buf_bytes(g->p_fft); }
 
 void launch_dual_fft(const Geometry *g, const float2 *hhat, const float *partial, const float *b, float *mu,
                      float *mu_bar, const float *winv, int lowdose, const double *scal, cudaStream_t st)
@@ -322,9 +511,14 @@ void launch_dual_fft_batched(const Geometry *g, const float2 *hhat, const float 
                              const double *scal, int batch, cudaStream_t st)
 {
     counted();
-    launch_kernel(k_dual_fft, dim3((g->n_views + 1) / 2, batch), dim3(FFT_T), dual_fft_smem(g), st, hhat, partial,
-                  proj_bands(g->n), b, mu_in, mu_out, mu_bar, winv, lowdose, g->d_views, scal, g->n_views, g->n_bins,
-                  g->n_fft, g->d_tw);
+    with_length(g->p_fft, [&](auto L) {
+        constexpr int P = decltype(L)::value;
+        const bool wide = wide_grid(g, batch);
+        const DualArgs a{hhat, g->d_tw, partial, proj_bands(g->n), b, mu_in, mu_out, mu_bar, winv, lowdose,
+                         g->d_views, scal, g->n_views, g->n_bins};
+        launch_kernel(wide ? k_dual_fft<P, true> : k_dual_fft<P, false>, fft_grid<P>((g->n_views + 1) / 2, batch),
+                      dim3(wide ? wide_threads(P) : block_threads(P)), block_smem(P), st, a);
+    });
 }
 
 // Adjoint of one dual step (Step 3 and the next Step 1) for the pair of
@@ -340,74 +534,84 @@ void launch_dual_fft_batched(const Geometry *g, const float2 *hhat, const float 
 //   gmu = gm1 - W gr - gmb + sigma W h    (dL/dmu)
 // and writes r and v = W (mu' - mu) for the tap correlations
 // dL/dt += sigma (gm1 * r) - sigma (gmb * v).  Few-view drops every W term.
-__global__ void __launch_bounds__(FFT_T)
+template <int P>
+__global__ void __launch_bounds__(block_threads(P), min_blocks(P))
 k_dual_bwd_fft(const float2 *__restrict__ hhat, const float *__restrict__ partial, int nb,
                const float *__restrict__ b, const float *__restrict__ winv, const float *__restrict__ mu,
                const float *__restrict__ mu1, const float *__restrict__ gm, const float *__restrict__ gmb,
-               float *__restrict__ gmu_out, float *__restrict__ gr_out, float *__restrict__ gm1_out,
+               float *__restrict__ gmu_out, float *__restrict__ gr_out, float *gm1_out,
                float *__restrict__ r_out, float *__restrict__ v_out, int lowdose,
-               const ViewP *__restrict__ views, const double *__restrict__ scal, int V, int B, int P,
+               const ViewP *__restrict__ views, const double *__restrict__ scal, int V, int B,
                const float2 *__restrict__ tw)
 {
     extern __shared__ float2 fsm[];
-    float2 *a = fsm, *bb = fsm + fft_elems(P);
-    float *h_s = reinterpret_cast<float *>(fsm + 2 * fft_elems(P));   // 2 x B: D^T gmb
-    float *g1_s = h_s + 2 * B;                             // 2 x B: gm1
-    const size_t so = (size_t)blockIdx.y * V * B;
-    partial += (size_t)blockIdx.y * nb * V * B;
-    const int v0 = 2 * blockIdx.x, v1 = v0 + 1;
-    const bool has1 = v1 < V;
-    const size_t VB = (size_t)V * B;
-    const size_t o0 = so + (size_t)v0 * B, o1 = so + (size_t)(has1 ? v1 : v0) * B;
+    pdl_wait();
+    constexpr int T = fft_threads(P);
+    const Place<P> pl(fsm);
+    const int v0 = 2 * pl.which, v1 = v0 + 1;
+    const bool has0 = v0 < V, has1 = v1 < V;
+    const size_t VB = (size_t)V * B, so = (size_t)blockIdx.y * VB;
+    const size_t o0 = so + (size_t)(has0 ? v0 : 0) * B, o1 = so + (size_t)(has1 ? v1 : 0) * B;
+    partial += (size_t)blockIdx.y * (nb - 1) * VB;
     const float sigma = fscal(scal, F_SIGMA);
     const float invP = 1.0f / (float)P;
+    const float sc0 = has0 ? views[v0].scale : 0.0f, sc1 = has1 ? views[v1].scale : 0.0f;
 
-    // h = D^T gmb
-    for (int i = threadIdx.x; i < P; i += blockDim.x)
-        a[fp(i)] = i < B ? make_float2(gmb[o0 + i], has1 ? gmb[o1 + i] : 0.0f) : make_float2(0.0f, 0.0f);
-    float2 *f = fft_block(whole_block(), a, bb, P, tw, false);
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const float2 h = hhat[i];
-        f[fp(i)] = cmul(f[fp(i)], make_float2(h.x, -h.y));
+    // pass 0: h = D^T gmb, which forms gm1 = gm + 2 gmb - sigma W h; pass 1: gr = sigma D^T gm1
+    float2 v[8], hr[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = pl.t + r * T;
+        v[r] = make_float2(i < B && has0 ? gmb[o0 + i] : 0.0f, i < B && has1 ? gmb[o1 + i] : 0.0f);
+        v[r + 4] = make_float2(0.0f, 0.0f);
     }
-    float2 *res = fft_block(whole_block(), f, f == a ? bb : a, P, tw, true);
-    float2 *other = res == a ? bb : a;
-    // gm1 = gm + 2 gmb - sigma W h ; stage gm1 for D^T
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        float g0 = 0.0f, g1v = 0.0f;
-        if (i < B) {
-            const float h0 = res[fp(i)].x * invP, h1 = res[fp(i)].y * invP;
-            h_s[i] = h0;
-            h_s[B + i] = h1;
-            g0 = gm[o0 + i] + 2.0f * gmb[o0 + i];
-            g1v = has1 ? gm[o1 + i] + 2.0f * gmb[o1 + i] : 0.0f;
-            if (lowdose) {
-                g0 -= sigma * winv[o0 + i] * h0;
-                if (has1) g1v -= sigma * winv[o1 + i] * h1;
+    int ph = 0;
+#pragma unroll 1
+    for (int pass = 0;; ++pass) {
+        fft_apply<P, true, true>(whole_block(), pl.t, v, pl.buf, ph, hhat, tw);
+        if (pass) break;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int i = pl.t + r * T;
+            float g0 = 0.0f, g1 = 0.0f;
+            hr[r] = make_float2(v[r].x * invP, v[r].y * invP);
+            if (i < B && has0) {
+                g0 = gm[o0 + i] + 2.0f * gmb[o0 + i];
+                if (lowdose) g0 -= sigma * winv[o0 + i] * hr[r].x;
+                gm1_out[o0 + i] = g0;
             }
-            g1_s[i] = g0;
-            g1_s[B + i] = g1v;
+            if (i < B && has1) {
+                g1 = gm[o1 + i] + 2.0f * gmb[o1 + i];
+                if (lowdose) g1 -= sigma * winv[o1 + i] * hr[r].y;
+                gm1_out[o1 + i] = g1;
+            }
+            v[r] = make_float2(g0, g1);
+            v[r + 4] = make_float2(0.0f, 0.0f);
         }
-        other[fp(i)] = make_float2(g0, g1v);
     }
-    f = fft_block(whole_block(), other, res, P, tw, false);
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const float2 h = hhat[i];
-        f[fp(i)] = cmul(f[fp(i)], make_float2(h.x, -h.y));
+    // the rest element by element, in a loop (for the code's size): the
+    // thread's own D^T gm1 and h wait in the free exchange buffer
+    float2 *st = pl.buf + ph * fft_elems(P);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = pl.t + r * T;
+        st[fp(i)] = v[r];
+        st[fp(P / 2 + i)] = hr[r];
     }
-    res = fft_block(whole_block(), f, f == a ? bb : a, P, tw, true);
-    const float sc0 = views[v0].scale, sc1 = has1 ? views[v1].scale : 0.0f;
-    for (int i = threadIdx.x; i < B; i += blockDim.x) {
-        // two views: k = 0 -> v0, k = 1 -> v1
-        for (int k = 0; k < (has1 ? 2 : 1); ++k) {
+    if (!has0) return;
+#pragma unroll 1
+    for (int i = pl.t; i < B; i += T) {
+        float s[2];
+        band_sum2(partial + o0 + i, partial + (has1 ? o1 : o0) + i, VB, nb, s[0], s[1]);
+        const float2 res = st[fp(i)], h = st[fp(P / 2 + i)];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (k == 1 && !has1) break;
             const size_t o = (k == 0 ? o0 : o1) + i;
-            const float gr = sigma * ((k == 0 ? res[fp(i)].x : res[fp(i)].y) * invP);
-            const float g1v = g1_s[k * B + i], hv = h_s[k * B + i];
+            const float gr = sigma * ((k == 0 ? res.x : res.y) * invP);
+            const float g1v = gm1_out[o], hv = k == 0 ? h.x : h.y;
             float gmu = g1v - gmb[o];
-            float acc = 0.0f;
-            const float *pp = partial + (o - so);
-            for (int q = 0; q < nb; ++q) acc += pp[q * VB];
-            float r = acc * (k == 0 ? sc0 : sc1) - b[o];
+            float r = s[k] * (k == 0 ? sc0 : sc1) - b[o];
             float vv = 0.0f;
             if (lowdose) {
                 gmu += -winv[o] * gr + sigma * winv[o] * hv;
@@ -416,14 +620,11 @@ k_dual_bwd_fft(const float2 *__restrict__ hhat, const float *__restrict__ partia
             }
             gmu_out[o] = gmu;
             gr_out[o] = gr;
-            gm1_out[o] = g1v;
             r_out[o] = r;
             v_out[o] = vv;
         }
     }
 }
-
-size_t dual_bwd_smem(const Geometry *g) { return sizeof(float2) * 2 * fft_elems(g->n_fft) + sizeof(float) * 4 * g->n_bins; }
 
 void launch_dual_bwd_fft(const Geometry *g, const float2 *hhat, const float *partial, const float *b,
                          const float *winv, const float *mu, const float *mu1, const float *gm, const float *gmb,
@@ -431,24 +632,33 @@ void launch_dual_bwd_fft(const Geometry *g, const float2 *hhat, const float *par
                          int batch, cudaStream_t st)
 {
     counted();
-    k_dual_bwd_fft<<<dim3((g->n_views + 1) / 2, batch), FFT_T, dual_bwd_smem(g), st>>>(
-        hhat, partial, proj_bands(g->n), b, winv, mu, mu1, gm, gmb, gmu, gr, gm1, r, v, lowdose, g->d_views,
-        scal, g->n_views, g->n_bins, g->n_fft, g->d_tw);
+    with_length(g->p_fft, [&](auto L) {
+        constexpr int P = decltype(L)::value;
+        launch_kernel(k_dual_bwd_fft<P>, fft_grid<P>((g->n_views + 1) / 2, batch), dim3(block_threads(P)),
+                      block_smem(P), st, hhat, partial, proj_bands(g->n), b, winv, mu, mu1, gm, gmb, gmu, gr, gm1, r,
+                      v, lowdose, g->d_views, scal, g->n_views, g->n_bins, g->d_tw);
+    });
 }
 
 bool fft_supported(const Geometry *g) { return g->n_fft <= FFT_MAX_P; }
 
 void kernel_attrs_fft()
 {
-    const int smax = (int)(sizeof(float2) * 2 * fft_elems(FFT_MAX_P) + sizeof(float) * 4 * (FFT_MAX_P / 2));
-    cudaFuncSetAttribute(k_hhat, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-    cudaFuncSetAttribute(k_filter_fft<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-    cudaFuncSetAttribute(k_filter_fft<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-    cudaFuncSetAttribute(k_dual_fft, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-    cudaFuncSetAttribute(k_dual_bwd_fft, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-    cudaFuncSetAttribute(k_filter_sv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-    cudaFuncSetAttribute(k_filter_sv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
-    cudaFuncSetAttribute(k_dual_sv, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
+    for (int p = 64; p <= FFT_MAX_P; p <<= 1)
+        with_length(p, [&](auto L) {
+            constexpr int P = decltype(L)::value;
+            const int sm = (int)block_smem(P);
+            cudaFuncSetAttribute(k_hhat<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            cudaFuncSetAttribute(k_filter_fft<P, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            cudaFuncSetAttribute(k_filter_fft<P, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            cudaFuncSetAttribute(k_filter_fft<P, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            cudaFuncSetAttribute(k_dual_fft<P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            cudaFuncSetAttribute(k_dual_fft<P, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            cudaFuncSetAttribute(k_dual_bwd_fft<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            cudaFuncSetAttribute(k_filter_sv<P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            cudaFuncSetAttribute(k_filter_sv<P, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            cudaFuncSetAttribute(k_dual_sv<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        });
 }
 
 }  // namespace ctpd

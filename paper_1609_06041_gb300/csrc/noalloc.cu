@@ -2,7 +2,7 @@
 // allocation, for callers that must not allocate (see include/ctpd.h).
 //
 // ct_ramp_filter needs a scratch buffer for the frequency response of the
-// taps (n_fft complex values); it takes that buffer from the stream-ordered
+// taps (p_fft complex values); it takes that buffer from the stream-ordered
 // allocator.  This variant keeps the scratch in a file-scope device array
 // instead, sized for the largest transform of the frequency-domain filter.
 #include <mutex>
@@ -85,9 +85,9 @@ extern "C" ct_status ct_ramp_filter_noalloc(const ct_geometry *geom, const float
         return CT_ERR_CUDA;
     }
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    // k_hhat writes all n_fft entries, so the shared array needs no clearing
+    // k_hhat writes all p_fft entries, so the shared array needs no clearing
     ctpd::launch_hhat(g, taps, half_len, hhat, st);
-    ctpd::launch_filter_fft(g, hhat, in, out, nullptr, nullptr, 0, nullptr, batch, st);
+    ctpd::launch_filter_fft(g, hhat, in, out, nullptr, nullptr, 0, nullptr, batch, st, true);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         ctpd::set_error("ct_ramp_filter_noalloc: %s", cudaGetErrorString(e));

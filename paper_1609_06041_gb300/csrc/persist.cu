@@ -26,7 +26,7 @@
 // The item bodies are those of the single-slice kernels (body_*.cuh), run
 // by the whole 1024-thread block (the work-balanced projector's unit ranges) or
 // by groups with their own named barriers (eight 128-thread orbit tiles,
-// four 256-thread view pairs of the dual update, two 512-thread TV tiles),
+// the view pairs of the dual update, two 512-thread TV tiles),
 // so A, A^T and the dual update keep the 32 warps per SM of their own
 // kernels; the block's 64 registers per thread are fewer than the TV
 // prox's own kernel uses, so the prox here holds regions of 48 rows.  All counters live in the slices' scalar blocks,
@@ -50,7 +50,6 @@ constexpr int PS_THREADS = 1024;
 constexpr int PS_MAX = 96;                         // slices per launch (kernel parameter space)
 enum { PH_ORBIT = 0, PH_OREDUCE, PH_TV, PH_QUAD, PH_DUAL, PH_N };
 constexpr int ORB_GROUPS = PS_THREADS / ORB_TH;    // orbit tiles per item
-constexpr int DUAL_GROUPS = PS_THREADS / FFT_T;    // view pairs per item
 constexpr int RED_PIX = PS_THREADS * 8;            // pixels per slice-reduction item
 constexpr int QUAD_PG = PS_THREADS / 64;           // projector view-pair items per block
 constexpr int TV_GROUPS = PS_THREADS / TV_THREADS; // TV tiles per item
@@ -60,13 +59,13 @@ constexpr int TV_GROUPS = PS_THREADS / TV_THREADS; // TV tiles per item
 constexpr int PS_TV_J = 3;
 constexpr int PS_TV_PUB = (TV_WARPS * PS_TV_J + 2) * 32;   // float2 per published field
 static_assert(TV_GROUPS * TV_THREADS == PS_THREADS && QUAD_PG == PG, "whole groups");
-static_assert(1 + ORB_GROUPS + DUAL_GROUPS + TV_GROUPS <= 16, "named barriers 1..15");
-static_assert(ORB_GROUPS * ORB_TH == PS_THREADS && DUAL_GROUPS * FFT_T == PS_THREADS, "whole groups");
+static_assert(1 + ORB_GROUPS + TV_GROUPS <= 16, "named barriers 1..15");
+static_assert(ORB_GROUPS * ORB_TH == PS_THREADS, "whole groups");
 
 struct PSlice {
     int N, V, B, P, nb, lowdose, al;
     int n_row_items, n_col_items, qseg;   // qseg: one projector item per staged band pair (segment)
-    int nsl, q16, orb_smem, dual_smem;
+    int nsl, q16, orb_smem;
     int tv_tc, tv_tr, tv_ncb, tv_nrb, ntv, fgp;
     int n_items[PH_N], pre[PH_N], per_iter;
     const ViewP *views;
@@ -101,6 +100,22 @@ __device__ __forceinline__ unsigned long long global_ns()
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
+}
+
+// The dual update of the PS_THREADS / (P/8) view pairs of item i.  Groups
+// of at least 128 threads share a named barrier (the orbit tiles' numbers:
+// the two phases never run together).
+template <int P>
+__device__ __noinline__ void dual_item(const PSlice &S, int i, unsigned char *psm)
+{
+    constexpr int T = fft_threads(P), GS = T < ORB_TH ? ORB_TH : T;
+    const int tid = threadIdx.x, sub = tid / T, g = tid / GS;
+    const int pair = i * (PS_THREADS / T) + sub, t = tid % T;
+    float2 *buf = reinterpret_cast<float2 *>(psm) + (size_t)sub * fft_elems(P);
+    const DualArgs a{S.hhat, S.tw, S.band, S.nb, S.b, S.mu, S.mu, S.mubar, S.winv, S.lowdose, S.views, S.scal, S.V,
+                     S.B};
+    dual_stage<P, false>(t, T, pair, 0, buf, a);
+    dual_update<P, false, false>(GroupCtx{tid % GS, GS, 1 + g}, t, pair, 0, buf, a);
 }
 
 // One work item of slice S: phase p of iteration k, item i of the phase.
@@ -140,7 +155,7 @@ __device__ __forceinline__ void run_item(const PSlice &S, int p, int k, int i, u
             float2 *pub_x = reinterpret_cast<float2 *>(psm) + (size_t)g * 2 * PS_TV_PUB;
             float2 *pub_y = pub_x + PS_TV_PUB;
             const int bx = j % S.tv_ncb, by = j / S.tv_ncb;
-            const GroupCtx c{tid % TV_THREADS, TV_THREADS, 1 + ORB_GROUPS + DUAL_GROUPS + g};
+            const GroupCtx c{tid % TV_THREADS, TV_THREADS, 1 + ORB_GROUPS + g};
             if (S.fgp)
                 tv_body<true, false, GroupCtx, PS_TV_J>(c, bx, by, 0, 1, pub_x, pub_y, S.z, S.p[k & 1],
                                                         S.p[(k + 1) & 1], S.x, S.N, S.ntv, 1, S.tv_tc, S.tv_tr,
@@ -174,12 +189,17 @@ __device__ __forceinline__ void run_item(const PSlice &S, int p, int k, int i, u
                                     reinterpret_cast<int *>(psm + quad_smem(S.N)), S.x, S.views, S.row_items,
                                     S.col_items, S.N, S.V, S.B, S.band);
     } else if (p == PH_DUAL) {
-        // residual, Step 3 and the next Step 1 for one view pair per group
-        const int g = tid / FFT_T, vp = i * DUAL_GROUPS + g;
-        if (2 * vp < S.V)
-            dual_fft_body(GroupCtx{tid % FFT_T, FFT_T, 1 + ORB_GROUPS + g}, vp, 0,
-                          reinterpret_cast<float2 *>(psm + (size_t)g * S.dual_smem), S.hhat, S.band, S.nb, S.b, S.mu,
-                          S.mu, S.mubar, S.winv, S.lowdose, S.views, S.scal, S.V, S.B, S.P, S.tw);
+        // residual, Step 3 and the next Step 1: one view pair per transform
+        switch (S.P) {
+        case 64: dual_item<64>(S, i, psm); break;
+        case 128: dual_item<128>(S, i, psm); break;
+        case 256: dual_item<256>(S, i, psm); break;
+        case 512: dual_item<512>(S, i, psm); break;
+        case 1024: dual_item<1024>(S, i, psm); break;
+        case 2048: dual_item<2048>(S, i, psm); break;
+        case 4096: dual_item<4096>(S, i, psm); break;
+        default: dual_item<8192>(S, i, psm); break;
+        }
     } else {
         // after the last iteration: the iteration count, and the result check
         unsigned f = 0;
@@ -304,7 +324,7 @@ ct_status launch_persistent(int n, const ct_geometry *const *geoms, const float 
             S.N = g->n;
             S.V = g->n_views;
             S.B = g->n_bins;
-            S.P = g->n_fft;
+            S.P = g->p_fft;
             S.nb = proj_bands(g->n);
             S.lowdose = prm.mode == CT_LOWDOSE;
             S.al = g->n_bins % 4 == 0;   // workspace buffers are 256-byte aligned
@@ -313,7 +333,6 @@ ct_status launch_persistent(int n, const ct_geometry *const *geoms, const float 
             S.nsl = orbit_slices(g, false);
             S.q16 = (g->n / 2 + ORB_T - 1) / ORB_T;
             S.orb_smem = (int)a16(orbit_smem_bytes());
-            S.dual_smem = (int)a16(dual_fft_smem(g));
             S.ntv = prm.tv_iters > 0 ? prm.tv_iters : 10;
             S.fgp = prm.tv_accel == 1;
             // TV tiles: the batch's tiles together fill the GPU about twice
@@ -334,7 +353,8 @@ ct_status launch_persistent(int n, const ct_geometry *const *geoms, const float 
                 S.qseg = nr <= 2 * nbp;
                 S.n_items[PH_QUAD] = S.qseg ? 2 * nbp : (int)std::min((long long)g->n_sm, nr);
             }
-            S.n_items[PH_DUAL] = ((g->n_views + 1) / 2 + DUAL_GROUPS - 1) / DUAL_GROUPS;
+            const int dual_pairs = PS_THREADS / fft_threads(g->p_fft);   // view pairs per item
+            S.n_items[PH_DUAL] = ((g->n_views + 1) / 2 + dual_pairs - 1) / dual_pairs;
             S.per_iter = 0;
             for (int q = 0; q < PH_N; ++q) {
                 S.pre[q] = S.per_iter;
@@ -359,7 +379,7 @@ ct_status launch_persistent(int n, const ct_geometry *const *geoms, const float 
             S.scal = sb.scal;
             const size_t tv_smem = sizeof(float2) * 2 * PS_TV_PUB * TV_GROUPS;
             smem = std::max({smem, (size_t)ORB_GROUPS * S.orb_smem, tv_smem, quad_smem(g->n) + 16,
-                             (size_t)DUAL_GROUPS * S.dual_smem});
+                             (size_t)dual_pairs * dual_fft_smem(g)});
             n_sm = std::max(n_sm, g->n_sm);
         }
         // queue order: iteration, phase, slice, item

@@ -40,7 +40,7 @@ UL layout(const Geometry *g, int S, int half, int iters, int ntv)
     size_t o = 0;
     L.scal = o;  o += a256(sizeof(double) * S_COUNT);
     L.scal2 = o; o += a256(sizeof(double) * S_COUNT);
-    L.hhat = o;  o += a256(sizeof(float2) * g->n_fft);
+    L.hhat = o;  o += a256(sizeof(float2) * g->p_fft);
     L.winv = o;  o += a256(F * S * I);
     L.ck = o;    o += a256(F * L.ck_stride * (iters + 1));
     L.zk = o;    o += a256(F * S * J * (size_t)std::max(iters, 1));                       // z_k
