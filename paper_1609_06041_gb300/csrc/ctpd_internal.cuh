@@ -181,6 +181,14 @@ struct Block2D {
 __device__ __forceinline__ float2 pk(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+// 1/sqrt(a) by the approximate instruction, subnormal a taken as 0
+__device__ __forceinline__ float rsqrt_ftz(float a)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
 __device__ __forceinline__ float2 psub(float2 a, float2 b)
 {
     unsigned long long A, Bv, D;

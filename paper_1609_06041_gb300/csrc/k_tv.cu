@@ -13,14 +13,15 @@
 // p_out) because neighbouring blocks read the old p in their halos.
 //
 // The held region is 64 columns (lane l owns columns 2l, 2l+1) by up to
-// TV_ROWS rows (warp w owns rows w + 16 j), so tc = 64 - 2H.  Every cell's
-// z, p and x stay in registers for the whole call; left/right neighbours
-// come from the adjacent lane by shuffle, and each phase publishes the one
-// field its vertical neighbours need (x for the dual step, p_y for the
-// divergence) in shared memory.  Outside the image, and where a forward
-// difference does not exist (p_x on the last column, p_y on the last row),
-// p is zero and stays zero: the dual step's factor is 0 there, so the
-// divergence needs no boundary tests.
+// TV_ROWS rows (warp w owns the J rows from w J), so tc = 64 - 2H.  Every
+// cell's z, p and x stay in registers for the whole call; left/right
+// neighbours come from the adjacent lane by shuffle, vertical ones from the
+// thread's own rows and, at the ends of a warp's run of rows, through shared
+// memory (tv_body).  Where a forward difference does not exist (p_x on the
+// last column, p_y on the last row) and just before the first column and
+// row, p is zero and stays zero: the dual step's factor is 0 there, so the
+// divergence needs no boundary tests, and the cells outside the image never
+// reach it.
 #include <algorithm>
 
 #include "body_tv.cuh"
@@ -51,17 +52,16 @@ static TvTiles tv_tiles(int N, int steps, int n_sm, int min_tr, bool even = fals
     return t;
 }
 
-template <bool FGP, bool TRAJ>
+template <bool FGP, bool TRAJ, int J>
 __global__ void __launch_bounds__(TV_THREADS, 1)
 k_tv(const float *__restrict__ z, const float *__restrict__ p_in, float *__restrict__ p_out,
      float *__restrict__ x, int N, int steps, int final_, int tc, int tr, const double *__restrict__ scal,
      float *__restrict__ traj)
 {
-    __shared__ float2 pub_x[(TV_ROWS + 2) * 32];
-    __shared__ float2 pub_y[(TV_ROWS + 2) * 32];
+    __shared__ TvPub pub;
     pdl_wait();
-    tv_body<FGP, TRAJ>(whole_block(), blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z, pub_x, pub_y, z, p_in, p_out, x,
-                       N, steps, final_, tc, tr, scal, traj);
+    tv_body<FGP, TRAJ, J>(whole_block(), blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z, pub, z, p_in, p_out, x, N,
+                          steps, final_, tc, tr, scal, traj);
 }
 
 void tv_tile_shape(int n, int steps, int n_sm, int min_rows, int *tc, int *tr, int *ncb, int *nrb, int rows)
@@ -84,7 +84,17 @@ void launch_tv(const float *z, const float *p_in, float *p_out, float *x,
                                traj != nullptr);
     const dim3 grid(t.ncb, t.nrb, std::max(1, batch));
     counted();
-    auto kern = traj ? k_tv<false, true> : fgp ? k_tv<true, false> : k_tv<false, false>;
+    // rows per warp: as few as hold the region, so that all 16 warps carry a share of it
+    const int rows = t.tr + 2 * tv_halo(steps, traj != nullptr);
+    auto pick = [&](auto k1, auto k2, auto k3, auto k4, auto k5) {
+        return rows <= TV_WARPS ? k1 : rows <= 2 * TV_WARPS ? k2 : rows <= 3 * TV_WARPS ? k3 : rows <= 4 * TV_WARPS ? k4 : k5;
+    };
+    auto kern = traj  ? pick(k_tv<false, true, 1>, k_tv<false, true, 2>, k_tv<false, true, 3>, k_tv<false, true, 4>,
+                             k_tv<false, true, 5>)
+                : fgp ? pick(k_tv<true, false, 1>, k_tv<true, false, 2>, k_tv<true, false, 3>, k_tv<true, false, 4>,
+                             k_tv<true, false, 5>)
+                      : pick(k_tv<false, false, 1>, k_tv<false, false, 2>, k_tv<false, false, 3>, k_tv<false, false, 4>,
+                             k_tv<false, false, 5>);
     launch_kernel(kern, grid, dim3(TV_THREADS), 0, st, z, p_in, p_out, x, n, steps, final_, t.tc, t.tr, scal, traj);
 }
 

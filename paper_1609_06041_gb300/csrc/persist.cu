@@ -57,7 +57,6 @@ constexpr int TV_GROUPS = PS_THREADS / TV_THREADS; // TV tiles per item
 // prox kernel's five, so that its cells fit the 64 registers a thread of a
 // 1024-thread block has (with five they spill), at more halo work
 constexpr int PS_TV_J = 3;
-constexpr int PS_TV_PUB = (TV_WARPS * PS_TV_J + 2) * 32;   // float2 per published field
 static_assert(TV_GROUPS * TV_THREADS == PS_THREADS && QUAD_PG == PG, "whole groups");
 static_assert(1 + ORB_GROUPS + TV_GROUPS <= 16, "named barriers 1..15");
 static_assert(ORB_GROUPS * ORB_TH == PS_THREADS, "whole groups");
@@ -152,18 +151,15 @@ __device__ __forceinline__ void run_item(const PSlice &S, int p, int k, int i, u
         // p[k & 1] and written to p[(k + 1) & 1]
         const int g = tid / TV_THREADS, j = i * TV_GROUPS + g;
         if (j < S.tv_ncb * S.tv_nrb) {
-            float2 *pub_x = reinterpret_cast<float2 *>(psm) + (size_t)g * 2 * PS_TV_PUB;
-            float2 *pub_y = pub_x + PS_TV_PUB;
+            TvPub &pub = reinterpret_cast<TvPub *>(psm)[g];
             const int bx = j % S.tv_ncb, by = j / S.tv_ncb;
             const GroupCtx c{tid % TV_THREADS, TV_THREADS, 1 + ORB_GROUPS + g};
             if (S.fgp)
-                tv_body<true, false, GroupCtx, PS_TV_J>(c, bx, by, 0, 1, pub_x, pub_y, S.z, S.p[k & 1],
-                                                        S.p[(k + 1) & 1], S.x, S.N, S.ntv, 1, S.tv_tc, S.tv_tr,
-                                                        S.scal, nullptr);
+                tv_body<true, false, PS_TV_J>(c, bx, by, 0, 1, pub, S.z, S.p[k & 1], S.p[(k + 1) & 1], S.x, S.N, S.ntv,
+                                              1, S.tv_tc, S.tv_tr, S.scal, nullptr);
             else
-                tv_body<false, false, GroupCtx, PS_TV_J>(c, bx, by, 0, 1, pub_x, pub_y, S.z, S.p[k & 1],
-                                                         S.p[(k + 1) & 1], S.x, S.N, S.ntv, 1, S.tv_tc, S.tv_tr,
-                                                         S.scal, nullptr);
+                tv_body<false, false, PS_TV_J>(c, bx, by, 0, 1, pub, S.z, S.p[k & 1], S.p[(k + 1) & 1], S.x, S.N,
+                                               S.ntv, 1, S.tv_tc, S.tv_tr, S.scal, nullptr);
         }
     } else if (p == PH_QUAD) {
         // band partial sums of A x^{k+1}: item i takes the i-th of the
@@ -377,7 +373,7 @@ ct_status launch_persistent(int n, const ct_geometry *const *geoms, const float 
             S.band = sb.band;
             S.orb = sb.orb;
             S.scal = sb.scal;
-            const size_t tv_smem = sizeof(float2) * 2 * PS_TV_PUB * TV_GROUPS;
+            const size_t tv_smem = sizeof(TvPub) * TV_GROUPS;
             smem = std::max({smem, (size_t)ORB_GROUPS * S.orb_smem, tv_smem, quad_smem(g->n) + 16,
                              (size_t)dual_pairs * dual_fft_smem(g)});
             n_sm = std::max(n_sm, g->n_sm);
