@@ -55,9 +55,9 @@ __device__ __forceinline__ void dft4(float2 &a0, float2 &a1, float2 &a2, float2 
     a3 = make_float2(__fmaf_rn(-s, d.y, t1.x), __fmaf_rn(s, d.x, t1.y));
 }
 
-// FUSE: the multiplication by 1/sqrt 2 and the following addition round once
-// (D in the filters and the dual step); otherwise each rounds (Hhat and the
-// adjoint of the dual step).
+// FUSE: the multiplication by 1/sqrt 2 of w8^3 and the addition after it
+// round once (the filters and the dual step); otherwise each rounds (Hhat and
+// the adjoint of the dual step).
 template <bool FUSE>
 __device__ __forceinline__ float mul_add(float a, float b, float c)
 {
@@ -78,8 +78,8 @@ __device__ __forceinline__ void dft8(float2 *v, float s)
     const float2 u3 = make_float2(__fmaf_rn(s, o3.y, -o3.x), __fmaf_rn(s, o3.x, o3.y));
     v[0] = cadd(e0, o0);
     v[4] = csub(e0, o0);
-    v[1] = make_float2(mul_add<FUSE>(c, u1.x, e1.x), mul_add<FUSE>(c, u1.y, e1.y));
-    v[5] = make_float2(mul_add<FUSE>(-c, u1.x, e1.x), mul_add<FUSE>(-c, u1.y, e1.y));
+    v[1] = make_float2(__fmaf_rn(c, u1.x, e1.x), __fmaf_rn(c, u1.y, e1.y));
+    v[5] = make_float2(__fmaf_rn(-c, u1.x, e1.x), __fmaf_rn(-c, u1.y, e1.y));
     v[2] = make_float2(__fmaf_rn(s, o2.y, e2.x), __fmaf_rn(-s, o2.x, e2.y));
     v[6] = make_float2(__fmaf_rn(-s, o2.y, e2.x), __fmaf_rn(s, o2.x, e2.y));
     v[3] = make_float2(mul_add<FUSE>(c, u3.x, e3.x), mul_add<FUSE>(-c, u3.y, e3.y));
