@@ -103,7 +103,9 @@ void ct_geometry_destroy(ct_geometry *geom);
  * computed).  Five shapes are held by the geometry:
  *   items_per_block  view pairs (v, V-v) sharing one staged band pair in the
  *                    projector, 64 threads each (4..16; 4..12 when
- *                    proj_rows is 4);
+ *                    proj_rows is 4).  The tuner also times other thread
+ *                    counts per item and the built-in rule's own shape,
+ *                    which it keeps without showing them here;
  *   proj_rows        steps a projector thread evaluates per pass of a ray
  *                    walk (2 or 4: more loads in flight, more registers;
  *                    the same sums either way);
@@ -118,15 +120,15 @@ void ct_geometry_destroy(ct_geometry *geom);
  *   proj_form        how the projector's work is cut into blocks (1 or 2):
  *                    1, each block stages one band pair and walks a few
  *                    groups of items_per_block items on it, the grid sized
- *                    by a wave-count model; 2, the work is cut into units
+ *                    by a model of its time; 2, the work is cut into units
  *                    (band pair, item, 64 rays) and each block, with
  *                    64 x items_per_block threads, takes an equal range of
  *                    them, as many blocks as fit on the device at once,
  *                    its warps taking the units of each staged band pair
  *                    from a shared counter.  Both give the same sums.
- * 0 selects the built-in rule (a wave-count model for items_per_block, 2
- * steps per pass, 4 slices, 16 rows; form 2 with 16 items' threads when
- * form 1 would need two waves of blocks or more, else form 1).  The
+ * 0 selects the built-in rule (for the projector a model of the time of
+ * each shape of both forms: 2 steps per pass in form 1, 4 with 12 items'
+ * threads in form 2; 4 slices; 16 rows).  The
  * projector's shapes (items_per_block, proj_rows, proj_form) and tv_rows
  * leave every result bit unchanged; orbit_slices changes the order in
  * which the backprojector's slice sums are added, so results can differ in

@@ -451,6 +451,11 @@ ct_status ct_geometry_create(int n, int n_views, int n_bins, const double *angle
     g->n = n;
     g->n_views = n_views;
     g->n_bins = n_bins;
+    g->proj_plans = proj_plans_create();
+    if (!g->proj_plans) {
+        ct_geometry_destroy(g);
+        return fail(CT_ERR_OOM, "ct_geometry_create: out of host memory");
+    }
     g->n_fft = 1;
     while (g->n_fft < 2 * n_bins) g->n_fft <<= 1;
     g->p_fft = fft_length(n_bins);
@@ -505,16 +510,23 @@ ct_status ct_geometry_create(int n, int n_views, int n_bins, const double *angle
         const double sc = 1.0 / fmax(fabs(c), fabs(s));
         ht[v] = make_float4((float)c, (float)s, (float)sc, (float)(1.0 - 0.5 * sc));
     }
-    // view-pair work items of the projector (default angles only)
+    // work items of the projector: view pairs (v, V - v) at the default angles
     g->vpair = !angles;
-    int2 *hri = new int2[n_views + 1], *hci = new int2[n_views + 1];
+    QuadItem *hri = new QuadItem[n_views + 1], *hci = new QuadItem[n_views + 1];
     g->n_row_items = g->n_col_items = 0;
-    if (g->vpair) {
-        hri[g->n_row_items++] = make_int2(0, -1);
+    auto item = [&](int v, int vp) {
+        const ViewP &P = hv[v];
+        return QuadItem{v, vp, P.stride, P.a, P.m, P.inv_m, {0, 0}};
+    };
+    if (!g->vpair) {
+        // no view mirror among given angles: every view by itself
+        for (int v = 0; v < n_views; ++v) (hv[v].rows ? hri[g->n_row_items++] : hci[g->n_col_items++]) = item(v, -1);
+    } else {
+        hri[g->n_row_items++] = item(0, -1);
         for (int v = 1; v < n_views; ++v) {
-            if (4 * v <= n_views) hri[g->n_row_items++] = make_int2(v, n_views - v);
-            else if (4 * v < 3 * n_views && 2 * v < n_views) hci[g->n_col_items++] = make_int2(v, n_views - v);
-            else if (2 * v == n_views) hci[g->n_col_items++] = make_int2(v, -1);
+            if (4 * v <= n_views) hri[g->n_row_items++] = item(v, n_views - v);
+            else if (4 * v < 3 * n_views && 2 * v < n_views) hci[g->n_col_items++] = item(v, n_views - v);
+            else if (2 * v == n_views) hci[g->n_col_items++] = item(v, -1);
         }
     }
     // twiddles of the frequency-domain D (none above its longest transform)
@@ -531,12 +543,12 @@ ct_status ct_geometry_create(int n, int n_views, int n_bins, const double *angle
     if (e == cudaSuccess) e = cudaMemcpy(g->d_views, hv, sizeof(ViewP) * n_views, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(g->d_row_list, rl, sizeof(int) * n_views, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(g->d_col_list, cl, sizeof(int) * n_views, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&g->d_row_items, sizeof(int2) * (n_views + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&g->d_col_items, sizeof(int2) * (n_views + 1));
+    if (e == cudaSuccess) e = cudaMalloc(&g->d_row_items, sizeof(QuadItem) * (n_views + 1));
+    if (e == cudaSuccess) e = cudaMalloc(&g->d_col_items, sizeof(QuadItem) * (n_views + 1));
     if (e == cudaSuccess && g->n_row_items)
-        e = cudaMemcpy(g->d_row_items, hri, sizeof(int2) * g->n_row_items, cudaMemcpyHostToDevice);
+        e = cudaMemcpy(g->d_row_items, hri, sizeof(QuadItem) * g->n_row_items, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && g->n_col_items)
-        e = cudaMemcpy(g->d_col_items, hci, sizeof(int2) * g->n_col_items, cudaMemcpyHostToDevice);
+        e = cudaMemcpy(g->d_col_items, hci, sizeof(QuadItem) * g->n_col_items, cudaMemcpyHostToDevice);
     delete[] hri;
     delete[] hci;
     delete[] hv;
@@ -577,6 +589,7 @@ void ct_geometry_destroy(ct_geometry *g)
     if (g->d_qbounds) cudaFree(g->d_qbounds);
     eps_cache_free(g);
     graph_cache_free(g);
+    proj_plans_free(g->proj_plans);
     delete[] g->h_angles;
     delete g;
 }

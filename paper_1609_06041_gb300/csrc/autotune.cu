@@ -4,11 +4,13 @@
 // Five shapes are tuned, each by timing every candidate on synthetic data
 // of the geometry's size with CUDA events (one warm-up launch, then the mean
 // of three):
-//   - the projector's view items per block (k_project_quad: 64 threads per
-//     view pair, pg pairs share one staged band pair), pg = 4 .. 16, jointly
-//     with its steps per pass of a ray walk (2, or 4 with pg <= 12) and its
-//     form (one band pair per block, or the work-balanced k_project_qbal
-//     with 8, 12 or 16 items' threads per block);
+//   - the projector's view items per block (k_project_quad: pg items share
+//     one staged band pair), pg = 4 .. 16, jointly with the threads per item
+//     (32 .. 512), its steps per pass of a ray walk (2, or 4 with pg <= 12)
+//     and its form (one band pair per block, or the work-balanced
+//     k_project_qbal with 8, 12 or 16 items' threads per block), and against
+//     the built-in rule's own shape (N a multiple of 32 up to 637 and default
+//     angles; the rule serves elsewhere);
 //   - the backprojector's base-view slices (grid.z), 1 .. 8, for its
 //     cluster form (k_backproject_orbit_cl: the slices' blocks add their
 //     sums through distributed shared memory) and for its slice-image form
@@ -57,8 +59,6 @@ float time_launches(F f, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1)
     return cudaGetLastError() == cudaSuccess ? ms / 3.0f : -1.0f;
 }
 
-bool quad_path(const Geometry *g) { return g->vpair && g->n % 32 == 0 && g->n + 3 <= 640; }
-
 }  // namespace
 
 extern "C" ct_status ct_geometry_get_tuning(const ct_geometry *g, int *items_per_block, int *proj_rows,
@@ -105,10 +105,12 @@ extern "C" ct_status ct_geometry_set_tuning(ct_geometry *g, int items_per_block,
         return CT_ERR_ARG;
     }
     g->tune_pg = items_per_block;
+    g->tune_tpi = 0;
     g->tune_qrows = proj_rows;
     g->tune_orb = g->tune_orb_si = orbit_slices;
     g->tune_tv = tv_rows;
     g->tune_qbal = proj_form;
+    proj_plans_clear(g);
     graph_cache_clear(g);
     return CT_OK;
 }
@@ -123,7 +125,7 @@ extern "C" ct_status ct_geometry_autotune(ct_geometry *g, int batch, void *strea
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const int N = g->n;
     const size_t J = (size_t)N * N, I = (size_t)g->n_views * g->n_bins;
-    const int old_pg = g->tune_pg, old_rows = g->tune_qrows, old_orb = g->tune_orb, old_tv = g->tune_tv;
+    const int old_pg = g->tune_pg, old_tpi = g->tune_tpi, old_rows = g->tune_qrows, old_orb = g->tune_orb, old_tv = g->tune_tv;
     const int old_orb_si = g->tune_orb_si;
     const int old_qbal = g->tune_qbal;
     Buffers buf;
@@ -158,23 +160,33 @@ extern "C" ct_status ct_geometry_autotune(ct_geometry *g, int batch, void *strea
 
     ct_status result = CT_OK;
     float t;
-    if (quad_path(g)) {
+    if (g->vpair && g->n % 32 == 0 && g->n + 3 <= 640) {   // elsewhere the built-in rule serves
         float best = -1.0f;
-        int best_pg = 0, best_rows = 0, best_form = 1;
+        int best_pg = 0, best_tpi = 0, best_rows = 0, best_form = 1;
+        static const int tpis[] = {32, 64, 96, 128, 192, 256, 384, 512};
         for (int form = 1; form <= 2 && result == CT_OK; ++form) {
             for (int rows = 2; rows <= 4 && result == CT_OK; rows += 2) {
                 for (int pg = form == 1 ? 4 : 8; pg <= (rows == 4 ? 12 : 16) && result == CT_OK;
                      pg += form == 1 ? 1 : 4) {
-                    g->tune_pg = pg;
-                    g->tune_qrows = rows;
-                    g->tune_qbal = form;
-                    t = time_launches([&] { launch_project_bands(g, x, band, batch, st); }, st, e0, e1);
-                    if (t < 0.0f) result = CT_ERR_CUDA;
-                    else if (best < 0.0f || t < best) {
-                        best = t;
-                        best_pg = pg;
-                        best_rows = rows;
-                        best_form = form;
+                    for (int tpi : tpis) {
+                        if (result != CT_OK || (form == 2 && tpi != 64)) continue;
+                        if (form == 1 && (pg * tpi < 64 || pg * tpi > (rows == 4 ? 768 : 1024) ||
+                                          (tpi > 64 && tpi >= (g->n_bins + 1) / 2 + 64)))
+                            continue;
+                        g->tune_pg = pg;
+                        g->tune_tpi = form == 1 ? tpi : 0;
+                        g->tune_qrows = rows;
+                        g->tune_qbal = form;
+                        proj_plans_clear(g);
+                        t = time_launches([&] { launch_project_bands(g, x, band, batch, st); }, st, e0, e1);
+                        if (t < 0.0f) result = CT_ERR_CUDA;
+                        else if (best < 0.0f || t < best) {
+                            best = t;
+                            best_pg = pg;
+                            best_tpi = g->tune_tpi;
+                            best_rows = rows;
+                            best_form = form;
+                        }
                     }
                 }
             }
@@ -182,6 +194,15 @@ extern "C" ct_status ct_geometry_autotune(ct_geometry *g, int batch, void *strea
         g->tune_pg = best_pg;
         g->tune_qrows = best_rows;
         g->tune_qbal = best_form;
+        // the built-in rule's shape, which may share a band pair among fewer items
+        g->tune_tpi = -1;
+        proj_plans_clear(g);
+        if (result == CT_OK) {
+            t = time_launches([&] { launch_project_bands(g, x, band, batch, st); }, st, e0, e1);
+            if (t < 0.0f) result = CT_ERR_CUDA;
+            else if (t > best) g->tune_tpi = best_tpi;
+        }
+        proj_plans_clear(g);
         // the balanced form's unit ranges for one image, from measured block times
         if (result == CT_OK) result = qbal_balance(g, x, band, st);
     }
@@ -227,11 +248,13 @@ extern "C" ct_status ct_geometry_autotune(ct_geometry *g, int batch, void *strea
     graph_cache_clear(g);
     if (result != CT_OK) {
         g->tune_pg = old_pg;
+        g->tune_tpi = old_tpi;
         g->tune_qrows = old_rows;
         g->tune_orb = old_orb;
         g->tune_orb_si = old_orb_si;
         g->tune_tv = old_tv;
         g->tune_qbal = old_qbal;
+        proj_plans_clear(g);
         cudaError_t le = cudaGetLastError();
         set_error("ct_geometry_autotune: %s", cudaGetErrorString(le));
         return result;

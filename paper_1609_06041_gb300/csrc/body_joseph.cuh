@@ -1,5 +1,4 @@
-// body_joseph.cuh -- bodies of the Joseph projector (view pairs and mirrored
-// bands) and of the rotation-orbit backprojector, shared by their kernels
+// body_joseph.cuh -- bodies of the mirrored Joseph projector and of the rotation-orbit backprojector, shared by their kernels
 // (k_joseph.cu) and the persistent batched kernel (persist.cu).  Each body
 // takes its block index and shared memory explicitly and runs on the
 // threads of a context (a whole block or a group of a persistent block).
@@ -35,24 +34,37 @@ __device__ __forceinline__ void step_range(float q, float m, float inv_m, float 
     hi = min(s_hi, (int)ceilf(smax) + 1);
 }
 
-// Shared memory of the view-pair projector's block at image side N.
-__host__ __device__ __forceinline__ size_t quad_smem(int N) { return sizeof(float2) * (size_t)2 * MR * ((N + 3) | 1); }
+// Shared memory of the mirrored projector's staged band pair at image side
+// N: float4 entries (one per step and pair), or raw (float2 pixel pairs).
+__host__ __device__ __forceinline__ size_t quad_smem(int N, bool raw = false)
+{
+    return raw ? sizeof(float2) * (size_t)MR * ((N + 4) | 1) : sizeof(float4) * (size_t)MR * ((N + 3) | 1);
+}
+// Band pairs of N image lines: pair bp holds the lines s0 .. s0 + 15, s0 = 16
+// bp, of the first half (the middle line of an odd N included) and their
+// mirrors N-1-s.
+__host__ __device__ __forceinline__ int quad_bands(int N) { return (N + 2 * MR - 1) / (2 * MR); }
 
 // ---------------------------------------------------------------------
-// Forward projection with the detector mirror and the view mirror (default
-// angles t_v = v pi / V).  View V-v is view v reflected in the image's
-// vertical axis: its a and m are those of view v with the signs a row view
-// (a -> -a, m -> -m) or a column view (m -> -m) gets from t -> pi - t.
-// For a row view that puts ray d of view V-v at coordinate N-1-u on the
-// same row; for a column view ray d of view V-v meets column N-1-c where
-// ray d of view v meets column c, i.e. the other band's line.  Either way
-// the reflected sample sits at pair N-2-i0 of a staged line with weight
-// -g: one evaluation of (u', g) at (d, s) yields four samples, two of view
-// v (bands A, B as in k_project_mirror) and two of view V-v:
+// Forward projection with the detector mirror and, at the default angles t_v
+// = v pi / V, the view mirror.  Ray B-1-d meets step N-1-s at the mirrored
+// coordinate N-1-u of ray d at step s, so a block that stages band A (steps
+// s0 .. s0+15) and band B (steps N-1-s0-15 .. N-1-s0) turned by 180 degrees
+// (step and pair order reversed) reads, for one evaluation of (u', g) at (d,
+// s), the sample of ray d in band A and of ray B-1-d in band B at the same
+// shared offset.  View V-v is view v reflected in the image's vertical axis:
+// its a and m are those of view v with the signs a row view (a -> -a, m ->
+// -m) or a column view (m -> -m) gets from t -> pi - t.  For a row view that
+// puts ray d of view V-v at coordinate N-1-u on the same row; for a column
+// view ray d of view V-v meets column N-1-c where ray d of view v meets
+// column c, i.e. the other band's line.  Either way the reflected sample
+// sits at pair N-2-i0 of a staged line with weight -g: one evaluation yields
+// four samples, two of view v and two of view V-v:
 //     rows:    A[i0] (v, d)  B[i0] (v, B-1-d)  A[N-2-i0] (V-v, d)    B[N-2-i0] (V-v, B-1-d)
 //     columns: A[i0] (v, d)  B[i0] (v, B-1-d)  A[N-2-i0] (V-v, B-1-d) B[N-2-i0] (V-v, d)
-// Work items are view pairs (v, V-v) and the views without a partner
-// (v = 0, and v = V/2 for even V), pg items per block, 64 threads per item.
+// Work items are view pairs (v, V-v) and the views without a partner (v = 0,
+// v = V/2 for even V; at custom angles every view), pg items per block, tpi
+// threads per item.
 // ---------------------------------------------------------------------
 // Walks one ray through the staged steps lo..hi (ROWS steps per pass, one
 // coordinate evaluation per step) and returns its four sums: band A and
@@ -61,16 +73,39 @@ __host__ __device__ __forceinline__ size_t quad_smem(int N) { return sizeof(floa
 // serves both bands and the two bands' samples are one packed two-wide
 // FMA, mid + g delta, into a pair accumulator (the reflected pair with -g).
 // The coordinates of two steps are evaluated as one packed pair as well.
+// RAW: the staged entries are the bands' pixels (A_i, B_i) instead, and a
+// sample reads the entries i and i + 1: with mid = (a + b) / 2 and delta =
+// b - a formed on the fly, mid + g delta is rounded exactly as from float4
+// entries, at half the shared memory and two more packed operations.
 // A pass of ROWS = 4 is two passes of ROWS = 2 whose loads are issued
 // together: the same coordinates (u' = (s - h) m + q for even steps,
 // (s - 1 - h) m + (q + m) for odd ones), the same two accumulators (even
 // and odd steps) updated in the same order and the same tail, so both
 // give the same sums to the bit.
-template <bool PAIR, int ROWS>
-__device__ __forceinline__ float4 quad_walk(const float4 *__restrict__ Q, int SP, float q, float m, int lo, int hi,
+template <bool PAIR, int ROWS, bool RAW>
+__device__ __forceinline__ float4 quad_walk(const void *Qv, int SP, float q, float m, int lo, int hi,
                                             int s0, float h, unsigned top)
 {
     static_assert(ROWS == 2 || ROWS == 4, "steps are evaluated in pairs, one or two pairs per pass");
+    // one sample's entry: (mid A, mid B, delta A, delta B), or raw pixels (A_i, B_i, A_i+1, B_i+1)
+    auto entry = [&](int k) {
+        if constexpr (RAW) {
+            const float2 *R = static_cast<const float2 *>(Qv);
+            const float2 x0 = R[k], x1 = R[k + 1];
+            return make_float4(x0.x, x0.y, x1.x, x1.y);
+        } else {
+            return static_cast<const float4 *>(Qv)[k];
+        }
+    };
+    // acc + mid + g delta: acc + mid rounds, then the FMA
+    auto sample = [&](float2 acc, const float4 &p, float g) {
+        if constexpr (RAW) {
+            const float2 x0 = pk(p.x, p.y), x1 = pk(p.z, p.w);
+            return pfma(pk(g, g), psub(x1, x0), pfma(pk(0.5f, 0.5f), padd(x0, x1), acc));
+        } else {
+            return pfma(pk(g, g), pk(p.z, p.w), padd(acc, pk(p.x, p.y)));
+        }
+    };
     const float2 qk = pk(q, __fmaf_rn(1.0f, m, q));   // q + k m for the steps k = 0, 1 of a pair
     const float2 mm = pk(m, m), bias = pk(JOSEPH_BIAS, JOSEPH_BIAS);
     float spk = (float)lo - h;
@@ -85,19 +120,19 @@ __device__ __forceinline__ float4 quad_walk(const float4 *__restrict__ Q, int SP
         g = psub(up, tb);
         const unsigned i0 = min((unsigned)(__float_as_int(t.x) - (JOSEPH_BIAS_BITS - 2)), top);
         const unsigned i1 = min((unsigned)(__float_as_int(t.y) - (JOSEPH_BIAS_BITS - 2)), top);
-        p0 = Q[rr + (int)i0];
-        p1 = Q[rr + SP + (int)i1];
+        p0 = entry(rr + (int)i0);
+        p1 = entry(rr + SP + (int)i1);
         if (PAIR) {
-            r0 = Q[rr + (int)(top - i0)];
-            r1 = Q[rr + SP + (int)(top - i1)];
+            r0 = entry(rr + (int)(top - i0));
+            r1 = entry(rr + SP + (int)(top - i1));
         }
     };
     auto pair_add = [&](const float4 &p0, const float4 &p1, const float4 &r0, const float4 &r1, float2 g) {
-        ab[0] = pfma(pk(g.x, g.x), pk(p0.z, p0.w), padd(ab[0], pk(p0.x, p0.y)));
-        ab[1] = pfma(pk(g.y, g.y), pk(p1.z, p1.w), padd(ab[1], pk(p1.x, p1.y)));
+        ab[0] = sample(ab[0], p0, g.x);
+        ab[1] = sample(ab[1], p1, g.y);
         if (PAIR) {
-            ce[0] = pfma(pk(-g.x, -g.x), pk(r0.z, r0.w), padd(ce[0], pk(r0.x, r0.y)));
-            ce[1] = pfma(pk(-g.y, -g.y), pk(r1.z, r1.w), padd(ce[1], pk(r1.x, r1.y)));
+            ce[0] = sample(ce[0], r0, -g.x);
+            ce[1] = sample(ce[1], r1, -g.y);
         }
     };
     int s = lo;
@@ -127,130 +162,106 @@ __device__ __forceinline__ float4 quad_walk(const float4 *__restrict__ Q, int SP
         const float t = __fadd_rn(up, JOSEPH_BIAS);
         const unsigned i = min((unsigned)(__float_as_int(t) - (JOSEPH_BIAS_BITS - 2)), top);
         const float g = __fsub_rn(up, __fsub_rn(t, JOSEPH_BIAS));
-        const float4 pv = Q[ridx + (int)i];
-        ab[0] = pfma(pk(g, g), pk(pv.z, pv.w), padd(ab[0], pk(pv.x, pv.y)));
-        if (PAIR) {
-            const float4 rv = Q[ridx + (int)(top - i)];
-            ce[0] = pfma(pk(-g, -g), pk(rv.z, rv.w), padd(ce[0], pk(rv.x, rv.y)));
-        }
+        ab[0] = sample(ab[0], entry(ridx + (int)i), g);
+        if (PAIR) ce[0] = sample(ce[0], entry(ridx + (int)(top - i)), -g);
     }
     ab[0] = padd(ab[0], ab[1]);
     ce[0] = padd(ce[0], ce[1]);
     return make_float4(ab[0].x, ab[0].y, ce[0].x, ce[0].y);
 }
 
-// Stages band pair s0 of image img into Q: pair i (stored at i + 2) of step
-// t holds (A mid, B mid, A delta, B delta), band A the image line s0 + t
-// and band B the line N-1-s0-t read backwards (image value at N-1-i); the
-// lines are image rows (rows) or columns.  Runs on the threads of c and
-// ends without a barrier.
-template <bool DEEP, class Ctx>
-__device__ __forceinline__ void quad_stage(const Ctx &c, float4 *Q, const float *img, int N, int s0, bool rows)
+// Stages band pair s0 of image img: entry i of step t (stored at i + 2,
+// -2 <= i <= N) holds (A mid, B mid, A delta, B delta), band A the image line
+// s0 + t and band B the line N-1-s0-t read backwards (image value at N-1-i);
+// the lines are image rows (rows) or columns.  RAW: the pixels (A_i, B_i),
+// i <= N + 1.  Steps past the first half hold zeros, as does band B on the
+// middle line of an odd N (band A has it).  Every pixel is loaded once and
+// its neighbour comes by shuffle; a thread issues the loads of four entries
+// before it stores any, and the index arithmetic has no division (staging a
+// 512-line segment took 170 instructions per 32 entries with both, about 30
+// now).  Runs on the threads of c and ends without a barrier.
+template <bool RAW, class Ctx>
+__device__ __forceinline__ void quad_stage(const Ctx &c, void *Qv, const float *img, int N, int s0, bool rows)
 {
-    static_assert(MR == 16, "column staging: a warp's lanes take the 16 steps of two pairs");
-    const int CW = N + 3, SP = CW | 1;
-    const int tid = c.tid(), nth = c.nth();
-    // one thread forms both bands' pairs of (t, i) and stores them as one float4
-    const int lx = tid & 31, nw = nth >> 5;
-    if constexpr (DEEP) {
-        // each thread issues the loads of SU pairs before it stores any, so
-        // that SU L2 round trips overlap (grids of few blocks, whose threads
-        // each stage many pairs)
-        constexpr int SU = 4;
-        float a0[SU], a1[SU], b0[SU], b1[SU];
-        if (rows) {
-            const int nch = (CW + 31) >> 5, nc = MR * nch;
-            for (int c0 = tid >> 5; c0 < nc; c0 += SU * nw) {
+    static_assert(MR == 16, "a warp's lanes take the 16 steps of two entries (columns)");
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int SU = 4;
+    const int CW = RAW ? N + 4 : N + 3, SP = CW | 1;
+    const int lane = c.tid() & 31, nw = c.nth() >> 5;
+    const int na = min(MR, (N + 1) / 2 - s0), nb = min(MR, N / 2 - s0);   // lines of bands A and B
+    const int last = N * N - 1;                                            // N N < 2^31
+    auto store = [&](int at, float a0, float a1, float b0, float b1) {
+        if constexpr (RAW) static_cast<float2 *>(Qv)[at] = make_float2(a0, b0);
+        else
+            static_cast<float4 *>(Qv)[at] = make_float4(0.5f * (a0 + a1), 0.5f * (b0 + b1), a1 - a0, b1 - b0);
+    };
+    if (rows) {
+        // a warp takes a chunk of 31 entries (RAW: 32) of one step; lane 31 loads the last entry's neighbour
+        constexpr int CH = RAW ? 32 : 31;
+        const int nc = MR * ((CW + CH - 1) / CH);
+        for (int k0 = c.tid() >> 5; k0 < nc; k0 += SU * nw) {
+            float av[SU], bv[SU];
 #pragma unroll
-                for (int u = 0; u < SU; ++u) {
-                    const int ch = c0 + u * nw;
-                    const int t = ch / nch, ii = ((ch - t * nch) << 5) + lx;
-                    const bool ok = ch < nc && ii < CW;
-                    const int i = ii - 2;
-                    const float *ra = img + (size_t)(s0 + t) * N, *rb = img + (size_t)(N - 1 - s0 - t) * N;
-                    a0[u] = (ok && i >= 0 && i < N) ? ra[i] : 0.0f;
-                    a1[u] = (ok && i + 1 >= 0 && i + 1 < N) ? ra[i + 1] : 0.0f;
-                    b0[u] = (ok && N - 1 - i >= 0 && N - 1 - i < N) ? rb[N - 1 - i] : 0.0f;
-                    b1[u] = (ok && N - 2 - i >= 0 && N - 2 - i < N) ? rb[N - 2 - i] : 0.0f;
-                }
-#pragma unroll
-                for (int u = 0; u < SU; ++u) {
-                    const int ch = c0 + u * nw;
-                    const int t = ch / nch, ii = ((ch - t * nch) << 5) + lx;
-                    if (ch < nc && ii < CW)
-                        Q[t * SP + ii] = make_float4(0.5f * (a0[u] + a1[u]), 0.5f * (b0[u] + b1[u]), a1[u] - a0[u],
-                                                     b1[u] - b0[u]);
-                }
+            for (int u = 0; u < SU; ++u) {
+                const int k = k0 + u * nw, t = k & (MR - 1), i = (k >> 4) * CH + lane - 2, o = (s0 + t) * N + i;
+                const bool in = k < nc && (unsigned)i < (unsigned)N;
+                av[u] = in && t < na ? img[o] : 0.0f;
+                bv[u] = in && t < nb ? img[last - o] : 0.0f;
             }
-        } else {
-            const int t = lx & 15;
-            const float *ia = img + (s0 + t), *ib = img + (N - 1 - s0 - t);   // columns of bands A, B
-            const int nc = (CW + 1) >> 1;
-            for (int c0 = tid >> 5; c0 < nc; c0 += SU * nw) {
 #pragma unroll
-                for (int u = 0; u < SU; ++u) {
-                    const int ii = 2 * (c0 + u * nw) + (lx >> 4);
-                    const bool ok = c0 + u * nw < nc && ii < CW;
-                    const int i = ii - 2;   // rows i, i + 1 (band A), N-1-i, N-2-i (band B); N N < 2^31
-                    a0[u] = (ok && i >= 0 && i < N) ? ia[i * N] : 0.0f;
-                    a1[u] = (ok && i + 1 >= 0 && i + 1 < N) ? ia[(i + 1) * N] : 0.0f;
-                    b0[u] = (ok && N - 1 - i >= 0 && N - 1 - i < N) ? ib[(N - 1 - i) * N] : 0.0f;
-                    b1[u] = (ok && N - 2 - i >= 0 && N - 2 - i < N) ? ib[(N - 2 - i) * N] : 0.0f;
+            for (int u = 0; u < SU; ++u) {
+                const int k = k0 + u * nw, t = k & (MR - 1), ii = (k >> 4) * CH + lane;
+                float a1 = 0.0f, b1 = 0.0f;
+                if (!RAW) {
+                    a1 = __shfl_down_sync(FULL, av[u], 1);
+                    b1 = __shfl_down_sync(FULL, bv[u], 1);
                 }
-#pragma unroll
-                for (int u = 0; u < SU; ++u) {
-                    const int ii = 2 * (c0 + u * nw) + (lx >> 4);
-                    if (c0 + u * nw < nc && ii < CW)
-                        Q[t * SP + ii] = make_float4(0.5f * (a0[u] + a1[u]), 0.5f * (b0[u] + b1[u]), a1[u] - a0[u],
-                                                     b1[u] - b0[u]);
-                }
-            }
-        }
-    } else if (rows) {
-        // warps take 32-pair chunks of the 16 steps, lanes neighbouring pairs
-        const int nch = (CW + 31) >> 5;
-        for (int ch = tid >> 5; ch < MR * nch; ch += nw) {
-            const int t = ch / nch, ii = ((ch - t * nch) << 5) + lx;
-            if (ii < CW) {
-                const int i = ii - 2;
-                const float *ra = img + (size_t)(s0 + t) * N, *rb = img + (size_t)(N - 1 - s0 - t) * N;
-                const float a0 = (i >= 0 && i < N) ? ra[i] : 0.0f;
-                const float a1 = (i + 1 >= 0 && i + 1 < N) ? ra[i + 1] : 0.0f;
-                const float b0 = (N - 1 - i >= 0 && N - 1 - i < N) ? rb[N - 1 - i] : 0.0f;
-                const float b1 = (N - 2 - i >= 0 && N - 2 - i < N) ? rb[N - 2 - i] : 0.0f;
-                Q[(size_t)t * SP + ii] = make_float4(0.5f * (a0 + a1), 0.5f * (b0 + b1), a1 - a0, b1 - b0);
+                if (k < nc && lane < CH && ii < CW) store(t * SP + ii, av[u], a1, bv[u], b1);
             }
         }
     } else {
-        // lanes take the 16 steps (columns) of two neighbouring pairs:
-        // 64-byte row segments in, conflict-free float4 stores (odd SP)
-        const int t = lx & 15, ca = s0 + t, cb = N - 1 - s0 - t;
-        for (int ch = tid >> 5; 2 * ch < CW; ch += nw) {
-            const int ii = 2 * ch + (lx >> 4);
-            if (ii < CW) {
-                const int i = ii - 2;
-                const float a0 = (i >= 0 && i < N) ? img[(size_t)i * N + ca] : 0.0f;
-                const float a1 = (i + 1 >= 0 && i + 1 < N) ? img[(size_t)(i + 1) * N + ca] : 0.0f;
-                const float b0 = (N - 1 - i >= 0 && N - 1 - i < N) ? img[(size_t)(N - 1 - i) * N + cb] : 0.0f;
-                const float b1 = (N - 2 - i >= 0 && N - 2 - i < N) ? img[(size_t)(N - 2 - i) * N + cb] : 0.0f;
-                Q[(size_t)t * SP + ii] = make_float4(0.5f * (a0 + a1), 0.5f * (b0 + b1), a1 - a0, b1 - b0);
+        // a warp takes 2 SU neighbouring entries: the lane's step t, entries e0 + 2 u + (lane >> 4) (64-byte row
+        // segments in, conflict-free stores: odd SP)
+        const int t = lane & 15, hf = lane >> 4;
+        const bool ina = t < na, inb = t < nb;
+        for (int e0 = 2 * SU * (c.tid() >> 5); e0 < CW; e0 += 2 * SU * nw) {
+            constexpr int SL = RAW ? SU : SU + 1;   // one more for the last entry's neighbour
+            float av[SL], bv[SL];
+#pragma unroll
+            for (int u = 0; u < SL; ++u) {
+                const int i = e0 + 2 * u + hf - 2, o = i * N + s0 + t;
+                const bool in = (unsigned)i < (unsigned)N && (u < SU || hf == 0);
+                av[u] = in && ina ? img[o] : 0.0f;
+                bv[u] = in && inb ? img[last - o] : 0.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < SU; ++u) {
+                const int ii = e0 + 2 * u + hf;
+                float a1 = 0.0f, b1 = 0.0f;
+                if constexpr (!RAW) {   // the other half-warp's entry after this one
+                    a1 = __shfl_xor_sync(FULL, hf ? av[u] : av[u + 1], 16);
+                    b1 = __shfl_xor_sync(FULL, hf ? bv[u] : bv[u + 1], 16);
+                }
+                if (ii < CW) store(t * SP + ii, av[u], a1, bv[u], b1);
             }
         }
     }
 }
 
 // Walks ray position idx of view-pair item (v, vp) through the staged band
-// pair (steps s0 .. s0 + MR - 1) and stores its band sums into the partial
+// pair (steps s0 .. s1) and stores its band sums into the partial
 // slot out (V x B): ray d and its detector mirror B-1-d of view v and, for
 // vp >= 0, of view vp.  Positions map to rays in whole blocks of 8 cs
 // positions, where the eight lanes of a quarter warp take rays cs apart,
 // spreading their 16-byte loads over the bank groups; the last partial
 // block maps to itself.
-template <int ROWS>
-__device__ __forceinline__ void quad_position(const float4 *Q, int SP, float a, float m, float inv_m, int cs, int v,
-                                              int vp, bool rows, int idx, int npair, int N, int B, int s0, float h,
-                                              float hq, unsigned top, float *out)
+template <int ROWS, bool RAW>
+__device__ __forceinline__ void quad_position(const void *Q, int SP, const QuadItem &it, bool rows, int idx, int npair,
+                                              int N, int B, int s0, int s1, float h, float hq, unsigned top,
+                                              float *out)
 {
+    const float a = it.a, m = it.m, inv_m = it.inv_m;
+    const int cs = it.stride, v = it.v, vp = it.vp;
     int d = idx;
     {
         const int blk = 8 * cs, b = idx / blk, r = idx - b * blk;
@@ -264,9 +275,9 @@ __device__ __forceinline__ void quad_position(const float4 *Q, int SP, float a, 
         const int dd = which == 0 ? d : dm;
         const float q = joseph_q(joseph_dp(dd, B), a, hq);
         int lo, hi;
-        step_range(q, m, inv_m, h, -2.5f, (float)N + 0.5f, s0, s0 + MR - 1, lo, hi);
-        const float4 r = vp >= 0 ? quad_walk<true, ROWS>(Q, SP, q, m, lo, hi, s0, h, top)
-                                 : quad_walk<false, ROWS>(Q, SP, q, m, lo, hi, s0, h, top);
+        step_range(q, m, inv_m, h, -2.5f, (float)N + 0.5f, s0, s1, lo, hi);
+        const float4 r = vp >= 0 ? quad_walk<true, ROWS, RAW>(Q, SP, q, m, lo, hi, s0, h, top)
+                                 : quad_walk<false, ROWS, RAW>(Q, SP, q, m, lo, hi, s0, h, top);
         ov[which] += r.x;
         ov[1 - which] += r.y;
         if (rows) {
@@ -296,18 +307,18 @@ __device__ __forceinline__ void quad_position(const float4 *Q, int SP, float a, 
 }
 
 // Body of block (bx, by, bz) of a grid of nbp band pairs: smraw holds
-// quad_smem(N) bytes, the block's c.nth() = 64 pg threads.  The block
+// quad_smem(N) bytes, the block's c.nth() = tpi pg threads.  The block
 // stages its band pair once and then walks gpb groups of pg view-pair
 // items of one class (rows or columns) one after the other, so that the
 // staging is spread over gpb groups.
-template <int ROWS, bool DEEP, class Ctx>
+template <int ROWS, class Ctx>
 __device__ __forceinline__ void quad_body(const Ctx &c, int bx, int by, int bz, int nbp, unsigned char *smraw,
-                                          const float *x, const ViewP *views, const int2 *row_items, int n_row,
-                                          const int2 *col_items, int n_col, int N, int V, int B, int pg, int gpb,
+                                          const float *x, const QuadItem *row_items, int n_row,
+                                          const QuadItem *col_items, int n_col, int N, int V, int B, int pg, int gpb, int tpi,
                                           float *partial)
 {
     const int SP = (N + 3) | 1;
-    float4 *Q = reinterpret_cast<float4 *>(smraw);   // [step][pair]: band A pair, band B pair
+    void *Q = smraw;   // [step][pair]: band A pair, band B pair
 
     const int bp = bx;
     const int row_groups = (n_row + pg - 1) / pg, col_groups = (n_col + pg - 1) / pg;
@@ -315,53 +326,63 @@ __device__ __forceinline__ void quad_body(const Ctx &c, int bx, int by, int bz, 
     const bool rows = by < row_blocks;
     const int grp0 = (rows ? by : by - row_blocks) * gpb;
     const int ngrp = min(gpb, (rows ? row_groups : col_groups) - grp0);
-    const int2 *list = rows ? row_items : col_items;
+    const QuadItem *list = rows ? row_items : col_items;
     const int nl = rows ? n_row : n_col;
     float *out = partial + ((size_t)bz * nbp + bp) * V * B;
-    const int s0 = bp * MR;
+    const int s0 = bp * MR, s1 = min(s0 + MR, (N + 1) / 2) - 1;
     const float h = joseph_h(N), hq = joseph_hq(N);
     const int tid = c.tid();
 
-    quad_stage<DEEP>(c, Q, x + (size_t)bz * N * N, N, s0, rows);
+    // the first item's constants arrive while the band pair is staged
+    const int vi = tid / tpi;
+    QuadItem it = list[min(grp0 * pg + vi, nl - 1)];
+    quad_stage<false>(c, Q, x + (size_t)bz * N * N, N, s0, rows);
     c.sync();
     const int npair = (B + 1) / 2;
     const unsigned top = (unsigned)(N + 2);
-    const int vi = tid >> 6;
     for (int gi = 0; gi < ngrp; ++gi) {
         const int grp = grp0 + gi;
         if (vi >= min(pg, nl - grp * pg)) break;
-        const int2 it = list[grp * pg + vi];
-        const ViewP &vw = views[it.x];
-        const float a = vw.a, m = vw.m, inv_m = vw.inv_m;
-        const int cs = vw.stride;
-        for (int idx = tid & 63; idx < npair; idx += 64)
-            quad_position<ROWS>(Q, SP, a, m, inv_m, cs, it.x, it.y, rows, idx, npair, N, B, s0, h, hq, top, out);
+        if (gi > 0) it = list[grp * pg + vi];
+        for (int idx = tid - vi * tpi; idx < npair; idx += tpi)
+            quad_position<ROWS, false>(Q, SP, it, rows, idx, npair, N, B, s0, s1, h, hq, top,
+                                       out);
     }
 }
 
 // Work-balanced form of the same projection.  The work of a batch is cut
-// into units (slice, class, band pair, item, chunk of 64 ray positions),
-// ordered so that the units of one staged band pair (a segment) are
-// consecutive; each block takes the equal range [u0, u1) of units, stages
+// into units (slice, class, band pair, item, chunk of 32 or 64 ray
+// positions), ordered so that the units of one staged band pair (a segment)
+// are consecutive; each block takes the range [u0, u1) of units, stages
 // each segment the range touches once, and its warps take the segment's
 // units one at a time from a shared counter.  Blocks thus carry equal work
 // whatever the number of items, and a block holds as many warps as its
 // registers allow.  The sums are those of quad_body, unit for unit.
 struct QuadUnits {
-    int nch;        // 64-position chunks per item
+    int upl;        // ray positions of a unit per lane (1 or 2)
+    int nch;        // chunks of 32 upl positions per item
     int u_rows;     // units of one row-class segment: n_row items x nch
     int u_cols;     // units of one column-class segment
-    long long u_z;  // units per slice: nbp (u_rows + u_cols)
+    long long u_z;  // units per slice: band pairs x (u_rows + u_cols)
 };
+__host__ __device__ __forceinline__ QuadUnits quad_units(int N, int B, int n_row, int n_col, int upl)
+{
+    QuadUnits U;
+    U.upl = upl;
+    U.nch = ((B + 1) / 2 + 32 * upl - 1) / (32 * upl);
+    U.u_rows = n_row * U.nch;
+    U.u_cols = n_col * U.nch;
+    U.u_z = (long long)quad_bands(N) * (U.u_rows + U.u_cols);
+    return U;
+}
 
-template <int ROWS, bool DEEP, class Ctx>
+template <int ROWS, bool RAW, class Ctx>
 __device__ __forceinline__ void quad_balanced_body(const Ctx &c, long long u0, long long u1, const QuadUnits &U,
                                                    unsigned char *smraw, int *next, const float *x,
-                                                   const ViewP *views, const int2 *row_items,
-                                                   const int2 *col_items, int N, int V, int B, float *partial)
+                                                   const QuadItem *row_items, const QuadItem *col_items, int N,
+                                                   int V, int B, float *partial)
 {
-    const int SP = (N + 3) | 1, nbp = N / (2 * MR);
-    float4 *Q = reinterpret_cast<float4 *>(smraw);
+    const int SP = RAW ? (N + 4) | 1 : (N + 3) | 1, nbp = quad_bands(N);
     const float h = joseph_h(N), hq = joseph_hq(N);
     const int npair = (B + 1) / 2;
     const unsigned top = (unsigned)(N + 2);
@@ -370,36 +391,33 @@ __device__ __forceinline__ void quad_balanced_body(const Ctx &c, long long u0, l
     long long u = u0;
     while (u < u1) {
         // the segment of unit u: slice z, class, band pair bp
-        const long long z = u / U.u_z, r = u - z * U.u_z;
+        const long long z = u < U.u_z ? 0 : u / U.u_z, r = u - z * U.u_z;
         const bool rows = r < rows_all;
         const long long r2 = rows ? r : r - rows_all;
         const int per = rows ? U.u_rows : U.u_cols;
-        const int bp = (int)(r2 / per);
+        const int bp = r2 < 0x7fffffffLL ? (int)((unsigned)r2 / (unsigned)per) : (int)(r2 / per);
         const long long seg0 = u - (r2 - (long long)bp * per);
         const long long e = min(u1, seg0 + per);
-        const int s0 = bp * MR;
-        quad_stage<DEEP>(c, Q, x + (size_t)z * N * N, N, s0, rows);
-        if (tid == 0) *next = (int)(u - seg0);
-        c.sync();
-        const int2 *list = rows ? row_items : col_items;
+        const int s0 = bp * MR, s1 = min(s0 + MR, (N + 1) / 2) - 1;
+        const QuadItem *list = rows ? row_items : col_items;
         float *out = partial + ((size_t)z * nbp + bp) * V * B;
         const int n_units = (int)(e - seg0);
+        quad_stage<RAW>(c, smraw, x + (size_t)z * N * N, N, s0, rows);
+        if (tid == 0) *next = (int)(u - seg0);
+        c.sync();
         for (;;) {
             int w = 0;
             if (lane == 0) w = atomicAdd(next, 1);
             w = __shfl_sync(0xffffffffu, w, 0);
             if (w >= n_units) break;
-            const int item = w / U.nch, chunk = w - item * U.nch;
-            const int2 it = list[item];
-            const ViewP &vw = views[it.x];
-            const float a = vw.a, m = vw.m, inv_m = vw.inv_m;
-            const int cs = vw.stride;
+            const int item = (int)((unsigned)w / (unsigned)U.nch), chunk = w - item * U.nch;
+            const QuadItem it = list[item];
 #pragma unroll 1
-            for (int k = 0; k < 2; ++k) {
-                const int idx = chunk * 64 + k * 32 + lane;
+            for (int k = 0; k < U.upl; ++k) {
+                const int idx = (chunk * U.upl + k) * 32 + lane;
                 if (idx < npair)
-                    quad_position<ROWS>(Q, SP, a, m, inv_m, cs, it.x, it.y, rows, idx, npair, N, B, s0, h, hq, top,
-                                        out);
+                    quad_position<ROWS, RAW>(smraw, SP, it, rows, idx, npair, N, B, s0, s1, h,
+                                             hq, top, out);
             }
         }
         c.sync();

@@ -27,7 +27,15 @@ struct ViewP {
     float inv_m;   // 1/m (0 when m = 0), for the ray->step range
     int rows;      // 1: steps along rows; 0: along columns
     int three;     // 1: a pixel's candidate-ray window can hold three rays
-    int stride;    // view-pair projector: rays of one quarter warp are `stride` apart (bank spread)
+    int stride;    // mirrored projector: rays of one quarter warp are `stride` apart (bank spread)
+};
+
+// Work item of the mirrored projector: views (v, V-v), or one view (vp = -1),
+// with view v's constants (one 32-byte load).
+struct __align__(16) QuadItem {
+    int v, vp, stride;
+    float a, m, inv_m;
+    int pad[2];
 };
 
 struct Geometry {
@@ -44,11 +52,13 @@ struct Geometry {
     int orbit;            // default angles with V and N even: A^T by rotation orbits
     int vpair;            // default angles: A by view pairs (v, V-v)
     int n_row_items, n_col_items;
-    int2 *d_row_items;    // device, (v, V-v) for 1 <= v <= V/4, and (0, -1)
-    int2 *d_col_items;    // device, (v, V-v) for V/4 < v < V/2, and (V/2, -1) for even V
+    QuadItem *d_row_items;   // device, (v, V-v) for 1 <= v <= V/4, and (0, -1); custom angles: (v, -1) each
+    QuadItem *d_col_items;   // device, (v, V-v) for V/4 < v < V/2, and (V/2, -1) for even V; custom: (v, -1) each
     int n_sm;             // multiprocessors of the device
     // launch shapes chosen by ct_geometry_autotune (0: the built-in rule)
     int tune_pg;          // projector view items per block (4..16; 4..12 with 4 steps per pass)
+    int tune_tpi;         // projector threads per view item of the band-pair form (0: 64 with tune_pg set, else
+                          // the rule; -1: the tuner found the rule's own shape best)
     int tune_qrows;       // projector steps per pass of a ray walk (2 or 4)
     int tune_orb;         // A^T orbit base-view slices (1..8), slices added in a cluster
     int tune_orb_si;      // the same for the slice-image form (solves side by side, the persistent kernel)
@@ -62,6 +72,7 @@ struct Geometry {
     unsigned long long *d_qtimes;   // device: the tuner's per-block start and end times while it measures
     double *h_angles;     // host copy
     void *eps_cache;      // eigenbases of D for the error-tolerant form (eps.cu)
+    void *proj_plans;     // the projector's launch shapes by batch size (k_joseph.cu)
     void *graph_cache;    // instantiated CUDA graphs of repeated solves (api.cu)
 };
 
@@ -352,7 +363,7 @@ ct_status launch_persistent(int n, const ct_geometry *const *geoms, const float 
 // (cluster false) of its slice-image form
 int orbit_slices(const Geometry *g, bool cluster = true);
 size_t orbit_smem_bytes();                      // shared memory of one orbit block
-bool quad_ok(const Geometry *g);                // the view-pair projector serves this geometry
+bool quad_ok(const Geometry *g);                // the mirrored projector serves this geometry (N <= about 1800)
 // TV prox tiles of one image spread over n_sm blocks (k_tv.cu's rule)
 void tv_tile_shape(int n, int steps, int n_sm, int min_rows, int *tc, int *tr, int *ncb, int *nrb, int rows = 0);
 size_t dual_fft_smem(const Geometry *g);       // one exchange buffer of the dual update's transform
@@ -377,7 +388,14 @@ void launch_trace(const Geometry *g, const float *partial, const float *b, const
 // partial holds n_bands(N) x V x B floats per image.
 constexpr int PROJ_R = 32;
 inline int proj_bands(int n) { return (n + PROJ_R - 1) / PROJ_R; }
-void launch_project_bands(const Geometry *g, const float *x, float *partial, int batch, cudaStream_t st);
+// plain: one unmirrored 32-line band per block whatever the geometry (the
+// unrolled form on sides that are not a multiple of 32).
+void launch_project_bands(const Geometry *g, const float *x, float *partial, int batch, cudaStream_t st,
+                          bool plain = false);
+// The geometry's cache of projector launch shapes; clear it when a tuning changes.
+void *proj_plans_create();
+void proj_plans_free(void *p);
+void proj_plans_clear(Geometry *g);
 // out = scale_v * sum_b partial[b]   (mode 0), minus b and winv*mu (mode 1),
 // minus b (mode 2).
 void launch_band_reduce(const Geometry *g, const float *partial, float *out, int mode,

@@ -3,6 +3,8 @@
 // deterministic (fixed summation orders, no atomics).
 #include <algorithm>
 #include <cmath>
+#include <mutex>
+#include <new>
 #include <vector>
 
 #include <cooperative_groups.h>
@@ -13,7 +15,9 @@ namespace ctpd {
 
 
 // =====================================================================
-// Forward projection.
+// Forward projection without mirrors: images of over about 1800 pixels a
+// side (a mirrored band pair does not fit in shared memory) and the unrolled
+// form on sides that are not a multiple of 32.
 // A block owns a band of PROJ_R consecutive steps (rows for row-stepping
 // views, columns for column-stepping views) and a group of PG views of one
 // class.  It stages the band in shared memory as interpolation pairs
@@ -30,6 +34,7 @@ constexpr int PROJ_CW = 640;   // pairs per staged band row
 
 static int proj_cw(int n) { return (n + 3) < PROJ_CW ? (n + 3) : PROJ_CW; }
 static int proj_stride(int n) { return proj_cw(n) | 1; }   // odd: spreads smem banks
+constexpr int QUAD_SMEM_MAX = 227 * 1024;   // shared memory a block may have
 static size_t proj_smem(int n) { return sizeof(float2) * (size_t)PROJ_R * proj_stride(n) + sizeof(ViewP) * PG + 64; }
 
 __device__ __forceinline__ int d_proj_cw(int n) { return (n + 3) < PROJ_CW ? (n + 3) : PROJ_CW; }
@@ -158,156 +163,18 @@ k_project_bands(const float *__restrict__ x, const ViewP *__restrict__ views,
     }
 }
 
-// ---------------------------------------------------------------------
-// Forward projection with the detector mirror (N a multiple of 32, one
-// staged pass).  Ray B-1-d meets step N-1-s at the mirrored coordinate
-// N-1-u of ray d at step s, so a block staging band A (steps s0 .. s0+15)
-// and band B (steps N-1-s0-15 .. N-1-s0) turned by 180 degrees (step and
-// pair order reversed) reads, for one evaluation of (u', g) at (d, s), the
-// sample of ray d in band A and of ray B-1-d in band B at the same shared
-// offset.  A thread takes the ray pair (d, B-1-d) and walks both rays; each
-// ray's partial covers both bands.  Partial slots: N/32 per image, like the
-// plain kernel's 32-step bands.
-// ---------------------------------------------------------------------
-static_assert(PG * 64 == PT, "one view of the group per 64 threads");
-static_assert(2 * MR == 32, "staging maps 32 lines (two bands) to 32 thread rows");
-
-__global__ void __launch_bounds__(PT)
-k_project_mirror(const float *__restrict__ x, const ViewP *__restrict__ views,
-                 const int *__restrict__ row_list, int n_row, const int *__restrict__ col_list, int n_col,
-                 int N, int V, int B, float *__restrict__ partial)
-{
-    extern __shared__ __align__(16) unsigned char smraw[];
-    const int CW = N + 3, SP = CW | 1;
-    float2 *PA = reinterpret_cast<float2 *>(smraw);
-    float2 *PB = PA + (size_t)MR * SP;
-    ViewP *sv = reinterpret_cast<ViewP *>(PB + (size_t)MR * SP);
-    int *svi = reinterpret_cast<int *>(sv + PG);
-
-    const int bp = blockIdx.x, nbp = gridDim.x;
-    const int row_groups = (n_row + PG - 1) / PG;
-    const bool rows = (int)blockIdx.y < row_groups;
-    const int grp = rows ? blockIdx.y : blockIdx.y - row_groups;
-    const int *list = rows ? row_list : col_list;
-    const int nl = rows ? n_row : n_col;
-    const int nv = min(PG, nl - grp * PG);
-    const float *img = x + (size_t)blockIdx.z * N * N;
-    float *out = partial + ((size_t)blockIdx.z * nbp + bp) * V * B;
-    const int s0 = bp * MR;
-    const float h = joseph_h(N), hq = joseph_hq(N);
-    const int tid = threadIdx.x;
-
-    if (tid < nv) {
-        svi[tid] = list[grp * PG + tid];
-        sv[tid] = views[svi[tid]];
-    }
-    // pair i (stored at i + 2) of step t: band A the image line s0 + t, band B
-    // the line N-1-s0-t read backwards (image value at N-1-i).  Threads as
-    // 32 x 32: rows class -> lanes along the line; column class -> lanes
-    // across the 32 lines of both bands (coalesced image rows).
-    {
-        const int lx = tid & 31, ly = tid >> 5;
-        if (rows) {
-            const int band = ly >= MR, t = ly - band * MR;
-            const int line = band == 0 ? s0 + t : N - 1 - s0 - t;
-            const float *rowp = img + (size_t)line * N;
-            float2 *dst = (band == 0 ? PA : PB) + t * SP;
-            for (int ii = lx; ii < CW; ii += 32) {
-                const int i = ii - 2;
-                const int ia = band == 0 ? i : N - 1 - i, ib = band == 0 ? i + 1 : N - 2 - i;
-                const float a = (ia >= 0 && ia < N) ? rowp[ia] : 0.0f;
-                const float b = (ib >= 0 && ib < N) ? rowp[ib] : 0.0f;
-                dst[ii] = make_float2(0.5f * (a + b), b - a);
-            }
-        } else {
-            const int band = lx >= MR, t = lx - band * MR;
-            const int line = band == 0 ? s0 + t : N - 1 - s0 - t;
-            float2 *dst = (band == 0 ? PA : PB) + t * SP;
-            for (int ii = ly; ii < CW; ii += 32) {
-                const int i = ii - 2;
-                const int ia = band == 0 ? i : N - 1 - i, ib = band == 0 ? i + 1 : N - 2 - i;
-                const float a = (ia >= 0 && ia < N) ? img[(size_t)ia * N + line] : 0.0f;
-                const float b = (ib >= 0 && ib < N) ? img[(size_t)ib * N + line] : 0.0f;
-                dst[ii] = make_float2(0.5f * (a + b), b - a);
-            }
-        }
-    }
-    __syncthreads();
-    const int npair = (B + 1) / 2;
-    const unsigned top = (unsigned)(N + 2);
-    // thread -> view tid / 64 of the group, ray pairs (tid % 64) + 64 j
-    const int vi = tid >> 6;
-    if (vi >= nv) return;
-    for (int d = tid & 63; d < npair; d += 64) {
-        const int dm = B - 1 - d;
-        const float a = sv[vi].a, m = sv[vi].m, inv_m = sv[vi].inv_m;
-        float accA[2] = {0.0f, 0.0f}, accB[2] = {0.0f, 0.0f};   // [0]: ray d, [1]: ray dm
-#pragma unroll
-        for (int which = 0; which < 2; ++which) {
-            if (which == 1 && dm == d) break;
-            const int dd = which == 0 ? d : dm;
-            const float q = joseph_q(joseph_dp(dd, B), a, hq);
-            int lo, hi;
-            step_range(q, m, inv_m, h, -2.5f, (float)N + 0.5f, s0, s0 + MR - 1, lo, hi);
-            const float qu1 = __fadd_rn(q, m);
-            float spk = (float)lo - h;
-            int ridx = (lo - s0) * SP;
-            float a0 = 0.0f, a1 = 0.0f, b0 = 0.0f, b1 = 0.0f;
-            int s = lo;
-            for (; s + 1 <= hi; s += 2) {
-                const float up0 = joseph_u(spk, m, q), up1 = joseph_u(spk, m, qu1);
-                const float t0 = __fadd_rn(up0, JOSEPH_BIAS), t1 = __fadd_rn(up1, JOSEPH_BIAS);
-                const unsigned i0 = min((unsigned)(__float_as_int(t0) - (JOSEPH_BIAS_BITS - 2)), top);
-                const unsigned i1 = min((unsigned)(__float_as_int(t1) - (JOSEPH_BIAS_BITS - 2)), top);
-                const float g0 = __fsub_rn(up0, __fsub_rn(t0, JOSEPH_BIAS));
-                const float g1 = __fsub_rn(up1, __fsub_rn(t1, JOSEPH_BIAS));
-                const float2 pa0 = PA[ridx + (int)i0], pb0 = PB[ridx + (int)i0];
-                const float2 pa1 = PA[ridx + SP + (int)i1], pb1 = PB[ridx + SP + (int)i1];
-                a0 += __fmaf_rn(g0, pa0.y, pa0.x);
-                b0 += __fmaf_rn(g0, pb0.y, pb0.x);
-                a1 += __fmaf_rn(g1, pa1.y, pa1.x);
-                b1 += __fmaf_rn(g1, pb1.y, pb1.x);
-                spk = __fadd_rn(spk, 2.0f);
-                ridx += 2 * SP;
-            }
-            if (s <= hi) {
-                const float up0 = joseph_u(spk, m, q);
-                const float t0 = __fadd_rn(up0, JOSEPH_BIAS);
-                const unsigned i0 = min((unsigned)(__float_as_int(t0) - (JOSEPH_BIAS_BITS - 2)), top);
-                const float g0 = __fsub_rn(up0, __fsub_rn(t0, JOSEPH_BIAS));
-                const float2 pa0 = PA[ridx + (int)i0], pb0 = PB[ridx + (int)i0];
-                a0 += __fmaf_rn(g0, pa0.y, pa0.x);
-                b0 += __fmaf_rn(g0, pb0.y, pb0.x);
-            }
-            // band A sample of ray dd; band B sample of its mirror ray
-            accA[which] = a0 + a1;
-            accB[1 - which] = b0 + b1;
-        }
-        float *o = out + (size_t)svi[vi] * B;
-        if (dm == d) {
-            o[d] = accA[0] + accB[1];
-        } else {
-            o[d] = accA[0] + accB[0];
-            o[dm] = accA[1] + accB[1];
-        }
-    }
-}
-
-// ROWS = 2: up to 16 items (1024 threads, 64 registers); ROWS = 4: more
-// loads in flight per thread, up to 12 items (768 threads, 85 registers).
-// DEEP: the staging issues the loads of four pairs per thread before it
-// stores them, for grids of few blocks whose threads each stage many pairs
-// (few views); otherwise one pair at a time (fewer registers).
-template <int ROWS, bool DEEP>
+// ROWS = 2: up to 1024 threads (64 registers); ROWS = 4: more loads in flight
+// per thread, up to 768 threads (85 registers).
+template <int ROWS>
 __global__ void __launch_bounds__(ROWS == 2 ? 1024 : 768)
-k_project_quad(const float *__restrict__ x, const ViewP *__restrict__ views,
-               const int2 *__restrict__ row_items, int n_row, const int2 *__restrict__ col_items, int n_col,
-               int N, int V, int B, int pg, int gpb, float *__restrict__ partial)
+k_project_quad(const float *__restrict__ x, const QuadItem *__restrict__ row_items, int n_row,
+               const QuadItem *__restrict__ col_items, int n_col, int N, int V, int B, int pg, int gpb, int tpi,
+               float *__restrict__ partial)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     pdl_wait();
-    quad_body<ROWS, DEEP>(whole_block(), blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, smraw, x, views, row_items,
-                          n_row, col_items, n_col, N, V, B, pg, gpb, partial);
+    quad_body<ROWS>(whole_block(), blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, smraw, x, row_items, n_row,
+                    col_items, n_col, N, V, B, pg, gpb, tpi, partial);
 }
 
 // The work-balanced form: block b takes units [total b / nb, total (b+1) / nb)
@@ -324,11 +191,11 @@ __device__ __forceinline__ unsigned long long global_time()
 // before the wait for the previous kernel); else equal unit counts.
 // times (optional): block b writes its start and end times (ns) to
 // times[2b], times[2b+1].
-template <int ROWS, bool DEEP>
+template <int ROWS, bool RAW>
 __global__ void __launch_bounds__(ROWS == 2 ? 1024 : 768)
-k_project_qbal(const float *__restrict__ x, const ViewP *__restrict__ views, const int2 *__restrict__ row_items,
-               const int2 *__restrict__ col_items, int N, int V, int B, QuadUnits U, long long total,
-               const long long *__restrict__ bounds, unsigned long long *__restrict__ times,
+k_project_qbal(const float *__restrict__ x, const QuadItem *__restrict__ row_items,
+               const QuadItem *__restrict__ col_items, int N, int V, int B, QuadUnits U, long long total,
+               long long share, const long long *__restrict__ bounds, unsigned long long *__restrict__ times,
                float *__restrict__ partial)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -338,13 +205,14 @@ k_project_qbal(const float *__restrict__ x, const ViewP *__restrict__ views, con
         u0 = min(max(bounds[blockIdx.x], 0LL), total);
         u1 = min(max(bounds[blockIdx.x + 1], u0), total);
     } else {
-        u0 = total * blockIdx.x / nb;
-        u1 = total * (blockIdx.x + 1) / nb;
+        // equal counts, the first blocks one more
+        u0 = (long long)blockIdx.x * share + min((long long)blockIdx.x, total - share * nb);
+        u1 = u0 + share + (blockIdx.x < total - share * nb ? 1 : 0);
     }
     pdl_wait();
     const unsigned long long t0 = times ? global_time() : 0ull;
-    quad_balanced_body<ROWS, DEEP>(whole_block(), u0, u1, U, smraw, reinterpret_cast<int *>(smraw + quad_smem(N)),
-                                   x, views, row_items, col_items, N, V, B, partial);
+    quad_balanced_body<ROWS, RAW>(whole_block(), u0, u1, U, smraw, reinterpret_cast<int *>(smraw + quad_smem(N, RAW)),
+                                  x, row_items, col_items, N, V, B, partial);
     if (times) {
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -354,111 +222,212 @@ k_project_qbal(const float *__restrict__ x, const ViewP *__restrict__ views, con
     }
 }
 
-// Launch shape of k_project_quad: items per group (pg, 64 threads each) and
-// groups per block (gpb, walked one after the other on one staged band
-// pair), by the fewest waves of blocks (one block per SM, shared memory)
-// times the per-block work, staging counted as three items.  pg_fixed > 0
-// fixes pg (the tuner's choice) and picks gpb for it.
-static void quad_shape(const Geometry *g, int batch, int max_pg, int pg_fixed, int *pg_out, int *gpb_out)
+// Launch shapes of the mirrored projector.
+//
+// k_project_quad: a block stages one band pair and walks gpb groups of pg
+// items, tpi threads an item.  k_project_qbal: about one block an SM, each
+// with an equal range of units.  The built-in rule takes the shape with the
+// least modelled time, in SM cycles:
+//   staging a band pair: 45 instructions per 32 entries, and a round trip of
+//     700 cycles per four entries of a thread;
+//   walking a ray position (both of its rays): 800 instructions per warp
+//     (450 for an item of one view), a chain of 1100 cycles;
+//   an SM issues 2.4 instructions a cycle for its resident blocks.
+// The constants are fitted to a sweep of (pg, tpi) over 16 geometries, 32^2
+// to 512^2, 12 to 720 views.  What it is for: with 64 threads an item, few-view
+// grids left most warp slots empty and each thread six positions of serial
+// walk (512^2 / 32 views: 80 blocks of 8 warps 13.6 us, 144 blocks of 24 warps
+// 8.4 us; 256^2 / 90: 8.9 and 6.8 us).  Launches in a graph, warm cache, with
+// the staging of quad_stage: 512^2 / 32 views 18.1 -> 8.3 us, 64^2 / 90 5.4 ->
+// 4.3, 256^2 / 180 11.9 -> 9.5, 512^2 / 720 69.9 -> 65.3.  Sides that are not a
+// multiple of 32, over 637, or custom angles took unmirrored or unpaired
+// kernels before: 1024^2 / 720 718 -> 313 us, 900^2 / 300 258 -> 82, 2 x 333^2
+// / 101 27.2 -> 16.8, 512^2 / 720 golden angles 97.8 -> 77.7.
+struct QuadShape {
+    int pg, gpb, tpi;
+    double cost;
+};
+static double stage_cycles(int N, int warps, double share)
 {
-    const long bands = g->n / (2 * MR);
-    long best_cost = -1;
-    for (int pg = pg_fixed > 0 ? pg_fixed : 4; pg <= (pg_fixed > 0 ? pg_fixed : max_pg); ++pg) {
+    const double entries = MR * ((N + 33) / 32);
+    return entries * 45.0 * share / 2.4 + ceil(entries / (4.0 * warps)) * 700.0;
+}
+static double walk_instr(const Geometry *g) { return g->vpair ? 800.0 : 450.0; }
+
+// the projector's settings in force: all by the rule when the tuner found the rule's shape best
+struct ProjSettings {
+    int pg, tpi, rows, form;
+};
+static ProjSettings settings(const Geometry *g)
+{
+    if (g->tune_tpi < 0) return ProjSettings{0, 0, 0, 0};
+    return ProjSettings{g->tune_pg, g->tune_tpi, g->tune_qrows, g->tune_qbal};
+}
+
+static QuadShape quad_shape(const Geometry *g, int batch, int rows4)
+{
+    const ProjSettings t = settings(g);
+    const int N = g->n, npair = (g->n_bins + 1) / 2, bands = quad_bands(N);
+    const int max_threads = rows4 ? 768 : 1024;
+    const int by_smem = std::max(1, QUAD_SMEM_MAX / (int)(quad_smem(N) + 1024));
+    static const int tpis[] = {32, 64, 96, 128, 192, 256, 384, 512};
+    QuadShape best{0, 1, 64, -1.0};
+    const int pg_fix = t.pg;
+    for (int pg = pg_fix > 0 ? pg_fix : 1; pg <= (pg_fix > 0 ? pg_fix : PG); ++pg) {
         const long rg = (g->n_row_items + pg - 1) / pg, cg = (g->n_col_items + pg - 1) / pg;
-        for (int gpb = 1; gpb <= 8; ++gpb) {
-            const long blocks = bands * ((rg + gpb - 1) / gpb + (cg + gpb - 1) / gpb) * batch;
-            const long cost = ((blocks + g->n_sm - 1) / g->n_sm) * ((long)gpb * pg + 3);
-            if (best_cost < 0 || cost < best_cost) {
-                best_cost = cost;
-                *pg_out = pg;
-                *gpb_out = gpb;
+        for (int tpi : tpis) {
+            if (t.tpi > 0 ? tpi != t.tpi : pg_fix > 0 && tpi != 64) continue;
+            const int threads = pg * tpi;
+            if (threads > max_threads || threads < 64 || (tpi > 64 && tpi >= npair + 64)) continue;
+            const int occ = std::max(1, std::min(by_smem, max_threads / threads));
+            for (int gpb = 1; gpb <= 8; ++gpb) {
+                const long blocks = bands * ((rg + gpb - 1) / gpb + (cg + gpb - 1) / gpb) * (long)batch;
+                const double share = (double)std::min<long>(occ, (blocks + g->n_sm - 1) / g->n_sm);
+                const double waves = ceil((double)blocks / ((double)g->n_sm * occ));
+                const double walk = gpb * pg * (double)((npair + 31) / 32) * walk_instr(g) * share / 2.4 +
+                                    gpb * (double)((npair + tpi - 1) / tpi) * 1100.0;
+                const double cost = waves * (stage_cycles(N, threads / 32, share) + walk);
+                if (best.cost < 0.0 || cost < best.cost) best = QuadShape{pg, gpb, tpi, cost};
+                if (rg <= gpb && cg <= gpb) break;
             }
         }
     }
+    return best;
 }
 
 // Launch shape of the work-balanced form: as many blocks as fit on the
 // device at once (fewer when the work would leave a warp under two units).
+// Four steps a pass and 12 items' threads unless set (512^2 / 720 views: 64.6
+// us, against 66.5 with two steps and 16 items' threads).
 struct QbalShape {
     QuadUnits U;
     long long total;
-    int rows4, pgb, threads, blocks, key;
+    int rows4, raw, pgb, threads, blocks, key;
     size_t smem;
+    double cost;
 };
+using QbalKernel = decltype(&k_project_qbal<2, false>);
+static QbalKernel qbal_kernel(const QbalShape &q)
+{
+    return q.rows4 ? (q.raw ? k_project_qbal<4, true> : k_project_qbal<4, false>)
+                   : (q.raw ? k_project_qbal<2, true> : k_project_qbal<2, false>);
+}
+static bool quad_raw(const Geometry *g) { return quad_smem(g->n) + 16 > (size_t)QUAD_SMEM_MAX; }
 static QbalShape qbal_shape(const Geometry *g, int batch)
 {
     QbalShape q;
+    const ProjSettings t = settings(g);
     const int N = g->n;
-    q.rows4 = g->tune_qrows == 4;
+    q.rows4 = t.rows == 4 || (t.rows == 0 && t.pg <= 12);
+    q.raw = quad_raw(g);
     const int max_pg = q.rows4 ? 12 : PG;
-    q.pgb = g->tune_pg > 0 ? std::min(g->tune_pg, max_pg) : max_pg;
+    q.pgb = t.pg > 0 ? std::min(t.pg, max_pg) : max_pg;
     q.threads = q.pgb * 64;
-    q.key = 64 * q.rows4 + q.pgb;
-    const int npair = (g->n_bins + 1) / 2, nch = (npair + 63) / 64;
-    q.U.nch = nch;
-    q.U.u_rows = g->n_row_items * nch;
-    q.U.u_cols = g->n_col_items * nch;
-    q.U.u_z = (long long)(N / (2 * MR)) * (q.U.u_rows + q.U.u_cols);
-    q.total = q.U.u_z * batch;
-    q.smem = quad_smem(N) + 16;
-    auto kern = q.rows4 ? k_project_qbal<4, true> : k_project_qbal<2, true>;
+    q.smem = quad_smem(N, q.raw) + 16;
     // blocks per SM, queried once per (steps per pass, items) for the geometry
     int &occ_slot = const_cast<Geometry *>(g)->qbal_occ[q.rows4][q.pgb];
     int occ = occ_slot;
     if (occ < 1) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, q.threads, q.smem) != cudaSuccess || occ < 1)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, qbal_kernel(q), q.threads, q.smem) != cudaSuccess ||
+            occ < 1)
             occ = 1;
         occ_slot = occ;
     }
+    // units of 64 positions, or of 32 when a warp would take fewer than eight of the former
+    q.U = quad_units(N, g->n_bins, g->n_row_items, g->n_col_items, 2);
+    if (q.U.u_z * batch < (long long)g->n_sm * occ * q.pgb * 2 * 8)
+        q.U = quad_units(N, g->n_bins, g->n_row_items, g->n_col_items, 1);
+    q.total = q.U.u_z * batch;
+    q.key = (q.U.upl * 2 + q.rows4) * 64 + q.pgb;
     const long long by_work = (q.total + 4 * q.pgb - 1) / (4 * q.pgb);   // two units per warp
     q.blocks = (int)std::max(1LL, std::min((long long)g->n_sm * occ, by_work));
+    const double share = std::min<double>(occ, ceil((double)q.blocks / g->n_sm));
+    const double segs = 1.0 + (double)(2 * quad_bands(N)) * batch / q.blocks;   // segments a block's range touches
+    q.cost = segs * stage_cycles(N, q.pgb * 2, share) +
+             (double)q.total / q.blocks * q.U.upl * walk_instr(g) * share / 2.4 + 2.0 * q.U.upl * 1100.0;
     return q;
 }
 
-void launch_project_bands(const Geometry *g, const float *x, float *partial, int batch, cudaStream_t st)
+// The mirrored projector's launch for one batch size, kept in the geometry
+// (the shape model is too slow for every call) until its tuning changes.
+struct ProjPlan {
+    int batch = 0, balanced, rows4;
+    QuadShape quad;
+    QbalShape qbal;
+};
+struct ProjPlans {
+    std::mutex mu;
+    ProjPlan p[4];
+    int next = 0;
+};
+static ProjPlan make_plan(const Geometry *g, int batch)
+{
+    ProjPlan p;
+    p.batch = batch;
+    const ProjSettings t = settings(g);
+    p.rows4 = t.rows == 4;
+    p.qbal = qbal_shape(g, batch);
+    p.balanced = quad_raw(g) || t.form == 2;
+    // The factor is fitted: without it the rule took the balanced form for 4 x
+    // 384^2 / 90 views (27.4 us against 25.3), 512^2 / 90 (17.2, 15.0) and 4 x
+    // 512^2 / 32 (21.5, 18.3); with it, it still takes it for 512^2 / 720 (65.3
+    // us against 66.5) and 512^2 / 360.
+    if (!p.balanced) {
+        p.quad = quad_shape(g, batch, p.rows4);
+        p.balanced = p.quad.cost < 0.0 || (t.form == 0 && 1.16 * p.qbal.cost < p.quad.cost);
+    }
+    return p;
+}
+static ProjPlan proj_plan(const Geometry *g, int batch)
+{
+    ProjPlans &c = *static_cast<ProjPlans *>(g->proj_plans);
+    std::lock_guard<std::mutex> lock(c.mu);
+    for (const ProjPlan &p : c.p)
+        if (p.batch == batch) return p;
+    ProjPlan &p = c.p[c.next];
+    c.next = (c.next + 1) % 4;
+    p = make_plan(g, batch);
+    return p;
+}
+void *proj_plans_create() { return new (std::nothrow) ProjPlans; }
+void proj_plans_free(void *p) { delete static_cast<ProjPlans *>(p); }
+void proj_plans_clear(Geometry *g)
+{
+    ProjPlans &c = *static_cast<ProjPlans *>(g->proj_plans);
+    std::lock_guard<std::mutex> lock(c.mu);
+    for (ProjPlan &p : c.p) p.batch = 0;
+}
+
+void launch_project_bands(const Geometry *g, const float *x, float *partial, int batch, cudaStream_t st, bool plain)
 {
     const int N = g->n;
-    dim3 grd(proj_bands(N), (g->n_row + PG - 1) / PG + (g->n_col + PG - 1) / PG, batch);
-    const size_t smem = proj_smem(N);
     counted();
-    if (g->vpair && N % (2 * MR) == 0 && N + 3 <= PROJ_CW) {
-        // view pairs and two mirrored 16-step bands per block: N/32 partial slots
-        const int rows4 = g->tune_qrows == 4;
-        const int max_pg = rows4 ? 12 : PG;
-        int pg = 0, gpb = 1;
-        quad_shape(g, batch, max_pg, g->tune_pg > 0 ? std::min(g->tune_pg, max_pg) : 0, &pg, &gpb);
-        const int rg = (g->n_row_items + pg - 1) / pg, cg = (g->n_col_items + pg - 1) / pg;
-        const int blocks_y = (rg + gpb - 1) / gpb + (cg + gpb - 1) / gpb;
-        const dim3 grd2(N / (2 * MR), blocks_y, batch);
-        const long static_blocks = (long)grd2.x * grd2.y * grd2.z;
-        // the built-in rule takes the work-balanced form when one band pair
-        // per block would need two waves of blocks or more
-        if (g->tune_qbal == 2 || (g->tune_qbal == 0 && static_blocks >= 2L * g->n_sm)) {
-            const QbalShape q = qbal_shape(g, batch);
-            auto kern = q.rows4 ? k_project_qbal<4, true> : k_project_qbal<2, true>;
+    if (quad_ok(g) && !plain) {
+        // mirrored 16-step bands: ceil(N/32) partial slots
+        const ProjPlan p = proj_plan(g, batch);
+        if (p.balanced) {
+            const QbalShape &q = p.qbal;
             // the tuner's measured-balance ranges, for the launch they were made for
             const long long *bounds =
                 batch == 1 && g->d_qbounds && g->qbounds_nb > 0 && g->qbounds_nb == q.blocks && g->qbounds_key == q.key
                     ? g->d_qbounds
                     : nullptr;
-            launch_kernel(kern, dim3(q.blocks), dim3(q.threads), q.smem, st, x, g->d_views, g->d_row_items,
-                          g->d_col_items, N, g->n_views, g->n_bins, q.U, q.total, bounds, g->d_qtimes, partial);
+            launch_kernel(qbal_kernel(q), dim3(q.blocks), dim3(q.threads), q.smem, st, x, g->d_row_items,
+                          g->d_col_items, N, g->n_views, g->n_bins, q.U, q.total, q.total / q.blocks, bounds,
+                          g->d_qtimes, partial);
             return;
         }
-        const size_t smem2 = quad_smem(N);
-        // few blocks (few views): each thread stages many pairs, so issue their loads four at a time
-        const bool deep = static_blocks < 2L * g->n_sm;
-        auto kern = rows4 ? (deep ? k_project_quad<4, true> : k_project_quad<4, false>)
-                          : (deep ? k_project_quad<2, true> : k_project_quad<2, false>);
-        launch_kernel(kern, grd2, dim3(pg * 64), smem2, st, x, g->d_views, g->d_row_items, g->n_row_items,
-                      g->d_col_items, g->n_col_items, N, g->n_views, g->n_bins, pg, gpb, partial);
-    } else if (N % (2 * MR) == 0 && N + 3 <= PROJ_CW) {
-        // two mirrored 16-step bands per block: N/32 partial slots, as below
-        dim3 grd2(N / (2 * MR), grd.y, batch);
-        const size_t smem2 = sizeof(float2) * (size_t)2 * MR * ((N + 3) | 1) + sizeof(ViewP) * PG + 64;
-        k_project_mirror<<<grd2, PT, smem2, st>>>(x, g->d_views, g->d_row_list, g->n_row, g->d_col_list, g->n_col,
-                                                 N, g->n_views, g->n_bins, partial);
-    } else if (N + 3 <= PROJ_CW)
+        const QuadShape &q = p.quad;
+        const int rg = (g->n_row_items + q.pg - 1) / q.pg, cg = (g->n_col_items + q.pg - 1) / q.pg;
+        const dim3 grd(quad_bands(N), (rg + q.gpb - 1) / q.gpb + (cg + q.gpb - 1) / q.gpb, batch);
+        launch_kernel(p.rows4 ? k_project_quad<4> : k_project_quad<2>, grd, dim3(q.pg * q.tpi), quad_smem(N), st, x,
+                      g->d_row_items, g->n_row_items, g->d_col_items, g->n_col_items, N, g->n_views, g->n_bins, q.pg,
+                      q.gpb, q.tpi, partial);
+        return;
+    }
+    dim3 grd(proj_bands(N), (g->n_row + PG - 1) / PG + (g->n_col + PG - 1) / PG, batch);
+    const size_t smem = proj_smem(N);
+    if (N + 3 <= PROJ_CW)
         k_project_bands<false><<<grd, PT, smem, st>>>(x, g->d_views, g->d_row_list, g->n_row, g->d_col_list,
                                                       g->n_col, N, g->n_views, g->n_bins, partial);
     else
@@ -718,7 +687,7 @@ int orbit_slices(const Geometry *g, bool cluster)
     return t > 0 ? t : ORB_SL;
 }
 size_t orbit_smem_bytes() { return orbit_smem(); }
-bool quad_ok(const Geometry *g) { return g->vpair && g->n % (2 * MR) == 0 && g->n + 3 <= PROJ_CW; }
+bool quad_ok(const Geometry *g) { return quad_smem(g->n, true) + 16 <= (size_t)QUAD_SMEM_MAX; }
 
 // Measured balance of the work-balanced projector for one image.  Equal
 // unit counts per block leave the blocks' times about 20 % apart at
@@ -740,7 +709,7 @@ constexpr int QB_CAP = 4096;
 ct_status qbal_balance(Geometry *g, const float *x, float *band, cudaStream_t st)
 {
     g->qbounds_nb = 0;   // no table until a better one is written
-    if (!quad_ok(g) || g->tune_qbal != 2) return CT_OK;
+    if (!quad_ok(g) || !proj_plan(g, 1).balanced) return CT_OK;
     const QbalShape q = qbal_shape(g, 1);
     const int nb = q.blocks;
     if (nb < 2 || nb + 1 > QB_CAP) return CT_OK;
@@ -880,13 +849,10 @@ void kernel_attrs_joseph()
     cudaFuncSetAttribute(k_backproject_orbit<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
     cudaFuncSetAttribute(k_backproject_orbit_cl<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
     cudaFuncSetAttribute(k_backproject_orbit_cl<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
-    cudaFuncSetAttribute(k_project_mirror, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj_smem(8192));
-    cudaFuncSetAttribute(k_project_quad<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj_smem(8192));
-    cudaFuncSetAttribute(k_project_quad<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj_smem(8192));
-    cudaFuncSetAttribute(k_project_quad<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj_smem(8192));
-    cudaFuncSetAttribute(k_project_quad<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj_smem(8192));
-    cudaFuncSetAttribute(k_project_qbal<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj_smem(8192));
-    cudaFuncSetAttribute(k_project_qbal<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj_smem(8192));
+    for (auto k : {k_project_quad<2>, k_project_quad<4>})
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, QUAD_SMEM_MAX);
+    for (auto k : {k_project_qbal<2, false>, k_project_qbal<2, true>, k_project_qbal<4, false>, k_project_qbal<4, true>})
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, QUAD_SMEM_MAX);
     cudaFuncSetAttribute(k_project_bands<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj_smem(8192));
     cudaFuncSetAttribute(k_project_bands<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj_smem(8192));
 }

@@ -68,7 +68,7 @@ struct PSlice {
     int tv_tc, tv_tr, tv_ncb, tv_nrb, ntv, fgp;
     int n_items[PH_N], pre[PH_N], per_iter;
     const ViewP *views;
-    const int2 *row_items, *col_items;
+    const QuadItem *row_items, *col_items;
     const float4 *trig;
     const float2 *tw, *hhat;
     const float *b, *winv;
@@ -165,24 +165,19 @@ __device__ __forceinline__ void run_item(const PSlice &S, int p, int k, int i, u
         // band partial sums of A x^{k+1}: item i takes the i-th of the
         // phase's equal ranges of (band pair, view pair, 64-ray) units, as a
         // block of the work-balanced projector does
-        const int npair = (S.B + 1) / 2;
-        QuadUnits U;
-        U.nch = (npair + 63) / 64;
-        U.u_rows = S.n_row_items * U.nch;
-        U.u_cols = S.n_col_items * U.nch;
-        U.u_z = (long long)(S.N / (2 * MR)) * (U.u_rows + U.u_cols);
+        const QuadUnits U = quad_units(S.N, S.B, S.n_row_items, S.n_col_items, 2);
         const long long nq = S.n_items[PH_QUAD];
         long long u0 = U.u_z * i / nq, u1 = U.u_z * (i + 1) / nq;
         if (S.qseg) {
             // small slices: item i is segment i (row-class band pairs, then column-class)
-            const int nbp = S.N / (2 * MR);
+            const int nbp = quad_bands(S.N);
             const bool rows = i < nbp;
             const int bp = rows ? i : i - nbp;
             u0 = rows ? (long long)bp * U.u_rows : (long long)nbp * U.u_rows + (long long)bp * U.u_cols;
             u1 = u0 + (rows ? U.u_rows : U.u_cols);
         }
-        quad_balanced_body<2, true>(BlockCtx{}, u0, u1, U, psm,
-                                    reinterpret_cast<int *>(psm + quad_smem(S.N)), S.x, S.views, S.row_items,
+        quad_balanced_body<2, false>(BlockCtx{}, u0, u1, U, psm,
+                                    reinterpret_cast<int *>(psm + quad_smem(S.N)), S.x, S.row_items,
                                     S.col_items, S.N, S.V, S.B, S.band);
     } else if (p == PH_DUAL) {
         // residual, Step 3 and the next Step 1: one view pair per transform
@@ -292,7 +287,7 @@ int batched_form() { return g_form.load(); }
 bool persistent_slice_ok(const Geometry *g, const ct_pdtv_params *p, int iters0)
 {
     const int ntv = p->tv_iters > 0 ? p->tv_iters : 10;
-    return g->orbit && quad_ok(g) && fft_supported(g) && orbit_slices_ok(g, orbit_slices(g, false)) &&
+    return g->orbit && g->n % (2 * MR) == 0 && g->n + 3 <= 640 && fft_supported(g) && orbit_slices_ok(g, orbit_slices(g, false)) &&
            (p->precond == 0 || p->precond == 1 || p->precond == 3) && !(p->eps > 0.0) && ntv <= TV_MAX_STEPS &&
            p->iters == iters0 && p->iters > 0 && !p->resume;
 }

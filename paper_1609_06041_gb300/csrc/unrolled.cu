@@ -133,6 +133,15 @@ bool tv_fused(double tau, double beta, int mode, int ntv)
     return ntv >= 1 && ntv <= tv_max_steps() && lam > 0.0;
 }
 
+// A in the unrolled form.  On sides that are not a multiple of 32 it keeps
+// the plain band sums: the gradients pass through the prox's kinks, where
+// another rounding of A moves tap gradients by up to 1e-4 of their norm, so
+// there their values stay what they were.
+void project(const Geometry *g, const float *x, float *band, int S, cudaStream_t st)
+{
+    launch_project_bands(g, x, band, S, st, g->vpair && g->n % 32 != 0);
+}
+
 void backproject(const Geometry *g, const float *y, float *out, int mode, const float *xin, const double *scal,
                  int S, char *ws, const UL &L, cudaStream_t st)
 {
@@ -191,7 +200,7 @@ extern "C" ct_status ct_unrolled_forward(const ct_geometry *geom, const float *b
             // the prox, writing its intermediate dual fields for the backward pass
             launch_tv(z, c.p, n.p, n.x, N, g->n_sm, TV_UNROLL_ROWS, tv_iters, 1, scal, st, false, S,
                       tv_iters > 1 ? traj_at(ws, L, g, S, tv_iters, k, 1) : nullptr);
-            launch_project_bands(g, n.x, band, S, st);
+            project(g, n.x, band, S, st);
             launch_dual_fft_batched(g, hhat, band, b, c.mu, n.mu, n.mubar, winv, lowdose, scal, S, st);
             continue;
         }
@@ -206,7 +215,7 @@ extern "C" ct_status ct_unrolled_forward(const ct_geometry *geom, const float *b
             }
         }
         launch_tv_final(z, n.p, n.x, N, S, scal, st);                               // x_{k+1}
-        launch_project_bands(g, n.x, band, S, st);
+        project(g, n.x, band, S, st);
         launch_dual_fft_batched(g, hhat, band, b, c.mu, n.mu, n.mubar, winv, lowdose, scal, S, st);
     }
     cudaMemcpyAsync(x_out, ck_at(ws, L, g, S, iters).x, sizeof(float) * S * J, cudaMemcpyDeviceToDevice, st);
@@ -294,7 +303,7 @@ extern "C" ct_status ct_unrolled_backward(const ct_geometry *geom, const float *
         std::swap(gp, gp2);   // gp: dL/dp_k
         // x_k enters through z_k only: dL/dx_k = dL/dz_k; dL/dmubar_k = -tau A dL/dz_k
         std::swap(gx, gz);
-        launch_project_bands(g, gx, band, S, st);
+        project(g, gx, band, S, st);
         if (fk) fork_end(fk, st);   // the correlations are done with gmb, gm1, rr and vv
         launch_band_reduce_scaled(g, band, gmb, scal + S_RED0, S, st);
         std::swap(gm, gmu);   // dL/dmu_k
