@@ -132,7 +132,7 @@ extern "C" ct_status ct_geometry_autotune(ct_geometry *g, int batch, void *strea
     float *x = nullptr, *sino = nullptr, *band = nullptr, *orb = nullptr, *img = nullptr, *tvb = nullptr;
     float *scalf = nullptr;
     cudaError_t e = buf.alloc(&x, J * batch);
-    if (e == cudaSuccess) e = buf.alloc(&sino, I * batch);
+    if (e == cudaSuccess) e = buf.alloc(&sino, (size_t)g->n_views * g->ld * batch);
     if (e == cudaSuccess) e = buf.alloc(&band, (size_t)proj_bands(N) * I * batch);
     if (e == cudaSuccess) e = buf.alloc(&orb, orbit_partial_floats(g, batch));
     if (e == cudaSuccess) e = buf.alloc(&img, J * batch);
@@ -154,7 +154,7 @@ extern "C" ct_status ct_geometry_autotune(ct_geometry *g, int batch, void *strea
     launch_scalars(scal, SC_SET, 0.05, 0, 0, S_LAMBDA, st);
     launch_scalars(scal, SC_SET, 1.0 / (8.0 * 0.05), 0, 0, S_INV8LAM, st);
     launch_fill(x, 0.5f, J * batch, st);
-    launch_fill(sino, 1.0f, I * batch, st);
+    launch_fill(sino, 1.0f, (size_t)g->n_views * g->ld * batch, st);
     launch_fill(tvb, 0.0f, 6 * J, st);
     launch_fill(tvb, 0.5f, J, st);
 

@@ -299,7 +299,7 @@ struct DualArgs {
     int lowdose;
     const ViewP *views;
     const double *scal;
-    int V, B;
+    int V, B, ld;   // ld: row stride of mu_bar, zeros written past B
 };
 
 template <int P, bool DBL>
@@ -337,7 +337,8 @@ __device__ __forceinline__ void dual_update(const Ctx &c, int t, int pair, int b
     const size_t so = (size_t)by * V * B;
     const size_t o0 = so + (size_t)(has0 ? v0 : 0) * B, o1 = so + (size_t)(has1 ? v1 : 0) * B;
     const float *winv = g.winv, *mu_in = g.mu_in;
-    float *mu = g.mu, *mu_bar = g.mu_bar;
+    float *mu = g.mu;
+    float *mb0 = g.mu_bar + ((size_t)by * V + (has0 ? v0 : 0)) * g.ld, *mb1 = has1 ? mb0 + g.ld : mb0;
     const float sp = fscal(g.scal, F_SIGMA) * (1.0f / (float)P);
     const float2 *stage = buf + (DBL ? fft_elems(P) : 0);
     int ph = 0;
@@ -373,12 +374,14 @@ __device__ __forceinline__ void dual_update(const Ctx &c, int t, int pair, int b
                 }
                 if (!KEEP || !lowdose) {   // Alg. 2: mu_bar = 2 mu' - mu, no second filter
                     mu[o0 + i] = n.x;
-                    mu_bar[o0 + i] = e.x;
+                    mb0[i] = e.x;
                     if (has1) {
                         mu[o1 + i] = n.y;
-                        mu_bar[o1 + i] = e.y;
+                        mb1[i] = e.y;
                     }
                 }
+            } else if (i < g.ld && has0) {
+                mb0[i] = mb1[i] = 0.0f;
             }
             v[r] = d;
         }
@@ -391,10 +394,10 @@ __device__ __forceinline__ void dual_update(const Ctx &c, int t, int pair, int b
         const int i = t + r * T;
         if (i < B && has0) {
             if constexpr (KEEP) mu[o0 + i] = mn[r].x;
-            mu_bar[o0 + i] = __fmaf_rn(-sp, v[r].x, KEEP ? mo[KEEP ? r : 0].x : mu_bar[o0 + i]);
+            mb0[i] = __fmaf_rn(-sp, v[r].x, KEEP ? mo[KEEP ? r : 0].x : mb0[i]);
             if (has1) {
                 if constexpr (KEEP) mu[o1 + i] = mn[r].y;
-                mu_bar[o1 + i] = __fmaf_rn(-sp, v[r].y, KEEP ? mo[KEEP ? r : 0].y : mu_bar[o1 + i]);
+                mb1[i] = __fmaf_rn(-sp, v[r].y, KEEP ? mo[KEEP ? r : 0].y : mb1[i]);
             }
         }
     }

@@ -456,12 +456,6 @@ constexpr int ORB_VC = 8;        // base views staged per chunk
 constexpr int ORB_RW = 36;       // values per window: pairs (k, k+1), k <= ORB_RW - 2
 constexpr int ORB_MAXS = 1024;   // base views per slice (V <= 8192)
 
-__device__ __forceinline__ void cp_async4(float *dst, const float *src, bool valid)
-{
-    const unsigned sdst = (unsigned)__cvta_generic_to_shared(dst);
-    const int n = valid ? 4 : 0;   // 0: fill with zeros, read nothing
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(sdst), "l"(src), "r"(n) : "memory");
-}
 __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool valid)
 {
     const unsigned sdst = (unsigned)__cvta_generic_to_shared(dst);
@@ -473,12 +467,18 @@ template <int K>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(K) : "memory"); }
 
 // Body of block (bx, by, bz) (c.nth() = ORB_TH threads, as ORB_T x ORB_TY);
-// osm holds orbit_smem() bytes.  CL: instead of storing its sums, the
+// osm holds orbit_smem() bytes.  y: V rows of B values per image, ld floats
+// apart, ld a multiple of 4, zeros past the B-th, 16-byte aligned: so every
+// window, whose start is a multiple of 4, is copied in aligned 16-byte
+// pieces, each wholly on or wholly off the padded row (rows of B floats with
+// B % 4 != 0 were copied by 4-byte pieces: 92 us against 67 at 512^2 / 720
+// views, 738 and 736 bins).  AL: B % 4 == 0, which makes the mirrored windows'
+// place a constant (otherwise one more addition a view, 68.5 against 67 us).  CL: instead of storing its sums, the
 // block leaves them in osm, entry (k ORB_PX + j) ORB_TH + tid for rotation
 // k of the thread's pixel orbit j, for a cluster reduction over slices.
 template <bool AL, class Ctx, bool CL = false>
 __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz, unsigned char *osm, const float *y,
-                                           float *partial, const float4 *trig, int N, int V, int B, int nsl,
+                                           int ld, float *partial, const float4 *trig, int N, int V, int B, int nsl,
                                            int fin, float *out, const float *xin, const double *scal)
 {
     // raw[buffer][view][row (v, v+V/2)][window (e, mirror e, e90, mirror e90)][value]
@@ -494,7 +494,8 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
     const bool inside = r < half && c < N;
     const float h = 0.5f * (float)(N - 1), hb = 0.5f * (float)(B - 1), hb_lo = hb - 0.5f;
     const float xq = (float)c - h, yq = (float)r - h;               // P = (x, y); R90 P = (-y, x)
-    const float *ys = y + (size_t)img * V * B;
+    const float *ys = y + (size_t)img * V * ld;
+    const int ms = AL ? 3 : (B - ORB_RW + 3) & 3;   // see the mirrored windows below
     const int vb0 = (int)((long long)V2 * slice / nsl), vb1 = (int)((long long)V2 * (slice + 1) / nsl);
     const int nvs = vb1 - vb0;
     float acc[ORB_PX][4];   // per pixel orbit: P, R90 P, R180 P, R270 P
@@ -521,8 +522,8 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
     }
     cb.sync();
 
-    // raw window values y[start + w], w < ORB_RW, start = wb (windows e, e90)
-    // or B - ORB_RW - wb (their mirrors, holding pair B-2-f at ORB_RW-2 - (f - wb));
+    // raw window values y[start + w], w < ORB_RW, start = wb (windows e, e90) or, for their mirrors, the multiple of
+    // 4 at or below B - ORB_RW + 3 - wb, so that pair B-2-f sits at ORB_RW-5 + ms - (f - wb), ms = 0 .. 3;
     // per view (cos, sin, |a|^2, |a| (1 - |a|/2)): the hat weights times |a|
     auto issue = [&](int v0, int nv, int buf) {
         float *dst0 = raw + (size_t)buf * ORB_VC * 8 * ORB_RW;
@@ -530,16 +531,14 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
             const float4 T = trig[v0 + tid];
             tt[buf * ORB_VC + tid] = make_float4(T.x, T.y, T.z * T.z, T.z * T.w);
         }
-        constexpr int CH = AL ? ORB_RW / 4 : ORB_RW;   // copies per window
+        constexpr int CH = ORB_RW / 4;   // copies per window
         for (int k = tid; k < nv * 8 * CH; k += ORB_TH) {
             const int q = k / CH, j = k - q * CH;
             const int win = q & 3, row = (q >> 2) & 1, vi = q >> 3;
             const int base = wbs[2 * (v0 - vb0 + vi) + (win >> 1)];
-            const int d = ((win & 1) ? B - ORB_RW - base : base) + (AL ? 4 * j : j);
+            const int d = ((win & 1) ? B - ORB_RW + 3 - ms - base : base) + 4 * j;
             const bool ok = d >= 0 && d < B;
-            const float *src = ys + (size_t)(v0 + vi + row * V2) * B + (ok ? d : 0);
-            if (AL) cp_async16(dst0 + (size_t)q * ORB_RW + 4 * j, src, ok);
-            else cp_async4(dst0 + (size_t)q * ORB_RW + j, src, ok);
+            cp_async16(dst0 + (size_t)q * ORB_RW + 4 * j, ys + (size_t)(v0 + vi + row * V2) * ld + (ok ? d : 0), ok);
         }
         cp_async_commit();
     };
@@ -570,14 +569,14 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
                     const float e9 = fmaf(xq, T.y, fmaf(-yy, T.x, hb_lo));
                     const float t = __fadd_rn(e, JOSEPH_BIAS), t9 = __fadd_rn(e9, JOSEPH_BIAS);
                     const unsigned k = min((unsigned)(__float_as_int(t) - (JOSEPH_BIAS_BITS + wb.x)),
-                                           (unsigned)(ORB_RW - 2));
+                                           (unsigned)(ORB_RW - 5));
                     const unsigned k9 = min((unsigned)(__float_as_int(t9) - (JOSEPH_BIAS_BITS + wb.y)),
-                                            (unsigned)(ORB_RW - 2));
+                                            (unsigned)(ORB_RW - 5));
                     const float g = __fsub_rn(e, __fsub_rn(t, JOSEPH_BIAS));
                     const float g9 = __fsub_rn(e9, __fsub_rn(t9, JOSEPH_BIAS));
                     const float w0 = fmaxf(0.0f, fmaf(-g, T.z, T.w)), w1 = fmaxf(0.0f, fmaf(g, T.z, T.w));
                     const float w09 = fmaxf(0.0f, fmaf(-g9, T.z, T.w)), w19 = fmaxf(0.0f, fmaf(g9, T.z, T.w));
-                    const unsigned km = ORB_RW - 2 - k, km9 = ORB_RW - 2 - k9;
+                    const unsigned km = ORB_RW - 5 + ms - k, km9 = ORB_RW - 5 + ms - k9;
                     cP = fmaf(w0, e_v[k], fmaf(w1, e_v[k + 1], cP));             // P at v
                     c180 = fmaf(w1, m_v[km], fmaf(w0, m_v[km + 1], c180));       // R180 P at v
                     c90 = fmaf(w0, e_w[k], fmaf(w1, e_w[k + 1], c90));           // R90 P at v + V/2

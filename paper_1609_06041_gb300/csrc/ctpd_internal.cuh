@@ -42,6 +42,7 @@ struct Geometry {
     int n, n_views, n_bins, device;
     int n_fft;            // P = 2^ceil(log2(2B)), the period of the taps
     int p_fft;            // transform length of D's convolution: n_fft, at least 64
+    int ld;               // row stride of the sinograms A^T reads inside the library: n_bins rounded up to 4
     int n_row, n_col;     // views stepping along rows / columns
     float win_eps;        // candidate-window margin (bins) of the backprojector
     ViewP *d_views;       // device, n_views entries
@@ -406,19 +407,26 @@ void launch_band_reduce(const Geometry *g, const float *partial, float *out, int
 // thread-block cluster (cluster, or partial NULL), or through slice images
 // in `partial` (orbit_partial_floats() floats) and a reduction pass: the
 // form for solves run side by side, whose clusters would wait for a GPC's
-// SMs to free together.
+// SMs to free together.  The orbit form's y has rows of g->ld floats, zeros
+// past n_bins, 16-byte aligned (launch_pad_rows copies a sinogram so); the
+// general form's rows are ld floats apart.
 bool orbit_ok(const Geometry *g);
 size_t orbit_partial_floats(const Geometry *g, int batch);
 bool orbit_slices_ok(const Geometry *g, int nsl);
 void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int mode, const float *xin,
                               const double *scal, int batch, float *partial, cudaStream_t st, bool cluster = true);
-void launch_backproject(const Geometry *g, const float *y, float *out, int mode,
+void launch_pad_rows(const Geometry *g, const float *in, float *out, int batch, cudaStream_t st);
+void launch_backproject(const Geometry *g, const float *y, int ld, float *out, int mode,
                         const float *xin, const double *scal, int batch, cudaStream_t st);
 
+// Sinograms that A^T reads inside the library (mu_bar, the adjoint's dL/dr)
+// have rows of g->ld floats; the kernels below that write one take its row
+// stride ldo and write zeros past n_bins (launch_filter, launch_dual_update
+// and launch_eps_step leave what is there).
 // Filter: out = post .* (D (pre .* in)) * (scal ? -sigma : 1); pre/post
 // may be NULL.  mode 0 plain, 1 "-sigma D in" (start of the iteration).
 void launch_filter(const Geometry *g, const float *taps, int half, const float *in,
-                   float *out, const float *pre, const float *post, int mode,
+                   float *out, int ldo, const float *pre, const float *post, int mode,
                    const double *scal, int batch, cudaStream_t st);
 // Fused Step 3 + next Step 1 for one iteration, per view:
 //   mu' = mu + sigma D r;  mu_bar = 2 mu' - mu [- sigma D (winv .* (mu' - mu))].
@@ -443,11 +451,11 @@ void launch_hhat(const Geometry *g, const float *taps, int half, float2 *hhat, c
 // post are complete when the kernel starts and only hhat is waited for
 void launch_filter_fft(const Geometry *g, const float2 *hhat, const float *in, float *out,
                        const float *pre, const float *post, int mode, const double *scal, int batch,
-                       cudaStream_t st, bool early = false);
+                       cudaStream_t st, int ldo, bool early = false);
 // out = D (A x) with A x given as the projector's band partial sums
 void launch_filter_fft_bands(const Geometry *g, const float2 *hhat, const float *partial, float *out, int batch,
-                             cudaStream_t st);
-// fused residual + Step 3 + next Step 1 (as launch_dual_update)
+                             cudaStream_t st, int ldo);
+// fused residual + Step 3 + next Step 1 (as launch_dual_update; mu_bar with rows of g->ld)
 void launch_dual_fft(const Geometry *g, const float2 *hhat, const float *partial, const float *b, float *mu,
                      float *mu_bar, const float *winv, int lowdose, const double *scal, cudaStream_t st);
 // The shift-variant preconditioner D = T_lo + S T_hi S (k_fft.cu; low-dose,
@@ -457,9 +465,9 @@ void launch_sv_hhat(const Geometry *g, const float *taps_lo, const float *taps_h
                     cudaStream_t st);
 void launch_filter_sv(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv, const float *in,
                       float *out, const float *pre, const float *post, int mode, const double *scal, int batch,
-                      cudaStream_t st);
+                      cudaStream_t st, int ldo);
 void launch_filter_sv_bands(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv,
-                            const float *partial, float *out, int batch, cudaStream_t st);
+                            const float *partial, float *out, int batch, cudaStream_t st, int ldo);
 void launch_dual_sv(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv, const float *partial,
                     const float *b, float *mu, float *mu_bar, const float *winv, const double *scal,
                     cudaStream_t st);
@@ -526,7 +534,7 @@ int tv_max_steps();
 // (Q as B x B row-major floats, lambda) for a geometry, precond and tau,
 // computed from the device taps (2B - 1 values) on first use and cached.
 // launch_eps_step: out = the proximal map of q (see eps.cu), out2 (may be
-// NULL) = 2 out - mu0; Q = NULL means D = I.  wbuf: V x B floats, s and w2:
+// NULL) = 2 out - mu0; their rows are ldo and ld2 floats apart.  Q = NULL means D = I.  wbuf: V x B floats, s and w2:
 // B floats each, part: eps_partial_floats(g) floats.
 bool toeplitz_eig(const double *t, int n, double *q, double *lambda);
 ct_status eps_basis(const Geometry *g, int precond, double tau_key, const float *taps, cudaStream_t st,
@@ -535,7 +543,8 @@ void eps_cache_free(Geometry *g);
 // whether eps_basis has the basis already (so a solve needs no host step)
 bool eps_basis_ready(const Geometry *g, int precond, double tau_key);
 size_t eps_partial_floats(const Geometry *g);
-void launch_eps_step(const Geometry *g, const float *q, float *out, float *out2, const float *mu0, const float *Q,
+void launch_eps_step(const Geometry *g, const float *q, float *out, int ldo, float *out2, int ld2, const float *mu0,
+                     const float *Q,
                      const float *lambda, double eps, double *scal, float *wbuf, float *s, float *w2, float *part,
                      cudaStream_t st);
 

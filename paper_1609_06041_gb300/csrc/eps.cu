@@ -299,8 +299,14 @@ k_eps_sum_w2(const float *__restrict__ part, int ks, int V, int B, float *__rest
 
 // after the second map: out = sum_z part[z] (chunks in order), out2 =
 // 2 out - mu0
-__global__ void k_eps_sum_out(const float *__restrict__ part, int ks, size_t n, float *__restrict__ out,
-                              float *__restrict__ out2, const float *__restrict__ mu0)
+// the place of element i (rows of B) in rows ld apart
+__device__ __forceinline__ size_t in_rows(size_t i, int B, int ld)
+{
+    return ld == B ? i : i + (i / (unsigned)B) * (unsigned)(ld - B);
+}
+
+__global__ void k_eps_sum_out(const float *__restrict__ part, int ks, size_t n, int B, float *__restrict__ out, int ldo,
+                              float *__restrict__ out2, int ld2, const float *__restrict__ mu0)
 {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         float pz[EG_KS];
@@ -309,21 +315,21 @@ __global__ void k_eps_sum_out(const float *__restrict__ part, int ks, size_t n, 
         float a = 0.0f;
 #pragma unroll
         for (int z = 0; z < EG_KS; ++z) a += pz[z];
-        out[i] = a;
-        if (out2) out2[i] = 2.0f * a - mu0[i];
+        out[in_rows(i, B, ldo)] = a;
+        if (out2) out2[in_rows(i, B, ld2)] = 2.0f * a - mu0[i];
     }
 }
 
 // out = X s (per column j; in place allowed), out2 = 2 out - mu0: the map
 // when D = I
-__global__ void k_eps_scale(const float *X, const float *__restrict__ s, float *out,
-                            float *__restrict__ out2, const float *__restrict__ mu0, int V, int B)
+__global__ void k_eps_scale(const float *X, const float *__restrict__ s, float *out, int ldo,
+                            float *__restrict__ out2, int ld2, const float *__restrict__ mu0, int V, int B)
 {
     const size_t n = (size_t)V * B;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float v = X[i] * s[i % B];
-        out[i] = v;
-        if (out2) out2[i] = 2.0f * v - mu0[i];
+        out[in_rows(i, B, ldo)] = v;
+        if (out2) out2[in_rows(i, B, ld2)] = 2.0f * v - mu0[i];
     }
 }
 
@@ -460,8 +466,8 @@ k_eps_root(const float *__restrict__ w2g, const float *__restrict__ lambda, int 
     if (tid == 0) *uslot = (zero || all) ? 0.0f : u;
 }
 
-void launch_eps_step(const Geometry *g, const float *q, float *out, float *out2, const float *mu0, const float *Q,
-                     const float *lambda, double eps, double *scal, float *wbuf, float *s, float *w2, float *part,
+void launch_eps_step(const Geometry *g, const float *q, float *out, int ldo, float *out2, int ld2, const float *mu0,
+                     const float *Q, const float *lambda, double eps, double *scal, float *wbuf, float *s, float *w2, float *part,
                      cudaStream_t st)
 {
     const int V = g->n_views, B = g->n_bins;
@@ -475,12 +481,12 @@ void launch_eps_step(const Geometry *g, const float *q, float *out, float *out2,
         k_eps_sum_w2<<<(B + 31) / 32, dim3(32, 8), 0, st>>>(part, ks, V, B, wbuf, w2);
         k_eps_root<<<1, EPS_ROOT_T, 0, st>>>(w2, lambda, B, scal, (float)eps, s);
         k_eps_gemm<true><<<grid, tb, 0, st>>>(wbuf, Q, s, part, V, B, kchunk);
-        k_eps_sum_out<<<eblocks, 256, 0, st>>>(part, ks, n, out, out2, mu0);
+        k_eps_sum_out<<<eblocks, 256, 0, st>>>(part, ks, n, B, out, ldo, out2, ld2, mu0);
     } else {
         counted(3);
         k_eps_w2<<<(B + 127) / 128, 128, 0, st>>>(q, V, B, w2);
         k_eps_root<<<1, EPS_ROOT_T, 0, st>>>(w2, nullptr, B, scal, (float)eps, s);
-        k_eps_scale<<<eblocks, 256, 0, st>>>(q, s, out, out2, mu0, V, B);
+        k_eps_scale<<<eblocks, 256, 0, st>>>(q, s, out, ldo, out2, ld2, mu0, V, B);
     }
 }
 

@@ -151,7 +151,7 @@ void launch_hhat(const Geometry *g, const float *taps, int half, float2 *hhat, c
 template <int P, bool BANDS, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? wide_threads(P) : block_threads(P),
                                   WIDE ? 1 : BANDS ? min_blocks(P) : 4 * min_blocks(P) / 3)
-k_filter_fft(const float2 *__restrict__ hhat, const float *__restrict__ in, float *__restrict__ out,
+k_filter_fft(const float2 *__restrict__ hhat, const float *__restrict__ in, float *__restrict__ out, int ldo,
              const float *__restrict__ pre, const float *__restrict__ post, int mode,
              const double *__restrict__ scal, int V, int B, const float2 *__restrict__ tw, int nb,
              const ViewP *__restrict__ views, int early)
@@ -201,6 +201,7 @@ k_filter_fft(const float2 *__restrict__ hhat, const float *__restrict__ in, floa
     const GroupCtx ctx{(int)threadIdx.x, block_threads(P), 1};
     fft_apply<P, false, true>(ctx, pl.t, v, pl.buf, ph, hhat, tw);
     const float sc = ((mode == 1) ? -fscal(scal, F_SIGMA) : 1.0f) / (float)P;
+    float *q0 = out + ((size_t)blockIdx.y * V + (has0 ? v0 : 0)) * ldo, *q1 = has1 ? q0 + ldo : q0;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         const int i = pl.t + r * T;
@@ -210,8 +211,10 @@ k_filter_fft(const float2 *__restrict__ hhat, const float *__restrict__ in, floa
                 y0 *= post[o0 + i];
                 if (has1) y1 *= post[o1 + i];
             }
-            out[o0 + i] = y0;
-            if (has1) out[o1 + i] = y1;
+            q0[i] = y0;
+            if (has1) q1[i] = y1;
+        } else if (i < ldo && has0) {
+            q0[i] = q1[i] = 0.0f;
         }
     }
 }
@@ -225,7 +228,7 @@ static dim3 fft_grid(int transforms, int batch)
 
 // out = D (A x) from the projector's band partial sums
 void launch_filter_fft_bands(const Geometry *g, const float2 *hhat, const float *partial, float *out, int batch,
-                             cudaStream_t st)
+                             cudaStream_t st, int ldo)
 {
     counted();
     with_length(g->p_fft, [&](auto L) {
@@ -233,21 +236,21 @@ void launch_filter_fft_bands(const Geometry *g, const float2 *hhat, const float 
         const bool wide = wide_grid(g, batch);
         launch_kernel(wide ? k_filter_fft<P, true, true> : k_filter_fft<P, true, false>,
                       fft_grid<P>((g->n_views + 1) / 2, batch), dim3(wide ? wide_threads(P) : block_threads(P)),
-                      block_smem(P), st, hhat, partial, out, nullptr, nullptr, 0, nullptr, g->n_views, g->n_bins,
+                      block_smem(P), st, hhat, partial, out, ldo, nullptr, nullptr, 0, nullptr, g->n_views, g->n_bins,
                       g->d_tw, proj_bands(g->n), g->d_views, 0);
     });
 }
 
 void launch_filter_fft(const Geometry *g, const float2 *hhat, const float *in, float *out,
                        const float *pre, const float *post, int mode, const double *scal, int batch,
-                       cudaStream_t st, bool early)
+                       cudaStream_t st, int ldo, bool early)
 {
     counted();
     PdlScope pdl(early || t_pdl);
     with_length(g->p_fft, [&](auto L) {
         constexpr int P = decltype(L)::value;
         launch_kernel(k_filter_fft<P, false, false>, fft_grid<P>((g->n_views + 1) / 2, batch), dim3(block_threads(P)),
-                      block_smem(P), st, hhat, in, out, pre, post, mode, scal, g->n_views, g->n_bins, g->d_tw, 0,
+                      block_smem(P), st, hhat, in, out, ldo, pre, post, mode, scal, g->n_views, g->n_bins, g->d_tw, 0,
                       nullptr, early ? 1 : 0);
     });
 }
@@ -351,7 +354,7 @@ __device__ __forceinline__ float band_sum(const float *__restrict__ p, size_t VB
 template <int P, bool BANDS>
 __global__ void __launch_bounds__(block_threads(P), min_blocks(P))
 k_filter_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const float *__restrict__ sv,
-            const float *__restrict__ in, float *__restrict__ out, const float *__restrict__ pre,
+            const float *__restrict__ in, float *__restrict__ out, int ldo, const float *__restrict__ pre,
             const float *__restrict__ post, int mode, const double *__restrict__ scal, int V, int B,
             const float2 *__restrict__ tw, int nb, const ViewP *__restrict__ views)
 {
@@ -383,6 +386,7 @@ k_filter_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const 
     }
     int ph = 0;
     sv_apply<P>(pl.t, v, pl.buf, ph, hs, hd, tw);
+    float *q = out + ((size_t)blockIdx.y * V + vw) * ldo;
     const float sc = ((mode == 1) ? -fscal(scal, F_SIGMA) : 1.0f) / (float)P;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -390,31 +394,33 @@ k_filter_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const 
         if (i < B && has) {
             float y = fmaf(s[i], v[r].y, v[r].x) * sc;
             if (post) y *= post[o + i];
-            out[o + i] = y;
+            q[i] = y;
+        } else if (i < ldo && has) {
+            q[i] = 0.0f;
         }
     }
 }
 
 void launch_filter_sv(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv, const float *in,
                       float *out, const float *pre, const float *post, int mode, const double *scal, int batch,
-                      cudaStream_t st)
+                      cudaStream_t st, int ldo)
 {
     counted();
     with_length(g->p_fft, [&](auto L) {
         constexpr int P = decltype(L)::value;
         launch_kernel(k_filter_sv<P, false>, fft_grid<P>(g->n_views, batch), dim3(block_threads(P)), block_smem(P), st,
-                      hs, hd, sv, in, out, pre, post, mode, scal, g->n_views, g->n_bins, g->d_tw, 0, nullptr);
+                      hs, hd, sv, in, out, ldo, pre, post, mode, scal, g->n_views, g->n_bins, g->d_tw, 0, nullptr);
     });
 }
 
 void launch_filter_sv_bands(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv,
-                            const float *partial, float *out, int batch, cudaStream_t st)
+                            const float *partial, float *out, int batch, cudaStream_t st, int ldo)
 {
     counted();
     with_length(g->p_fft, [&](auto L) {
         constexpr int P = decltype(L)::value;
         launch_kernel(k_filter_sv<P, true>, fft_grid<P>(g->n_views, batch), dim3(block_threads(P)), block_smem(P), st,
-                      hs, hd, sv, partial, out, nullptr, nullptr, 0, nullptr, g->n_views, g->n_bins, g->d_tw,
+                      hs, hd, sv, partial, out, ldo, nullptr, nullptr, 0, nullptr, g->n_views, g->n_bins, g->d_tw,
                       proj_bands(g->n), g->d_views);
     });
 }
@@ -427,7 +433,7 @@ template <int P>
 __global__ void __launch_bounds__(block_threads(P), min_blocks(P))
 k_dual_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const float *__restrict__ sv,
           const float *__restrict__ partial, int nb, const float *__restrict__ b, float *mu,
-          float *__restrict__ mu_bar, const float *__restrict__ winv, const ViewP *__restrict__ views,
+          float *__restrict__ mu_bar, int ld, const float *__restrict__ winv, const ViewP *__restrict__ views,
           const double *__restrict__ scal, int V, int B, const float2 *__restrict__ tw)
 {
     extern __shared__ float2 fsm[];
@@ -479,7 +485,9 @@ k_dual_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const fl
         const int i = pl.t + r * T;
         if (i < B && has) {
             mu[o + i] = mn[r];
-            mu_bar[o + i] = fmaf(-sp, fmaf(s[i], v[r].y, v[r].x), mo[r]);
+            mu_bar[(size_t)vw * ld + i] = fmaf(-sp, fmaf(s[i], v[r].y, v[r].x), mo[r]);
+        } else if (i < ld && has) {
+            mu_bar[(size_t)vw * ld + i] = 0.0f;
         }
     }
 }
@@ -492,7 +500,7 @@ void launch_dual_sv(const Geometry *g, const float2 *hs, const float2 *hd, const
     with_length(g->p_fft, [&](auto L) {
         constexpr int P = decltype(L)::value;
         launch_kernel(k_dual_sv<P>, fft_grid<P>(g->n_views, 1), dim3(block_threads(P)), block_smem(P), st, hs, hd, sv,
-                      partial, proj_bands(g->n), b, mu, mu_bar, winv, g->d_views, scal, g->n_views, g->n_bins,
+                      partial, proj_bands(g->n), b, mu, mu_bar, g->ld, winv, g->d_views, scal, g->n_views, g->n_bins,
                       g->d_tw);
     });
 }
@@ -515,7 +523,7 @@ void launch_dual_fft_batched(const Geometry *g, const float2 *hhat, const float 
         constexpr int P = decltype(L)::value;
         const bool wide = wide_grid(g, batch);
         const DualArgs a{hhat, g->d_tw, partial, proj_bands(g->n), b, mu_in, mu_out, mu_bar, winv, lowdose,
-                         g->d_views, scal, g->n_views, g->n_bins};
+                         g->d_views, scal, g->n_views, g->n_bins, g->ld};
         launch_kernel(wide ? k_dual_fft<P, true> : k_dual_fft<P, false>, fft_grid<P>((g->n_views + 1) / 2, batch),
                       dim3(wide ? wide_threads(P) : block_threads(P)), block_smem(P), st, a);
     });
@@ -541,7 +549,7 @@ k_dual_bwd_fft(const float2 *__restrict__ hhat, const float *__restrict__ partia
                const float *__restrict__ mu1, const float *__restrict__ gm, const float *__restrict__ gmb,
                float *__restrict__ gmu_out, float *__restrict__ gr_out, float *gm1_out,
                float *__restrict__ r_out, float *__restrict__ v_out, int lowdose,
-               const ViewP *__restrict__ views, const double *__restrict__ scal, int V, int B,
+               const ViewP *__restrict__ views, const double *__restrict__ scal, int V, int B, int ld,
                const float2 *__restrict__ tw)
 {
     extern __shared__ float2 fsm[];
@@ -599,6 +607,12 @@ k_dual_bwd_fft(const float2 *__restrict__ hhat, const float *__restrict__ partia
         st[fp(P / 2 + i)] = hr[r];
     }
     if (!has0) return;
+    // dL/dr, the adjoint's input of A^T: rows of ld, zeros past B
+    float *gp = gr_out + ((size_t)blockIdx.y * V + v0) * ld;
+    for (int i = B + pl.t; i < ld; i += T) {
+        gp[i] = 0.0f;
+        if (has1) gp[ld + i] = 0.0f;
+    }
 #pragma unroll 1
     for (int i = pl.t; i < B; i += T) {
         float s[2];
@@ -619,7 +633,7 @@ k_dual_bwd_fft(const float2 *__restrict__ hhat, const float *__restrict__ partia
                 vv = winv[o] * (mu1[o] - mu[o]);
             }
             gmu_out[o] = gmu;
-            gr_out[o] = gr;
+            gp[(size_t)k * ld + i] = gr;
             r_out[o] = r;
             v_out[o] = vv;
         }
@@ -636,7 +650,7 @@ void launch_dual_bwd_fft(const Geometry *g, const float2 *hhat, const float *par
         constexpr int P = decltype(L)::value;
         launch_kernel(k_dual_bwd_fft<P>, fft_grid<P>((g->n_views + 1) / 2, batch), dim3(block_threads(P)),
                       block_smem(P), st, hhat, partial, proj_bands(g->n), b, winv, mu, mu1, gm, gmb, gmu, gr, gm1, r,
-                      v, lowdose, g->d_views, scal, g->n_views, g->n_bins, g->d_tw);
+                      v, lowdose, g->d_views, scal, g->n_views, g->n_bins, g->ld, g->d_tw);
     });
 }
 

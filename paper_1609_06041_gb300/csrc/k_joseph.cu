@@ -506,7 +506,7 @@ constexpr int BWW = 32;         // staged ray pairs per view (>= 15 (|cos|+|sin|
 
 template <int MODE>
 __global__ void __launch_bounds__(BTH)
-k_backproject_tiles(const float *__restrict__ y, float *__restrict__ out,
+k_backproject_tiles(const float *__restrict__ y, int ld, float *__restrict__ out,
                     const float4 *__restrict__ trig, int N, int V, int B,
                     const float *__restrict__ xin, const double *__restrict__ scal)
 {
@@ -519,7 +519,7 @@ k_backproject_tiles(const float *__restrict__ y, float *__restrict__ out,
     const int slice = tid >> 6, l = tid & 63;
     const int R0 = blockIdx.y * BT, C0 = blockIdx.x * BT;
     const int r = R0 + (l >> 2), c0 = C0 + (l & 3) * 4;
-    const float *ys = y + (size_t)blockIdx.z * V * B;
+    const float *ys = y + (size_t)blockIdx.z * V * ld;
     const float h = 0.5f * (float)(N - 1);
     const float hb_lo = 0.5f * (float)(B - 1) - 0.5f;   // e - 1/2 is rounded to find floor(e)
     const float yr = (float)r - h;
@@ -549,7 +549,7 @@ k_backproject_tiles(const float *__restrict__ y, float *__restrict__ out,
         for (int k = tid; k < nv * BWW; k += BTH) {
             const int vi = k / BWW, w = k - vi * BWW;
             const int d = wbase[vi] + w;
-            const float *yv = ys + (size_t)(v0 + vi) * B;
+            const float *yv = ys + (size_t)(v0 + vi) * ld;
             const float sc = sv[vi].z;
             const float y0 = (d >= 0 && d < B) ? yv[d] : 0.0f;
             const float y1 = (d + 1 >= 0 && d + 1 < B) ? yv[d + 1] : 0.0f;
@@ -593,18 +593,15 @@ k_backproject_tiles(const float *__restrict__ y, float *__restrict__ out,
     }
 }
 
-// AL: B % 4 == 0 and y 16-byte aligned, so every window (its base a
-// multiple of 4) is copied in aligned 16-byte pieces, each wholly on or
-// wholly off the detector.
 template <bool AL>
 __global__ void __launch_bounds__(ORB_TH, 8)
-k_backproject_orbit(const float *__restrict__ y, float *__restrict__ partial, const float4 *__restrict__ trig,
+k_backproject_orbit(const float *__restrict__ y, int ld, float *__restrict__ partial, const float4 *__restrict__ trig,
                     int N, int V, int B, int nsl, int fin, float *out, const float *xin,
                     const double *__restrict__ scal)
 {
     extern __shared__ __align__(16) unsigned char osm[];
     pdl_wait();
-    orbit_body<AL>(Block2D{}, blockIdx.x, blockIdx.y, blockIdx.z, osm, y, partial, trig, N, V, B, nsl, fin, out, xin,
+    orbit_body<AL>(Block2D{}, blockIdx.x, blockIdx.y, blockIdx.z, osm, y, ld, partial, trig, N, V, B, nsl, fin, out, xin,
                    scal);
 }
 
@@ -617,12 +614,12 @@ k_backproject_orbit(const float *__restrict__ y, float *__restrict__ partial, co
 // reduction pass runs.
 template <bool AL>
 __global__ void __launch_bounds__(ORB_TH, 8)
-k_backproject_orbit_cl(const float *__restrict__ y, const float4 *__restrict__ trig, int N, int V, int B, int nsl,
+k_backproject_orbit_cl(const float *__restrict__ y, int ld, const float4 *__restrict__ trig, int N, int V, int B, int nsl,
                        int mode, float *out, const float *xin, const double *__restrict__ scal)
 {
     extern __shared__ __align__(16) unsigned char osm[];
     pdl_wait();
-    orbit_body<AL, Block2D, true>(Block2D{}, blockIdx.x, blockIdx.y, blockIdx.z, osm, y, nullptr, trig, N, V, B, nsl, 0,
+    orbit_body<AL, Block2D, true>(Block2D{}, blockIdx.x, blockIdx.y, blockIdx.z, osm, y, ld, nullptr, trig, N, V, B, nsl, 0,
                                   nullptr, nullptr, scal);
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
@@ -804,6 +801,23 @@ ct_status qbal_balance(Geometry *g, const float *x, float *band, cudaStream_t st
     return CT_OK;
 }
 
+// out rows of ld >= B floats: the B values of each row, then zeros
+__global__ void k_pad_rows(const float *__restrict__ in, float *__restrict__ out, size_t n, int B, int ld)
+{
+    const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const size_t row = i / (unsigned)ld;
+    const int d = (int)(i - row * ld);
+    out[i] = d < B ? in[row * B + d] : 0.0f;
+}
+
+void launch_pad_rows(const Geometry *g, const float *in, float *out, int batch, cudaStream_t st)
+{
+    const size_t n = (size_t)batch * g->n_views * g->ld;
+    counted();
+    k_pad_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, out, n, g->n_bins, g->ld);
+}
+
 void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int mode, const float *xin,
                               const double *scal, int batch, float *partial, cudaStream_t st, bool cluster)
 {
@@ -811,44 +825,45 @@ void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int
     const bool cl = cluster || !partial;
     const int nsl = orbit_slices(g, cl);
     dim3 grd((q + ORB_T - 1) / ORB_T, (q + ORB_T - 1) / ORB_T, nsl * batch);
-    const bool al = g->n_bins % 4 == 0 && reinterpret_cast<uintptr_t>(y) % 16 == 0;
+    const bool al = g->ld == g->n_bins;
     if (nsl > 1 && cl) {
         // several slices: their sums are added in a cluster of the slices' blocks
         counted();
         launch_kernel_cluster(al ? k_backproject_orbit_cl<true> : k_backproject_orbit_cl<false>, grd,
-                              dim3(ORB_T, ORB_TY), orbit_smem(), st, dim3(1, 1, nsl), y, (const float4 *)g->d_trig,
-                              g->n, g->n_views, g->n_bins, nsl, mode != 0 ? 1 : 0, out, xin, scal);
+                              dim3(ORB_T, ORB_TY), orbit_smem(), st, dim3(1, 1, nsl), y, g->ld,
+                              (const float4 *)g->d_trig, g->n, g->n_views, g->n_bins, nsl, mode != 0 ? 1 : 0, out, xin,
+                              scal);
         return;
     }
     // one slice: the block's sums are complete and it writes the result;
     // several slices without a cluster: slice images, then k_orbit_reduce
     const int fin = nsl == 1 ? 1 + (mode != 0) : 0;
     counted(fin ? 1 : 2);
-    launch_kernel(al ? k_backproject_orbit<true> : k_backproject_orbit<false>, grd, dim3(ORB_T, ORB_TY), orbit_smem(),
-                  st, y, partial, g->d_trig, g->n, g->n_views, g->n_bins, nsl, fin, out, xin, scal);
+    launch_kernel(al ? k_backproject_orbit<true> : k_backproject_orbit<false>, grd, dim3(ORB_T, ORB_TY), orbit_smem(), st,
+                  y, g->ld, partial, g->d_trig, g->n, g->n_views, g->n_bins, nsl, fin, out, xin, scal);
     if (fin) return;
     const size_t NN = (size_t)g->n * g->n;
     launch_kernel(mode == 0 ? k_orbit_reduce<0> : k_orbit_reduce<1>, dim3((unsigned)((NN + 255) / 256), batch),
                   dim3(256), 0, st, (const float *)partial, out, xin, scal, NN, nsl);
 }
 
-void launch_backproject(const Geometry *g, const float *y, float *out, int mode,
+void launch_backproject(const Geometry *g, const float *y, int ld, float *out, int mode,
                         const float *xin, const double *scal, int batch, cudaStream_t st)
 {
     dim3 grd((g->n + BT - 1) / BT, (g->n + BT - 1) / BT, batch);
     counted();
     if (mode == 0)
-        k_backproject_tiles<0><<<grd, BTH, 0, st>>>(y, out, g->d_trig, g->n, g->n_views, g->n_bins, xin, scal);
+        k_backproject_tiles<0><<<grd, BTH, 0, st>>>(y, ld, out, g->d_trig, g->n, g->n_views, g->n_bins, xin, scal);
     else
-        k_backproject_tiles<1><<<grd, BTH, 0, st>>>(y, out, g->d_trig, g->n, g->n_views, g->n_bins, xin, scal);
+        k_backproject_tiles<1><<<grd, BTH, 0, st>>>(y, ld, out, g->d_trig, g->n, g->n_views, g->n_bins, xin, scal);
 }
 
 void kernel_attrs_joseph()
 {
-    cudaFuncSetAttribute(k_backproject_orbit<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
-    cudaFuncSetAttribute(k_backproject_orbit<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
-    cudaFuncSetAttribute(k_backproject_orbit_cl<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
-    cudaFuncSetAttribute(k_backproject_orbit_cl<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
+    for (auto k : {k_backproject_orbit<true>, k_backproject_orbit<false>})
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
+    for (auto k : {k_backproject_orbit_cl<true>, k_backproject_orbit_cl<false>})
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
     for (auto k : {k_project_quad<2>, k_project_quad<4>})
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, QUAD_SMEM_MAX);
     for (auto k : {k_project_qbal<2, false>, k_project_qbal<2, true>, k_project_qbal<4, false>, k_project_qbal<4, true>})

@@ -87,7 +87,7 @@ extern "C" ct_status ct_ramp_filter_noalloc(const ct_geometry *geom, const float
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     // k_hhat writes all p_fft entries, so the shared array needs no clearing
     ctpd::launch_hhat(g, taps, half_len, hhat, st);
-    ctpd::launch_filter_fft(g, hhat, in, out, nullptr, nullptr, 0, nullptr, batch, st, true);
+    ctpd::launch_filter_fft(g, hhat, in, out, nullptr, nullptr, 0, nullptr, batch, st, g->n_bins, true);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         ctpd::set_error("ct_ramp_filter_noalloc: %s", cudaGetErrorString(e));

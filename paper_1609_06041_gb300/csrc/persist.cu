@@ -62,7 +62,7 @@ static_assert(1 + ORB_GROUPS + TV_GROUPS <= 16, "named barriers 1..15");
 static_assert(ORB_GROUPS * ORB_TH == PS_THREADS, "whole groups");
 
 struct PSlice {
-    int N, V, B, P, nb, lowdose, al;
+    int N, V, B, ld, P, nb, lowdose;
     int n_row_items, n_col_items, qseg;   // qseg: one projector item per staged band pair (segment)
     int nsl, q16, orb_smem;
     int tv_tc, tv_tr, tv_ncb, tv_nrb, ntv, fgp;
@@ -112,7 +112,7 @@ __device__ __noinline__ void dual_item(const PSlice &S, int i, unsigned char *ps
     const int pair = i * (PS_THREADS / T) + sub, t = tid % T;
     float2 *buf = reinterpret_cast<float2 *>(psm) + (size_t)sub * fft_elems(P);
     const DualArgs a{S.hhat, S.tw, S.band, S.nb, S.b, S.mu, S.mu, S.mubar, S.winv, S.lowdose, S.views, S.scal, S.V,
-                     S.B};
+                     S.B, S.ld};
     dual_stage<P, false>(t, T, pair, 0, buf, a);
     dual_update<P, false, false>(GroupCtx{tid % GS, GS, 1 + g}, t, pair, 0, buf, a);
 }
@@ -129,11 +129,11 @@ __device__ __forceinline__ void run_item(const PSlice &S, int p, int k, int i, u
             const GroupCtx c{tid % ORB_TH, ORB_TH, 1 + g};
             unsigned char *sm = psm + (size_t)g * S.orb_smem;
             const int fin = S.nsl == 1 ? 2 : 0;
-            if (S.al)
-                orbit_body<true>(c, bx, by, bz, sm, S.mubar, S.orb, S.trig, S.N, S.V, S.B, S.nsl, fin, S.z, S.x,
+            if (S.ld == S.B)
+                orbit_body<true>(c, bx, by, bz, sm, S.mubar, S.ld, S.orb, S.trig, S.N, S.V, S.B, S.nsl, fin, S.z, S.x,
                                  S.scal);
             else
-                orbit_body<false>(c, bx, by, bz, sm, S.mubar, S.orb, S.trig, S.N, S.V, S.B, S.nsl, fin, S.z, S.x,
+                orbit_body<false>(c, bx, by, bz, sm, S.mubar, S.ld, S.orb, S.trig, S.N, S.V, S.B, S.nsl, fin, S.z, S.x,
                                   S.scal);
         }
     } else if (p == PH_OREDUCE) {
@@ -315,10 +315,10 @@ ct_status launch_persistent(int n, const ct_geometry *const *geoms, const float 
             S.N = g->n;
             S.V = g->n_views;
             S.B = g->n_bins;
+            S.ld = g->ld;
             S.P = g->p_fft;
             S.nb = proj_bands(g->n);
             S.lowdose = prm.mode == CT_LOWDOSE;
-            S.al = g->n_bins % 4 == 0;   // workspace buffers are 256-byte aligned
             S.n_row_items = g->n_row_items;
             S.n_col_items = g->n_col_items;
             S.nsl = orbit_slices(g, false);

@@ -36,7 +36,8 @@ UL layout(const Geometry *g, int S, int half, int iters, int ntv)
 {
     UL L;
     const size_t J = (size_t)g->n * g->n, I = (size_t)g->n_views * g->n_bins, F = sizeof(float);
-    L.ck_stride = (size_t)S * (4 * J + 2 * I);
+    const size_t Ip = (size_t)g->n_views * g->ld;   // mu_bar and dL/dr, the inputs of A^T
+    L.ck_stride = ((size_t)S * (3 * J + Ip + I) + 63) & ~(size_t)63;
     size_t o = 0;
     L.scal = o;  o += a256(sizeof(double) * S_COUNT);
     L.scal2 = o; o += a256(sizeof(double) * S_COUNT);
@@ -53,7 +54,7 @@ UL layout(const Geometry *g, int S, int half, int iters, int ntv)
     L.gm = o;    o += a256(F * S * I);
     L.gmb = o;   o += a256(F * S * I);
     L.gmu = o;   o += a256(F * S * I);
-    L.gr = o;    o += a256(F * S * I);
+    L.gr = o;    o += a256(F * S * Ip);
     L.gm1 = o;   o += a256(F * S * I);
     L.rr = o;    o += a256(F * S * I);
     L.vv = o;    o += a256(F * S * I);
@@ -75,13 +76,14 @@ struct CK {
 
 CK ck_at(char *ws, const UL &L, const Geometry *g, int S, int k)
 {
-    const size_t J = (size_t)g->n * g->n, I = (size_t)g->n_views * g->n_bins;
+    // x first, then mu_bar: both 16-byte aligned where the orbit backprojector serves (N even)
+    const size_t J = (size_t)g->n * g->n, I = (size_t)g->n_views * g->n_bins, Ip = (size_t)g->n_views * g->ld;
     float *base = (float *)(ws + L.ck) + (size_t)k * L.ck_stride;
     CK c;
     c.x = base;
-    c.mu = c.x + S * J;
-    c.mubar = c.mu + S * I;
-    c.p = c.mubar + S * I;
+    c.mubar = c.x + S * J;
+    c.p = c.mubar + S * Ip;
+    c.mu = c.p + S * 2 * J;
     return c;
 }
 
@@ -146,7 +148,7 @@ void backproject(const Geometry *g, const float *y, float *out, int mode, const 
                  int S, char *ws, const UL &L, cudaStream_t st)
 {
     if (orbit_ok(g)) launch_backproject_orbit(g, y, out, mode, xin, scal, S, (float *)(ws + L.orb), st);
-    else launch_backproject(g, y, out, mode, xin, scal, S, st);
+    else launch_backproject(g, y, g->ld, out, mode, xin, scal, S, st);
 }
 
 }  // namespace
@@ -190,7 +192,7 @@ extern "C" ct_status ct_unrolled_forward(const ct_geometry *geom, const float *b
     cudaMemsetAsync(c0.x, 0, sizeof(float) * S * J, st);
     cudaMemsetAsync(c0.mu, 0, sizeof(float) * S * I, st);
     cudaMemsetAsync(c0.p, 0, sizeof(float) * S * 2 * J, st);
-    launch_filter_fft(g, hhat, b, c0.mubar, nullptr, nullptr, 1, scal, S, st);      // mubar_0 = -sigma D b
+    launch_filter_fft(g, hhat, b, c0.mubar, nullptr, nullptr, 1, scal, S, st, g->ld);      // mubar_0 = -sigma D b
     const bool fused = tv_fused(tau, beta, mode, tv_iters);
     for (int k = 0; k < iters; ++k) {
         CK c = ck_at(ws, L, g, S, k), n = ck_at(ws, L, g, S, k + 1);
