@@ -29,7 +29,10 @@
  * caller (for example torch tensor storage), contiguous, 16-byte aligned;
  * the library never frees it.  Host pointers are marked "host".  A
  * geometry handle owns a few KB of device memory (per-view constants) on
- * the device that was current at creation; use it on that device only.
+ * the device that was current at creation; use it on that device only.  It
+ * also owns the pool of ct_project's and ct_backproject's stream-ordered
+ * scratch, which keeps up to 256 MB of freed scratch until the handle is
+ * destroyed.
  *
  * Streams.  `stream` is a cudaStream_t passed as void* (NULL = legacy
  * default stream).  Calls enqueue work and return without synchronising,
@@ -156,7 +159,9 @@ ct_status ct_geometry_get_tuning(const ct_geometry *geom, int *items_per_block, 
 
 /*
  * Forward projection sino = A img (A of Eq. 1; Joseph interpolation).
- * img: batch x N x N, sino: batch x V x B (overwritten).
+ * img: batch x N x N, sino: batch x V x B (overwritten).  Takes
+ * stream-ordered scratch for the band partial sums (none for images of up to
+ * 96 pixels a side in small batches); CT_ERR_OOM when that fails.
  */
 ct_status ct_project(const ct_geometry *geom, const float *img, float *sino,
                      int batch, void *stream);
@@ -183,6 +188,8 @@ ct_status ct_project_bands(const ct_geometry *geom, const float *img, float *par
  * Backprojection img = A^T sino (the A^T of Eq. 19), a pixel-driven gather
  * over the two rays around each pixel's detector coordinate; deterministic
  * and free of atomics.  sino: batch x V x B, img: batch x N x N (overwritten).
+ * With the default angles, N and V even and B % 4 != 0 it takes
+ * stream-ordered scratch for padded rows (CT_ERR_OOM when that fails).
  */
 ct_status ct_backproject(const ct_geometry *geom, const float *sino, float *img,
                          int batch, void *stream);

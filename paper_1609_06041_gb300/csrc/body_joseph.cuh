@@ -248,25 +248,24 @@ __device__ __forceinline__ void quad_stage(const Ctx &c, void *Qv, const float *
     }
 }
 
-// Walks ray position idx of view-pair item (v, vp) through the staged band
-// pair (steps s0 .. s1) and stores its band sums into the partial
-// slot out (V x B): ray d and its detector mirror B-1-d of view v and, for
-// vp >= 0, of view vp.  Positions map to rays in whole blocks of 8 cs
-// positions, where the eight lanes of a quarter warp take rays cs apart,
-// spreading their 16-byte loads over the bank groups; the last partial
-// block maps to itself.
+// Ray position idx of an item: rays d and its detector mirror B-1-d.
+// Positions map to rays in whole blocks of 8 stride positions, where the
+// eight lanes of a quarter warp take rays `stride` apart, spreading their
+// 16-byte loads over the bank groups; the last partial block maps to itself.
+__device__ __forceinline__ int quad_ray(int idx, int cs, int npair)
+{
+    const int blk = 8 * cs, b = idx / blk, r = idx - b * blk;
+    return (b + 1) * blk <= npair ? b * blk + (r & 7) * cs + (r >> 3) : idx;
+}
+
+// Walks rays d and dm = B-1-d of item `it` through the staged band pair
+// (steps s0 .. s1): the band sums of view v in (x, y) and, for vp >= 0, of
+// view vp in (z, w), ray d first (in x and z alone when dm == d).
 template <int ROWS, bool RAW>
-__device__ __forceinline__ void quad_position(const void *Q, int SP, const QuadItem &it, bool rows, int idx, int npair,
-                                              int N, int B, int s0, int s1, float h, float hq, unsigned top,
-                                              float *out)
+__device__ __forceinline__ float4 quad_sums(const void *Q, int SP, const QuadItem &it, bool rows, int d, int N, int B,
+                                            int s0, int s1, float h, float hq, unsigned top)
 {
     const float a = it.a, m = it.m, inv_m = it.inv_m;
-    const int cs = it.stride, v = it.v, vp = it.vp;
-    int d = idx;
-    {
-        const int blk = 8 * cs, b = idx / blk, r = idx - b * blk;
-        if ((b + 1) * blk <= npair) d = b * blk + (r & 7) * cs + (r >> 3);
-    }
     const int dm = B - 1 - d;
     float ov[2] = {0.0f, 0.0f}, op[2] = {0.0f, 0.0f};   // view v / vp: [0] ray d, [1] ray dm
 #pragma unroll
@@ -276,8 +275,8 @@ __device__ __forceinline__ void quad_position(const void *Q, int SP, const QuadI
         const float q = joseph_q(joseph_dp(dd, B), a, hq);
         int lo, hi;
         step_range(q, m, inv_m, h, -2.5f, (float)N + 0.5f, s0, s1, lo, hi);
-        const float4 r = vp >= 0 ? quad_walk<true, ROWS, RAW>(Q, SP, q, m, lo, hi, s0, h, top)
-                                 : quad_walk<false, ROWS, RAW>(Q, SP, q, m, lo, hi, s0, h, top);
+        const float4 r = it.vp >= 0 ? quad_walk<true, ROWS, RAW>(Q, SP, q, m, lo, hi, s0, h, top)
+                                    : quad_walk<false, ROWS, RAW>(Q, SP, q, m, lo, hi, s0, h, top);
         ov[which] += r.x;
         ov[1 - which] += r.y;
         if (rows) {
@@ -288,21 +287,28 @@ __device__ __forceinline__ void quad_position(const void *Q, int SP, const QuadI
             op[which] += r.w;
         }
     }
-    float *o = out + (size_t)v * B;
     if (dm == d) {
-        o[d] = ov[0] + ov[1];
-    } else {
-        o[d] = ov[0];
-        o[dm] = ov[1];
+        ov[0] = ov[0] + ov[1];
+        op[0] = op[0] + op[1];
     }
-    if (vp >= 0) {
-        float *o2 = out + (size_t)vp * B;
-        if (dm == d) {
-            o2[d] = op[0] + op[1];
-        } else {
-            o2[d] = op[0];
-            o2[dm] = op[1];
-        }
+    return make_float4(ov[0], ov[1], op[0], op[1]);
+}
+
+// quad_sums of position idx, stored into the partial slot out (V x B).
+template <int ROWS, bool RAW>
+__device__ __forceinline__ void quad_position(const void *Q, int SP, const QuadItem &it, bool rows, int idx, int npair,
+                                              int N, int B, int s0, int s1, float h, float hq, unsigned top,
+                                              float *out)
+{
+    const int d = quad_ray(idx, it.stride, npair), dm = B - 1 - d;
+    const float4 r = quad_sums<ROWS, RAW>(Q, SP, it, rows, d, N, B, s0, s1, h, hq, top);
+    float *o = out + (size_t)it.v * B;
+    o[d] = r.x;
+    if (dm != d) o[dm] = r.y;
+    if (it.vp >= 0) {
+        float *o2 = out + (size_t)it.vp * B;
+        o2[d] = r.z;
+        if (dm != d) o2[dm] = r.w;
     }
 }
 

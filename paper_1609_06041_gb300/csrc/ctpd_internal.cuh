@@ -72,6 +72,7 @@ struct Geometry {
     int qbounds_key;      // ... and 64 (4 steps per pass) + items per block
     unsigned long long *d_qtimes;   // device: the tuner's per-block start and end times while it measures
     double *h_angles;     // host copy
+    cudaMemPool_t pool;   // scratch of ct_project and ct_backproject (see ct_geometry_create)
     void *eps_cache;      // eigenbases of D for the error-tolerant form (eps.cu)
     void *proj_plans;     // the projector's launch shapes by batch size (k_joseph.cu)
     void *graph_cache;    // instantiated CUDA graphs of repeated solves (api.cu)
@@ -393,6 +394,9 @@ inline int proj_bands(int n) { return (n + PROJ_R - 1) / PROJ_R; }
 // unrolled form on sides that are not a multiple of 32).
 void launch_project_bands(const Geometry *g, const float *x, float *partial, int batch, cudaStream_t st,
                           bool plain = false);
+// out = A x of small images (project_direct_ok) in one launch, no partial sums.
+bool project_direct_ok(const Geometry *g, int batch);
+void launch_project_direct(const Geometry *g, const float *x, float *out, int batch, cudaStream_t st);
 // The geometry's cache of projector launch shapes; clear it when a tuning changes.
 void *proj_plans_create();
 void proj_plans_free(void *p);

@@ -177,6 +177,97 @@ k_project_quad(const float *__restrict__ x, const QuadItem *__restrict__ row_ite
                     col_items, n_col, N, V, B, pg, gpb, tpi, partial);
 }
 
+// A x of small images in one launch, without partial sums.  A block takes one
+// item: it stages all band pairs of the item's line class (at most
+// DIRECT_BANDS, 76 KB at N = 96), a thread walks one of a position's two rays
+// through one band pair, and the sums meet in shared memory, where each ray's
+// are added in quad_position's and k_band_reduce's order and scaled (the same
+// bits).  Such a projection is a call's latency: one kernel and no scratch,
+// instead of two kernels and an allocation (64^2 / 90 views: 21 us a call),
+// and walks as short as can be (8 items a block with both rays and all bands
+// on one thread took 10.5 us, six SMs busy).
+constexpr int DIRECT_BANDS = 3;
+constexpr int DIRECT_THREADS = 1024;
+
+__global__ void __launch_bounds__(DIRECT_THREADS)
+k_project_direct(const float *__restrict__ x, const QuadItem *__restrict__ row_items, int n_row,
+                 const QuadItem *__restrict__ col_items, int N, int V, int B, int tpi,
+                 const ViewP *__restrict__ views, float *__restrict__ out)
+{
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const bool rows = (int)blockIdx.x < n_row;
+    const QuadItem it = rows ? row_items[blockIdx.x] : col_items[blockIdx.x - n_row];
+    const int nb = quad_bands(N), SP = (N + 3) | 1, npair = (B + 1) / 2;
+    const float *img = x + (size_t)blockIdx.y * N * N;
+    for (int b = 0; b < nb; ++b)
+        quad_stage<false>(whole_block(), smraw + b * quad_smem(N), img, N, b * MR, rows);
+    float4 *red = reinterpret_cast<float4 *>(smraw + nb * quad_smem(N));   // [2 band + ray][position]
+    __syncthreads();
+    const int part = threadIdx.x / tpi, idx = threadIdx.x - part * tpi, b = part >> 1;
+    const int d = idx < npair ? quad_ray(idx, it.stride, npair) : 0, dm = B - 1 - d;
+    float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (idx < npair && !((part & 1) && dm == d)) {
+        const float q = joseph_q(joseph_dp((part & 1) ? dm : d, B), it.a, joseph_hq(N));
+        const int s0 = b * MR, s1 = min(s0 + MR, (N + 1) / 2) - 1;
+        const float h = joseph_h(N);
+        const unsigned top = (unsigned)(N + 2);
+        const void *Q = smraw + b * quad_smem(N);
+        int lo, hi;
+        step_range(q, it.m, it.inv_m, h, -2.5f, (float)N + 0.5f, s0, s1, lo, hi);
+        r = it.vp >= 0 ? quad_walk<true, 2, false>(Q, SP, q, it.m, lo, hi, s0, h, top)
+                       : quad_walk<false, 2, false>(Q, SP, q, it.m, lo, hi, s0, h, top);
+    }
+    red[part * tpi + idx] = r;
+    __syncthreads();
+    if (part != 0 || idx >= npair) return;
+    float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // view v: rays d, dm; view vp: rays d, dm
+    for (int k = 0; k < nb; ++k) {
+        const float4 u = red[2 * k * tpi + idx], v = red[(2 * k + 1) * tpi + idx];   // the walks of rays d and dm
+        float o0 = u.x + v.y, o1 = u.y + v.x;
+        float p0 = rows ? u.z + v.w : u.w + v.z, p1 = rows ? u.w + v.z : u.z + v.w;
+        if (dm == d) {   // one walk: both its sums are ray d's
+            o0 = u.x + u.y;
+            p0 = rows ? u.z + u.w : u.w + u.z;
+        }
+        acc.x += o0;
+        acc.y += o1;
+        acc.z += p0;
+        acc.w += p1;
+    }
+    float *o = out + (size_t)blockIdx.y * V * B + (size_t)it.v * B;
+    const float sc = views[it.v].scale;
+    o[d] = acc.x * sc;
+    if (dm != d) o[dm] = acc.y * sc;
+    if (it.vp >= 0) {
+        float *o2 = out + (size_t)blockIdx.y * V * B + (size_t)it.vp * B;
+        const float sp = views[it.vp].scale;
+        o2[d] = acc.z * sp;
+        if (dm != d) o2[dm] = acc.w * sp;
+    }
+}
+
+// Served by k_project_direct: the whole image's bands staged at once, the
+// threads of one item in a block, and few enough blocks that staging an
+// image per item does not show (16 x 64^2 / 90 views, 720 blocks: as fast as
+// the band-pair form and its reduction).
+bool project_direct_ok(const Geometry *g, int batch)
+{
+    const int nb = quad_bands(g->n), tpi = ((g->n_bins + 1) / 2 + 31) / 32 * 32;
+    return nb <= DIRECT_BANDS && 2 * nb * tpi <= DIRECT_THREADS &&
+           (long long)(g->n_row_items + g->n_col_items) * batch <= 8LL * g->n_sm;
+}
+
+static size_t direct_smem(int n, int tpi) { return quad_bands(n) * (quad_smem(n) + 2 * sizeof(float4) * tpi); }
+
+void launch_project_direct(const Geometry *g, const float *x, float *out, int batch, cudaStream_t st)
+{
+    const int tpi = ((g->n_bins + 1) / 2 + 31) / 32 * 32;
+    counted();
+    k_project_direct<<<dim3(g->n_row_items + g->n_col_items, batch), 2 * quad_bands(g->n) * tpi,
+                       direct_smem(g->n, tpi), st>>>(x, g->d_row_items, g->n_row_items, g->d_col_items, g->n,
+                                                     g->n_views, g->n_bins, tpi, g->d_views, out);
+}
+
 // The work-balanced form: block b takes units [total b / nb, total (b+1) / nb)
 // (see quad_balanced_body); its unit counter sits after the staged pairs.
 __device__ __forceinline__ unsigned long long global_time()
@@ -860,6 +951,8 @@ void launch_backproject(const Geometry *g, const float *y, int ld, float *out, i
 
 void kernel_attrs_joseph()
 {
+    cudaFuncSetAttribute(k_project_direct, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(DIRECT_BANDS * quad_smem(2 * MR * DIRECT_BANDS) + sizeof(float4) * DIRECT_THREADS));
     for (auto k : {k_backproject_orbit<true>, k_backproject_orbit<false>})
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
     for (auto k : {k_backproject_orbit_cl<true>, k_backproject_orbit_cl<false>})

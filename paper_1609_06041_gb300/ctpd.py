@@ -99,19 +99,22 @@ def _check(status):
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the raw handle: torch.cuda.current_stream() builds a Stream object, 3 us a call
+    torch.cuda._lazy_init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dev(t, name, shape_tail=None):
+    """The device address of a contiguous float32 CUDA tensor whose shape ends in shape_tail."""
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != torch.float32:
+    if t.dtype is not torch.float32:
         raise TypeError(f"{name} must be float32")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape_tail is not None and tuple(t.shape[-len(shape_tail):]) != tuple(shape_tail):
+    if shape_tail is not None and t.shape[-len(shape_tail):] != shape_tail:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected (..., {shape_tail})")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _buf(t, name, shape_tail=None):
@@ -123,11 +126,13 @@ def _buf(t, name, shape_tail=None):
             raise TypeError(f"{name} must be contiguous float32")
         if shape_tail is not None and tuple(t.shape[-len(shape_tail):]) != tuple(shape_tail):
             raise ValueError(f"{name} has shape {tuple(t.shape)}, expected (..., {shape_tail})")
-        return ctypes.c_void_p(t.data_ptr())
+        return t.data_ptr()
     return _dev(t, name, shape_tail)
 
 
 def _batch(t, ndim_tail):
+    if t.dim() == ndim_tail:
+        return 1
     b = 1
     for s in t.shape[:-ndim_tail]:
         b *= s
@@ -240,8 +245,10 @@ def ct_project(g: Geometry, img: torch.Tensor, out: torch.Tensor | None = None) 
     pi = _dev(img, "img", (g.n, g.n))
     if out is None:
         out = torch.empty(*img.shape[:-2], g.n_views, g.n_bins, device=img.device, dtype=torch.float32)
-    po = _dev(out, "out", (g.n_views, g.n_bins))
-    _check(_lib.ct_project(g.handle, pi, po, _batch(img, 2), _stream()))
+        po = out.data_ptr()
+    else:
+        po = _dev(out, "out", (g.n_views, g.n_bins))
+    _check(_lib.ct_project(g._h, pi, po, _batch(img, 2), _stream()))
     return out
 
 
@@ -265,8 +272,10 @@ def ct_backproject(g: Geometry, sino: torch.Tensor, out: torch.Tensor | None = N
     ps = _dev(sino, "sino", (g.n_views, g.n_bins))
     if out is None:
         out = torch.empty(*sino.shape[:-2], g.n, g.n, device=sino.device, dtype=torch.float32)
-    po = _dev(out, "out", (g.n, g.n))
-    _check(_lib.ct_backproject(g.handle, ps, po, _batch(sino, 2), _stream()))
+        po = out.data_ptr()
+    else:
+        po = _dev(out, "out", (g.n, g.n))
+    _check(_lib.ct_backproject(g._h, ps, po, _batch(sino, 2), _stream()))
     return out
 
 
@@ -288,8 +297,10 @@ def ct_ramp_filter(g: Geometry, taps: torch.Tensor, sino: torch.Tensor, out=None
     ps = _dev(sino, "sino", (g.n_views, g.n_bins))
     if out is None:
         out = torch.empty_like(sino)
-    po = _dev(out, "out", (g.n_views, g.n_bins))
-    _check(_lib.ct_ramp_filter(g.handle, pt, half, ps, po, _batch(sino, 2), _stream()))
+        po = out.data_ptr()
+    else:
+        po = _dev(out, "out", (g.n_views, g.n_bins))
+    _check(_lib.ct_ramp_filter(g._h, pt, half, ps, po, _batch(sino, 2), _stream()))
     return out
 
 

@@ -65,3 +65,25 @@ def test_solve_on_ragged_sides(N, V, B):
     xg, _ = P.ct_pdtv_solve(P.Geometry(N, V, B), to_gpu(b), to_gpu(w), prm)
     st, _ = O.pdtv(b, w, O.ramp_taps(0, V, B, tau, kappa), 0, 0.01, tau, 0.05, 5, 3, N)
     assert rel_l2(to_np(xg), st.x) <= 1e-3
+
+
+@pytest.mark.parametrize("kind", ["uniform", "custom"])
+@pytest.mark.parametrize("N,V,B,batch", [(1, 1, 1, 1), (5, 4, 9, 3), (17, 7, 24, 1), (32, 12, 47, 2), (33, 6, 340, 1),
+                                         (64, 90, 95, 1), (64, 11, 96, 40), (65, 10, 93, 1), (96, 8, 139, 2),
+                                         (96, 9, 341, 1)])
+def test_small_images_in_one_launch(N, V, B, batch, kind):
+    # up to three band pairs: ct_project adds the band sums itself, in band order, to the same bits (one launch, or
+    # two past the sizes that a block or the batch allows)
+    P = need_gpu()
+    import torch
+    ang = angles_of(kind, V)
+    g = P.Geometry(N, V, B, angles=ang)
+    xg = to_gpu(np.stack([f32(synth.random_image(N, 5 + i)) for i in range(batch)]))
+    parts = P.ct_project_bands(g, xg)
+    t = np.arange(V) * np.pi / V if ang is None else ang
+    rows = (4 * np.arange(V) <= V) | (4 * np.arange(V) >= 3 * V) if ang is None else np.abs(np.cos(t)) >= np.abs(np.sin(t))
+    scale = to_gpu(np.abs(1.0 / np.where(rows, np.cos(t), np.sin(t))))[:, None]
+    acc = torch.zeros_like(parts[:, 0])
+    for k in range(parts.shape[1]):
+        acc = acc + parts[:, k]
+    assert torch.equal(P.ct_project(g, xg), acc * scale)
