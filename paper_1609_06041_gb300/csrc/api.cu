@@ -244,8 +244,13 @@ void lanczos_norm(Op op, float *t, float *tp, float *w, size_t n, int k, double 
     launch_scalars(scal, SC_SET, sqrt((double)n), 0, 0, n0slot, st);
     for (int j = 0; j < k; ++j) {
         op(t, w);
-        launch_lanczos_step(w, tp, t, n, scal, base, n0slot, j, 0, partials, ticket, st);
-        launch_lanczos_step(w, tp, t, n, scal, base, n0slot, j, 1, partials, ticket, st);
+        // (the sinogram side's third buffer starts on an odd place when V B % 4 != 0)
+        if (n <= LANCZOS_FUSED && aligned16(w) && aligned16(tp) && aligned16(t)) {
+            launch_lanczos_fused(w, tp, t, n, scal, base, n0slot, j, st);
+        } else {
+            launch_lanczos_step(w, tp, t, n, scal, base, n0slot, j, 0, partials, ticket, st);
+            launch_lanczos_step(w, tp, t, n, scal, base, n0slot, j, 1, partials, ticket, st);
+        }
         float *x = tp;
         tp = t;
         t = w;
@@ -479,6 +484,7 @@ ct_status ct_geometry_create(int n, int n_views, int n_bins, const double *angle
         cudaGetLastError();
         g->n_sm = 1;
     }
+    g->orb_rule = orbit_slices_rule(g);
     g->h_angles = new double[n_views];
     // candidate-window margin of the backprojector (bins): a generous bound
     // on the float rounding of the Joseph coordinates at this size
@@ -641,7 +647,10 @@ ct_status ct_project(const ct_geometry *g, const float *img, float *sino, int ba
         return fail(CT_ERR_OOM, "ct_project: scratch allocation failed (%zu bytes)", bytes);
     }
     launch_project_bands(g, img, partial, batch, S(stream));
-    launch_band_reduce(g, partial, sino, 0, nullptr, nullptr, nullptr, batch, S(stream));
+    {
+        PdlScope pdl(true);   // launched as the projector ends; it waits for it
+        launch_band_reduce(g, partial, sino, 0, nullptr, nullptr, nullptr, batch, S(stream));
+    }
     cudaFreeAsync(partial, S(stream));
     return cuda_check("ct_project");
 }

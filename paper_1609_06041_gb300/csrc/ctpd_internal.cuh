@@ -62,6 +62,7 @@ struct Geometry {
                           // the rule; -1: the tuner found the rule's own shape best)
     int tune_qrows;       // projector steps per pass of a ray walk (2 or 4)
     int tune_orb;         // A^T orbit base-view slices (1..8), slices added in a cluster
+    int orb_rule;         // A^T base-view slices by the built-in rule
     int tune_orb_si;      // the same for the slice-image form (solves side by side, the persistent kernel)
     int tune_tv;          // fewest interior rows of a TV tile (4..64)
     int tune_qbal;        // projector form: 1 band pair per block, 2 work-balanced ranges (0: the rule)
@@ -413,12 +414,14 @@ void launch_band_reduce(const Geometry *g, const float *partial, float *out, int
 // form for solves run side by side, whose clusters would wait for a GPC's
 // SMs to free together.  The orbit form's y has rows of g->ld floats, zeros
 // past n_bins, 16-byte aligned (launch_pad_rows copies a sinogram so); the
-// general form's rows are ld floats apart.
+// general form's rows are ld floats apart.  slices > 0 fixes the slice count.
 bool orbit_ok(const Geometry *g);
 size_t orbit_partial_floats(const Geometry *g, int batch);
 bool orbit_slices_ok(const Geometry *g, int nsl);
 void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int mode, const float *xin,
-                              const double *scal, int batch, float *partial, cudaStream_t st, bool cluster = true);
+                              const double *scal, int batch, float *partial, cudaStream_t st, bool cluster = true,
+                              int slices = 0);
+int orbit_slices_rule(const Geometry *g);
 void launch_pad_rows(const Geometry *g, const float *in, float *out, int batch, cudaStream_t st);
 void launch_backproject(const Geometry *g, const float *y, int ld, float *out, int mode,
                         const float *xin, const double *scal, int batch, cudaStream_t st);
@@ -574,6 +577,11 @@ void launch_lanczos_max(double *scal, int base, int k, int out, cudaStream_t st)
 // zero-initialised counter (left at zero).
 void launch_lanczos_step(float *w, const float *tp, const float *tc, size_t n, double *scal, int base, int n0slot,
                          int j, int phase, double *partials, unsigned *ticket, cudaStream_t st);
+// Both halves in one launch (a cluster of at most 8 blocks), to the same bits,
+// for vectors of at most LANCZOS_FUSED elements, 16-byte aligned.
+constexpr size_t LANCZOS_FUSED = 32768;
+void launch_lanczos_fused(float *w, const float *tp, const float *tc, size_t n, double *scal, int base, int n0slot,
+                          int j, cudaStream_t st);
 // w -= scal[slot] * q
 void launch_axpy_neg(float *w, const float *q, size_t n, const double *scal, int slot, cudaStream_t st);
 

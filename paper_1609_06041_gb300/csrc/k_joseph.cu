@@ -533,6 +533,7 @@ __global__ void k_band_reduce(const float *__restrict__ partial, float *__restri
                               const float *__restrict__ b, const float *__restrict__ winv,
                               const float *__restrict__ mu)
 {
+    pdl_wait();
     const int d = blockIdx.x * blockDim.x + threadIdx.x, v = blockIdx.y;
     if (d >= B) return;
     const size_t VB = (size_t)V * B;
@@ -547,18 +548,54 @@ __global__ void k_band_reduce(const float *__restrict__ partial, float *__restri
     out[o] = val;
 }
 
+// The plain sum (mode 0) for B % 4 == 0, four bins a thread and four bands'
+// loads together: with the projector before it, 512^2 / 720 views 70.3 -> 68.7
+// us, 1024^2 / 720 341.6 -> 329.9 (eight and sixteen bands together are slower,
+// 71.0 and 71.4 us: more rows of the partial sums open at once).
+constexpr int BR_BANDS = 4;
+__global__ void __launch_bounds__(256)
+k_band_reduce4(const float4 *__restrict__ partial, float4 *__restrict__ out, const ViewP *__restrict__ views, int nb,
+               unsigned vb4, unsigned b4)
+{
+    pdl_wait();
+    const unsigned i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= vb4) return;
+    const float4 *p = partial + (size_t)blockIdx.y * nb * vb4 + i;
+    float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int k0 = 0; k0 < nb; k0 += BR_BANDS) {
+        float4 t[BR_BANDS];
+#pragma unroll
+        for (int k = 0; k < BR_BANDS; ++k)
+            t[k] = k0 + k < nb ? p[(size_t)(k0 + k) * vb4] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int k = 0; k < BR_BANDS; ++k)
+            if (k0 + k < nb) {
+                acc.x += t[k].x;
+                acc.y += t[k].y;
+                acc.z += t[k].z;
+                acc.w += t[k].w;
+            }
+    }
+    const float s = views[i / b4].scale;
+    out[(size_t)blockIdx.y * vb4 + i] = make_float4(acc.x * s, acc.y * s, acc.z * s, acc.w * s);
+}
+
 void launch_band_reduce(const Geometry *g, const float *partial, float *out, int mode,
                         const float *b, const float *winv, const float *mu, int batch, cudaStream_t st)
 {
     dim3 grd((g->n_bins + 255) / 256, g->n_views, batch);
     const int nb = proj_bands(g->n);
     counted();
-    if (mode == 0)
-        k_band_reduce<0><<<grd, 256, 0, st>>>(partial, out, g->d_views, nb, g->n_views, g->n_bins, b, winv, mu);
-    else if (mode == 1)
-        k_band_reduce<1><<<grd, 256, 0, st>>>(partial, out, g->d_views, nb, g->n_views, g->n_bins, b, winv, mu);
-    else
-        k_band_reduce<2><<<grd, 256, 0, st>>>(partial, out, g->d_views, nb, g->n_views, g->n_bins, b, winv, mu);
+    const unsigned b4 = g->n_bins / 4, vb4 = b4 * g->n_views;
+    // below 20000 rays the grid of four-bin threads is too small (256^2 / 32 views: 7.6 against 7.3 us)
+    if (mode == 0 && g->n_bins % 4 == 0 && 4 * vb4 >= 20000 &&
+        (reinterpret_cast<uintptr_t>(partial) | reinterpret_cast<uintptr_t>(out)) % 16 == 0) {
+        launch_kernel(k_band_reduce4, dim3((vb4 + 255) / 256, batch), dim3(256), 0, st, (const float4 *)partial,
+                      (float4 *)out, g->d_views, nb, vb4, b4);
+        return;
+    }
+    launch_kernel(mode == 0 ? k_band_reduce<0> : mode == 1 ? k_band_reduce<1> : k_band_reduce<2>, grd, dim3(256), 0, st,
+                  partial, out, g->d_views, nb, g->n_views, g->n_bins, b, winv, mu);
 }
 
 // out = fac * A x from the band partials (fac: one device double)
@@ -772,7 +809,33 @@ bool orbit_slices_ok(const Geometry *g, int nsl)
 int orbit_slices(const Geometry *g, bool cluster)
 {
     const int t = cluster ? g->tune_orb : g->tune_orb_si;
-    return t > 0 ? t : ORB_SL;
+    return t > 0 ? t : g->orb_rule;
+}
+
+// The built-in count of base-view slices: the least modelled time of A^T of
+// one image, in us, over 1 .. 8 slices of `tiles` blocks each.  A block costs
+// about 0.3 and, per base view, 0.19 alone on its SM, 0.135 with another,
+// 0.118 as one of three and 0.105 of four and more, the most blocks of any SM
+// counting; adding the slices in a cluster costs 1.  (Warm launches: 512^2 /
+// 32 views 7.1 us with one slice, 8.2 with four; 64^2 / 90 6.1 with four, 4.7
+// with eight; 256^2 / 180 9.9 and 9.0; 512^2 / 720 and 384^2 / 90 keep four.)
+int orbit_slices_rule(const Geometry *g)
+{
+    if (!g->orbit) return ORB_SL;
+    const int q = (g->n / 2 + ORB_T - 1) / ORB_T, tiles = q * q;
+    const double per[] = {0.19, 0.135, 0.118, 0.105};
+    int best = ORB_SL;
+    double cost = -1.0;
+    for (int nsl = 1; nsl <= ORB_SL_MAX; ++nsl) {
+        if (!orbit_slices_ok(g, nsl)) continue;
+        const int k = (tiles * nsl + g->n_sm - 1) / g->n_sm;
+        const double c = k * ((double)(g->n_views / 2) / nsl * per[std::min(k, 4) - 1] + 0.3) + (nsl > 1 ? 1.0 : 0.0);
+        if (cost < 0.0 || c < cost) {
+            cost = c;
+            best = nsl;
+        }
+    }
+    return best;
 }
 size_t orbit_smem_bytes() { return orbit_smem(); }
 bool quad_ok(const Geometry *g) { return quad_smem(g->n, true) + 16 <= (size_t)QUAD_SMEM_MAX; }
@@ -910,11 +973,11 @@ void launch_pad_rows(const Geometry *g, const float *in, float *out, int batch, 
 }
 
 void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int mode, const float *xin,
-                              const double *scal, int batch, float *partial, cudaStream_t st, bool cluster)
+                              const double *scal, int batch, float *partial, cudaStream_t st, bool cluster, int slices)
 {
     const int q = g->n / 2;
     const bool cl = cluster || !partial;
-    const int nsl = orbit_slices(g, cl);
+    const int nsl = slices > 0 ? slices : orbit_slices(g, cl);
     dim3 grd((q + ORB_T - 1) / ORB_T, (q + ORB_T - 1) / ORB_T, nsl * batch);
     const bool al = g->ld == g->n_bins;
     if (nsl > 1 && cl) {

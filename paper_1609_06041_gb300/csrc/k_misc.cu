@@ -4,6 +4,8 @@
 
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
 #include "ctpd_internal.cuh"
 
 namespace ctpd {
@@ -224,6 +226,7 @@ __global__ void k_scalars(double *s, int op, double a0, double a1, double a2, in
 __global__ void k_lanczos_max(double *s, int base, int k, int out)
 {
     __shared__ float ta[LANCZOS_MAX], tb[LANCZOS_MAX];
+    __shared__ double y[LANCZOS_MAX], inv_d[LANCZOS_MAX], od[LANCZOS_MAX];
     const int lane = threadIdx.x;
     for (int j = lane; j < k; j += 32) {
         ta[j] = (float)s[base + 2 * j];
@@ -269,29 +272,25 @@ __global__ void k_lanczos_max(double *s, int base, int k, int out)
     // y by two steps of inverse iteration with theta I - T (positive definite,
     // as theta is above every eigenvalue of T): tridiagonal elimination in
     // double on this one thread.
+    // One elimination serves both steps: the pivots' reciprocals are the only
+    // divisions (with a division per element and step the kernel took 35 us).
     const double theta = (double)(hi * big) * (1.0 + 1e-6);
-    double y[LANCZOS_MAX], cp[LANCZOS_MAX];
-    for (int j = 0; j < k; ++j) y[j] = 1.0;
-    for (int itr = 0; itr < 2; ++itr) {
-        double m = theta - s[base];
-        if (!(m > 0.0)) m = 1e-300;
-        cp[0] = k > 1 ? -s[base + 1] / m : 0.0;
-        y[0] = y[0] / m;
-        for (int j = 1; j < k; ++j) {
-            const double sub = -s[base + 2 * j - 1];
-            double d = (theta - s[base + 2 * j]) - sub * cp[j - 1];
-            if (!(d > 0.0)) d = 1e-300;
-            cp[j] = j + 1 < k ? -s[base + 2 * j + 1] / d : 0.0;
-            y[j] = (y[j] - sub * y[j - 1]) / d;
-        }
-        for (int j = k - 2; j >= 0; --j) y[j] -= cp[j] * y[j + 1];
-        double nrm = 0.0;
-        for (int j = 0; j < k; ++j) nrm += y[j] * y[j];
-        nrm = sqrt(nrm);
-        if (!(nrm > 0.0) || !isfinite(nrm)) break;
-        for (int j = 0; j < k; ++j) y[j] /= nrm;
+    for (int j = 0; j < k; ++j) {
+        double d = theta - s[base + 2 * j];
+        if (j > 0) d -= od[j - 1] * od[j - 1] * inv_d[j - 1];
+        if (!(d > 0.0)) d = 1e-300;
+        inv_d[j] = 1.0 / d;
+        od[j] = s[base + 2 * j + 1];   // T's off-diagonal; theta I - T holds -od
+        y[j] = 1.0;
     }
-    const double res = fabs(s[base + 2 * (k - 1) + 1] * y[k - 1]);
+    for (int itr = 0; itr < 2; ++itr) {
+        for (int j = 1; j < k; ++j) y[j] = fma(od[j - 1] * inv_d[j - 1], y[j - 1], y[j]);
+        y[k - 1] *= inv_d[k - 1];
+        for (int j = k - 2; j >= 0; --j) y[j] = fma(od[j], y[j + 1], y[j]) * inv_d[j];
+    }
+    double nrm = 0.0;
+    for (int j = 0; j < k; ++j) nrm += y[j] * y[j];
+    const double res = fabs(od[k - 1] * y[k - 1]) / sqrt(nrm);
     s[out] = isfinite(res) ? theta + res : theta;
 }
 
@@ -314,6 +313,7 @@ k_lanczos_step(float *__restrict__ w, const float *__restrict__ tp, const float 
 {
     __shared__ bool last;
     __shared__ float coef[3];
+    pdl_wait();
     const float *x2 = phase == 0 ? tp : tc;
     const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
     const bool vec = ((reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(tc) |
@@ -396,7 +396,129 @@ void launch_lanczos_step(float *w, const float *tp, const float *tc, size_t n, d
     const size_t groups = (n + 4 * (size_t)DOT_THREADS - 1) / (4 * (size_t)DOT_THREADS);
     const int blocks = (int)std::min<size_t>(std::max<size_t>(groups, 1), DOT_BLOCKS);
     counted();
-    k_lanczos_step<<<blocks, DOT_THREADS, 0, st>>>(w, tp, tc, n, scal, base, n0slot, j, phase, partials, ticket);
+    launch_kernel(k_lanczos_step, dim3(blocks), dim3(DOT_THREADS), 0, st, w, tp, tc, n, scal, base, n0slot, j, phase,
+                  partials, ticket);
+}
+
+// Both halves of a Lanczos step in one launch of a thread-block cluster, for
+// vectors of at most LANCZOS_FUSED elements: the halves of k_lanczos_step are
+// two launches whose work (a 64^2 or 256^2 image) is far shorter than their
+// launch and their ticket.  Groups of 256 threads stand in for that kernel's
+// blocks, each forming the same partial (four elements a thread, the same
+// trees), and every block adds all partials in that kernel's order, so the
+// coefficients are the same to the bit.  Eight blocks take 32768 elements in
+// one pass, the limit; on a 512^2 image they need eight and lose to the two
+// launches by about 14 us a step (64^2 / 90 views, with k_lanczos_max and the
+// backprojector's slice rule: 685 -> 603 us a solve).  Partials of both halves sit in the
+// first block's shared memory (distributed shared memory).
+constexpr int LF_THREADS = 1024;
+constexpr int LF_PARTS = (int)(LANCZOS_FUSED / (4 * DOT_THREADS));   // stand-in blocks
+static_assert(LANCZOS_FUSED % (4 * DOT_THREADS) == 0 && LF_PARTS <= DOT_THREADS, "one partial per thread of a group");
+
+__global__ void __launch_bounds__(LF_THREADS)
+k_lanczos_fused(float *w, const float *tp, const float *tc, size_t n, double *s, int base, int n0slot, int j)
+{
+    namespace cg = cooperative_groups;
+    __shared__ float part[2][LF_PARTS];
+    __shared__ float wsum[LF_THREADS / 32];
+    __shared__ float total, coef[3];
+    pdl_wait();
+    cg::cluster_group cl = cg::this_cluster();
+    const int grp = threadIdx.x >> 8, t = threadIdx.x & 255, ng = LF_THREADS / DOT_THREADS;
+    const size_t n4 = n / 4, done = n4 * 4;
+    const int nparts = (int)((n + 4 * (size_t)DOT_THREADS - 1) / (4 * (size_t)DOT_THREADS));
+    float4 *w4 = reinterpret_cast<float4 *>(w);
+    const float4 *tc4 = reinterpret_cast<const float4 *>(tc), *tp4 = reinterpret_cast<const float4 *>(tp);
+    if (threadIdx.x == 0) {   // from the double slots once per block (FP64 is slow here)
+        const float n0 = (float)(j == 0 ? s[n0slot] : s[base + 2 * j - 1]);
+        const float nm = (float)(j <= 1 ? s[n0slot] : s[base + 2 * j - 3]);
+        coef[0] = n0 > 0.0f ? 1.0f / n0 : 0.0f;
+        coef[1] = (j > 0 && nm > 0.0f) ? n0 / nm : 0.0f;
+        coef[2] = n0;
+    }
+    __syncthreads();
+    float c1 = coef[0], c2 = coef[1];
+    const float nj = coef[2];
+    const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 1
+    for (int phase = 0; phase < 2; ++phase) {
+        const float4 *x4 = phase == 0 ? tp4 : tc4;
+        const float *x2 = phase == 0 ? tp : tc;
+        for (int b0 = blockIdx.x * ng; b0 < nparts; b0 += gridDim.x * ng) {   // uniform over the block
+            const int b = b0 + grp;
+            const size_t i = (size_t)b * DOT_THREADS + t;
+            float acc = 0.0f;
+            if (b < nparts && i < n4) {
+                float4 a = w4[i], x = x4[i];
+                const float4 tt = phase == 0 ? tc4[i] : zero;
+                if (c2 == 0.0f) x = zero;   // t_{-1} is never read (it may hold anything)
+                a.x = fmaf(-c2, x.x, a.x * c1);
+                a.y = fmaf(-c2, x.y, a.y * c1);
+                a.z = fmaf(-c2, x.z, a.z * c1);
+                a.w = fmaf(-c2, x.w, a.w * c1);
+                w4[i] = a;
+                const float4 d = phase == 0 ? tt : a;
+                acc = fmaf(a.x, d.x, acc);
+                acc = fmaf(a.y, d.y, acc);
+                acc = fmaf(a.z, d.z, acc);
+                acc = fmaf(a.w, d.w, acc);
+            }
+            if (b < nparts && done + i < n) {   // the last one to three elements
+                float wi = w[done + i] * c1;
+                if (c2 != 0.0f) wi = fmaf(-c2, x2[done + i], wi);
+                w[done + i] = wi;
+                acc = fmaf(wi, phase == 0 ? tc[done + i] : wi, acc);
+            }
+            const float v = warp_sum(acc);
+            if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v;
+            __syncthreads();
+            if (t == 0 && b < nparts) {
+                float q = 0.0f;
+#pragma unroll
+                for (int k = 0; k < DOT_THREADS / 32; ++k) q += wsum[grp * (DOT_THREADS / 32) + k];
+                *cl.map_shared_rank(&part[phase][b], 0) = q;
+            }
+            __syncthreads();
+        }
+        cl.sync();
+        // every block adds the partials, as k_lanczos_step's last block does
+        if (grp == 0) {
+            float v = 0.0f;
+            if (t < nparts) v += *cl.map_shared_rank(&part[phase][t], 0);
+            v = warp_sum(v);
+            if ((t & 31) == 0) wsum[t >> 5] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            float q = 0.0f;
+#pragma unroll
+            for (int k = 0; k < DOT_THREADS / 32; ++k) q += wsum[k];
+            total = q;
+        }
+        __syncthreads();
+        const float tf = total;
+        if (phase == 0) {
+            const float alpha = nj > 0.0f ? tf / nj : 0.0f;
+            c2 = nj > 0.0f ? alpha / nj : 0.0f;
+            c1 = 1.0f;
+            if (blockIdx.x == 0 && threadIdx.x == 0) s[base + 2 * j] = (double)alpha;
+        } else if (blockIdx.x == 0 && threadIdx.x == 0) {
+            s[base + 2 * j + 1] = (double)sqrtf(fmaxf(tf, 0.0f));
+        }
+    }
+    cl.sync();   // the first block's partials outlive every read of them
+}
+
+void launch_lanczos_fused(float *w, const float *tp, const float *tc, size_t n, double *scal, int base, int n0slot,
+                          int j, cudaStream_t st)
+{
+    const int ng = LF_THREADS / DOT_THREADS;
+    const int nparts = (int)((n + 4 * (size_t)DOT_THREADS - 1) / (4 * (size_t)DOT_THREADS));
+    int blocks = 1;
+    while (blocks < 8 && blocks * ng < nparts) blocks *= 2;
+    counted();
+    launch_kernel_cluster(k_lanczos_fused, dim3(blocks), dim3(LF_THREADS), 0, st, dim3(blocks), w, tp, tc, n, scal,
+                          base, n0slot, j);
 }
 
 __global__ void k_axpy_neg(float *w, const float *q, size_t n, const double *scal, int slot)

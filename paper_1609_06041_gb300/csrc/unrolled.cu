@@ -77,7 +77,7 @@ struct CK {
 CK ck_at(char *ws, const UL &L, const Geometry *g, int S, int k)
 {
     // x first, then mu_bar: both 16-byte aligned where the orbit backprojector serves (N even)
-    const size_t J = (size_t)g->n * g->n, I = (size_t)g->n_views * g->n_bins, Ip = (size_t)g->n_views * g->ld;
+    const size_t J = (size_t)g->n * g->n, Ip = (size_t)g->n_views * g->ld;
     float *base = (float *)(ws + L.ck) + (size_t)k * L.ck_stride;
     CK c;
     c.x = base;
@@ -147,7 +147,11 @@ void project(const Geometry *g, const float *x, float *band, int S, cudaStream_t
 void backproject(const Geometry *g, const float *y, float *out, int mode, const float *xin, const double *scal,
                  int S, char *ws, const UL &L, cudaStream_t st)
 {
-    if (orbit_ok(g)) launch_backproject_orbit(g, y, out, mode, xin, scal, S, (float *)(ws + L.orb), st);
+    // four slices unless tuned, whatever the image: the order its slice sums are added in, and so the gradients'
+    // bits, stay what they were
+    if (orbit_ok(g))
+        launch_backproject_orbit(g, y, out, mode, xin, scal, S, (float *)(ws + L.orb), st, true,
+                                 g->tune_orb > 0 ? 0 : 4);
     else launch_backproject(g, y, g->ld, out, mode, xin, scal, S, st);
 }
 
