@@ -516,8 +516,13 @@ void launch_tv_final(const float *z, const float *p, float *x, int n, int batch,
 // scalar slots, deterministically (scratch: pair_sums_scratch_floats()).
 void launch_tv_final_bwd(const float *z, const float *p, const float *gx, const float *gp_next, float *gz,
                          float *gp, int n, int batch, const double *scal, float *part, cudaStream_t st);
-void launch_tv_step_bwd(const float *z, const float *p, const float *gp_next, float *gz, float *gp, int n,
-                        int batch, const double *scal, float *part, cudaStream_t st);
+// The adjoints of the prox's steps l_hi, l_hi - 1, .. (steps of them, at most
+// tv_bwd_max_steps()) in one launch: p before step 0 is p0, before step l traj
+// + (l - 1) tstride; gp_next -> gp, gz added to in place.
+int tv_bwd_max_steps();
+void launch_tv_bwd(const float *z, const float *p0, const float *traj, size_t tstride, int l_hi, int steps,
+                   const float *gp_next, float *gz, float *gp, int n, int n_sm, int batch, const double *scal,
+                   float *part, cudaStream_t st);
 size_t pair_sums_scratch_floats();
 void launch_pair_sums(const float *part, size_t npairs, float *scratch, double *scal, int slot_a, int slot_b,
                       cudaStream_t st);

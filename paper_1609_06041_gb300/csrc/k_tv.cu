@@ -98,7 +98,6 @@ void launch_tv(const float *z, const float *p_in, float *p_out, float *x,
     launch_kernel(kern, grid, dim3(TV_THREADS), 0, st, z, p_in, p_out, x, n, steps, final_, t.tc, t.tr, scal, traj);
 }
 
-void kernel_attrs_tv() {}
 
 
 // =====================================================================
@@ -139,11 +138,10 @@ __device__ __forceinline__ float2 tv_q(const float *z, const float *px, const fl
 __device__ __forceinline__ float2 proj_adj(float2 q, float2 g)
 {
     const float n2 = fmaf(q.x, q.x, q.y * q.y);
-    if (n2 <= 1.0f) return g;
     const float inv = rsqrtf(n2);
     const float hx = q.x * inv, hy = q.y * inv;
     const float d = hx * g.x + hy * g.y;
-    return make_float2((g.x - hx * d) * inv, (g.y - hy * d) * inv);
+    return n2 <= 1.0f ? g : make_float2((g.x - hx * d) * inv, (g.y - hy * d) * inv);
 }
 
 // Block sums of the per-thread float terms va, vb: a fixed shuffle tree per
@@ -246,157 +244,287 @@ k_tv_final_bwd(const float *__restrict__ z, const float *__restrict__ p, const f
 //   gq = J_Pi(q)^T gp_next;   gx = -inv8 div gq;   gs = gx [s > 0];
 //   gz += gs;   gp = gq - lam grad gs;
 // and the derivative terms <gq, grad x> (for inv8) and <gs, div p> (for
-// lam).  One block per BT_W x BT_H tile: p is staged with a halo of two,
-// s with a halo of one (one more column and row on the far side), gq with
-// a halo of one and gs one column and row past the tile, each phase
-// reading only shared memory and the phase before.  The tile is 28 columns
-// wide so that every staged row fits one warp: lane = column, warp = row.
-constexpr int BT_W = 28, BT_H = 16;
-constexpr int BP_H = BT_H + 4;   // p: origin (r0 - 2, c0 - 2), 32 columns
-constexpr int BS_H = BT_H + 3;   // s: origin (r0 - 1, c0 - 1), 31 columns
-constexpr int BQ_H = BT_H + 2;   // gq: origin (r0 - 1, c0 - 1), 30 columns
-constexpr int BG_H = BT_H + 1;   // gs: origin (r0, c0), 29 columns
-
-// INT: the tile and its halos lie inside the image, one cell away from the
-// last row and column (r0 >= 2, c0 >= 2, r0 + BT_H + 3 <= N, c0 + 31 <= N),
-// so every bounds and boundary test below is true and is left out.
-struct BwdTile {   // the staged regions (one per block, shared by both paths)
-    float PX[BP_H][32], PY[BP_H][32], SS[BS_H][32], QX[BQ_H][32], QY[BQ_H][32], GS[BG_H][32];
+// lam).
+//
+// Several steps run per launch, temporally blocked as the prox itself
+// (body_tv.cuh): a block holds a region of 64 columns by 16 J rows, lane l
+// the columns 2l and 2l + 1, warp w the J rows from w J, with z, gz and gp in
+// registers; its interior is the region minus a halo of steps + 1 (rounded up
+// to even) on every side.  A step reads its p from shared memory, copied there
+// by cp.async while the step before it computes; it publishes gq_y of a
+// warp's last row (for gs below) and gs of its first row (for gp above), with
+// a barrier after each.  One step per launch staged every field with halos
+// and read and wrote the adjoints each time: 17.7 us a step on 16 x 256^2; five
+// steps take 48 us, bound by their instructions (64 % of the issue slots, 16
+// warps an SM).  Both forms of a warp's cells (border tests or none), no masks
+// on cells whose values go nowhere, and a branch-free projection adjoint took
+// the five steps there from 60 us.
+constexpr int TVB_J = 4;       // most region rows per warp: 5 spill
+constexpr int TVB_STEPS = 5;   // most steps per launch: halo 6, 52 interior columns
+__host__ __device__ __forceinline__ int tvb_halo(int steps) { return (steps + 2) & ~1; }
+struct TvbPub {
+    float2 gqy[TV_WARPS + 1][32];   // gq_y of warp w - 1's last row; entry 0: zeros
+    float2 gs[TV_WARPS + 1][32];    // gs of warp w's first row; the last entry: zeros
 };
+template <int J>
+constexpr size_t tvb_smem() { return sizeof(TvbPub) + sizeof(float) * 2 * 2 * TV_WARPS * J * 64; }
 
-template <bool INT>
-__device__ __forceinline__ void tv_step_bwd_tile(BwdTile &t, const float *__restrict__ z, const float *__restrict__ px,
-                                                 const float *__restrict__ py, const float *__restrict__ gnx,
-                                                 const float *__restrict__ gny, float *__restrict__ gz,
-                                                 float *__restrict__ ox, float *__restrict__ oy, int N, int r0,
-                                                 int c0, float lam, float inv8, float &c_inv8, float &c_lam)
+// p0: p before the prox's first step (l = 0); traj: p before step l at traj +
+// (l - 1) tstride.  Runs the adjoints of steps l_hi, l_hi - 1, .., l_hi - steps + 1.
+template <int J>
+__global__ void __launch_bounds__(TV_THREADS, 1)
+k_tv_bwd(const float *__restrict__ z, const float *__restrict__ p0, const float *__restrict__ traj, size_t tstride,
+         int l_hi, int steps, const float *__restrict__ gp_next, float *__restrict__ gz, float *__restrict__ gp, int N,
+         int tc, int tr, const double *__restrict__ scal, float *__restrict__ part)
 {
-    auto &PX = t.PX;
-    auto &PY = t.PY;
-    auto &SS = t.SS;
-    auto &QX = t.QX;
-    auto &QY = t.QY;
-    auto &GS = t.GS;
-    const int lx = threadIdx.x, ly = threadIdx.y;
-    auto in_img = [&](int v) { return INT || (unsigned)v < (unsigned)N; };
-    auto below_last = [&](int v) { return INT || v < N - 1; };   // a forward difference exists
-    auto above_first = [&](int v) { return INT || v > 0; };
-    // image column of this lane in each region, and whether it is inside
-    const int bp = c0 - 2 + lx, bs = c0 - 1 + lx, bg = c0 + lx;
-    const bool inp = in_img(bp), ins = lx < 31 && in_img(bs);
-    const bool inq = lx < 30 && in_img(bs), ing = lx < 29 && in_img(bg);
-    // div p at image cell (a, b) = region p cell (i, j) (zero outside the image)
-    auto div_p = [&](int i, int j, int a, int b) {
-        return ((below_last(b) ? PX[i][j] : 0.0f) - (above_first(b) ? PX[i][j - 1] : 0.0f)) +
-               ((below_last(a) ? PY[i][j] : 0.0f) - (above_first(a) ? PY[i - 1][j] : 0.0f));
-    };
-
-    for (int i = ly; i < BP_H; i += 8) {
-        const int a = r0 - 2 + i;
-        const bool in = inp && in_img(a);
-        const size_t gi = (size_t)a * N + bp;
-        PX[i][lx] = in ? px[gi] : 0.0f;
-        PY[i][lx] = in ? py[gi] : 0.0f;
-    }
-    // every global load of the block goes out before the first barrier
-    float zr[3], gnr[3][2], gzr[2];
-#pragma unroll
-    for (int m = 0; m < 3; ++m) {
-        const int i = ly + 8 * m, a = r0 - 1 + i;
-        const bool in = ins && in_img(a);
-        const size_t gi = (size_t)a * N + bs;
-        zr[m] = (i < BS_H && in) ? z[gi] : 0.0f;
-        gnr[m][0] = (i < BQ_H && lx < 30 && in) ? gnx[gi] : 0.0f;
-        gnr[m][1] = (i < BQ_H && lx < 30 && in) ? gny[gi] : 0.0f;
-    }
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-        const int a = r0 + ly + 8 * m;
-        gzr[m] = (lx < BT_W && (INT || (bg < N && a < N))) ? gz[(size_t)a * N + bg] : 0.0f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < 3; ++m) {   // s = z + lam div p
-        const int i = ly + 8 * m, a = r0 - 1 + i;
-        if (i < BS_H && lx < 31)
-            SS[i][lx] = (ins && in_img(a)) ? fmaf(lam, div_p(i + 1, lx + 1, a, bs), zr[m]) : 0.0f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < 3; ++m) {   // gq = J_Pi(q)^T gp_next
-        const int i = ly + 8 * m, a = r0 - 1 + i;
-        if (i >= BQ_H) break;
-        float2 g = make_float2(0.0f, 0.0f);
-        if (inq && in_img(a)) {
-            const float x0 = fmaxf(0.0f, SS[i][lx]);
-            const float gxv = below_last(bs) ? fmaxf(0.0f, SS[i][lx + 1]) - x0 : 0.0f;
-            const float gyv = below_last(a) ? fmaxf(0.0f, SS[i + 1][lx]) - x0 : 0.0f;
-            const float2 q = make_float2(PX[i + 1][lx + 1] + gxv * inv8, PY[i + 1][lx + 1] + gyv * inv8);
-            g = proj_adj(q, make_float2(gnr[m][0], gnr[m][1]));
-            if (i >= 1 && i <= BT_H && lx >= 1 && lx <= BT_W) c_inv8 = fmaf(g.x, gxv, fmaf(g.y, gyv, c_inv8));
-        }
-        if (lx < 30) {
-            QX[i][lx] = g.x;
-            QY[i][lx] = g.y;
-        }
-    }
-    __syncthreads();
-    for (int i = ly; i < BG_H; i += 8) {   // gs = [s > 0] (-inv8 div gq)
-        const int a = r0 + i;
-        float v = 0.0f;
-        if (ing && in_img(a) && SS[i + 1][lx + 1] > 0.0f) {
-            const float d = ((below_last(bg) ? QX[i + 1][lx + 1] : 0.0f) - (above_first(bg) ? QX[i + 1][lx] : 0.0f)) +
-                            ((below_last(a) ? QY[i + 1][lx + 1] : 0.0f) - (above_first(a) ? QY[i][lx + 1] : 0.0f));
-            v = -inv8 * d;
-        }
-        if (lx < 29) GS[i][lx] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-        const int i = ly + 8 * m, a = r0 + i;
-        if (lx < BT_W && (INT || (bg < N && a < N))) {
-            const size_t gi = (size_t)a * N + bg;
-            const float gs0 = GS[i][lx];
-            gz[gi] = gzr[m] + gs0;
-            ox[gi] = QX[i + 1][lx + 1] - lam * (below_last(bg) ? GS[i][lx + 1] - gs0 : 0.0f);
-            oy[gi] = QY[i + 1][lx + 1] - lam * (below_last(a) ? GS[i + 1][lx] - gs0 : 0.0f);
-            c_lam = fmaf(gs0, div_p(i + 2, lx + 2, a, bg), c_lam);
-        }
-    }
-}
-
-__global__ void __launch_bounds__(256, 6)
-k_tv_step_bwd(const float *__restrict__ z, const float *__restrict__ p, const float *__restrict__ gp_next,
-              float *__restrict__ gz, float *__restrict__ gp, int N, const double *__restrict__ scal,
-              float *__restrict__ part)
-{
-    const int r0 = blockIdx.y * BT_H, c0 = blockIdx.x * BT_W;
+    extern __shared__ __align__(16) unsigned char tvsm[];
+    TvbPub &pub = *reinterpret_cast<TvbPub *>(tvsm);
+    float *P = reinterpret_cast<float *>(tvsm + sizeof(TvbPub));   // [buffer][x, y][row][column]
+    constexpr int ROWS = TV_WARPS * J;
+    constexpr unsigned FULL = 0xffffffffu;
+    pdl_wait();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int H = tvb_halo(steps), Sr = tr + 2 * H;
+    const int R0 = blockIdx.y * tr - H, C0 = blockIdx.x * tc - H, c0 = C0 + 2 * lane, l0 = w * J;
     const size_t NN = (size_t)N * N;
-    const float *px = p + blockIdx.z * 2 * NN;
-    const float *gnx = gp_next + blockIdx.z * 2 * NN;
-    float *ox = gp + blockIdx.z * 2 * NN;
+    z += blockIdx.z * NN;
+    gz += blockIdx.z * NN;
+    gp_next += blockIdx.z * 2 * NN;
+    gp += blockIdx.z * 2 * NN;
     const float lam = fscal(scal, F_LAMBDA), inv8 = fscal(scal, F_INV8LAM);
-    __shared__ BwdTile tile;
-    float c_inv8 = 0.0f, c_lam = 0.0f;
-    if (r0 >= 2 && c0 >= 2 && r0 + BT_H + 3 <= N && c0 + 31 <= N)
-        tv_step_bwd_tile<true>(tile, z + blockIdx.z * NN, px, px + NN, gnx, gnx + NN, gz + blockIdx.z * NN, ox, ox + NN,
-                               N, r0, c0, lam, inv8, c_inv8, c_lam);
-    else
-        tv_step_bwd_tile<false>(tile, z + blockIdx.z * NN, px, px + NN, gnx, gnx + NN, gz + blockIdx.z * NN, ox, ox + NN,
-                                N, r0, c0, lam, inv8, c_inv8, c_lam);
-    block_pair_to(c_inv8, c_lam, part);
+    bool in[2], lt[2], gt[2], own[2];   // columns: inside, before the last, after the first, interior of the tile
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int c = c0 + e, lj = 2 * lane + e;
+        in[e] = (unsigned)c < (unsigned)N;
+        lt[e] = c < N - 1;
+        gt[e] = c > 0;
+        own[e] = in[e] && lj >= H && lj < H + tc;
+    }
+    auto row_in = [&](int li) { return li < Sr && (unsigned)(R0 + li) < (unsigned)N; };
+
+    // the region's p before step l into buffer b (zeros outside the image)
+    auto fetch = [&](int l, int b) {
+        const float *src = (l == 0 ? p0 : traj + (size_t)(l - 1) * tstride) + blockIdx.z * 2 * NN;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const int li = l0 + j;
+            const size_t gi = (size_t)(R0 + li) * N + c0;
+            const bool ok = row_in(li);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                float *dst = P + ((b * 2 + k) * ROWS + li) * 64 + 2 * lane;
+                const float *sp = src + k * NN;
+                const unsigned sd = (unsigned)__cvta_generic_to_shared(dst);
+                if ((N & 1) == 0) {   // C0 is even: an aligned pair, inside or outside as a whole
+                    const int n = ok && in[0] ? 8 : 0;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(sd), "l"(n ? sp + gi : src), "r"(n)
+                                 : "memory");
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int n = ok && in[e] ? 4 : 0;
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(sd + 4 * e),
+                                     "l"(n ? sp + gi + e : src), "r"(n)
+                                     : "memory");
+                    }
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch(l_hi, 0);
+    for (int i = threadIdx.x; i < (int)(sizeof(TvbPub) / sizeof(float2)); i += TV_THREADS)
+        reinterpret_cast<float2 *>(tvsm)[i] = make_float2(0.0f, 0.0f);
+
+    float zr[J + 1][2], gzr[J][2], gx[J][2], gy[J][2];   // gx, gy: the adjoint field gp
+#pragma unroll
+    for (int j = 0; j <= J; ++j) {
+        const int li = l0 + j;
+        const bool rin = row_in(li), rown = li >= H && li < H + tr;
+        const size_t gi = (size_t)(R0 + li) * N + c0;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            zr[j][e] = rin && in[e] ? z[gi + e] : 0.0f;
+            if (j < J) {
+                gx[j < J ? j : 0][e] = rin && in[e] ? gp_next[gi + e] : 0.0f;
+                gy[j < J ? j : 0][e] = rin && in[e] ? gp_next[NN + gi + e] : 0.0f;
+                gzr[j < J ? j : 0][e] = rin && rown && own[e] ? gz[gi + e] : 0.0f;
+            }
+        }
+    }
+    FSum si[2], sl[2];   // <gq, grad x>, <gs, div p> of a column
+    si[0] = si[1] = sl[0] = sl[1] = FSum{0.0f, 0.0f};
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    const bool busy = l0 < Sr;
+    // No value of a cell outside the image, or beyond the region's good part,
+    // reaches an interior cell: its differences across the border are dropped
+    // and the halo takes the rest, so only the sums and the stores ask whether
+    // a cell is the tile's own.  Warps whose cells all have four neighbours in
+    // the image take the form without the border's tests.
+    const bool inner = C0 >= 1 && C0 + 64 < N && R0 + l0 >= 1 && R0 + l0 + J < N - 1;
+    for (int st = 0; st < steps; ++st) {
+        const int b = st & 1;
+        if (st + 1 < steps) fetch(l_hi - st - 1, b ^ 1);
+        const float *PX = P + (b * 2) * ROWS * 64 + 2 * lane, *PY = PX + ROWS * 64;
+        float s[J + 1][2], dv[J][2], qx[J][2], qy[J][2], gs[J][2];
+        float ti[2] = {0.0f, 0.0f}, tl[2] = {0.0f, 0.0f};
+        auto first = [&](auto form) {   // s and gq
+            constexpr bool INT = decltype(form)::value;
+            const bool lt0 = INT || lt[0], lt1 = INT || lt[1], gt0 = INT || gt[0];
+            float2 pu = l0 > 0 ? *reinterpret_cast<const float2 *>(PY + (l0 - 1) * 64) : make_float2(0.0f, 0.0f);
+            float px[J][2], py[J][2];
+#pragma unroll
+            for (int j = 0; j <= J; ++j) {   // s = z + lam div p, the run and the row below it
+                const int li = l0 + j, a = R0 + li;
+                const bool rlt = INT || a < N - 1, rgt = INT || a > 0;
+                float2 vx = make_float2(0.0f, 0.0f), vy = vx;
+                if (j < J || li < ROWS) {
+                    vx = *reinterpret_cast<const float2 *>(PX + li * 64);
+                    vy = *reinterpret_cast<const float2 *>(PY + li * 64);
+                }
+                const float left = __shfl_up_sync(FULL, vx.y, 1);
+                const float d0 = ((lt0 ? vx.x : 0.0f) - (gt0 ? left : 0.0f)) + ((rlt ? vy.x : 0.0f) - (rgt ? pu.x : 0.0f));
+                const float d1 = ((lt1 ? vx.y : 0.0f) - vx.x) + ((rlt ? vy.y : 0.0f) - (rgt ? pu.y : 0.0f));
+                s[j][0] = fmaf(lam, d0, zr[j][0]);
+                s[j][1] = fmaf(lam, d1, zr[j][1]);
+                if (j < J) {
+                    const int jj = j < J ? j : 0;
+                    px[jj][0] = vx.x;
+                    px[jj][1] = vx.y;
+                    py[jj][0] = vy.x;
+                    py[jj][1] = vy.y;
+                    dv[jj][0] = d0;
+                    dv[jj][1] = d1;
+                }
+                pu = vy;
+            }
+#pragma unroll
+            for (int j = 0; j < J; ++j) {   // gq = J_Pi(q)^T gp_next
+                const int li = l0 + j;
+                const bool rlt = INT || R0 + li < N - 1;
+                const float right = __shfl_down_sync(FULL, s[j][0], 1);
+                const bool rown = li >= H && li < H + tr;
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float x0 = fmaxf(0.0f, s[j][e]), sr = e == 0 ? s[j][1] : right;
+                    const float gxv = (e == 0 ? lt0 : lt1) ? fmaxf(0.0f, sr) - x0 : 0.0f;
+                    const float gyv = rlt ? fmaxf(0.0f, s[j + 1][e]) - x0 : 0.0f;
+                    const float2 q = make_float2(px[j][e] + gxv * inv8, py[j][e] + gyv * inv8);
+                    const float2 g = proj_adj(q, make_float2(gx[j][e], gy[j][e]));
+                    qx[j][e] = g.x;
+                    qy[j][e] = g.y;
+                    if (rown) ti[e] = fmaf(g.x, gxv, fmaf(g.y, gyv, ti[e]));
+                }
+            }
+            pub.gqy[w + 1][lane] = make_float2(qy[J - 1][0], qy[J - 1][1]);
+        };
+        auto second = [&](auto form) {   // gs
+            constexpr bool INT = decltype(form)::value;
+            const bool lt0 = INT || lt[0], lt1 = INT || lt[1], gt0 = INT || gt[0];
+            float2 qu = pub.gqy[w][lane];
+#pragma unroll
+            for (int j = 0; j < J; ++j) {   // gs = [s > 0] (-inv8 div gq)
+                const int li = l0 + j, a = R0 + li;
+                const bool rlt = INT || a < N - 1, rgt = INT || a > 0, rown = li >= H && li < H + tr;
+                const float left = __shfl_up_sync(FULL, qx[j][1], 1);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float ql = e == 0 ? left : qx[j][0], qup = e == 0 ? qu.x : qu.y;
+                    const float d = (((e == 0 ? lt0 : lt1) ? qx[j][e] : 0.0f) - ((e == 1 || gt0) ? ql : 0.0f)) +
+                                    ((rlt ? qy[j][e] : 0.0f) - (rgt ? qup : 0.0f));
+                    const float v = s[j][e] > 0.0f ? -inv8 * d : 0.0f;
+                    gs[j][e] = v;
+                    gzr[j][e] = gzr[j][e] + v;
+                    if (rown) tl[e] = fmaf(v, dv[j][e], tl[e]);
+                }
+                qu = make_float2(qy[j][0], qy[j][1]);
+            }
+            pub.gs[w][lane] = make_float2(gs[0][0], gs[0][1]);
+        };
+        auto third = [&](auto form) {   // gp
+            constexpr bool INT = decltype(form)::value;
+            const bool lt0 = INT || lt[0], lt1 = INT || lt[1];
+            const float2 dn = pub.gs[w + 1][lane];
+#pragma unroll
+            for (int j = 0; j < J; ++j) {   // gp = gq - lam grad gs
+                const bool rlt = INT || R0 + l0 + j < N - 1;
+                const float right = __shfl_down_sync(FULL, gs[j][0], 1);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float g0 = gs[j][e], gr = e == 0 ? gs[j][1] : right;
+                    const float gd = j + 1 < J ? gs[j + 1 < J ? j + 1 : 0][e] : (e == 0 ? dn.x : dn.y);
+                    gx[j][e] = qx[j][e] - lam * ((e == 0 ? lt0 : lt1) ? gr - g0 : 0.0f);
+                    gy[j][e] = qy[j][e] - lam * (rlt ? gd - g0 : 0.0f);
+                }
+            }
+        };
+        constexpr std::true_type yes{};
+        constexpr std::false_type no{};
+        if (busy) inner ? first(yes) : first(no);
+        __syncthreads();
+        if (busy) inner ? second(yes) : second(no);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");   // the next step's p
+        __syncthreads();
+        if (busy) inner ? third(yes) : third(no);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            fsum_add(si[e], ti[e]);
+            fsum_add(sl[e], tl[e]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        const int li = l0 + j;
+        if (li >= H && li < H + tr && row_in(li)) {
+            const size_t gi = (size_t)(R0 + li) * N + c0;
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                if (own[e]) {
+                    gz[gi + e] = gzr[j][e];
+                    gp[gi + e] = gx[j][e];
+                    gp[NN + gi + e] = gy[j][e];
+                }
+        }
+    }
+    // block sums of the derivative terms: a fixed shuffle tree per warp, then the warps in order
+    float va = 0.0f, vb = 0.0f;
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+        if (own[e]) {
+            va += si[e].s + si[e].c;
+            vb += sl[e].s + sl[e].c;
+        }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        va += __shfl_down_sync(FULL, va, o);
+        vb += __shfl_down_sync(FULL, vb, o);
+    }
+    float2 *red = &pub.gqy[0][0];   // read by every warp before the last barrier
+    if (lane == 0) red[w] = make_float2(va, vb);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        FSum ta{0.0f, 0.0f}, tb{0.0f, 0.0f};
+        for (int k = 0; k < TV_WARPS; ++k) {
+            fsum_add(ta, red[k].x);
+            fsum_add(tb, red[k].y);
+        }
+        const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        part[2 * blk] = ta.s + ta.c;
+        part[2 * blk + 1] = tb.s + tb.c;
+    }
 }
 
 namespace {
 dim3 tv_px_grid(int n, int batch) { return dim3((n + 31) / 32, (n + 7) / 8, batch); }
 }
 
-// partials (two floats per block) of the adjoint kernels: the larger grid
+// partials (two floats per block) of the adjoint kernels: the final step's grid, the larger one (its blocks hold 32 x
+// 8 pixels, k_tv_bwd's at least 34 x 8)
 size_t tv_px_blocks(int n, int batch)
 {
-    const size_t px = (size_t)((n + 31) / 32) * ((n + 7) / 8), tl = (size_t)((n + BT_W - 1) / BT_W) * ((n + BT_H - 1) / BT_H);
-    return 2 * std::max(px, tl) * batch;
+    return 2 * (size_t)((n + 31) / 32) * ((n + 7) / 8) * batch;
 }
 
 void launch_tv_step(const float *z, const float *p_in, float *p_out, int n, int batch, const double *scal,
@@ -419,12 +547,37 @@ void launch_tv_final_bwd(const float *z, const float *p, const float *gx, const 
     k_tv_final_bwd<<<tv_px_grid(n, batch), dim3(32, 8), 0, st>>>(z, p, gx, gp_next, gz, gp, n, scal, part);
 }
 
-void launch_tv_step_bwd(const float *z, const float *p, const float *gp_next, float *gz, float *gp, int n,
-                        int batch, const double *scal, float *part, cudaStream_t st)
+int tv_bwd_max_steps() { return TVB_STEPS; }
+
+void launch_tv_bwd(const float *z, const float *p0, const float *traj, size_t tstride, int l_hi, int steps,
+                   const float *gp_next, float *gz, float *gp, int n, int n_sm, int batch, const double *scal,
+                   float *part, cudaStream_t st)
 {
+    // row tiles by the least rows per warp times waves of blocks (one block an SM);
+    // the row below the run is computed too, hence j + 1
+    const int H = tvb_halo(steps), tc = 64 - 2 * H, ncb = (n + tc - 1) / tc;
+    int best_j = 0, best_tr = 0;
+    long best = -1;
+    for (int j = 2; j <= TVB_J; ++j) {
+        const int most = TV_WARPS * j - 2 * H;
+        if (most < 8) continue;
+        const int nrb = (n + most - 1) / most, tr = (n + nrb - 1) / nrb;
+        const long blocks = (long)ncb * nrb * batch, cost = (blocks + n_sm - 1) / n_sm * (j + 1);
+        if (best < 0 || cost < best) {
+            best = cost;
+            best_j = j;
+            best_tr = std::max(tr, 8);
+        }
+    }
+    const dim3 grid(ncb, (n + best_tr - 1) / best_tr, batch);
     counted();
-    k_tv_step_bwd<<<dim3((n + BT_W - 1) / BT_W, (n + BT_H - 1) / BT_H, batch), dim3(32, 8), 0, st>>>(
-        z, p, gp_next, gz, gp, n, scal, part);
+    auto go = [&](auto kern, size_t smem) {
+        launch_kernel(kern, grid, dim3(TV_THREADS), smem, st, z, p0, traj, tstride, l_hi, steps, gp_next, gz, gp, n, tc,
+                      best_tr, scal, part);
+    };
+    if (best_j == 2) go(k_tv_bwd<2>, tvb_smem<2>());
+    else if (best_j == 3) go(k_tv_bwd<3>, tvb_smem<3>());
+    else go(k_tv_bwd<4>, tvb_smem<4>());
 }
 
 // scal[slot_a] += sum of part[2 i], scal[slot_b] += sum of part[2 i + 1],
@@ -489,6 +642,13 @@ void launch_pair_sums(const float *part, size_t npairs, float *scratch, double *
     counted(2);
     k_pair_sums<<<PS_BLOCKS, 256, 0, st>>>(part, npairs, scratch);
     k_pair_final<<<1, 32, 0, st>>>(scratch, PS_BLOCKS, scal, slot_a, slot_b);
+}
+
+void kernel_attrs_tv()
+{
+    cudaFuncSetAttribute(k_tv_bwd<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tvb_smem<2>());
+    cudaFuncSetAttribute(k_tv_bwd<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tvb_smem<3>());
+    cudaFuncSetAttribute(k_tv_bwd<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tvb_smem<4>());
 }
 
 }  // namespace ctpd

@@ -301,8 +301,14 @@ extern "C" ct_status ct_unrolled_backward(const ct_geometry *geom, const float *
         const float *trn = tp(tv_iters);
         launch_tv_final_bwd(z, trn, gx, gp, gz, gp2, N, S, scal, part, st);
         part += npx;
-        for (int l = tv_iters - 1; l >= 0; --l) {
-            launch_tv_step_bwd(z, tp(l), gp2, gz, gp, N, S, scal, part, st);
+        // (p before step l >= 1 sits in the trajectory), in equal chunks of at most tv_bwd_max_steps()
+        const size_t tstride = (size_t)S * 2 * J;
+        int left = tv_iters;
+        for (int c_ = (tv_iters + tv_bwd_max_steps() - 1) / tv_bwd_max_steps(); c_ > 0; --c_) {
+            const int steps = (left + c_ - 1) / c_;
+            launch_tv_bwd(z, c.p, tv_iters > 1 ? traj_at(ws, L, g, S, tv_iters, k, 1) : nullptr, tstride, left - 1, steps,
+                          gp2, gz, gp, N, g->n_sm, S, scal, part, st);
+            left -= steps;
             part += npx;
             std::swap(gp, gp2);
         }
