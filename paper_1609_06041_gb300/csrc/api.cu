@@ -224,24 +224,23 @@ int quad_lane_stride(double a, int npair)
 }
 
 // Largest eigenvalue of the symmetric positive semi-definite operator `op`
-// (n-vectors) by k Lanczos steps from the all-ones vector, into scal[slot]:
+// (n-vectors) by k Lanczos steps, into scal[slot]:
 //   w = op(q_j) - beta_{j-1} q_{j-1};  alpha_j = <w, q_j>;  w -= alpha_j q_j;
 //   beta_j = |w|;  q_{j+1} = w / beta_j,
 // then the largest eigenvalue of the tridiagonal (alpha, beta) (Sturm
 // multisection).  The vectors are kept unnormalised (t_j = beta_{j-1} q_j,
-// t_0 = ones with norm sqrt(n)), the scaling folded into the two fused
+// t_0 of norm sqrt(n)), the scaling folded into the two fused
 // update-and-reduce kernels of each step.  Coefficients go to scal[base ..
 // base + 2k), the norm of t_0 to scal[n0slot].  t, tp, w are n-vector
 // buffers; the whole recurrence stays on the device.
+// t holds the start vector, scal[n0slot] its norm sqrt(n): +-1 by a hash of
+// the index, as the all-ones vector is invariant under the geometry's
+// rotations and reflections and has no component along a top eigenvector of
+// another symmetry class.
 template <class Op>
 void lanczos_norm(Op op, float *t, float *tp, float *w, size_t n, int k, double *scal, int base, int n0slot,
                   double *partials, unsigned *ticket, int slot, cudaStream_t st)
 {
-    // start vector: +-1 by a hash of the index (norm sqrt(n)); the all-ones
-    // vector is invariant under the geometry's rotations and reflections and
-    // has no component along a top eigenvector of another symmetry class
-    launch_fill_sign(t, n, st);
-    launch_scalars(scal, SC_SET, sqrt((double)n), 0, 0, n0slot, st);
     for (int j = 0; j < k; ++j) {
         op(t, w);
         // (the sinogram side's third buffer starts on an odd place when V B % 4 != 0)
@@ -961,44 +960,48 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
         cudaMemsetAsync(scal, 0, sizeof(double) * S_COUNT, st);
     }
     // the input checks: w > 0 and finite (low-dose), b finite; bits in the flag word
-    cudaMemsetAsync(flags, 0, sizeof(unsigned), st);
-    launch_check_inputs(b, lowdose ? w : nullptr, I, flags, st);
-    if (!prm->resume) {
-        cudaMemsetAsync(ticket, 0, sizeof(unsigned), st);
-        cudaMemsetAsync(ticket2, 0, sizeof(unsigned), st);
+    if (prm->resume) {
+        cudaMemsetAsync(flags, 0, sizeof(unsigned), st);
+        launch_check_inputs(b, lowdose ? w : nullptr, I, flags, st);
+    } else {
+        const bool norms = !(prm->sigma > 0.0);
+        float *sw = lowdose && norms ? aux : nullptr;   // W^-1/2 and the start vectors, for the norms below
+        launch_setup_data(b, lowdose ? w : nullptr, I, winv, sw, sw ? mu : nullptr, norms ? z : nullptr, J, partials,
+                          flags, ticket, ticket2, st);
         // mu_bar's row padding, where its kernels do not write it
         if (g->ld != g->n_bins && (epsf || !use_fft))
             cudaMemsetAsync(mubar, 0, sizeof(float) * (size_t)g->n_views * g->ld, st);
-        if (lowdose) {
-            launch_recip(w, winv, I, st);
-            launch_dot(winv, nullptr, I, scal, S_RED0, partials, st);
-            launch_scalars(scal, SC_KAPPA_FROM_SUM, (double)I, 0, 0, 0, st);
-        }
-        launch_scalars(scal, SC_TAU, prm->tau, (double)g->n_views, 0, mode, st);
-        if (sv_d) {
-            launch_taps(g, CT_TAPS_LOW_BAND, scal, 0.0, 0.0, taps, st);
-            launch_taps(g, CT_TAPS_HIGH_BAND, scal, 0.0, 0.0, taps2, st);
-            launch_sv_hhat(g, taps, taps2, half, hhat, hhat2, st);
-            launch_sv_scale(w, scal, sv, I, st);
-        } else if (prm->precond == 3) {
+        double kappa3 = 0.0;
+        if (prm->precond == 3) {
             // few-view smoothed ramp: Eq. 24's form with kappa = tau l (l the mean
-            // diagonal of A A^T, from the view constants), tau as SC_TAU sets it
+            // diagonal of A A^T, from the view constants), tau as the setup sets it
             double sa = 0.0;
             for (int v = 0; v < g->n_views; ++v) {
                 const double t = g->h_angles[v];
                 sa += 1.0 / std::max(fabs(cos(t)), fabs(sin(t)));
             }
             const double ell = (2.0 / 3.0) * ((double)g->n * g->n / g->n_bins) * (sa / g->n_views);
-            const double tau_h = prm->tau > 0.0 ? prm->tau : 0.01;
-            launch_scalars(scal, SC_SET, tau_h * ell, 0, 0, S_KAPPA, st);
-            launch_taps(g, CT_LOWDOSE, scal, 0.0, 0.0, taps, st);
-            if (use_fft) launch_hhat(g, taps, half, hhat, st);
-        } else {
-            if (prm->precond) launch_taps(g, mode, scal, 0.0, 0.0, taps, st);
-            else launch_fill(taps, 1.0f, 1, st);
-            if (use_fft) launch_hhat(g, taps, half, hhat, st);
+            kappa3 = (prm->tau > 0.0 ? prm->tau : 0.01) * ell;
         }
-        if (!(prm->sigma > 0.0)) {
+        {
+            PdlScope pdl(true);
+            launch_setup_scalars(scal, partials, mode, I, J, prm->tau, g->n_views, kappa3, norms ? sqrt((double)J) : 0.0,
+                                 sw ? sqrt((double)I) : 0.0, st);
+            if (sv_d) {
+                launch_taps(g, CT_TAPS_LOW_BAND, scal, 0.0, 0.0, taps, st);
+                launch_taps(g, CT_TAPS_HIGH_BAND, scal, 0.0, 0.0, taps2, st);
+            } else if (prm->precond) {
+                launch_taps(g, prm->precond == 3 ? CT_LOWDOSE : mode, scal, 0.0, 0.0, taps, st);
+            } else {
+                launch_fill(taps, 1.0f, 1, st);
+            }
+            if (!sv_d && use_fft) launch_hhat(g, taps, half, hhat, st);
+        }
+        if (sv_d) {
+            launch_sv_hhat(g, taps, taps2, half, hhat, hhat2, st);
+            launch_sv_scale(w, scal, sv, I, st);
+        }
+        if (norms) {
             // ||W^-1/2 D W^-1/2|| by Lanczos on the sinogram side (low-dose),
             // on a second stream beside the image-side run when D is applied
             // by FFT (the two then share no buffers)
@@ -1011,8 +1014,6 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
             if (lowdose) {
                 cudaStream_t s2 = st;
                 if (fk) s2 = fork_begin(fk, st);
-                float *sw = aux;
-                launch_sqrt(winv, sw, I, s2);
                 auto op_wdw = [&](const float *v, float *out) { filter(v, out, g->n_bins, sw, sw, 0, s2); };
                 lanczos_norm(op_wdw, mu, r, aux + I, I, nlz, scal, S_LZ2, S_LN0B, partials2, ticket2, S_NWDW, s2);
             }
@@ -1037,13 +1038,9 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
             }
             if (fk) fork_end(fk, st);
         }
-        launch_scalars(scal, SC_SIGMA, prm->sigma, rho, 0, mode, st);
-        launch_scalars(scal, SC_LAMBDA, lowdose ? prm->beta : 0.0, 0, 0, mode, st);
         // ---- x^0 = mu^0 = 0, p = 0; Step 1 at k = 0: mu_bar = -sigma D b ----
-        launch_fill(x_out, 0.0f, J, st);
-        launch_fill(pbuf[0], 0.0f, 2 * J, st);
-        launch_fill(pbuf[1], 0.0f, 2 * J, st);
-        launch_fill(mu, 0.0f, I, st);
+        launch_setup_finish(scal, prm->sigma, rho, mode, lowdose ? prm->beta : 0.0, x_out, pbuf[0], pbuf[1], J, mu, I,
+                            st);
         if (epsf) filter(b, r, g->n_bins, nullptr, nullptr, 1, st);   // its proximal map goes to mu_bar below
         else filter(b, mubar, g->ld, nullptr, nullptr, 1, st);
     }
@@ -1096,7 +1093,7 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
         if (epsf)
             launch_eps_step(g, mu, mu, g->n_bins, mubar, g->ld, r, eQ, eLam, prm->eps, scal, aux, es, ew2, epart, st);
     }
-    launch_scalars(scal, SC_SET, (double)(k0 + prm->iters), 0, 0, S_K, st);
+    launch_scalars(scal, SC_SET, (double)(k0 + prm->iters), 0, S_K, st);
     launch_check_finite(x_out, J, flags, CHK_NONFINITE_RESULT, st);
     launch_check_finite(mu, I, flags, CHK_NONFINITE_RESULT, st);   // x >= 0 clamps a diverged x, not mu
     cs = cuda_check("ct_pdtv_solve");

@@ -150,9 +150,9 @@ extern "C" ct_status ct_geometry_autotune(ct_geometry *g, int batch, void *strea
     }
     double *scal = reinterpret_cast<double *>(scalf);
     cudaMemsetAsync(scal, 0, sizeof(double) * S_COUNT, st);
-    launch_scalars(scal, SC_SET, 1.0, 0, 0, S_TAU, st);
-    launch_scalars(scal, SC_SET, 0.05, 0, 0, S_LAMBDA, st);
-    launch_scalars(scal, SC_SET, 1.0 / (8.0 * 0.05), 0, 0, S_INV8LAM, st);
+    launch_scalars(scal, SC_SET, 1.0, 0, S_TAU, st);
+    launch_scalars(scal, SC_SET, 0.05, 0, S_LAMBDA, st);
+    launch_scalars(scal, SC_SET, 1.0 / (8.0 * 0.05), 0, S_INV8LAM, st);
     launch_fill(x, 0.5f, J * batch, st);
     launch_fill(sino, 1.0f, (size_t)g->n_views * g->ld * batch, st);
     launch_fill(tvb, 0.0f, 6 * J, st);

@@ -480,8 +480,6 @@ void launch_dual_sv(const Geometry *g, const float2 *hs, const float2 *hd, const
                     cudaStream_t st);
 // s = sqrt(kappa w), kappa = scal[S_KAPPA]
 void launch_sv_scale(const float *w, const double *scal, float *s, size_t n, cudaStream_t st);
-// out[i] = +-1 from an integer hash of i (the Lanczos start vector)
-void launch_fill_sign(float *out, size_t n, cudaStream_t st);
 void kernel_attrs_fft();
 void launch_dual_fft_batched(const Geometry *g, const float2 *hhat, const float *partial, const float *b,
                              const float *mu_in, float *mu_out, float *mu_bar, const float *winv, int lowdose,
@@ -563,16 +561,26 @@ void launch_eps_step(const Geometry *g, const float *q, float *out, int ldo, flo
 // Small helpers
 void launch_fill(float *p, float v, size_t n, cudaStream_t st);
 void launch_recip(const float *w, float *winv, size_t n, cudaStream_t st);
-void launch_sqrt(const float *a, float *out, size_t n, cudaStream_t st);
 void launch_scale_by(const float *in, const float *s, int sqrt_s, float *out, size_t n, cudaStream_t st);
-// scal[slot] = sum(a .* b) (b may be NULL: sum(a)), deterministic two-pass.
-void launch_dot(const float *a, const float *b, size_t n, double *scal, int slot,
-                double *partials, cudaStream_t st);
-// scalar program: set tau/sigma/lambda from norms and parameters
-void launch_scalars(double *scal, int op, double a0, double a1, double a2, int i0,
-                    cudaStream_t st);
-enum { SC_KAPPA_FROM_SUM = 0, SC_TAU, SC_NORM_FROM_DOT, SC_SIGMA, SC_LAMBDA, SC_SET, SC_COPY,
-       SC_NORM_SQRT, SC_AXPY_SLOT };
+// A solve's setup around its Lanczos runs (n = V B).  First the input checks
+// into flags, winv = 1 / w with its partial sums (w NULL: neither), sw =
+// sqrt(winv), the start vectors t_sino (n) and t_img (n_img) (each may be
+// NULL), and the reductions' counters at zero; then kappa, tau and the start
+// vectors' norms (kappa > 0: given); at the end sigma, lambda and x = p0 = p1
+// = mu = 0.  partials: dot_partials_doubles().
+void launch_setup_data(const float *b, const float *w, size_t n, float *winv, float *sw, float *t_sino, float *t_img,
+                       size_t n_img, double *partials, unsigned *flags, unsigned *ticket, unsigned *ticket2,
+                       cudaStream_t st);
+void launch_setup_scalars(double *scal, const double *partials, int mode, size_t n, size_t n_img, double tau,
+                          int n_views, double kappa, double norm_img, double norm_sino, cudaStream_t st);
+void launch_setup_finish(double *scal, double sigma, double rho, int mode, double beta, float *x, float *p0,
+                         float *p1, size_t J, float *mu, size_t I, cudaStream_t st);
+// the unrolled form's scalars; acc_a, acc_b: accumulator slots, set to zero
+void launch_unrolled_scalars(double *scal, double *scal2, double tau, double sigma, double lam, int acc_a, int acc_b,
+                             cudaStream_t st);
+// one scalar: scal[i0] = a0 (SC_SET) or scal[i0] += a0 scal[(int)a1] (SC_AXPY_SLOT)
+enum { SC_SET = 0, SC_AXPY_SLOT };
+void launch_scalars(double *scal, int op, double a0, double a1, int i0, cudaStream_t st);
 // scal[out] = largest eigenvalue of the Lanczos tridiagonal of k steps with
 // coefficients at scal[base ..]
 void launch_lanczos_max(double *scal, int base, int k, int out, cudaStream_t st);
@@ -587,8 +595,6 @@ void launch_lanczos_step(float *w, const float *tp, const float *tc, size_t n, d
 constexpr size_t LANCZOS_FUSED = 32768;
 void launch_lanczos_fused(float *w, const float *tp, const float *tc, size_t n, double *scal, int base, int n0slot,
                           int j, cudaStream_t st);
-// w -= scal[slot] * q
-void launch_axpy_neg(float *w, const float *q, size_t n, const double *scal, int slot, cudaStream_t st);
 
 size_t dot_partials_doubles();
 void kernel_attrs_filter();

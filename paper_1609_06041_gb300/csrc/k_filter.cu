@@ -195,6 +195,7 @@ void kernel_attrs_filter()
 __global__ void k_taps(int mode, int m, int P, int B, const double *__restrict__ scal,
                        float tau_h, float kappa_h, float *__restrict__ taps)
 {
+    pdl_wait();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= B) return;
@@ -232,8 +233,8 @@ void launch_taps(const Geometry *g, int mode, const double *scal, double tau, do
     int threads = 256, warps_per = threads / 32;
     int blocks = (g->n_bins + warps_per - 1) / warps_per;
     counted();
-    k_taps<<<blocks, threads, 0, st>>>(mode, g->n_views, g->n_fft, g->n_bins, scal,
-                                       (float)tau, (float)kappa, taps);
+    launch_kernel(k_taps, dim3(blocks), dim3(threads), 0, st, mode, g->n_views, g->n_fft, g->n_bins, scal, (float)tau,
+                  (float)kappa, taps);
 }
 
 }  // namespace ctpd

@@ -40,18 +40,6 @@ void launch_recip(const float *w, float *winv, size_t n, cudaStream_t st)
     k_recip<<<grid_for(n, 256), 256, 0, st>>>(w, winv, n);
 }
 
-__global__ void k_sqrt(const float *a, float *out, size_t n)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        out[i] = sqrtf(a[i]);
-}
-
-void launch_sqrt(const float *a, float *out, size_t n, cudaStream_t st)
-{
-    counted();
-    k_sqrt<<<grid_for(n, 256), 256, 0, st>>>(a, out, n);
-}
-
 // s = sqrt(kappa w): the diagonal of the shift-variant preconditioner
 __global__ void k_sv_scale(const float *w, const double *scal, float *s, size_t n)
 {
@@ -66,25 +54,17 @@ void launch_sv_scale(const float *w, const double *scal, float *s, size_t n, cud
     k_sv_scale<<<grid_for(n, 256), 256, 0, st>>>(w, scal, s, n);
 }
 
-// out[i] = +-1 from a 32-bit integer hash of i (the lowbias32 mixing of
-// C. Wellons): a start vector with components in every symmetry class
-__global__ void k_fill_sign(float *out, size_t n)
+// +-1 from a 32-bit integer hash of i (the lowbias32 mixing of C. Wellons):
+// a start vector with components in every symmetry class
+__device__ __forceinline__ float hash_sign(size_t i)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        unsigned x = (unsigned)i * 2654435761u + 12345u;
-        x ^= x >> 16;
-        x *= 0x7feb352du;
-        x ^= x >> 15;
-        x *= 0x846ca68bu;
-        x ^= x >> 16;
-        out[i] = (x & 1u) ? 1.0f : -1.0f;
-    }
-}
-
-void launch_fill_sign(float *out, size_t n, cudaStream_t st)
-{
-    counted();
-    k_fill_sign<<<grid_for(n, 256), 256, 0, st>>>(out, n);
+    unsigned x = (unsigned)i * 2654435761u + 12345u;
+    x ^= x >> 16;
+    x *= 0x7feb352du;
+    x ^= x >> 15;
+    x *= 0x846ca68bu;
+    x ^= x >> 16;
+    return (x & 1u) ? 1.0f : -1.0f;
 }
 
 // out = in * s (sqrt_s: in * sqrt(s))
@@ -143,77 +123,171 @@ __device__ __forceinline__ float partials_sum(const double *partials, int np)
     return block_sum(t);
 }
 
-__global__ void __launch_bounds__(DOT_THREADS)
-k_dot_partial(const float *a, const float *b, size_t n, double *partials)
+// The float copies of the scalars the per-iteration kernels read
+__device__ __forceinline__ void float_copies(double *s)
 {
-    float acc = 0.0f;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        acc = fmaf(a[i], b ? b[i] : 1.0f, acc);
-    const float t = block_sum(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = (double)t;
-}
-
-__global__ void __launch_bounds__(DOT_THREADS) k_dot_final(const double *partials, int np, double *scal, int slot)
-{
-    const float t = partials_sum(partials, np);
-    if (threadIdx.x == 0) scal[slot] = (double)t;
-}
-
-void launch_dot(const float *a, const float *b, size_t n, double *scal, int slot,
-                double *partials, cudaStream_t st)
-{
-    counted();
-    k_dot_partial<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(a, b, n, partials);
-    counted();
-    k_dot_final<<<1, DOT_THREADS, 0, st>>>(partials, DOT_BLOCKS, scal, slot);
-}
-
-// One-thread scalar program (keeps the whole setup on the device, so a
-// solve needs no host round trip).
-__global__ void k_scalars(double *s, int op, double a0, double a1, double a2, int i0)
-{
-    switch (op) {
-    case SC_KAPPA_FROM_SUM:             // kappa = mean(1/w), a0 = count (Eq. 24)
-        s[S_KAPPA] = s[S_RED0] / a0;
-        break;
-    case SC_TAU:                        // a0 = given tau (> 0) ; a1 = m ; i0 = mode
-        if (a0 > 0.0) s[S_TAU] = a0;
-        else s[S_TAU] = (i0 == CT_LOWDOSE) ? 3.14159265358979323846 * s[S_KAPPA] / (2.0 * a1) : 0.01;
-        break;
-    case SC_NORM_FROM_DOT:              // s[i0] = Rayleigh quotient <v, Mv>, |v| = 1
-        s[i0] = s[S_RED0];
-        break;
-    case SC_SIGMA: {                    // a0 = given sigma ; a1 = rho ; i0 = mode
-        if (a0 > 0.0) { s[S_SIGMA] = a0; break; }
-        double bound = 1.0 / (s[S_TAU] * s[S_NADA]);
-        if (i0 == CT_LOWDOSE && s[S_NWDW] > 0.0) bound = fmin(bound, 2.0 / s[S_NWDW]);
-        s[S_SIGMA] = a1 * bound;
-        break;
-    }
-    case SC_LAMBDA: {                   // a0 = beta ; i0 = mode
-        double lam = (i0 == CT_LOWDOSE) ? s[S_TAU] * a0 : s[S_TAU];
-        s[S_LAMBDA] = lam;
-        s[S_INV8LAM] = lam > 0.0 ? 1.0 / (8.0 * lam) : 0.0;
-        break;
-    }
-    case SC_SET:
-        s[i0] = a0;
-        break;
-    case SC_COPY:                       // s[i0] = s[(int)a0]
-        s[i0] = s[(int)a0];
-        break;
-    case SC_NORM_SQRT:                  // s[i0] = sqrt(s[(int)a0])
-        s[i0] = sqrt(s[(int)a0]);
-        break;
-    case SC_AXPY_SLOT:                  // s[i0] += a0 * s[(int)a1]
-        s[i0] += a0 * s[(int)a1];
-        break;
-    }
     float *f = reinterpret_cast<float *>(s + S_F32);
     f[F_TAU] = (float)s[S_TAU];
     f[F_SIGMA] = (float)s[S_SIGMA];
     f[F_LAMBDA] = (float)s[S_LAMBDA];
     f[F_INV8LAM] = (float)s[S_INV8LAM];
+}
+
+// The solve's setup around its Lanczos runs, in three launches.  Each part is
+// an element-wise pass or a few scalars, far shorter than a launch; as a
+// chain of some fifteen kernels and memsets they cost a 64^2 / 90-view solve
+// (20 iterations) 21 of its 607 us.
+//
+// First: the input checks (w > 0 and finite, b finite; bits in the flag
+// word), W^-1 and, where the Lanczos runs follow, W^-1/2 and both start
+// vectors; partial sums of 1 / w by the deterministic reduction above.
+__global__ void __launch_bounds__(DOT_THREADS)
+k_setup_data(const float *b, const float *w, size_t n, float *winv, float *sw, float *t_sino, float *t_img,
+             size_t n_img, double *partials, unsigned *flags, unsigned *ticket, unsigned *ticket2)
+{
+    const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+    if (tid == 0) {   // the reductions' counters
+        *ticket = 0u;
+        *ticket2 = 0u;
+    }
+    unsigned f = 0;
+    float acc = 0.0f;
+    for (size_t i = tid; i < n; i += stride) {
+        if (!isfinite(b[i])) f |= CHK_NONFINITE_INPUT;
+        if (w) {
+            const float wi = w[i], v = 1.0f / wi;
+            if (!isfinite(wi)) f |= CHK_NONFINITE_INPUT;
+            else if (!(wi > 0.0f)) f |= CHK_WEIGHT_NOT_POSITIVE;
+            winv[i] = v;
+            if (sw) sw[i] = sqrtf(v);
+            acc += v;
+        }
+        if (t_sino) t_sino[i] = hash_sign(i);
+    }
+    if (t_img)
+        for (size_t i = tid; i < n_img; i += stride) t_img[i] = hash_sign(i);
+    f = __reduce_or_sync(0xffffffffu, f);
+    if ((threadIdx.x & 31) == 0 && f) atomicOr(flags, f);
+    if (!w) return;
+    const float t = block_sum(acc);
+    if (threadIdx.x == 0) partials[blockIdx.x] = (double)t;
+}
+
+// blocks of the first launch: at most DOT_BLOCKS, fewer where each thread then
+// has one element at most (the blocks left out would add zeros)
+static int setup_blocks(size_t n, size_t n_img)
+{
+    return (int)std::min<size_t>((std::max(n, n_img) + DOT_THREADS - 1) / DOT_THREADS, DOT_BLOCKS);
+}
+
+void launch_setup_data(const float *b, const float *w, size_t n, float *winv, float *sw, float *t_sino, float *t_img,
+                       size_t n_img, double *partials, unsigned *flags, unsigned *ticket, unsigned *ticket2,
+                       cudaStream_t st)
+{
+    counted();
+    launch_kernel(k_setup_data, dim3(setup_blocks(n, n_img)), dim3(DOT_THREADS), 0, st, b, w, n, winv, sw, t_sino, t_img, n_img,
+                  partials, flags, ticket, ticket2);
+}
+
+// Second: kappa = mean(1/w) (Eq. 24; low-dose) or the given one, tau, and the
+// norms of the Lanczos start vectors.
+__global__ void __launch_bounds__(DOT_THREADS)
+k_setup_scalars(double *s, const double *partials, int np, int mode, double n, double tau, double n_views, double kappa,
+                double norm_img, double norm_sino)
+{
+    pdl_wait();
+    const float t = mode == CT_LOWDOSE ? partials_sum(partials, np) : 0.0f;
+    if (threadIdx.x != 0) return;
+    if (mode == CT_LOWDOSE) {
+        s[S_RED0] = (double)t;
+        s[S_KAPPA] = s[S_RED0] / n;
+    }
+    if (tau > 0.0) s[S_TAU] = tau;
+    else s[S_TAU] = mode == CT_LOWDOSE ? 3.14159265358979323846 * s[S_KAPPA] / (2.0 * n_views) : 0.01;
+    if (kappa > 0.0) s[S_KAPPA] = kappa;
+    s[S_LN0] = norm_img;
+    s[S_LN0B] = norm_sino;
+    float_copies(s);
+}
+
+void launch_setup_scalars(double *scal, const double *partials, int mode, size_t n, size_t n_img, double tau,
+                          int n_views, double kappa, double norm_img, double norm_sino, cudaStream_t st)
+{
+    counted();
+    launch_kernel(k_setup_scalars, dim3(1), dim3(DOT_THREADS), 0, st, scal, partials, setup_blocks(n, n_img), mode,
+                  (double)n, tau, (double)n_views, kappa, norm_img, norm_sino);
+}
+
+// Third, after the norms: sigma and lambda (thread 0), and x = p = mu = 0.
+// The arrays start on 16-byte boundaries.
+__global__ void __launch_bounds__(256)
+k_setup_finish(double *s, double sigma, double rho, int mode, double beta, float *x, float *p0, float *p1, size_t J,
+               float *mu, size_t I)
+{
+    const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+    if (tid == 0) {
+        if (sigma > 0.0) {
+            s[S_SIGMA] = sigma;
+        } else {
+            double bound = 1.0 / (s[S_TAU] * s[S_NADA]);
+            if (mode == CT_LOWDOSE && s[S_NWDW] > 0.0) bound = fmin(bound, 2.0 / s[S_NWDW]);
+            s[S_SIGMA] = rho * bound;
+        }
+        const double lam = mode == CT_LOWDOSE ? s[S_TAU] * beta : s[S_TAU];
+        s[S_LAMBDA] = lam;
+        s[S_INV8LAM] = lam > 0.0 ? 1.0 / (8.0 * lam) : 0.0;
+        float_copies(s);
+    }
+    auto zero = [&](float *a, size_t n) {
+        for (size_t i = tid; i < n / 4; i += stride)
+            reinterpret_cast<float4 *>(a)[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (tid < n % 4) a[n / 4 * 4 + tid] = 0.0f;
+    };
+    zero(x, J);
+    zero(p0, 2 * J);
+    zero(p1, 2 * J);
+    zero(mu, I);
+}
+
+void launch_setup_finish(double *scal, double sigma, double rho, int mode, double beta, float *x, float *p0,
+                         float *p1, size_t J, float *mu, size_t I, cudaStream_t st)
+{
+    counted();
+    k_setup_finish<<<grid_for(std::max(2 * J, I) / 4 + 1, 256), 256, 0, st>>>(scal, sigma, rho, mode, beta, x, p0, p1,
+                                                                              J, mu, I);
+}
+
+// The scalars of the unrolled form: tau, sigma, lambda and -tau (the factor
+// of mu_bar's adjoint) with both accumulators at zero, and in s2 the factor
+// of a backprojection that adds.  (As eight launches, twice per forward and
+// backward: 36 us more in 6000 at 16 x 256^2.)
+__global__ void k_unrolled_scalars(double *s, double *s2, double tau, double sigma, double lam, int acc_a, int acc_b)
+{
+    s[S_TAU] = tau;
+    s[S_SIGMA] = sigma;
+    s[S_LAMBDA] = lam;
+    s[S_INV8LAM] = lam > 0.0 ? 1.0 / (8.0 * lam) : 0.0;
+    s[S_RED0] = -tau;
+    s[acc_a] = 0.0;
+    s[acc_b] = 0.0;
+    float_copies(s);
+    s2[S_TAU] = -1.0;
+    float_copies(s2);
+}
+
+void launch_unrolled_scalars(double *scal, double *scal2, double tau, double sigma, double lam, int acc_a, int acc_b,
+                             cudaStream_t st)
+{
+    counted();
+    k_unrolled_scalars<<<1, 1, 0, st>>>(scal, scal2, tau, sigma, lam, acc_a, acc_b);
+}
+
+// One-thread scalar program: s[i0] = a0, or s[i0] += a0 s[(int)a1].
+__global__ void k_scalars(double *s, int op, double a0, double a1, int i0)
+{
+    if (op == SC_SET) s[i0] = a0;
+    else s[i0] += a0 * s[(int)a1];
+    float_copies(s);
 }
 
 // Largest eigenvalue of the Lanczos tridiagonal T_k (diagonal s[base + 2j],
@@ -226,11 +300,14 @@ __global__ void k_scalars(double *s, int op, double a0, double a1, double a2, in
 __global__ void k_lanczos_max(double *s, int base, int k, int out)
 {
     __shared__ float ta[LANCZOS_MAX], tb[LANCZOS_MAX];
-    __shared__ double y[LANCZOS_MAX], inv_d[LANCZOS_MAX], od[LANCZOS_MAX];
+    __shared__ double y[LANCZOS_MAX], inv_d[LANCZOS_MAX], da[LANCZOS_MAX], od[LANCZOS_MAX];
+    pdl_wait();
     const int lane = threadIdx.x;
     for (int j = lane; j < k; j += 32) {
-        ta[j] = (float)s[base + 2 * j];
-        tb[j] = (float)s[base + 2 * j + 1];
+        da[j] = s[base + 2 * j];
+        od[j] = s[base + 2 * j + 1];   // T's off-diagonal; theta I - T holds -od
+        ta[j] = (float)da[j];
+        tb[j] = (float)od[j];
     }
     __syncwarp();
     float glo = 0.0f, ghi = 0.0f;
@@ -276,11 +353,10 @@ __global__ void k_lanczos_max(double *s, int base, int k, int out)
     // divisions (with a division per element and step the kernel took 35 us).
     const double theta = (double)(hi * big) * (1.0 + 1e-6);
     for (int j = 0; j < k; ++j) {
-        double d = theta - s[base + 2 * j];
+        double d = theta - da[j];
         if (j > 0) d -= od[j - 1] * od[j - 1] * inv_d[j - 1];
         if (!(d > 0.0)) d = 1e-300;
         inv_d[j] = 1.0 / d;
-        od[j] = s[base + 2 * j + 1];   // T's off-diagonal; theta I - T holds -od
         y[j] = 1.0;
     }
     for (int itr = 0; itr < 2; ++itr) {
@@ -297,7 +373,7 @@ __global__ void k_lanczos_max(double *s, int base, int k, int out)
 void launch_lanczos_max(double *scal, int base, int k, int out, cudaStream_t st)
 {
     counted();
-    k_lanczos_max<<<1, 32, 0, st>>>(scal, base, k, out);
+    launch_kernel(k_lanczos_max, dim3(1), dim3(32), 0, st, scal, base, k, out);
 }
 
 // One half of a Lanczos step on unnormalised vectors (t_j = n_j q_j with
@@ -521,23 +597,10 @@ void launch_lanczos_fused(float *w, const float *tp, const float *tc, size_t n, 
                           base, n0slot, j);
 }
 
-__global__ void k_axpy_neg(float *w, const float *q, size_t n, const double *scal, int slot)
-{
-    const float c = (float)scal[slot];
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        w[i] = fmaf(-c, q[i], w[i]);
-}
-
-void launch_axpy_neg(float *w, const float *q, size_t n, const double *scal, int slot, cudaStream_t st)
+void launch_scalars(double *scal, int op, double a0, double a1, int i0, cudaStream_t st)
 {
     counted();
-    k_axpy_neg<<<grid_for(n, 256), 256, 0, st>>>(w, q, n, scal, slot);
-}
-
-void launch_scalars(double *scal, int op, double a0, double a1, double a2, int i0, cudaStream_t st)
-{
-    counted();
-    k_scalars<<<1, 1, 0, st>>>(scal, op, a0, a1, a2, i0);
+    k_scalars<<<1, 1, 0, st>>>(scal, op, a0, a1, i0);
 }
 
 }  // namespace ctpd

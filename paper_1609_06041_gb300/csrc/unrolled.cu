@@ -115,14 +115,7 @@ ct_status check_args(const Geometry *g, const float *b, const float *w, int batc
 void set_scalars(double *scal, double *scal2, double tau, double sigma, double beta, int mode, cudaStream_t st)
 {
     const double lam = mode == CT_LOWDOSE ? tau * beta : tau;
-    launch_scalars(scal, SC_SET, tau, 0, 0, S_TAU, st);
-    launch_scalars(scal, SC_SET, sigma, 0, 0, S_SIGMA, st);
-    launch_scalars(scal, SC_SET, lam, 0, 0, S_LAMBDA, st);
-    launch_scalars(scal, SC_SET, lam > 0.0 ? 1.0 / (8.0 * lam) : 0.0, 0, 0, S_INV8LAM, st);
-    launch_scalars(scal, SC_SET, -tau, 0, 0, S_RED0, st);       // factor of mubar's adjoint
-    launch_scalars(scal, SC_SET, 0.0, 0, 0, U_LAMACC, st);
-    launch_scalars(scal, SC_SET, 0.0, 0, 0, U_INV8ACC, st);
-    launch_scalars(scal2, SC_SET, -1.0, 0, 0, S_TAU, st);       // backprojection that adds
+    launch_unrolled_scalars(scal, scal2, tau, sigma, lam, U_LAMACC, U_INV8ACC, st);
 }
 
 // The prox steps of one iteration run as one register-resident launch
@@ -324,7 +317,7 @@ extern "C" ct_status ct_unrolled_backward(const ct_geometry *geom, const float *
     launch_tapcorr_acc(gmb, b, -sigma, nullptr, nullptr, 0.0, S * V, g->n_bins, half_len, tcorr, tacc, st);
     launch_pair_sums(pa, npx * ncall / 2, psum, scal, U_INV8ACC, U_LAMACC, st);
     // dL/dbeta = dL/dlambda dlambda/dbeta, dL/dlambda = lamacc + inv8acc d(1/(8 lam))/dlam
-    if (lam > 0.0) launch_scalars(scal, SC_AXPY_SLOT, -1.0 / (8.0 * lam * lam), (double)U_INV8ACC, 0, U_LAMACC, st);
+    if (lam > 0.0) launch_scalars(scal, SC_AXPY_SLOT, -1.0 / (8.0 * lam * lam), (double)U_INV8ACC, U_LAMACC, st);
     launch_grad_out(tacc, nl, scal, U_LAMACC, lowdose ? tau : 0.0, grad, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
