@@ -30,9 +30,9 @@
  * the library never frees it.  Host pointers are marked "host".  A
  * geometry handle owns a few KB of device memory (per-view constants) on
  * the device that was current at creation; use it on that device only.  It
- * also owns the pool of ct_project's and ct_backproject's stream-ordered
- * scratch, which keeps up to 256 MB of freed scratch until the handle is
- * destroyed.
+ * also shares, with the device's other geometries, the pool of ct_project's
+ * and ct_backproject's stream-ordered scratch, which keeps up to 256 MB of
+ * freed scratch until the last of them is destroyed.
  *
  * Streams.  `stream` is a cudaStream_t passed as void* (NULL = legacy
  * default stream).  Calls enqueue work and return without synchronising,
@@ -188,8 +188,9 @@ ct_status ct_project_bands(const ct_geometry *geom, const float *img, float *par
  * Backprojection img = A^T sino (the A^T of Eq. 19), a pixel-driven gather
  * over the two rays around each pixel's detector coordinate; deterministic
  * and free of atomics.  sino: batch x V x B, img: batch x N x N (overwritten).
- * With the default angles, N and V even and B % 4 != 0 it takes
- * stream-ordered scratch for padded rows (CT_ERR_OOM when that fails).
+ * With the default angles and N and V even, all but small calls take
+ * stream-ordered scratch for the sinogram with its row pairs interleaved
+ * (without scratch they read it as it is, more slowly, to the same bits).
  */
 ct_status ct_backproject(const ct_geometry *geom, const float *sino, float *img,
                          int batch, void *stream);

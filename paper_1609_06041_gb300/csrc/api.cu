@@ -145,7 +145,7 @@ Layout layout(const Geometry *g, const ct_pdtv_params *prm)
     L.sv = o;       o += align256(sizeof(float) * I);
     L.winv = o;     o += align256(sizeof(float) * I);
     L.mu = o;       o += align256(sizeof(float) * I);
-    L.mubar = o;    o += align256(sizeof(float) * (size_t)g->n_views * g->ld);   // rows of ld: the input of A^T
+    L.mubar = o;    o += align256(sizeof(float) * (size_t)g->n_views * g->ld);   // the input of A^T (at_rows)
     L.r = o;        o += align256(sizeof(float) * I);
     L.z = o;        o += align256(sizeof(float) * J);
     L.u = o;        o += align256(sizeof(float) * J);
@@ -165,11 +165,51 @@ Layout layout(const Geometry *g, const ct_pdtv_params *prm)
 }
 
 // Stream-ordered scratch of ct_project and ct_backproject comes from a pool
-// of the geometry's own that keeps up to this much across synchronisations:
-// the device's default pool gives its memory back at every one, and the next
-// call's allocation then takes some 200 us (ct_project at 64^2, waited for
-// each time: 220 us).  The pool goes with the geometry.
+// that keeps up to this much across synchronisations: the device's default
+// pool gives its memory back at every one, and the next call's allocation
+// then takes some 200 us (ct_project at 64^2, waited for each time: 220 us).
+// The geometries of a device share one, so that a new geometry's first call
+// finds it filled; it goes with the last of them.
 constexpr unsigned long long SCRATCH_KEEP = 256ull << 20;
+constexpr int SCRATCH_DEVICES = 64;
+struct ScratchPool {
+    cudaMemPool_t pool;
+    int users;
+};
+std::mutex g_scratch_mu;
+ScratchPool g_scratch[SCRATCH_DEVICES];
+
+// NULL: the default pool serves instead
+cudaMemPool_t scratch_pool_acquire(int dev)
+{
+    if (dev < 0 || dev >= SCRATCH_DEVICES) return nullptr;
+    std::lock_guard<std::mutex> lock(g_scratch_mu);
+    ScratchPool &p = g_scratch[dev];
+    if (p.users == 0) {
+        cudaMemPoolProps pp = {};
+        pp.allocType = cudaMemAllocationTypePinned;
+        pp.location.type = cudaMemLocationTypeDevice;
+        pp.location.id = dev;
+        unsigned long long keep = SCRATCH_KEEP;
+        if (cudaMemPoolCreate(&p.pool, &pp) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            cudaMemPoolDestroy(p.pool);
+            return nullptr;
+        }
+    }
+    ++p.users;
+    return p.pool;
+}
+
+void scratch_pool_release(int dev)
+{
+    std::lock_guard<std::mutex> lock(g_scratch_mu);
+    if (--g_scratch[dev].users == 0) cudaMemPoolDestroy(g_scratch[dev].pool);
+}
 
 cudaError_t scratch_alloc(const Geometry *g, float **p, size_t bytes, cudaStream_t st)
 {
@@ -580,19 +620,7 @@ ct_status ct_geometry_create(int n, int n_views, int n_bins, const double *angle
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? CT_ERR_OOM : CT_ERR_CUDA;
     }
-    {
-        cudaMemPoolProps pp = {};
-        pp.allocType = cudaMemAllocationTypePinned;
-        pp.location.type = cudaMemLocationTypeDevice;
-        pp.location.id = g->device;
-        unsigned long long keep = SCRATCH_KEEP;
-        if (cudaMemPoolCreate(&g->pool, &pp) != cudaSuccess ||
-            cudaMemPoolSetAttribute(g->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaGetLastError();   // the default pool serves instead
-            if (g->pool) cudaMemPoolDestroy(g->pool);
-            g->pool = nullptr;
-        }
-    }
+    g->pool = scratch_pool_acquire(g->device);
     kernel_attrs_filter();
     kernel_attrs_tv();
     kernel_attrs_joseph();
@@ -618,7 +646,7 @@ void ct_geometry_destroy(ct_geometry *g)
     if (g->d_row_items) cudaFree(g->d_row_items);
     if (g->d_col_items) cudaFree(g->d_col_items);
     if (g->d_qbounds) cudaFree(g->d_qbounds);
-    if (g->pool) cudaMemPoolDestroy(g->pool);
+    if (g->pool) scratch_pool_release(g->device);
     eps_cache_free(g);
     graph_cache_free(g);
     proj_plans_free(g->proj_plans);
@@ -679,24 +707,24 @@ ct_status ct_backproject(const ct_geometry *g, const float *sino, float *img, in
         launch_backproject(g, sino, g->n_bins, img, 0, nullptr, nullptr, batch, S(stream));
         return cuda_check("ct_backproject");
     }
-    if (g->ld == g->n_bins) {
-        launch_backproject_orbit(g, sino, img, 0, nullptr, nullptr, batch, nullptr, S(stream));
+    // views v and v + V/2 interleaved first (stream-ordered scratch), 2 to 3 us at 512^2 / 720 views; small sinograms,
+    // and calls for which there is no scratch, are read in their own rows
+    const size_t bytes = sizeof(float) * (size_t)batch * g->n_views * g->ld;
+    float *pairs = nullptr;
+    if (!orbit_plain_rows(g, batch) && scratch_alloc(g, &pairs, bytes, S(stream)) != cudaSuccess) {
+        cudaGetLastError();
+        pairs = nullptr;
+    }
+    if (!pairs) {
+        launch_backproject_orbit(g, sino, img, 0, nullptr, nullptr, batch, nullptr, S(stream), true, 0, true);
         return cuda_check("ct_backproject");
     }
-    // a detector of n_bins % 4 != 0: the rows padded to 16 bytes first (stream-ordered scratch), 2 to 3 us at 512^2 /
-    // 720 views against 25 us that 4-byte window copies cost
-    const size_t bytes = sizeof(float) * (size_t)batch * g->n_views * g->ld;
-    float *padded = nullptr;
-    if (scratch_alloc(g, &padded, bytes, S(stream)) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(CT_ERR_OOM, "ct_backproject: scratch allocation failed (%zu bytes)", bytes);
-    }
-    launch_pad_rows(g, sino, padded, batch, S(stream));
+    launch_pair_rows(g, sino, pairs, batch, S(stream));
     {
         PdlScope pdl(true);
-        launch_backproject_orbit(g, padded, img, 0, nullptr, nullptr, batch, nullptr, S(stream));
+        launch_backproject_orbit(g, pairs, img, 0, nullptr, nullptr, batch, nullptr, S(stream));
     }
-    cudaFreeAsync(padded, S(stream));
+    cudaFreeAsync(pairs, S(stream));
     return cuda_check("ct_backproject");
 }
 
@@ -917,7 +945,7 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
     float *taps2 = (float *)(ws + L.taps2), *sv = (float *)(ws + L.sv);
     float2 *hhat2 = (float2 *)(ws + L.hhat2);
     // out = post .* D(pre .* in) * (mode 1 ? -sigma : 1), and D applied to A x given as band sums
-    auto filter = [&](const float *in, float *out, int ldo, const float *pre, const float *post, int md,
+    auto filter = [&](const float *in, float *out, Rows ldo, const float *pre, const float *post, int md,
                       cudaStream_t s_) {
         if (sv_d) launch_filter_sv(g, hhat, hhat2, sv, in, out, pre, post, md, scal, 1, s_, ldo);
         else if (use_fft) launch_filter_fft(g, hhat, in, out, pre, post, md, scal, 1, s_, ldo);
@@ -1021,12 +1049,12 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
             auto op_ada = [&](const float *v, float *out) {
                 launch_project_bands(g, v, band, 1, st);
                 if (sv_d) {
-                    launch_filter_sv_bands(g, hhat, hhat2, sv, band, mubar, 1, st, g->ld);
+                    launch_filter_sv_bands(g, hhat, hhat2, sv, band, mubar, 1, st, at_rows(g));
                 } else if (use_fft) {
-                    launch_filter_fft_bands(g, hhat, band, mubar, 1, st, g->ld);
+                    launch_filter_fft_bands(g, hhat, band, mubar, 1, st, at_rows(g));
                 } else {
                     launch_band_reduce(g, band, r, 0, nullptr, nullptr, nullptr, 1, st);
-                    launch_filter(g, taps, half, r, mubar, g->ld, nullptr, nullptr, 0, nullptr, 1, st);
+                    launch_filter(g, taps, half, r, mubar, at_rows(g), nullptr, nullptr, 0, nullptr, 1, st);
                 }
                 backproject(mubar, out, 0, nullptr);
             };
@@ -1042,7 +1070,7 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
         launch_setup_finish(scal, prm->sigma, rho, mode, lowdose ? prm->beta : 0.0, x_out, pbuf[0], pbuf[1], J, mu, I,
                             st);
         if (epsf) filter(b, r, g->n_bins, nullptr, nullptr, 1, st);   // its proximal map goes to mu_bar below
-        else filter(b, mubar, g->ld, nullptr, nullptr, 1, st);
+        else filter(b, mubar, at_rows(g), nullptr, nullptr, 1, st);
     }
     ct_status cs = cuda_check("ct_pdtv_solve setup");
     // error-tolerant form: D's eigenbasis (precond 1, 3; none for D = I),
@@ -1051,7 +1079,7 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
     float *es = (float *)(ws + L.eps), *ew2 = es + g->n_bins, *epart = ew2 + g->n_bins;
     if (cs == CT_OK && epsf && prm->precond != 0) cs = eps_basis(g, prm->precond, prm->tau, taps, st, &eQ, &eLam);
     if (cs == CT_OK && epsf && !prm->resume)
-        launch_eps_step(g, r, mubar, g->ld, nullptr, 0, nullptr, eQ, eLam, prm->eps, scal, aux, es, ew2, epart, st);
+        launch_eps_step(g, r, mubar, at_rows(g), nullptr, 0, nullptr, eQ, eLam, prm->eps, scal, aux, es, ew2, epart, st);
     if (cs != CT_OK) {
         if (trace_d) cudaFreeAsync(trace_d, st);
         if (owned) cudaFreeAsync(ws, st);
@@ -1091,7 +1119,7 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
         // error-tolerant form: mu^{k+1} = the proximal map of Algorithm 2's
         // update, mu_bar = 2 mu^{k+1} - mu^k
         if (epsf)
-            launch_eps_step(g, mu, mu, g->n_bins, mubar, g->ld, r, eQ, eLam, prm->eps, scal, aux, es, ew2, epart, st);
+            launch_eps_step(g, mu, mu, g->n_bins, mubar, at_rows(g), r, eQ, eLam, prm->eps, scal, aux, es, ew2, epart, st);
     }
     launch_scalars(scal, SC_SET, (double)(k0 + prm->iters), 0, S_K, st);
     launch_check_finite(x_out, J, flags, CHK_NONFINITE_RESULT, st);

@@ -299,7 +299,8 @@ struct DualArgs {
     int lowdose;
     const ViewP *views;
     const double *scal;
-    int V, B, ld;   // ld: row stride of mu_bar, zeros written past B
+    int V, B;
+    Rows rows;   // of mu_bar; zeros are written past B
 };
 
 template <int P, bool DBL>
@@ -338,7 +339,10 @@ __device__ __forceinline__ void dual_update(const Ctx &c, int t, int pair, int b
     const size_t o0 = so + (size_t)(has0 ? v0 : 0) * B, o1 = so + (size_t)(has1 ? v1 : 0) * B;
     const float *winv = g.winv, *mu_in = g.mu_in;
     float *mu = g.mu;
-    float *mb0 = g.mu_bar + ((size_t)by * V + (has0 ? v0 : 0)) * g.ld, *mb1 = has1 ? mb0 + g.ld : mb0;
+    float *mb0 = g.mu_bar + g.rows.row(by, has0 ? v0 : 0, V);
+    // the second view's row from the first's
+    const int m1 = has1 ? (int)((ptrdiff_t)g.rows.row(0, v1, V) - (ptrdiff_t)g.rows.row(0, v0, V)) : 0;
+    const int rs = g.rows.step();
     const float sp = fscal(g.scal, F_SIGMA) * (1.0f / (float)P);
     const float2 *stage = buf + (DBL ? fft_elems(P) : 0);
     int ph = 0;
@@ -374,14 +378,14 @@ __device__ __forceinline__ void dual_update(const Ctx &c, int t, int pair, int b
                 }
                 if (!KEEP || !lowdose) {   // Alg. 2: mu_bar = 2 mu' - mu, no second filter
                     mu[o0 + i] = n.x;
-                    mb0[i] = e.x;
+                    mb0[i * rs] = e.x;
                     if (has1) {
                         mu[o1 + i] = n.y;
-                        mb1[i] = e.y;
+                        mb0[i * rs + m1] = e.y;
                     }
                 }
-            } else if (i < g.ld && has0) {
-                mb0[i] = mb1[i] = 0.0f;
+            } else if (i < g.rows.ld && has0) {
+                mb0[i * rs] = mb0[i * rs + m1] = 0.0f;
             }
             v[r] = d;
         }
@@ -394,10 +398,10 @@ __device__ __forceinline__ void dual_update(const Ctx &c, int t, int pair, int b
         const int i = t + r * T;
         if (i < B && has0) {
             if constexpr (KEEP) mu[o0 + i] = mn[r].x;
-            mb0[i] = __fmaf_rn(-sp, v[r].x, KEEP ? mo[KEEP ? r : 0].x : mb0[i]);
+            mb0[i * rs] = __fmaf_rn(-sp, v[r].x, KEEP ? mo[KEEP ? r : 0].x : mb0[i * rs]);
             if (has1) {
                 if constexpr (KEEP) mu[o1 + i] = mn[r].y;
-                mb1[i] = __fmaf_rn(-sp, v[r].y, KEEP ? mo[KEEP ? r : 0].y : mb1[i]);
+                mb0[i * rs + m1] = __fmaf_rn(-sp, v[r].y, KEEP ? mo[KEEP ? r : 0].y : mb0[i * rs + m1]);
             }
         }
     }

@@ -468,26 +468,38 @@ __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool va
     const int n = valid ? 16 : 0;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sdst), "l"(src), "r"(n) : "memory");
 }
+__device__ __forceinline__ void cp_async4(float *dst, const float *src, bool valid)
+{
+    const unsigned sdst = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = valid ? 4 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(sdst), "l"(src), "r"(n) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int K>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(K) : "memory"); }
 
 // Body of block (bx, by, bz) (c.nth() = ORB_TH threads, as ORB_T x ORB_TY);
-// osm holds orbit_smem() bytes.  y: V rows of B values per image, ld floats
-// apart, ld a multiple of 4, zeros past the B-th, 16-byte aligned: so every
-// window, whose start is a multiple of 4, is copied in aligned 16-byte
-// pieces, each wholly on or wholly off the padded row (rows of B floats with
-// B % 4 != 0 were copied by 4-byte pieces: 92 us against 67 at 512^2 / 720
-// views, 738 and 736 bins).  AL: B % 4 == 0, which makes the mirrored windows'
-// place a constant (otherwise one more addition a view, 68.5 against 67 us).  CL: instead of storing its sums, the
+// osm holds orbit_smem() bytes.  FORM ORB_PAIR: y holds per image V/2 pairs
+// of rows, views v and v + V/2 interleaved, ld values each, ld a multiple of
+// 4, zeros past the B-th, 16-byte aligned: so every window, whose start is a
+// multiple of 4, is copied in aligned 16-byte pieces, each wholly on or
+// wholly off the padded row, and one 8-byte load serves both views (their
+// windows, places and weights are the same).  A load per view took 5 us more
+// a launch at 512^2 / 720 views / 736 bins (a 30-iteration solve's 42: 6669
+// -> 6453 us); ct_backproject, which interleaves its input first, 66.7 ->
+// 63.8 us there, 238 -> 224 at 1024^2.  ORB_PAIR4: also B % 4 == 0, which makes the mirrored
+// windows' place a constant (one addition a view less, 2 %).  ORB_PLAIN: y
+// holds rows of B values, ld = B apart, copied value by value (25 us more
+// there: for small sinograms).  CL: instead of storing its sums, the
 // block leaves them in osm, entry (k ORB_PX + j) ORB_TH + tid for rotation
 // k of the thread's pixel orbit j, for a cluster reduction over slices.
-template <bool AL, class Ctx, bool CL = false>
+enum { ORB_PLAIN = 0, ORB_PAIR, ORB_PAIR4 };
+template <int FORM, class Ctx, bool CL = false>
 __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz, unsigned char *osm, const float *y,
                                            int ld, float *partial, const float4 *trig, int N, int V, int B, int nsl,
                                            int fin, float *out, const float *xin, const double *scal)
 {
-    // raw[buffer][view][row (v, v+V/2)][window (e, mirror e, e90, mirror e90)][value]
+    // raw[buffer][view][window (e, mirror e, e90, mirror e90)][value][row (v, v+V/2)]
     float *raw = reinterpret_cast<float *>(osm);                               // 2 x ORB_VC x 8 x ORB_RW
     float4 *tt = reinterpret_cast<float4 *>(raw + 2 * ORB_VC * 8 * ORB_RW);    // 2 x ORB_VC
     int *wbs = reinterpret_cast<int *>(tt + 2 * ORB_VC);                       // ORB_MAXS x 2
@@ -501,7 +513,7 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
     const float h = 0.5f * (float)(N - 1), hb = 0.5f * (float)(B - 1), hb_lo = hb - 0.5f;
     const float xq = (float)c - h, yq = (float)r - h;               // P = (x, y); R90 P = (-y, x)
     const float *ys = y + (size_t)img * V * ld;
-    const int ms = AL ? 3 : (B - ORB_RW + 3) & 3;   // see the mirrored windows below
+    const int ms = FORM == ORB_PAIR4 ? 3 : (B - ORB_RW + 3) & 3;   // see the mirrored windows below
     const int vb0 = (int)((long long)V2 * slice / nsl), vb1 = (int)((long long)V2 * (slice + 1) / nsl);
     const int nvs = vb1 - vb0;
     float acc[ORB_PX][4];   // per pixel orbit: P, R90 P, R180 P, R270 P
@@ -537,14 +549,26 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
             const float4 T = trig[v0 + tid];
             tt[buf * ORB_VC + tid] = make_float4(T.x, T.y, T.z * T.z, T.z * T.w);
         }
-        constexpr int CH = ORB_RW / 4;   // copies per window
-        for (int k = tid; k < nv * 8 * CH; k += ORB_TH) {
-            const int q = k / CH, j = k - q * CH;
-            const int win = q & 3, row = (q >> 2) & 1, vi = q >> 3;
-            const int base = wbs[2 * (v0 - vb0 + vi) + (win >> 1)];
-            const int d = ((win & 1) ? B - ORB_RW + 3 - ms - base : base) + 4 * j;
-            const bool ok = d >= 0 && d < B;
-            cp_async16(dst0 + (size_t)q * ORB_RW + 4 * j, ys + (size_t)(v0 + vi + row * V2) * ld + (ok ? d : 0), ok);
+        if (FORM != ORB_PLAIN) {
+            constexpr int CH = ORB_RW / 2;   // copies per window
+            for (int k = tid; k < nv * 4 * CH; k += ORB_TH) {
+                const int q = k / CH, j = k - q * CH;
+                const int win = q & 3, vi = q >> 2;
+                const int base = wbs[2 * (v0 - vb0 + vi) + (win >> 1)];
+                const int d = ((win & 1) ? B - ORB_RW + 3 - ms - base : base) + 2 * j;
+                const bool ok = d >= 0 && d < B;
+                cp_async16(dst0 + 2 * (size_t)q * ORB_RW + 4 * j, ys + 2 * ((size_t)(v0 + vi) * ld + (ok ? d : 0)), ok);
+            }
+        } else {
+            for (int k = tid; k < nv * 8 * ORB_RW; k += ORB_TH) {
+                const int q = k / ORB_RW, j = k - q * ORB_RW;
+                const int win = q & 3, row = (q >> 2) & 1, vi = q >> 3;
+                const int base = wbs[2 * (v0 - vb0 + vi) + (win >> 1)];
+                const int d = ((win & 1) ? B - ORB_RW + 3 - ms - base : base) + j;
+                const bool ok = d >= 0 && d < B;
+                cp_async4(dst0 + 2 * ((size_t)(vi * 4 + win) * ORB_RW + j) + row,
+                          ys + (size_t)(v0 + vi + row * V2) * ld + (ok ? d : 0), ok);
+            }
         }
         cp_async_commit();
     };
@@ -565,10 +589,9 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
             for (int vi = 0; vi < nv; ++vi) {
                 const float4 T = tv[vi];
                 const int2 wb = *reinterpret_cast<const int2 *>(wbs + 2 * (v0 - vb0 + vi));
-                const float *t8 = tb + (size_t)vi * 8 * ORB_RW;   // [row][win][value]
-                const float *e_v = t8, *m_v = t8 + ORB_RW, *e9_v = t8 + 2 * ORB_RW, *m9_v = t8 + 3 * ORB_RW;
-                const float *e_w = t8 + 4 * ORB_RW, *m_w = t8 + 5 * ORB_RW, *e9_w = t8 + 6 * ORB_RW,
-                            *m9_w = t8 + 7 * ORB_RW;
+                // [window][value](view v, view v + V/2)
+                const float2 *e_v = reinterpret_cast<const float2 *>(tb) + (size_t)vi * 4 * ORB_RW, *m_v = e_v + ORB_RW,
+                             *e9_v = e_v + 2 * ORB_RW, *m9_v = e_v + 3 * ORB_RW;
                 // the orbit of the pixel at (x, y) = (xq, yy): e - 1/2 of P and of R90 P
                 auto orbit = [&](float yy, float &cP, float &c90, float &c180, float &c270) {
                     const float e = fmaf(xq, T.x, fmaf(yy, T.y, hb_lo));
@@ -583,14 +606,16 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
                     const float w0 = fmaxf(0.0f, fmaf(-g, T.z, T.w)), w1 = fmaxf(0.0f, fmaf(g, T.z, T.w));
                     const float w09 = fmaxf(0.0f, fmaf(-g9, T.z, T.w)), w19 = fmaxf(0.0f, fmaf(g9, T.z, T.w));
                     const unsigned km = ORB_RW - 5 + ms - k, km9 = ORB_RW - 5 + ms - k9;
-                    cP = fmaf(w0, e_v[k], fmaf(w1, e_v[k + 1], cP));             // P at v
-                    c180 = fmaf(w1, m_v[km], fmaf(w0, m_v[km + 1], c180));       // R180 P at v
-                    c90 = fmaf(w0, e_w[k], fmaf(w1, e_w[k + 1], c90));           // R90 P at v + V/2
-                    c270 = fmaf(w1, m_w[km], fmaf(w0, m_w[km + 1], c270));       // R270 P at v + V/2
-                    c90 = fmaf(w09, e9_v[k9], fmaf(w19, e9_v[k9 + 1], c90));     // R90 P at v
-                    c270 = fmaf(w19, m9_v[km9], fmaf(w09, m9_v[km9 + 1], c270)); // R270 P at v
-                    c180 = fmaf(w09, e9_w[k9], fmaf(w19, e9_w[k9 + 1], c180));   // R180 P at v + V/2
-                    cP = fmaf(w19, m9_w[km9], fmaf(w09, m9_w[km9 + 1], cP));     // P at v + V/2
+                    const float2 e0 = e_v[k], e1 = e_v[k + 1], m0 = m_v[km], m1 = m_v[km + 1];
+                    const float2 f0 = e9_v[k9], f1 = e9_v[k9 + 1], n0 = m9_v[km9], n1 = m9_v[km9 + 1];
+                    cP = fmaf(w0, e0.x, fmaf(w1, e1.x, cP));           // P at v
+                    c180 = fmaf(w1, m0.x, fmaf(w0, m1.x, c180));       // R180 P at v
+                    c90 = fmaf(w0, e0.y, fmaf(w1, e1.y, c90));         // R90 P at v + V/2
+                    c270 = fmaf(w1, m0.y, fmaf(w0, m1.y, c270));       // R270 P at v + V/2
+                    c90 = fmaf(w09, f0.x, fmaf(w19, f1.x, c90));       // R90 P at v
+                    c270 = fmaf(w19, n0.x, fmaf(w09, n1.x, c270));     // R270 P at v
+                    c180 = fmaf(w09, f0.y, fmaf(w19, f1.y, c180));     // R180 P at v + V/2
+                    cP = fmaf(w19, n0.y, fmaf(w09, n1.y, cP));         // P at v + V/2
                 };
 #pragma unroll
                 for (int j = 0; j < ORB_PX; ++j)

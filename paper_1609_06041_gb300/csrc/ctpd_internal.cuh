@@ -73,7 +73,7 @@ struct Geometry {
     int qbounds_key;      // ... and 64 (4 steps per pass) + items per block
     unsigned long long *d_qtimes;   // device: the tuner's per-block start and end times while it measures
     double *h_angles;     // host copy
-    cudaMemPool_t pool;   // scratch of ct_project and ct_backproject (see ct_geometry_create)
+    cudaMemPool_t pool;   // the device's, for the scratch of ct_project and ct_backproject (NULL: the default pool)
     void *eps_cache;      // eigenbases of D for the error-tolerant form (eps.cu)
     void *proj_plans;     // the projector's launch shapes by batch size (k_joseph.cu)
     void *graph_cache;    // instantiated CUDA graphs of repeated solves (api.cu)
@@ -369,6 +369,24 @@ size_t orbit_smem_bytes();                      // shared memory of one orbit bl
 bool quad_ok(const Geometry *g);                // the mirrored projector serves this geometry (N <= about 1800)
 // TV prox tiles of one image spread over n_sm blocks (k_tv.cu's rule)
 void tv_tile_shape(int n, int steps, int n_sm, int min_rows, int *tc, int *tr, int *ncb, int *nrb, int rows = 0);
+// How a sinogram's rows lie: row v of image `img` starts at row() and its
+// elements are step() floats apart.  half 0: rows ld floats apart.  half > 0
+// (= V / 2; the orbit backprojector's input, which reads views v and v + half
+// at the same places): the two rows interleaved, 2 ld floats a pair.
+struct Rows {
+    int ld, half;
+    __host__ __device__ Rows(int ld_ = 0, int half_ = 0) : ld(ld_), half(half_) {}
+    __host__ __device__ size_t row(size_t img, int v, int V) const
+    {
+        const size_t o = img * V * ld;
+        if (half == 0) return o + (size_t)v * ld;
+        const int up = v >= half;
+        return o + (size_t)(v - up * half) * 2 * ld + up;
+    }
+    __host__ __device__ int step() const { return half ? 2 : 1; }
+};
+// the rows of mu_bar and dL/dr, the inputs of A^T (zeros past n_bins)
+inline Rows at_rows(const Geometry *g) { return Rows(g->ld, g->orbit ? g->n_views / 2 : 0); }
 size_t dual_fft_smem(const Geometry *g);       // one exchange buffer of the dual update's transform
 // Device pointers into a solve workspace (api.cu's layout).
 struct SolveBuffers {
@@ -412,17 +430,19 @@ void launch_band_reduce(const Geometry *g, const float *partial, float *out, int
 // thread-block cluster (cluster, or partial NULL), or through slice images
 // in `partial` (orbit_partial_floats() floats) and a reduction pass: the
 // form for solves run side by side, whose clusters would wait for a GPC's
-// SMs to free together.  The orbit form's y has rows of g->ld floats, zeros
-// past n_bins, 16-byte aligned (launch_pad_rows copies a sinogram so); the
-// general form's rows are ld floats apart.  slices > 0 fixes the slice count.
+// SMs to free together.  The orbit form's y is laid out by at_rows(g), zeros
+// past n_bins, 16-byte aligned (launch_pair_rows copies a sinogram so), or,
+// with plain set, in rows of n_bins floats; the general form's rows are ld
+// floats apart.  slices > 0 fixes the slice count.
 bool orbit_ok(const Geometry *g);
 size_t orbit_partial_floats(const Geometry *g, int batch);
 bool orbit_slices_ok(const Geometry *g, int nsl);
 void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int mode, const float *xin,
                               const double *scal, int batch, float *partial, cudaStream_t st, bool cluster = true,
-                              int slices = 0);
+                              int slices = 0, bool plain = false);
+bool orbit_plain_rows(const Geometry *g, int batch);
 int orbit_slices_rule(const Geometry *g);
-void launch_pad_rows(const Geometry *g, const float *in, float *out, int batch, cudaStream_t st);
+void launch_pair_rows(const Geometry *g, const float *in, float *out, int batch, cudaStream_t st);
 void launch_backproject(const Geometry *g, const float *y, int ld, float *out, int mode,
                         const float *xin, const double *scal, int batch, cudaStream_t st);
 
@@ -433,7 +453,7 @@ void launch_backproject(const Geometry *g, const float *y, int ld, float *out, i
 // Filter: out = post .* (D (pre .* in)) * (scal ? -sigma : 1); pre/post
 // may be NULL.  mode 0 plain, 1 "-sigma D in" (start of the iteration).
 void launch_filter(const Geometry *g, const float *taps, int half, const float *in,
-                   float *out, int ldo, const float *pre, const float *post, int mode,
+                   float *out, Rows ldo, const float *pre, const float *post, int mode,
                    const double *scal, int batch, cudaStream_t st);
 // Fused Step 3 + next Step 1 for one iteration, per view:
 //   mu' = mu + sigma D r;  mu_bar = 2 mu' - mu [- sigma D (winv .* (mu' - mu))].
@@ -458,10 +478,10 @@ void launch_hhat(const Geometry *g, const float *taps, int half, float2 *hhat, c
 // post are complete when the kernel starts and only hhat is waited for
 void launch_filter_fft(const Geometry *g, const float2 *hhat, const float *in, float *out,
                        const float *pre, const float *post, int mode, const double *scal, int batch,
-                       cudaStream_t st, int ldo, bool early = false);
+                       cudaStream_t st, Rows ldo, bool early = false);
 // out = D (A x) with A x given as the projector's band partial sums
 void launch_filter_fft_bands(const Geometry *g, const float2 *hhat, const float *partial, float *out, int batch,
-                             cudaStream_t st, int ldo);
+                             cudaStream_t st, Rows ldo);
 // fused residual + Step 3 + next Step 1 (as launch_dual_update; mu_bar with rows of g->ld)
 void launch_dual_fft(const Geometry *g, const float2 *hhat, const float *partial, const float *b, float *mu,
                      float *mu_bar, const float *winv, int lowdose, const double *scal, cudaStream_t st);
@@ -472,9 +492,9 @@ void launch_sv_hhat(const Geometry *g, const float *taps_lo, const float *taps_h
                     cudaStream_t st);
 void launch_filter_sv(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv, const float *in,
                       float *out, const float *pre, const float *post, int mode, const double *scal, int batch,
-                      cudaStream_t st, int ldo);
+                      cudaStream_t st, Rows ldo);
 void launch_filter_sv_bands(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv,
-                            const float *partial, float *out, int batch, cudaStream_t st, int ldo);
+                            const float *partial, float *out, int batch, cudaStream_t st, Rows ldo);
 void launch_dual_sv(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv, const float *partial,
                     const float *b, float *mu, float *mu_bar, const float *winv, const double *scal,
                     cudaStream_t st);
@@ -553,7 +573,7 @@ void eps_cache_free(Geometry *g);
 // whether eps_basis has the basis already (so a solve needs no host step)
 bool eps_basis_ready(const Geometry *g, int precond, double tau_key);
 size_t eps_partial_floats(const Geometry *g);
-void launch_eps_step(const Geometry *g, const float *q, float *out, int ldo, float *out2, int ld2, const float *mu0,
+void launch_eps_step(const Geometry *g, const float *q, float *out, Rows ldo, float *out2, Rows ld2, const float *mu0,
                      const float *Q,
                      const float *lambda, double eps, double *scal, float *wbuf, float *s, float *w2, float *part,
                      cudaStream_t st);

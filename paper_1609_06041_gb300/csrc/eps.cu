@@ -299,14 +299,16 @@ k_eps_sum_w2(const float *__restrict__ part, int ks, int V, int B, float *__rest
 
 // after the second map: out = sum_z part[z] (chunks in order), out2 =
 // 2 out - mu0
-// the place of element i (rows of B) in rows ld apart
-__device__ __forceinline__ size_t in_rows(size_t i, int B, int ld)
+// the place of element i (rows of B) of a sinogram in the given rows
+__device__ __forceinline__ size_t in_rows(size_t i, int V, int B, const Rows &rows)
 {
-    return ld == B ? i : i + (i / (unsigned)B) * (unsigned)(ld - B);
+    if (rows.half == 0 && rows.ld == B) return i;
+    const unsigned v = (unsigned)(i / (unsigned)B);
+    return rows.row(0, (int)v, V) + (i - (size_t)v * B) * rows.step();
 }
 
-__global__ void k_eps_sum_out(const float *__restrict__ part, int ks, size_t n, int B, float *__restrict__ out, int ldo,
-                              float *__restrict__ out2, int ld2, const float *__restrict__ mu0)
+__global__ void k_eps_sum_out(const float *__restrict__ part, int ks, size_t n, int V, int B, float *__restrict__ out, Rows ldo,
+                              float *__restrict__ out2, Rows ld2, const float *__restrict__ mu0)
 {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         float pz[EG_KS];
@@ -315,21 +317,21 @@ __global__ void k_eps_sum_out(const float *__restrict__ part, int ks, size_t n, 
         float a = 0.0f;
 #pragma unroll
         for (int z = 0; z < EG_KS; ++z) a += pz[z];
-        out[in_rows(i, B, ldo)] = a;
-        if (out2) out2[in_rows(i, B, ld2)] = 2.0f * a - mu0[i];
+        out[in_rows(i, V, B, ldo)] = a;
+        if (out2) out2[in_rows(i, V, B, ld2)] = 2.0f * a - mu0[i];
     }
 }
 
 // out = X s (per column j; in place allowed), out2 = 2 out - mu0: the map
 // when D = I
-__global__ void k_eps_scale(const float *X, const float *__restrict__ s, float *out, int ldo,
-                            float *__restrict__ out2, int ld2, const float *__restrict__ mu0, int V, int B)
+__global__ void k_eps_scale(const float *X, const float *__restrict__ s, float *out, Rows ldo,
+                            float *__restrict__ out2, Rows ld2, const float *__restrict__ mu0, int V, int B)
 {
     const size_t n = (size_t)V * B;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float v = X[i] * s[i % B];
-        out[in_rows(i, B, ldo)] = v;
-        if (out2) out2[in_rows(i, B, ld2)] = 2.0f * v - mu0[i];
+        out[in_rows(i, V, B, ldo)] = v;
+        if (out2) out2[in_rows(i, V, B, ld2)] = 2.0f * v - mu0[i];
     }
 }
 
@@ -466,7 +468,7 @@ k_eps_root(const float *__restrict__ w2g, const float *__restrict__ lambda, int 
     if (tid == 0) *uslot = (zero || all) ? 0.0f : u;
 }
 
-void launch_eps_step(const Geometry *g, const float *q, float *out, int ldo, float *out2, int ld2, const float *mu0,
+void launch_eps_step(const Geometry *g, const float *q, float *out, Rows ldo, float *out2, Rows ld2, const float *mu0,
                      const float *Q, const float *lambda, double eps, double *scal, float *wbuf, float *s, float *w2, float *part,
                      cudaStream_t st)
 {
@@ -481,7 +483,7 @@ void launch_eps_step(const Geometry *g, const float *q, float *out, int ldo, flo
         k_eps_sum_w2<<<(B + 31) / 32, dim3(32, 8), 0, st>>>(part, ks, V, B, wbuf, w2);
         k_eps_root<<<1, EPS_ROOT_T, 0, st>>>(w2, lambda, B, scal, (float)eps, s);
         k_eps_gemm<true><<<grid, tb, 0, st>>>(wbuf, Q, s, part, V, B, kchunk);
-        k_eps_sum_out<<<eblocks, 256, 0, st>>>(part, ks, n, B, out, ldo, out2, ld2, mu0);
+        k_eps_sum_out<<<eblocks, 256, 0, st>>>(part, ks, n, V, B, out, ldo, out2, ld2, mu0);
     } else {
         counted(3);
         k_eps_w2<<<(B + 127) / 128, 128, 0, st>>>(q, V, B, w2);

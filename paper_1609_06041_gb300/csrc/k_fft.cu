@@ -151,7 +151,7 @@ void launch_hhat(const Geometry *g, const float *taps, int half, float2 *hhat, c
 template <int P, bool BANDS, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? wide_threads(P) : block_threads(P),
                                   WIDE ? 1 : BANDS ? min_blocks(P) : 4 * min_blocks(P) / 3)
-k_filter_fft(const float2 *__restrict__ hhat, const float *__restrict__ in, float *__restrict__ out, int ldo,
+k_filter_fft(const float2 *__restrict__ hhat, const float *__restrict__ in, float *__restrict__ out, Rows ldo,
              const float *__restrict__ pre, const float *__restrict__ post, int mode,
              const double *__restrict__ scal, int V, int B, const float2 *__restrict__ tw, int nb,
              const ViewP *__restrict__ views, int early)
@@ -201,7 +201,8 @@ k_filter_fft(const float2 *__restrict__ hhat, const float *__restrict__ in, floa
     const GroupCtx ctx{(int)threadIdx.x, block_threads(P), 1};
     fft_apply<P, false, true>(ctx, pl.t, v, pl.buf, ph, hhat, tw);
     const float sc = ((mode == 1) ? -fscal(scal, F_SIGMA) : 1.0f) / (float)P;
-    float *q0 = out + ((size_t)blockIdx.y * V + (has0 ? v0 : 0)) * ldo, *q1 = has1 ? q0 + ldo : q0;
+    float *q0 = out + ldo.row(blockIdx.y, has0 ? v0 : 0, V), *q1 = has1 ? out + ldo.row(blockIdx.y, v1, V) : q0;
+    const int rs = ldo.step();
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
         const int i = pl.t + r * T;
@@ -211,10 +212,10 @@ k_filter_fft(const float2 *__restrict__ hhat, const float *__restrict__ in, floa
                 y0 *= post[o0 + i];
                 if (has1) y1 *= post[o1 + i];
             }
-            q0[i] = y0;
-            if (has1) q1[i] = y1;
-        } else if (i < ldo && has0) {
-            q0[i] = q1[i] = 0.0f;
+            q0[i * rs] = y0;
+            if (has1) q1[i * rs] = y1;
+        } else if (i < ldo.ld && has0) {
+            q0[i * rs] = q1[i * rs] = 0.0f;
         }
     }
 }
@@ -228,7 +229,7 @@ static dim3 fft_grid(int transforms, int batch)
 
 // out = D (A x) from the projector's band partial sums
 void launch_filter_fft_bands(const Geometry *g, const float2 *hhat, const float *partial, float *out, int batch,
-                             cudaStream_t st, int ldo)
+                             cudaStream_t st, Rows ldo)
 {
     counted();
     with_length(g->p_fft, [&](auto L) {
@@ -243,7 +244,7 @@ void launch_filter_fft_bands(const Geometry *g, const float2 *hhat, const float 
 
 void launch_filter_fft(const Geometry *g, const float2 *hhat, const float *in, float *out,
                        const float *pre, const float *post, int mode, const double *scal, int batch,
-                       cudaStream_t st, int ldo, bool early)
+                       cudaStream_t st, Rows ldo, bool early)
 {
     counted();
     PdlScope pdl(early || t_pdl);
@@ -354,7 +355,7 @@ __device__ __forceinline__ float band_sum(const float *__restrict__ p, size_t VB
 template <int P, bool BANDS>
 __global__ void __launch_bounds__(block_threads(P), min_blocks(P))
 k_filter_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const float *__restrict__ sv,
-            const float *__restrict__ in, float *__restrict__ out, int ldo, const float *__restrict__ pre,
+            const float *__restrict__ in, float *__restrict__ out, Rows ldo, const float *__restrict__ pre,
             const float *__restrict__ post, int mode, const double *__restrict__ scal, int V, int B,
             const float2 *__restrict__ tw, int nb, const ViewP *__restrict__ views)
 {
@@ -386,7 +387,8 @@ k_filter_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const 
     }
     int ph = 0;
     sv_apply<P>(pl.t, v, pl.buf, ph, hs, hd, tw);
-    float *q = out + ((size_t)blockIdx.y * V + vw) * ldo;
+    float *q = out + ldo.row(blockIdx.y, vw, V);
+    const int rs = ldo.step();
     const float sc = ((mode == 1) ? -fscal(scal, F_SIGMA) : 1.0f) / (float)P;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -394,16 +396,16 @@ k_filter_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const 
         if (i < B && has) {
             float y = fmaf(s[i], v[r].y, v[r].x) * sc;
             if (post) y *= post[o + i];
-            q[i] = y;
-        } else if (i < ldo && has) {
-            q[i] = 0.0f;
+            q[i * rs] = y;
+        } else if (i < ldo.ld && has) {
+            q[i * rs] = 0.0f;
         }
     }
 }
 
 void launch_filter_sv(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv, const float *in,
                       float *out, const float *pre, const float *post, int mode, const double *scal, int batch,
-                      cudaStream_t st, int ldo)
+                      cudaStream_t st, Rows ldo)
 {
     counted();
     with_length(g->p_fft, [&](auto L) {
@@ -414,7 +416,7 @@ void launch_filter_sv(const Geometry *g, const float2 *hs, const float2 *hd, con
 }
 
 void launch_filter_sv_bands(const Geometry *g, const float2 *hs, const float2 *hd, const float *sv,
-                            const float *partial, float *out, int batch, cudaStream_t st, int ldo)
+                            const float *partial, float *out, int batch, cudaStream_t st, Rows ldo)
 {
     counted();
     with_length(g->p_fft, [&](auto L) {
@@ -433,7 +435,7 @@ template <int P>
 __global__ void __launch_bounds__(block_threads(P), min_blocks(P))
 k_dual_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const float *__restrict__ sv,
           const float *__restrict__ partial, int nb, const float *__restrict__ b, float *mu,
-          float *__restrict__ mu_bar, int ld, const float *__restrict__ winv, const ViewP *__restrict__ views,
+          float *__restrict__ mu_bar, Rows rows, const float *__restrict__ winv, const ViewP *__restrict__ views,
           const double *__restrict__ scal, int V, int B, const float2 *__restrict__ tw)
 {
     extern __shared__ float2 fsm[];
@@ -485,9 +487,9 @@ k_dual_sv(const float2 *__restrict__ hs, const float2 *__restrict__ hd, const fl
         const int i = pl.t + r * T;
         if (i < B && has) {
             mu[o + i] = mn[r];
-            mu_bar[(size_t)vw * ld + i] = fmaf(-sp, fmaf(s[i], v[r].y, v[r].x), mo[r]);
-        } else if (i < ld && has) {
-            mu_bar[(size_t)vw * ld + i] = 0.0f;
+            mu_bar[rows.row(0, vw, V) + i * rows.step()] = fmaf(-sp, fmaf(s[i], v[r].y, v[r].x), mo[r]);
+        } else if (i < rows.ld && has) {
+            mu_bar[rows.row(0, vw, V) + i * rows.step()] = 0.0f;
         }
     }
 }
@@ -500,7 +502,7 @@ void launch_dual_sv(const Geometry *g, const float2 *hs, const float2 *hd, const
     with_length(g->p_fft, [&](auto L) {
         constexpr int P = decltype(L)::value;
         launch_kernel(k_dual_sv<P>, fft_grid<P>(g->n_views, 1), dim3(block_threads(P)), block_smem(P), st, hs, hd, sv,
-                      partial, proj_bands(g->n), b, mu, mu_bar, g->ld, winv, g->d_views, scal, g->n_views, g->n_bins,
+                      partial, proj_bands(g->n), b, mu, mu_bar, at_rows(g), winv, g->d_views, scal, g->n_views, g->n_bins,
                       g->d_tw);
     });
 }
@@ -523,7 +525,7 @@ void launch_dual_fft_batched(const Geometry *g, const float2 *hhat, const float 
         constexpr int P = decltype(L)::value;
         const bool wide = wide_grid(g, batch);
         const DualArgs a{hhat, g->d_tw, partial, proj_bands(g->n), b, mu_in, mu_out, mu_bar, winv, lowdose,
-                         g->d_views, scal, g->n_views, g->n_bins, g->ld};
+                         g->d_views, scal, g->n_views, g->n_bins, at_rows(g)};
         launch_kernel(wide ? k_dual_fft<P, true> : k_dual_fft<P, false>, fft_grid<P>((g->n_views + 1) / 2, batch),
                       dim3(wide ? wide_threads(P) : block_threads(P)), block_smem(P), st, a);
     });
@@ -549,7 +551,7 @@ k_dual_bwd_fft(const float2 *__restrict__ hhat, const float *__restrict__ partia
                const float *__restrict__ mu1, const float *__restrict__ gm, const float *__restrict__ gmb,
                float *__restrict__ gmu_out, float *__restrict__ gr_out, float *gm1_out,
                float *__restrict__ r_out, float *__restrict__ v_out, int lowdose,
-               const ViewP *__restrict__ views, const double *__restrict__ scal, int V, int B, int ld,
+               const ViewP *__restrict__ views, const double *__restrict__ scal, int V, int B, Rows rows,
                const float2 *__restrict__ tw)
 {
     extern __shared__ float2 fsm[];
@@ -607,12 +609,10 @@ k_dual_bwd_fft(const float2 *__restrict__ hhat, const float *__restrict__ partia
         st[fp(P / 2 + i)] = hr[r];
     }
     if (!has0) return;
-    // dL/dr, the adjoint's input of A^T: rows of ld, zeros past B
-    float *gp = gr_out + ((size_t)blockIdx.y * V + v0) * ld;
-    for (int i = B + pl.t; i < ld; i += T) {
-        gp[i] = 0.0f;
-        if (has1) gp[ld + i] = 0.0f;
-    }
+    // dL/dr, the adjoint's input of A^T: zeros past B
+    float *gp0 = gr_out + rows.row(blockIdx.y, v0, V), *gp1 = gr_out + rows.row(blockIdx.y, has1 ? v1 : v0, V);
+    const int rs = rows.step();
+    for (int i = B + pl.t; i < rows.ld; i += T) gp0[i * rs] = gp1[i * rs] = 0.0f;
 #pragma unroll 1
     for (int i = pl.t; i < B; i += T) {
         float s[2];
@@ -633,7 +633,7 @@ k_dual_bwd_fft(const float2 *__restrict__ hhat, const float *__restrict__ partia
                 vv = winv[o] * (mu1[o] - mu[o]);
             }
             gmu_out[o] = gmu;
-            gp[(size_t)k * ld + i] = gr;
+            (k == 0 ? gp0 : gp1)[i * rs] = gr;
             r_out[o] = r;
             v_out[o] = vv;
         }
@@ -650,7 +650,7 @@ void launch_dual_bwd_fft(const Geometry *g, const float2 *hhat, const float *par
         constexpr int P = decltype(L)::value;
         launch_kernel(k_dual_bwd_fft<P>, fft_grid<P>((g->n_views + 1) / 2, batch), dim3(block_threads(P)),
                       block_smem(P), st, hhat, partial, proj_bands(g->n), b, winv, mu, mu1, gm, gmb, gmu, gr, gm1, r,
-                      v, lowdose, g->d_views, scal, g->n_views, g->n_bins, g->ld, g->d_tw);
+                      v, lowdose, g->d_views, scal, g->n_views, g->n_bins, at_rows(g), g->d_tw);
     });
 }
 

@@ -42,7 +42,7 @@ static size_t filter_smem(int B) { return sizeof(float) * (size_t)(2 * B + 2 * (
 
 __global__ void __launch_bounds__(FT)
 k_filter(const float *__restrict__ taps, int half, const float *__restrict__ in,
-         float *__restrict__ out, int ldo, const float *__restrict__ pre, const float *__restrict__ post,
+         float *__restrict__ out, Rows ldo, const float *__restrict__ pre, const float *__restrict__ post,
          int mode, const double *__restrict__ scal, int V, int B)
 {
     extern __shared__ float sm[];
@@ -66,14 +66,14 @@ k_filter(const float *__restrict__ taps, int half, const float *__restrict__ in,
             if (d < B) {
                 float val = acc[i];
                 if (post) val *= post[off + d];
-                out[((size_t)blockIdx.y * V + blockIdx.x) * ldo + d] = sc * val;
+                out[ldo.row(blockIdx.y, blockIdx.x, V) + d * ldo.step()] = sc * val;
             }
         }
     }
 }
 
 void launch_filter(const Geometry *g, const float *taps, int half, const float *in,
-                   float *out, int ldo, const float *pre, const float *post, int mode,
+                   float *out, Rows ldo, const float *pre, const float *post, int mode,
                    const double *scal, int batch, cudaStream_t st)
 {
     size_t smem = filter_smem(g->n_bins);
@@ -89,7 +89,7 @@ void launch_filter(const Geometry *g, const float *taps, int half, const float *
 // mu is updated in place; the view's values are read before any write.
 __global__ void __launch_bounds__(FT)
 k_dual(const float *__restrict__ taps, int half, const float *__restrict__ partial, int nb,
-       const float *__restrict__ b, float *__restrict__ mu, float *__restrict__ mu_bar, int ldb,
+       const float *__restrict__ b, float *__restrict__ mu, float *__restrict__ mu_bar, Rows rows,
        const float *__restrict__ winv, int lowdose, const ViewP *__restrict__ views,
        const double *__restrict__ scal, int V, int B)
 {
@@ -136,7 +136,7 @@ k_dual(const float *__restrict__ taps, int half, const float *__restrict__ parti
                 int d = q * FT * FR + threadIdx.x + i * FT;
                 if (d < B) {
                     mu[off + d] = mun[q][i];
-                    mu_bar[(size_t)blockIdx.x * ldb + d] = 2.0f * mun[q][i] - mo[q][i];
+                    mu_bar[rows.row(0, blockIdx.x, V) + d * rows.step()] = 2.0f * mun[q][i] - mo[q][i];
                 }
             }
         }
@@ -163,7 +163,7 @@ k_dual(const float *__restrict__ taps, int half, const float *__restrict__ parti
             int d = q * FT * FR + threadIdx.x + i * FT;
             if (d < B) {
                 mu[off + d] = mun[q][i];
-                mu_bar[(size_t)blockIdx.x * ldb + d] = 2.0f * mun[q][i] - mo[q][i] - sigma * acc[i];
+                mu_bar[rows.row(0, blockIdx.x, V) + d * rows.step()] = 2.0f * mun[q][i] - mo[q][i] - sigma * acc[i];
             }
         }
     }
@@ -175,7 +175,7 @@ void launch_dual_update(const Geometry *g, const float *taps, int half, const fl
 {
     size_t smem = filter_smem(g->n_bins);
     counted();
-    k_dual<<<g->n_views, FT, smem, st>>>(taps, half, partial, proj_bands(g->n), b, mu, mu_bar, g->ld, winv,
+    k_dual<<<g->n_views, FT, smem, st>>>(taps, half, partial, proj_bands(g->n), b, mu, mu_bar, at_rows(g), winv,
                                          lowdose, g->d_views, scal, g->n_views, g->n_bins);
 }
 

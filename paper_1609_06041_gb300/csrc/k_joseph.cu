@@ -721,7 +721,7 @@ k_backproject_tiles(const float *__restrict__ y, int ld, float *__restrict__ out
     }
 }
 
-template <bool AL>
+template <int FORM>
 __global__ void __launch_bounds__(ORB_TH, 8)
 k_backproject_orbit(const float *__restrict__ y, int ld, float *__restrict__ partial, const float4 *__restrict__ trig,
                     int N, int V, int B, int nsl, int fin, float *out, const float *xin,
@@ -729,7 +729,7 @@ k_backproject_orbit(const float *__restrict__ y, int ld, float *__restrict__ par
 {
     extern __shared__ __align__(16) unsigned char osm[];
     pdl_wait();
-    orbit_body<AL>(Block2D{}, blockIdx.x, blockIdx.y, blockIdx.z, osm, y, ld, partial, trig, N, V, B, nsl, fin, out, xin,
+    orbit_body<FORM>(Block2D{}, blockIdx.x, blockIdx.y, blockIdx.z, osm, y, ld, partial, trig, N, V, B, nsl, fin, out, xin,
                    scal);
 }
 
@@ -740,14 +740,14 @@ k_backproject_orbit(const float *__restrict__ y, int ld, float *__restrict__ par
 // in slice order through distributed shared memory and writes the sum
 // (mode 0) or xin - tau sum (mode 1).  No slice images are written, and no
 // reduction pass runs.
-template <bool AL>
+template <int FORM>
 __global__ void __launch_bounds__(ORB_TH, 8)
 k_backproject_orbit_cl(const float *__restrict__ y, int ld, const float4 *__restrict__ trig, int N, int V, int B, int nsl,
                        int mode, float *out, const float *xin, const double *__restrict__ scal)
 {
     extern __shared__ __align__(16) unsigned char osm[];
     pdl_wait();
-    orbit_body<AL, Block2D, true>(Block2D{}, blockIdx.x, blockIdx.y, blockIdx.z, osm, y, ld, nullptr, trig, N, V, B, nsl, 0,
+    orbit_body<FORM, Block2D, true>(Block2D{}, blockIdx.x, blockIdx.y, blockIdx.z, osm, y, ld, nullptr, trig, N, V, B, nsl, 0,
                                   nullptr, nullptr, scal);
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
@@ -955,36 +955,53 @@ ct_status qbal_balance(Geometry *g, const float *x, float *band, cudaStream_t st
     return CT_OK;
 }
 
-// out rows of ld >= B floats: the B values of each row, then zeros
-__global__ void k_pad_rows(const float *__restrict__ in, float *__restrict__ out, size_t n, int B, int ld)
+// the rows of at_rows (half > 0): views v and v + V/2 interleaved, zeros past B
+__global__ void k_pair_rows(const float *__restrict__ in, float2 *__restrict__ out, size_t n, int B, int ld, int half)
 {
     const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const size_t row = i / (unsigned)ld;
-    const int d = (int)(i - row * ld);
-    out[i] = d < B ? in[row * B + d] : 0.0f;
+    const size_t pair = i / (unsigned)ld, row = pair + pair / (unsigned)half * (unsigned)half;   // of its first view
+    const int d = (int)(i - pair * ld);
+    out[i] = d < B ? make_float2(in[row * B + d], in[(row + half) * B + d]) : make_float2(0.0f, 0.0f);
 }
 
-void launch_pad_rows(const Geometry *g, const float *in, float *out, int batch, cudaStream_t st)
+void launch_pair_rows(const Geometry *g, const float *in, float *out, int batch, cudaStream_t st)
 {
-    const size_t n = (size_t)batch * g->n_views * g->ld;
+    const int half = g->n_views / 2;
+    const size_t n = (size_t)batch * half * g->ld;
     counted();
-    k_pad_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, out, n, g->n_bins, g->ld);
+    k_pair_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, reinterpret_cast<float2 *>(out), n, g->n_bins, g->ld,
+                                                             half);
+}
+
+// Whether a caller's sinogram is better read in its own rows than interleaved
+// first: where the pass and its launch (about 1.5 us) cost more than copying
+// the windows value by value, that is for little work and few views (64^2 / 90
+// views 5.1 against 6.0 us, 128^2 / 90 6.2 / 6.4, 256^2 / 32 5.8 / 6.6; but
+// 128^2 / 180 8.0 / 7.9, 64^2 / 720 17.1 / 13.1, 512^2 / 32 8.6 / 7.6).
+bool orbit_plain_rows(const Geometry *g, int batch)
+{
+    return g->n_views <= 128 && (double)g->n * g->n * g->n_views * batch <= 2.5e6;
 }
 
 void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int mode, const float *xin,
-                              const double *scal, int batch, float *partial, cudaStream_t st, bool cluster, int slices)
+                              const double *scal, int batch, float *partial, cudaStream_t st, bool cluster, int slices,
+                              bool plain)
 {
     const int q = g->n / 2;
     const bool cl = cluster || !partial;
     const int nsl = slices > 0 ? slices : orbit_slices(g, cl);
     dim3 grd((q + ORB_T - 1) / ORB_T, (q + ORB_T - 1) / ORB_T, nsl * batch);
     const bool al = g->ld == g->n_bins;
+    const int ld = plain ? g->n_bins : g->ld;
     if (nsl > 1 && cl) {
         // several slices: their sums are added in a cluster of the slices' blocks
         counted();
-        launch_kernel_cluster(al ? k_backproject_orbit_cl<true> : k_backproject_orbit_cl<false>, grd,
-                              dim3(ORB_T, ORB_TY), orbit_smem(), st, dim3(1, 1, nsl), y, g->ld,
+        launch_kernel_cluster(plain ? k_backproject_orbit_cl<ORB_PLAIN>
+                              : al  ? k_backproject_orbit_cl<ORB_PAIR4>
+                                    : k_backproject_orbit_cl<ORB_PAIR>,
+                              grd,
+                              dim3(ORB_T, ORB_TY), orbit_smem(), st, dim3(1, 1, nsl), y, ld,
                               (const float4 *)g->d_trig, g->n, g->n_views, g->n_bins, nsl, mode != 0 ? 1 : 0, out, xin,
                               scal);
         return;
@@ -993,8 +1010,10 @@ void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int
     // several slices without a cluster: slice images, then k_orbit_reduce
     const int fin = nsl == 1 ? 1 + (mode != 0) : 0;
     counted(fin ? 1 : 2);
-    launch_kernel(al ? k_backproject_orbit<true> : k_backproject_orbit<false>, grd, dim3(ORB_T, ORB_TY), orbit_smem(), st,
-                  y, g->ld, partial, g->d_trig, g->n, g->n_views, g->n_bins, nsl, fin, out, xin, scal);
+    launch_kernel(plain ? k_backproject_orbit<ORB_PLAIN>
+                  : al  ? k_backproject_orbit<ORB_PAIR4>
+                        : k_backproject_orbit<ORB_PAIR>,
+                  grd, dim3(ORB_T, ORB_TY), orbit_smem(), st, y, ld, partial, g->d_trig, g->n, g->n_views, g->n_bins, nsl, fin, out, xin, scal);
     if (fin) return;
     const size_t NN = (size_t)g->n * g->n;
     launch_kernel(mode == 0 ? k_orbit_reduce<0> : k_orbit_reduce<1>, dim3((unsigned)((NN + 255) / 256), batch),
@@ -1016,9 +1035,9 @@ void kernel_attrs_joseph()
 {
     cudaFuncSetAttribute(k_project_direct, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(DIRECT_BANDS * quad_smem(2 * MR * DIRECT_BANDS) + sizeof(float4) * DIRECT_THREADS));
-    for (auto k : {k_backproject_orbit<true>, k_backproject_orbit<false>})
+    for (auto k : {k_backproject_orbit<ORB_PLAIN>, k_backproject_orbit<ORB_PAIR>, k_backproject_orbit<ORB_PAIR4>})
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
-    for (auto k : {k_backproject_orbit_cl<true>, k_backproject_orbit_cl<false>})
+    for (auto k : {k_backproject_orbit_cl<ORB_PLAIN>, k_backproject_orbit_cl<ORB_PAIR>, k_backproject_orbit_cl<ORB_PAIR4>})
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
     for (auto k : {k_project_quad<2>, k_project_quad<4>})
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, QUAD_SMEM_MAX);

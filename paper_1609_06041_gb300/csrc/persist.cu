@@ -112,7 +112,7 @@ __device__ __noinline__ void dual_item(const PSlice &S, int i, unsigned char *ps
     const int pair = i * (PS_THREADS / T) + sub, t = tid % T;
     float2 *buf = reinterpret_cast<float2 *>(psm) + (size_t)sub * fft_elems(P);
     const DualArgs a{S.hhat, S.tw, S.band, S.nb, S.b, S.mu, S.mu, S.mubar, S.winv, S.lowdose, S.views, S.scal, S.V,
-                     S.B, S.ld};
+                     S.B, Rows(S.ld, S.V / 2)};
     dual_stage<P, false>(t, T, pair, 0, buf, a);
     dual_update<P, false, false>(GroupCtx{tid % GS, GS, 1 + g}, t, pair, 0, buf, a);
 }
@@ -130,10 +130,10 @@ __device__ __forceinline__ void run_item(const PSlice &S, int p, int k, int i, u
             unsigned char *sm = psm + (size_t)g * S.orb_smem;
             const int fin = S.nsl == 1 ? 2 : 0;
             if (S.ld == S.B)
-                orbit_body<true>(c, bx, by, bz, sm, S.mubar, S.ld, S.orb, S.trig, S.N, S.V, S.B, S.nsl, fin, S.z, S.x,
+                orbit_body<ORB_PAIR4>(c, bx, by, bz, sm, S.mubar, S.ld, S.orb, S.trig, S.N, S.V, S.B, S.nsl, fin, S.z, S.x,
                                  S.scal);
             else
-                orbit_body<false>(c, bx, by, bz, sm, S.mubar, S.ld, S.orb, S.trig, S.N, S.V, S.B, S.nsl, fin, S.z, S.x,
+                orbit_body<ORB_PAIR>(c, bx, by, bz, sm, S.mubar, S.ld, S.orb, S.trig, S.N, S.V, S.B, S.nsl, fin, S.z, S.x,
                                   S.scal);
         }
     } else if (p == PH_OREDUCE) {

@@ -189,7 +189,7 @@ extern "C" ct_status ct_unrolled_forward(const ct_geometry *geom, const float *b
     cudaMemsetAsync(c0.x, 0, sizeof(float) * S * J, st);
     cudaMemsetAsync(c0.mu, 0, sizeof(float) * S * I, st);
     cudaMemsetAsync(c0.p, 0, sizeof(float) * S * 2 * J, st);
-    launch_filter_fft(g, hhat, b, c0.mubar, nullptr, nullptr, 1, scal, S, st, g->ld);      // mubar_0 = -sigma D b
+    launch_filter_fft(g, hhat, b, c0.mubar, nullptr, nullptr, 1, scal, S, st, at_rows(g)); // mubar_0 = -sigma D b
     const bool fused = tv_fused(tau, beta, mode, tv_iters);
     for (int k = 0; k < iters; ++k) {
         CK c = ck_at(ws, L, g, S, k), n = ck_at(ws, L, g, S, k + 1);

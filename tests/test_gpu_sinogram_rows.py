@@ -1,5 +1,5 @@
-"""A^T on detectors of every length mod 4 (rows that are not whole 16-byte
-pieces are padded), from ones narrower than a staged window to past the
+"""A^T on detectors of every length mod 4 (its input's rows are padded to whole
+16-byte pieces, views v and v + V/2 interleaved), from ones narrower than a staged window to past the
 diagonal, against the FP64 oracle, and the solves that write padded rows: the
 paper's D, the shift-variant D, the few-view forms and the direct convolution
 above 4096 bins.
@@ -29,6 +29,21 @@ def test_backproject_rows(N, V, B):
     for i in range(3):
         assert rel_l2(to_np(out[i]), O.backproject(ys[i], N)) <= 2e-5
         assert torch.equal(P.ct_backproject(g, yg[i].clone()), out[i])
+
+
+@pytest.mark.parametrize("B", [1, 2, 3, 4, 30, 33, 35, 94, 95, 96, 97])
+@pytest.mark.parametrize("N,V", [(34, 10), (64, 18)])   # odd V/2: a transform's two views lie in different halves
+def test_interleaved_rows_equal_plain_rows(N, V, B):
+    # a batch of more than 2.5e6 pixel views is interleaved first, one image is not: the same bits
+    P = need_gpu()
+    import torch
+    g = P.Geometry(N, V, B)
+    batch = int(2.5e6 / (N * N * V)) + 2
+    gen = torch.Generator(device="cuda").manual_seed(B)
+    y = torch.randn(batch, V, B, device="cuda", generator=gen)
+    out = P.ct_backproject(g, y)
+    for i in (0, 1, batch // 2, batch - 1):
+        assert torch.equal(P.ct_backproject(g, y[i].clone()), out[i])
 
 
 @pytest.mark.parametrize("B", [70, 71, 72, 73, 4201])
