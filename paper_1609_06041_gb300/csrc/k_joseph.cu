@@ -779,7 +779,7 @@ k_backproject_orbit_cl(const float *__restrict__ y, int ld, const float4 *__rest
 
 static size_t orbit_smem()
 {
-    return sizeof(float) * 2 * ORB_VC * 8 * ORB_RW + sizeof(float4) * 2 * ORB_VC + sizeof(int) * 2 * ORB_MAXS;
+    return sizeof(float) * 2 * ORB_VC * 8 * ORB_RW + sizeof(float4) * 4 * ORB_VC + sizeof(int) * 2 * ORB_MAXS;
 }
 
 // out = sum of the slice images (mode 0), or xin - tau * sum (mode 1)
