@@ -47,8 +47,9 @@ SMEM_PEAK_TBPS = 152 * 128 * 2.070e9 / 1e12         # SMs x 128 shared-memory by
 # dram__bytes_write.sum); update together with the kernels, None when no
 # capture of the current kernel exists.  A: k_project_qbal<4> (the
 # work-balanced projector, 12 items' threads per block, 4 steps per pass);
-# AT: k_backproject_orbit_cl<true> (mu_bar and x read once).
-TRAFFIC_BYTES = {"A": 1.14304e6, "AT": 3.080704e6}
+# AT: k_backproject_orbit_cl (mu_bar and x read once; without ct_backproject's
+# pass that interleaves the rows).
+TRAFFIC_BYTES = {"A": 1.149952e6, "AT": 3.052032e6}
 
 
 def dist_info():

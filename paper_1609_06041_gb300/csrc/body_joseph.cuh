@@ -445,7 +445,7 @@ __device__ __forceinline__ void quad_balanced_body(const Ctx &c, long long u0, l
 // 16 ORB_TY threads takes the orbits of ORB_PX pixels of one tile column
 // (rows r, r + ORB_TY, ..), so the per-view constants, window bases and
 // loop control are shared by 8 ORB_PX pixel-views.  Base views are split into
-// nsl slices (grid.z; 4 unless tuned, at most ORB_SL_MAX), added in slice
+// nsl slices (grid.z; by rule or tuned, at most ORB_SL_MAX), added in slice
 // order: in a thread-block cluster of the slices' blocks
 // (k_backproject_orbit_cl), or from slice images (the persistent batched
 // kernel's reduction phase).  The weights are the
