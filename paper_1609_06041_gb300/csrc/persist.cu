@@ -209,11 +209,13 @@ __global__ void __launch_bounds__(PS_THREADS, 1) k_persistent(const __grid_const
 {
     extern __shared__ __align__(16) unsigned char psm[];
     __shared__ int cur[4];   // slice (< 0: leave), phase, iteration, item
+    __shared__ unsigned next;   // the next item's queue number (thread 0's)
     unsigned *queue = pslot(prm.sl[0].scal, S_PQUEUE), *err = pslot(prm.sl[0].scal, S_PERR);
+    if (threadIdx.x == 0) next = atomicAdd(queue, 1u);
     for (;;) {
         if (threadIdx.x == 0) {
             int s = -1, p = 0, k = 0, i = 0;
-            const unsigned t = atomicAdd(queue, 1u);
+            const unsigned t = next;
             if (t < (unsigned)prm.total && ld_relaxed(err) == 0) {
                 unsigned need;
                 if (t >= (unsigned)(prm.K * prm.R)) {   // a slice's closing item
@@ -264,8 +266,14 @@ __global__ void __launch_bounds__(PS_THREADS, 1) k_persistent(const __grid_const
         const int s = cur[0];
         if (s < 0) break;
         run_item(prm.sl[s], cur[1], cur[2], cur[3], psm);
+        // The next item is taken while other warps finish this one (the items
+        // before it are all taken, so the order of the queue still ends every
+        // wait), and this one is published by another warp than the one that
+        // then waits for the next's phase: 25.9 -> 25.5 ms for 12 mixed slices,
+        // 4.90 -> 4.70 for 16 of 256^2 / 32 views (a lone slice 2.21 -> 2.24).
+        if (threadIdx.x == 0) next = atomicAdd(queue, 1u);
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 32) {
             __threadfence();
             atomicAdd(pslot(prm.sl[s].scal, S_PDONE), 1u);
         }
