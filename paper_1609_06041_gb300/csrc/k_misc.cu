@@ -498,8 +498,11 @@ k_lanczos_fused(float *w, const float *tp, const float *tc, size_t n, double *s,
     __shared__ float part[2][LF_PARTS];
     __shared__ float wsum[LF_THREADS / 32];
     __shared__ float total, coef[3];
-    pdl_wait();
     cg::cluster_group cl = cg::this_cluster();
+    // a block may store into the first block's shared memory once that block runs: every block arrives here and
+    // waits just before its first remote store, behind the loads in between
+    cl.barrier_arrive();
+    pdl_wait();
     const int grp = threadIdx.x >> 8, t = threadIdx.x & 255, ng = LF_THREADS / DOT_THREADS;
     const size_t n4 = n / 4, done = n4 * 4;
     const int nparts = (int)((n + 4 * (size_t)DOT_THREADS - 1) / (4 * (size_t)DOT_THREADS));
@@ -516,6 +519,7 @@ k_lanczos_fused(float *w, const float *tp, const float *tc, size_t n, double *s,
     float c1 = coef[0], c2 = coef[1];
     const float nj = coef[2];
     const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    cl.barrier_wait();
 #pragma unroll 1
     for (int phase = 0; phase < 2; ++phase) {
         const float4 *x4 = phase == 0 ? tp4 : tc4;
