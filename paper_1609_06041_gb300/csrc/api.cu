@@ -523,7 +523,8 @@ ct_status ct_geometry_create(int n, int n_views, int n_bins, const double *angle
         cudaGetLastError();
         g->n_sm = 1;
     }
-    g->orb_rule = orbit_slices_rule(g);
+    g->orb_rule = orbit_slices_rule(g, false);
+    g->orb_rule_op = orbit_slices_rule(g, true);
     g->h_angles = new double[n_views];
     // candidate-window margin of the backprojector (bins): a generous bound
     // on the float rounding of the Joseph coordinates at this size
@@ -709,6 +710,8 @@ ct_status ct_backproject(const ct_geometry *g, const float *sino, float *img, in
     }
     // views v and v + V/2 interleaved first (stream-ordered scratch), 2 to 3 us at 512^2 / 720 views; small sinograms,
     // and calls for which there is no scratch, are read in their own rows
+    const int slices = g->tune_orb > 0 ? g->tune_orb : g->orb_rule_op;
+    const int blocks = g->tune_orb > 0 ? slices : orbit_blocks(g, slices, batch);
     const size_t bytes = sizeof(float) * (size_t)batch * g->n_views * g->ld;
     float *pairs = nullptr;
     if (!orbit_plain_rows(g, batch) && scratch_alloc(g, &pairs, bytes, S(stream)) != cudaSuccess) {
@@ -716,13 +719,14 @@ ct_status ct_backproject(const ct_geometry *g, const float *sino, float *img, in
         pairs = nullptr;
     }
     if (!pairs) {
-        launch_backproject_orbit(g, sino, img, 0, nullptr, nullptr, batch, nullptr, S(stream), true, 0, true);
+        launch_backproject_orbit(g, sino, img, 0, nullptr, nullptr, batch, nullptr, S(stream), true, slices, true, blocks);
         return cuda_check("ct_backproject");
     }
     launch_pair_rows(g, sino, pairs, batch, S(stream));
     {
         PdlScope pdl(true);
-        launch_backproject_orbit(g, pairs, img, 0, nullptr, nullptr, batch, nullptr, S(stream));
+        launch_backproject_orbit(g, pairs, img, 0, nullptr, nullptr, batch, nullptr, S(stream), true, slices, false,
+                                 blocks);
     }
     cudaFreeAsync(pairs, S(stream));
     return cuda_check("ct_backproject");

@@ -493,20 +493,35 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // there: for small sinograms).  CL: instead of storing its sums, the
 // block leaves them in osm, entry (k ORB_PX + j) ORB_TH + tid for rotation
 // k of the thread's pixel orbit j, for a cluster reduction over slices.
+// SEQ (nsl a power of two): bz counts the csz blocks of a tile, a divisor of
+// nsl, instead of the slices; each takes nsl / csz slices one after the other.
+// CL: the sums of those before its last are kept one by one in
+// orbit_kept(osm), the last one's are left as above.  Otherwise csz is 1: the
+// block adds its slices' sums up there and writes the result.
 enum { ORB_PLAIN = 0, ORB_PAIR, ORB_PAIR4 };
-template <int FORM, class Ctx, bool CL = false>
+constexpr int ORB_E = 4 * ORB_PX * ORB_TH;   // sums of a tile
+__device__ __forceinline__ float *orbit_kept(unsigned char *osm)
+{
+    return reinterpret_cast<float *>(osm) + 2 * ORB_VC * 8 * ORB_RW + 4 * 4 * ORB_VC;
+}
+// Sets of sums a block keeps: one of csz that share nsl slices.
+__host__ __device__ __forceinline__ int orbit_kept_sets(int nsl, int csz) { return csz == 1 ? 1 : nsl / csz - 1; }
+template <int FORM, class Ctx, bool CL = false, bool SEQ = false>
 __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz, unsigned char *osm, const float *y,
                                            int ld, float *partial, const float4 *trig, int N, int V, int B, int nsl,
-                                           int fin, float *out, const float *xin, const double *scal)
+                                           int fin, float *out, const float *xin, const double *scal, int csz = 1)
 {
     // raw[buffer][view][window (e, mirror e, e90, mirror e90)][value][row (v, v+V/2)]
     float *raw = reinterpret_cast<float *>(osm);                               // 2 x ORB_VC x 8 x ORB_RW
     float4 *tt = reinterpret_cast<float4 *>(raw + 2 * ORB_VC * 8 * ORB_RW);    // 2 x ORB_VC x 2
-    int *wbs = reinterpret_cast<int *>(tt + 4 * ORB_VC);                       // ORB_MAXS x 2
+    float *kept = orbit_kept(osm);                                             // SEQ: orbit_kept_sets x ORB_E
+    int *wbs = reinterpret_cast<int *>(kept + (SEQ ? orbit_kept_sets(nsl, csz) * ORB_E : 0));   // base views x 2
     const int tid = cb.tid();   // tid / ORB_T < ORB_TY
     const int tx = tid % ORB_T, ty = tid / ORB_T;
     const int half = N / 2, V2 = V / 2;
-    const int slice = bz % nsl, img = bz / nsl;
+    const int share = SEQ ? nsl / csz : 1, slice = SEQ ? bz % csz * share : bz % nsl, img = bz / (SEQ ? csz : nsl);
+    const int slice1 = slice + share;   // the block's slices: slice .. slice1 - 1
+    auto first_view = [&](int s) { return SEQ ? V2 * s >> (31 - __clz(nsl)) : (int)((long long)V2 * s / nsl); };
     const int r0 = by * ORB_T, c0 = half + bx * ORB_T;   // quadrant r < N/2, c >= N/2
     const int r = r0 + ty, c = c0 + tx;                  // pixels (r + j ORB_TY, c)
     const bool inside = r < half && c < N;
@@ -514,7 +529,7 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
     const float xq = (float)c - h, yq = (float)r - h;               // P = (x, y); R90 P = (-y, x)
     const float *ys = y + (size_t)img * V * ld;
     const int ms = FORM == ORB_PAIR4 ? 3 : (B - ORB_RW + 3) & 3;   // see the mirrored windows below
-    const int vb0 = (int)((long long)V2 * slice / nsl), vb1 = (int)((long long)V2 * (slice + 1) / nsl);
+    const int vb0 = first_view(slice), vb1 = first_view(slice1);
     const int nvs = vb1 - vb0;
     static_assert(ORB_PX == 2, "a thread's two orbits are packed");
     const float2 xq2 = pk(xq, xq), yq2 = pk(yq, yq + (float)ORB_TY), nyq2 = pk(-yq, -(yq + (float)ORB_TY));
@@ -576,6 +591,25 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
         }
         cp_async_commit();
     };
+    // SEQ: the sums of a slice that ends before view v are kept, and the next slice's start at zero
+    int cur = slice, bnd = 0x7fffffff;
+    auto bound = [&]() { bnd = cur + 1 < slice1 ? first_view(cur + 1) : 0x7fffffff; };
+    auto keep = [&](int v) {
+        while (v >= bnd) {
+            float *dst = kept + (CL ? (cur - slice) * ORB_E : 0) + tid;
+#pragma unroll
+            for (int j = 0; j < ORB_PX; ++j)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    float *q = dst + (k * ORB_PX + j) * ORB_TH;
+                    *q = !CL && cur > 0 ? *q + acc[j][k] : acc[j][k];
+                    acc[j][k] = 0.0f;
+                }
+            ++cur;
+            bound();
+        }
+    };
+    if constexpr (SEQ) bound();
     const int nch = (nvs + ORB_VC - 1) / ORB_VC;
     if (nch > 0) issue(vb0, min(ORB_VC, nvs), 0);
     for (int ch = 0; ch < nch; ++ch) {
@@ -589,47 +623,65 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
         cb.sync();
         const float *tb = raw + (size_t)(ch & 1) * ORB_VC * 8 * ORB_RW;
         const float4 *tv = tt + 2 * (ch & 1) * ORB_VC;
-        if (inside) {
-            for (int vi = 0; vi < nv; ++vi) {
-                const float4 Ta = tv[2 * vi], Tb = tv[2 * vi + 1];
-                const float2 Tx = pk(Ta.x, Ta.y), Ty = pk(Ta.z, Ta.w), Tz = pk(Tb.x, Tb.y), Tw = pk(Tb.z, Tb.w);
-                const int2 wb = *reinterpret_cast<const int2 *>(wbs + 2 * (v0 - vb0 + vi));
-                // [window][value](view v, view v + V/2)
-                const float2 *e_v = reinterpret_cast<const float2 *>(tb) + (size_t)vi * 4 * ORB_RW, *m_v = e_v + ORB_RW,
-                             *e9_v = e_v + 2 * ORB_RW, *m9_v = e_v + 3 * ORB_RW;
-                // e - 1/2 of P and of R90 P for the thread's two orbits, (x, y) = (xq, yq) and (xq, yq + ORB_TY),
-                // their windows' places and weights: packed (14 issue slots a view for 28; ct_backproject 63.8 -> 62.7 us
-                // at 512^2 / 720 views, each value rounded as before)
-                const float2 e = pfma(xq2, Tx, pfma(yq2, Ty, hb2)), e9 = pfma(xq2, Ty, pfma(nyq2, Tx, hb2));
-                const float2 t = padd(e, bias2), t9 = padd(e9, bias2);
-                const float2 u = psub(t, bias2), u9 = psub(t9, bias2);
-                const float2 g = psub(e, u), g9 = psub(e9, u9), ng = psub(u, e), ng9 = psub(u9, e9);
-                const float2 a0 = pfma(ng, Tz, Tw), a1 = pfma(g, Tz, Tw), a09 = pfma(ng9, Tz, Tw), a19 = pfma(g9, Tz, Tw);
-                auto orbit = [&](int j, float &cP, float &c90, float &c180, float &c270) {
-                    const unsigned k = min((unsigned)(__float_as_int((j ? t.y : t.x)) - (JOSEPH_BIAS_BITS + wb.x)),
-                                           (unsigned)(ORB_RW - 5));
-                    const unsigned k9 = min((unsigned)(__float_as_int((j ? t9.y : t9.x)) - (JOSEPH_BIAS_BITS + wb.y)),
-                                            (unsigned)(ORB_RW - 5));
-                    const float w0 = fmaxf(0.0f, (j ? a0.y : a0.x)), w1 = fmaxf(0.0f, (j ? a1.y : a1.x));
-                    const float w09 = fmaxf(0.0f, (j ? a09.y : a09.x)), w19 = fmaxf(0.0f, (j ? a19.y : a19.x));
-                    const unsigned km = ORB_RW - 5 + ms - k, km9 = ORB_RW - 5 + ms - k9;
-                    const float2 e0 = e_v[k], e1 = e_v[k + 1], m0 = m_v[km], m1 = m_v[km + 1];
-                    const float2 f0 = e9_v[k9], f1 = e9_v[k9 + 1], n0 = m9_v[km9], n1 = m9_v[km9 + 1];
-                    cP = fmaf(w0, e0.x, fmaf(w1, e1.x, cP));           // P at v
-                    c180 = fmaf(w1, m0.x, fmaf(w0, m1.x, c180));       // R180 P at v
-                    c90 = fmaf(w0, e0.y, fmaf(w1, e1.y, c90));         // R90 P at v + V/2
-                    c270 = fmaf(w1, m0.y, fmaf(w0, m1.y, c270));       // R270 P at v + V/2
-                    c90 = fmaf(w09, f0.x, fmaf(w19, f1.x, c90));       // R90 P at v
-                    c270 = fmaf(w19, n0.x, fmaf(w09, n1.x, c270));     // R270 P at v
-                    c180 = fmaf(w09, f0.y, fmaf(w19, f1.y, c180));     // R180 P at v + V/2
-                    cP = fmaf(w19, n0.y, fmaf(w09, n1.y, cP));         // P at v + V/2
-                };
+        auto view = [&](int vi) {
+            const float4 Ta = tv[2 * vi], Tb = tv[2 * vi + 1];
+            const float2 Tx = pk(Ta.x, Ta.y), Ty = pk(Ta.z, Ta.w), Tz = pk(Tb.x, Tb.y), Tw = pk(Tb.z, Tb.w);
+            const int2 wb = *reinterpret_cast<const int2 *>(wbs + 2 * (v0 - vb0 + vi));
+            // [window][value](view v, view v + V/2)
+            const float2 *e_v = reinterpret_cast<const float2 *>(tb) + (size_t)vi * 4 * ORB_RW, *m_v = e_v + ORB_RW,
+                         *e9_v = e_v + 2 * ORB_RW, *m9_v = e_v + 3 * ORB_RW;
+            // e - 1/2 of P and of R90 P for the thread's two orbits, (x, y) = (xq, yq) and (xq, yq + ORB_TY),
+            // their windows' places and weights: packed (14 issue slots a view for 28; ct_backproject 63.8 -> 62.7 us
+            // at 512^2 / 720 views, each value rounded as before)
+            const float2 e = pfma(xq2, Tx, pfma(yq2, Ty, hb2)), e9 = pfma(xq2, Ty, pfma(nyq2, Tx, hb2));
+            const float2 t = padd(e, bias2), t9 = padd(e9, bias2);
+            const float2 u = psub(t, bias2), u9 = psub(t9, bias2);
+            const float2 g = psub(e, u), g9 = psub(e9, u9), ng = psub(u, e), ng9 = psub(u9, e9);
+            const float2 a0 = pfma(ng, Tz, Tw), a1 = pfma(g, Tz, Tw), a09 = pfma(ng9, Tz, Tw), a19 = pfma(g9, Tz, Tw);
+            auto orbit = [&](int j, float &cP, float &c90, float &c180, float &c270) {
+                const unsigned k = min((unsigned)(__float_as_int((j ? t.y : t.x)) - (JOSEPH_BIAS_BITS + wb.x)),
+                                       (unsigned)(ORB_RW - 5));
+                const unsigned k9 = min((unsigned)(__float_as_int((j ? t9.y : t9.x)) - (JOSEPH_BIAS_BITS + wb.y)),
+                                        (unsigned)(ORB_RW - 5));
+                const float w0 = fmaxf(0.0f, (j ? a0.y : a0.x)), w1 = fmaxf(0.0f, (j ? a1.y : a1.x));
+                const float w09 = fmaxf(0.0f, (j ? a09.y : a09.x)), w19 = fmaxf(0.0f, (j ? a19.y : a19.x));
+                const unsigned km = ORB_RW - 5 + ms - k, km9 = ORB_RW - 5 + ms - k9;
+                const float2 e0 = e_v[k], e1 = e_v[k + 1], m0 = m_v[km], m1 = m_v[km + 1];
+                const float2 f0 = e9_v[k9], f1 = e9_v[k9 + 1], n0 = m9_v[km9], n1 = m9_v[km9 + 1];
+                cP = fmaf(w0, e0.x, fmaf(w1, e1.x, cP));           // P at v
+                c180 = fmaf(w1, m0.x, fmaf(w0, m1.x, c180));       // R180 P at v
+                c90 = fmaf(w0, e0.y, fmaf(w1, e1.y, c90));         // R90 P at v + V/2
+                c270 = fmaf(w1, m0.y, fmaf(w0, m1.y, c270));       // R270 P at v + V/2
+                c90 = fmaf(w09, f0.x, fmaf(w19, f1.x, c90));       // R90 P at v
+                c270 = fmaf(w19, n0.x, fmaf(w09, n1.x, c270));     // R270 P at v
+                c180 = fmaf(w09, f0.y, fmaf(w19, f1.y, c180));     // R180 P at v + V/2
+                cP = fmaf(w19, n0.y, fmaf(w09, n1.y, cP));         // P at v + V/2
+            };
 #pragma unroll
-                for (int j = 0; j < ORB_PX; ++j)
-                    orbit(j, acc[j][0], acc[j][1], acc[j][2], acc[j][3]);   // (a row past the quadrant is not stored)
+            for (int j = 0; j < ORB_PX; ++j)
+                orbit(j, acc[j][0], acc[j][1], acc[j][2], acc[j][3]);   // (a row past the quadrant is not stored)
+        };
+        if (inside) {
+            if constexpr (SEQ) {
+                for (int vi = 0; vi < nv;) {
+                    keep(v0 + vi);
+                    for (const int ve = min(nv, bnd - v0); vi < ve; ++vi) view(vi);
+                }
+            } else {
+                for (int vi = 0; vi < nv; ++vi) view(vi);
             }
         }
         cb.sync();   // the buffer is refilled two chunks later
+    }
+    if constexpr (SEQ) {
+        keep(vb1);
+        if constexpr (!CL) {   // the only block of the tile: the sums are complete
+            if (cur > 0)
+#pragma unroll
+                for (int j = 0; j < ORB_PX; ++j)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[j][k] = kept[(k * ORB_PX + j) * ORB_TH + tid] + acc[j][k];
+        }
     }
     if constexpr (CL) {
         float *red = reinterpret_cast<float *>(osm);   // the staging buffers are free again
@@ -642,7 +694,7 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
     // fin 0: the slice's partial image; with a single slice the sums are
     // complete and the block writes the result itself: fin 1 out = sum,
     // fin 2 out = xin - tau sum
-    float *pp = (fin ? out : partial) + ((size_t)img * (fin ? 1 : nsl) + slice) * N * N;
+    float *pp = (fin ? out : partial) + ((size_t)img * (fin ? 1 : nsl) + (fin ? 0 : slice)) * N * N;
     const float *xq0 = fin == 2 ? xin + (size_t)img * N * N : nullptr;
     const float tau = fin == 2 ? fscal(scal, F_TAU) : 0.0f;
 #pragma unroll

@@ -63,6 +63,7 @@ struct Geometry {
     int tune_qrows;       // projector steps per pass of a ray walk (2 or 4)
     int tune_orb;         // A^T orbit base-view slices (1..8), slices added in a cluster
     int orb_rule;         // A^T base-view slices by the built-in rule
+    int orb_rule_op;      // the same for ct_backproject: a power of two, shared out in batches
     int tune_orb_si;      // the same for the slice-image form (solves side by side, the persistent kernel)
     int tune_tv;          // fewest interior rows of a TV tile (4..64)
     int tune_qbal;        // projector form: 1 band pair per block, 2 work-balanced ranges (0: the rule)
@@ -433,15 +434,18 @@ void launch_band_reduce(const Geometry *g, const float *partial, float *out, int
 // SMs to free together.  The orbit form's y is laid out by at_rows(g), zeros
 // past n_bins, 16-byte aligned (launch_pair_rows copies a sinogram so), or,
 // with plain set, in rows of n_bins floats; the general form's rows are ld
-// floats apart.  slices > 0 fixes the slice count.
+// floats apart.  slices > 0 fixes the slice count; blocks > 0 (mode 0 in the
+// cluster form; a divisor of the slices): that many blocks share a tile's
+// slices, to the same bits.
 bool orbit_ok(const Geometry *g);
 size_t orbit_partial_floats(const Geometry *g, int batch);
 bool orbit_slices_ok(const Geometry *g, int nsl);
 void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int mode, const float *xin,
                               const double *scal, int batch, float *partial, cudaStream_t st, bool cluster = true,
-                              int slices = 0, bool plain = false);
+                              int slices = 0, bool plain = false, int blocks = 0);
 bool orbit_plain_rows(const Geometry *g, int batch);
-int orbit_slices_rule(const Geometry *g);
+int orbit_slices_rule(const Geometry *g, bool pow2);
+int orbit_blocks(const Geometry *g, int nsl, int images);
 void launch_pair_rows(const Geometry *g, const float *in, float *out, int batch, cudaStream_t st);
 void launch_backproject(const Geometry *g, const float *y, int ld, float *out, int mode,
                         const float *xin, const double *scal, int batch, cudaStream_t st);

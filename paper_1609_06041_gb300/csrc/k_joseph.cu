@@ -777,9 +777,59 @@ k_backproject_orbit_cl(const float *__restrict__ y, int ld, const float4 *__rest
     cl.sync();   // no block leaves while its partial sums may still be read
 }
 
-static size_t orbit_smem()
+// The same sums with fewer blocks than slices: the csz blocks of a tile share
+// the nsl slices (orbit_body, SEQ), whose sums are added in slice order still,
+// so the result has k_backproject_orbit_cl's bits whatever csz is.  CL: csz >
+// 1 blocks in a cluster; else one block, which writes its sums itself.
+template <int FORM, bool CL>
+__global__ void __launch_bounds__(ORB_TH, 8)
+k_backproject_orbit_seq(const float *__restrict__ y, int ld, const float4 *__restrict__ trig, int N, int V, int B,
+                        int nsl, int csz, float *__restrict__ out)
 {
-    return sizeof(float) * 2 * ORB_VC * 8 * ORB_RW + sizeof(float4) * 4 * ORB_VC + sizeof(int) * 2 * ORB_MAXS;
+    extern __shared__ __align__(16) unsigned char osm[];
+    pdl_wait();
+    orbit_body<FORM, Block2D, CL, true>(Block2D{}, blockIdx.x, blockIdx.y, blockIdx.z, osm, y, ld, nullptr, trig, N, V,
+                                        B, nsl, 1, out, nullptr, nullptr, csz);
+    if constexpr (CL) {
+        namespace cg = cooperative_groups;
+        cg::cluster_group cl = cg::this_cluster();
+        cl.sync();   // every slice's sums are in its block's shared memory
+        const int rank = blockIdx.z % csz, img = blockIdx.z / csz;
+        const int sets = orbit_kept_sets(nsl, csz), lg = 31 - __clz(sets + 1);   // a block's slices: sets + 1 = 2^lg
+        float *red = reinterpret_cast<float *>(osm), *kept = orbit_kept(osm);
+        const int half = N / 2;
+        float *o_img = out + (size_t)img * N * N;
+        for (int e = ORB_E / csz * rank + (int)(threadIdx.y * blockDim.x + threadIdx.x); e < ORB_E / csz * (rank + 1);
+             e += ORB_TH) {
+            // the loads of all slices are issued together
+            float p[ORB_SL_MAX];
+#pragma unroll
+            for (int s = 0; s < ORB_SL_MAX; ++s) {
+                const int l = s & sets;
+                if (s < nsl) p[s] = *cl.map_shared_rank(l < sets ? kept + l * ORB_E + e : red + e, s >> lg);
+            }
+            float t = p[0];
+#pragma unroll
+            for (int s = 1; s < ORB_SL_MAX; ++s)
+                if (s < nsl) t += p[s];
+            const int k = e / (ORB_PX * ORB_TH), rem = e - k * (ORB_PX * ORB_TH);
+            const int j = rem / ORB_TH, th = rem - j * ORB_TH;
+            const int rj = blockIdx.y * ORB_T + th / ORB_T + j * ORB_TY, c = half + blockIdx.x * ORB_T + th % ORB_T;
+            if (rj < half && c < N)
+                o_img[k == 0   ? (size_t)rj * N + c
+                      : k == 1 ? (size_t)c * N + (N - 1 - rj)
+                      : k == 2 ? (size_t)(N - 1 - rj) * N + (N - 1 - c)
+                               : (size_t)(N - 1 - c) * N + rj] = t;
+        }
+        cl.sync();   // no block leaves while its sums may still be read
+    }
+}
+
+// shared memory of a block that holds the window bases of `views` base views, and `kept` sets of sums
+static size_t orbit_smem(int views = ORB_MAXS, int kept = 0)
+{
+    return sizeof(float) * 2 * ORB_VC * 8 * ORB_RW + sizeof(float4) * 4 * ORB_VC + sizeof(float) * ORB_E * kept +
+           sizeof(int) * 2 * views;
 }
 
 // out = sum of the slice images (mode 0), or xin - tau * sum (mode 1)
@@ -812,27 +862,58 @@ int orbit_slices(const Geometry *g, bool cluster)
     return t > 0 ? t : g->orb_rule;
 }
 
-// The built-in count of base-view slices: the least modelled time of A^T of
-// one image, in us, over 1 .. 8 slices of `tiles` blocks each.  A block costs
-// about 0.3 and, per base view, 0.19 alone on its SM, 0.135 with another,
-// 0.118 as one of three and 0.105 of four and more, the most blocks of any SM
-// counting; adding the slices in a cluster costs 1.  (Warm launches: 512^2 /
-// 32 views 7.1 us with one slice, 8.2 with four; 64^2 / 90 6.1 with four, 4.7
-// with eight; 256^2 / 180 9.9 and 9.0; 512^2 / 720 and 384^2 / 90 keep four.)
-int orbit_slices_rule(const Geometry *g)
+// Modelled time, in us, of A^T of `images` images by `blocks` blocks a tile,
+// each taking `share` slices of `views` base views.  A block costs about 0.3,
+// 0.07 per slice after its first and, per base view, 0.19 alone on its SM,
+// 0.135 with another, 0.118 as one of three and 0.105 of four and more, the
+// most blocks of any SM counting; adding the blocks' sums in a cluster costs 1.
+static double orbit_cost(const Geometry *g, int images, int blocks, int share, double views)
+{
+    static const double per[] = {0.19, 0.135, 0.118, 0.105};
+    const int q = (g->n / 2 + ORB_T - 1) / ORB_T;
+    const long long k = ((long long)q * q * images * blocks + g->n_sm - 1) / g->n_sm;
+    return (double)k * (share * views * per[std::min(k, 4LL) - 1] + 0.3 + 0.07 * (share - 1)) + (blocks > 1 ? 1.0 : 0.0);
+}
+
+// The built-in count of base-view slices, which fixes the order of the sums:
+// the least modelled time of one image over 1 .. 8 slices, or over 1, 2, 4
+// and 8 (pow2; ct_backproject, whose batches share them out, orbit_blocks).
+// (Warm launches: 512^2 / 32 views 7.1 us with one slice, 8.2 with four;
+// 64^2 / 90 6.1 with four, 4.7 with eight; 256^2 / 180 9.9 and 9.0; 512^2 /
+// 720 and 384^2 / 90 keep four.)
+int orbit_slices_rule(const Geometry *g, bool pow2)
 {
     if (!g->orbit) return ORB_SL;
-    const int q = (g->n / 2 + ORB_T - 1) / ORB_T, tiles = q * q;
-    const double per[] = {0.19, 0.135, 0.118, 0.105};
     int best = ORB_SL;
     double cost = -1.0;
     for (int nsl = 1; nsl <= ORB_SL_MAX; ++nsl) {
-        if (!orbit_slices_ok(g, nsl)) continue;
-        const int k = (tiles * nsl + g->n_sm - 1) / g->n_sm;
-        const double c = k * ((double)(g->n_views / 2) / nsl * per[std::min(k, 4) - 1] + 0.3) + (nsl > 1 ? 1.0 : 0.0);
+        if (!orbit_slices_ok(g, nsl) || (pow2 && (nsl & (nsl - 1)))) continue;
+        const double c = orbit_cost(g, 1, nsl, 1, (double)(g->n_views / 2) / nsl);
         if (cost < 0.0 || c < cost) {
             cost = c;
             best = nsl;
+        }
+    }
+    return best;
+}
+
+// Blocks that share a tile's nsl slices (a power of two) in a launch of
+// several images, by the same model: a batch that fills the device wants
+// fewer than a lone image.  The count of slices stays, so an image has the
+// same bits in any batch.  (Launches in a graph, a block per slice of a lone
+// image's eight -> the rule's blocks; with four slices always: 16 x 64^2 / 90
+// 7.4 -> 7.6, 7.9; 64 x 64^2 / 90 16.4 -> 15.2, 14.4; 256 x 64^2 / 90 51.2 ->
+// 38.2, 43.0; 64 x 128^2 / 60 42.7 -> 26.9, 32.4; 4 x 256^2 / 90 15.8 ->
+// 14.7, 13.9; 16 x 256^2 / 180 73.7 -> 63.3, 66.0 us.)
+int orbit_blocks(const Geometry *g, int nsl, int images)
+{
+    int best = nsl;
+    double cost = -1.0;
+    for (int c = nsl; c >= 1; c /= 2) {
+        const double t = orbit_cost(g, images, c, nsl / c, (double)(g->n_views / 2) / nsl);
+        if (cost < 0.0 || t < cost) {
+            cost = t;
+            best = c;
         }
     }
     return best;
@@ -986,38 +1067,64 @@ bool orbit_plain_rows(const Geometry *g, int batch)
 
 void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int mode, const float *xin,
                               const double *scal, int batch, float *partial, cudaStream_t st, bool cluster, int slices,
-                              bool plain)
+                              bool plain, int blocks)
 {
     const int q = g->n / 2;
     const bool cl = cluster || !partial;
     const int nsl = slices > 0 ? slices : orbit_slices(g, cl);
-    dim3 grd((q + ORB_T - 1) / ORB_T, (q + ORB_T - 1) / ORB_T, nsl * batch);
+    const int csz = blocks > 0 ? blocks : nsl;
     const bool al = g->ld == g->n_bins;
     const int ld = plain ? g->n_bins : g->ld;
-    if (nsl > 1 && cl) {
-        // several slices: their sums are added in a cluster of the slices' blocks
-        counted();
-        launch_kernel_cluster(plain ? k_backproject_orbit_cl<ORB_PLAIN>
-                              : al  ? k_backproject_orbit_cl<ORB_PAIR4>
-                                    : k_backproject_orbit_cl<ORB_PAIR>,
-                              grd,
-                              dim3(ORB_T, ORB_TY), orbit_smem(), st, dim3(1, 1, nsl), y, ld,
-                              (const float4 *)g->d_trig, g->n, g->n_views, g->n_bins, nsl, mode != 0 ? 1 : 0, out, xin,
-                              scal);
-        return;
-    }
-    // one slice: the block's sums are complete and it writes the result;
-    // several slices without a cluster: slice images, then k_orbit_reduce
-    const int fin = nsl == 1 ? 1 + (mode != 0) : 0;
-    counted(fin ? 1 : 2);
-    launch_kernel(plain ? k_backproject_orbit<ORB_PLAIN>
-                  : al  ? k_backproject_orbit<ORB_PAIR4>
-                        : k_backproject_orbit<ORB_PAIR>,
-                  grd, dim3(ORB_T, ORB_TY), orbit_smem(), st, y, ld, partial, g->d_trig, g->n, g->n_views, g->n_bins, nsl, fin, out, xin, scal);
-    if (fin) return;
     const size_t NN = (size_t)g->n * g->n;
-    launch_kernel(mode == 0 ? k_orbit_reduce<0> : k_orbit_reduce<1>, dim3((unsigned)((NN + 255) / 256), batch),
-                  dim3(256), 0, st, (const float *)partial, out, xin, scal, NN, nsl);
+    // grid.z holds 65535: larger batches go in several launches
+    const int most = 65535 / csz;
+    for (int i0 = 0; i0 < batch; i0 += most, y += (size_t)most * g->n_views * ld, out += most * NN) {
+        const int images = std::min(most, batch - i0);
+        const dim3 grd((q + ORB_T - 1) / ORB_T, (q + ORB_T - 1) / ORB_T, csz * images);
+        const float *xi = xin ? xin + (size_t)i0 * NN : nullptr;
+        if (csz < nsl) {
+            const int views = g->n_views / 2 / csz + 1;
+            const size_t smem = orbit_smem(views, orbit_kept_sets(nsl, csz));
+            const float4 *trig = g->d_trig;
+            counted();
+            if (csz > 1)
+                launch_kernel_cluster(plain ? k_backproject_orbit_seq<ORB_PLAIN, true>
+                                      : al  ? k_backproject_orbit_seq<ORB_PAIR4, true>
+                                            : k_backproject_orbit_seq<ORB_PAIR, true>,
+                                      grd, dim3(ORB_T, ORB_TY), smem, st, dim3(1, 1, csz), y, ld, trig, g->n,
+                                      g->n_views, g->n_bins, nsl, csz, out);
+            else
+                launch_kernel(plain ? k_backproject_orbit_seq<ORB_PLAIN, false>
+                              : al  ? k_backproject_orbit_seq<ORB_PAIR4, false>
+                                    : k_backproject_orbit_seq<ORB_PAIR, false>,
+                              grd, dim3(ORB_T, ORB_TY), smem, st, y, ld, trig, g->n, g->n_views, g->n_bins, nsl, csz,
+                              out);
+            continue;
+        }
+        if (nsl > 1 && cl) {
+            // several slices: their sums are added in a cluster of the slices' blocks
+            counted();
+            launch_kernel_cluster(plain ? k_backproject_orbit_cl<ORB_PLAIN>
+                                  : al  ? k_backproject_orbit_cl<ORB_PAIR4>
+                                        : k_backproject_orbit_cl<ORB_PAIR>,
+                                  grd, dim3(ORB_T, ORB_TY), orbit_smem(), st, dim3(1, 1, nsl), y, ld,
+                                  (const float4 *)g->d_trig, g->n, g->n_views, g->n_bins, nsl, mode != 0 ? 1 : 0, out,
+                                  xi, scal);
+            continue;
+        }
+        // one slice: the block's sums are complete and it writes the result;
+        // several slices without a cluster: slice images, then k_orbit_reduce
+        const int fin = nsl == 1 ? 1 + (mode != 0) : 0;
+        counted(fin ? 1 : 2);
+        launch_kernel(plain ? k_backproject_orbit<ORB_PLAIN>
+                      : al  ? k_backproject_orbit<ORB_PAIR4>
+                            : k_backproject_orbit<ORB_PAIR>,
+                      grd, dim3(ORB_T, ORB_TY), orbit_smem(), st, y, ld, partial, g->d_trig, g->n, g->n_views,
+                      g->n_bins, nsl, fin, out, xi, scal);
+        if (fin) continue;
+        launch_kernel(mode == 0 ? k_orbit_reduce<0> : k_orbit_reduce<1>, dim3((unsigned)((NN + 255) / 256), images),
+                      dim3(256), 0, st, (const float *)partial, out, xi, scal, NN, nsl);
+    }
 }
 
 void launch_backproject(const Geometry *g, const float *y, int ld, float *out, int mode,
@@ -1039,6 +1146,11 @@ void kernel_attrs_joseph()
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
     for (auto k : {k_backproject_orbit_cl<ORB_PLAIN>, k_backproject_orbit_cl<ORB_PAIR>, k_backproject_orbit_cl<ORB_PAIR4>})
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
+    // at most all base views with one set of kept sums, or half of them with three
+    for (auto k : {k_backproject_orbit_seq<ORB_PLAIN, true>, k_backproject_orbit_seq<ORB_PAIR, true>,
+                   k_backproject_orbit_seq<ORB_PAIR4, true>, k_backproject_orbit_seq<ORB_PLAIN, false>,
+                   k_backproject_orbit_seq<ORB_PAIR, false>, k_backproject_orbit_seq<ORB_PAIR4, false>})
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem(4 * ORB_MAXS + 1, 3));
     for (auto k : {k_project_quad<2>, k_project_quad<4>})
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, QUAD_SMEM_MAX);
     for (auto k : {k_project_qbal<2, false>, k_project_qbal<2, true>, k_project_qbal<4, false>, k_project_qbal<4, true>})
