@@ -490,7 +490,9 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // 63.8 us there, 238 -> 224 at 1024^2.  ORB_PAIR4: also B % 4 == 0, which makes the mirrored
 // windows' place a constant (one addition a view less, 2 %).  ORB_PLAIN: y
 // holds rows of B values, ld = B apart, copied value by value (25 us more
-// there: for small sinograms).  CL: instead of storing its sums, the
+// there: for small sinograms).  ORB_PLAIN4: such rows with B % 4 == 0, copied
+// in 16-byte pieces, two 4-byte loads for a pair's two views (for all but large
+// sinograms: no pass before it).  CL: instead of storing its sums, the
 // block leaves them in osm, entry (k ORB_PX + j) ORB_TH + tid for rotation
 // k of the thread's pixel orbit j, for a cluster reduction over slices.
 // SEQ (nsl a power of two): bz counts the csz blocks of a tile, a divisor of
@@ -498,7 +500,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // CL: the sums of those before its last are kept one by one in
 // orbit_kept(osm), the last one's are left as above.  Otherwise csz is 1: the
 // block adds its slices' sums up there and writes the result.
-enum { ORB_PLAIN = 0, ORB_PAIR, ORB_PAIR4 };
+enum { ORB_PLAIN = 0, ORB_PLAIN4, ORB_PAIR, ORB_PAIR4 };
 constexpr int ORB_E = 4 * ORB_PX * ORB_TH;   // sums of a tile
 __device__ __forceinline__ float *orbit_kept(unsigned char *osm)
 {
@@ -511,7 +513,7 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
                                            int ld, float *partial, const float4 *trig, int N, int V, int B, int nsl,
                                            int fin, float *out, const float *xin, const double *scal, int csz = 1)
 {
-    // raw[buffer][view][window (e, mirror e, e90, mirror e90)][value][row (v, v+V/2)]
+    // raw[buffer][view][window (e, mirror e, e90, mirror e90)][value][row (v, v+V/2)]; ORB_PLAIN4: [row][window][value]
     float *raw = reinterpret_cast<float *>(osm);                               // 2 x ORB_VC x 8 x ORB_RW
     float4 *tt = reinterpret_cast<float4 *>(raw + 2 * ORB_VC * 8 * ORB_RW);    // 2 x ORB_VC x 2
     float *kept = orbit_kept(osm);                                             // SEQ: orbit_kept_sets x ORB_E
@@ -528,7 +530,7 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
     const float h = 0.5f * (float)(N - 1), hb = 0.5f * (float)(B - 1), hb_lo = hb - 0.5f;
     const float xq = (float)c - h, yq = (float)r - h;               // P = (x, y); R90 P = (-y, x)
     const float *ys = y + (size_t)img * V * ld;
-    const int ms = FORM == ORB_PAIR4 ? 3 : (B - ORB_RW + 3) & 3;   // see the mirrored windows below
+    const int ms = FORM == ORB_PAIR4 || FORM == ORB_PLAIN4 ? 3 : (B - ORB_RW + 3) & 3;   // see the mirrored windows below
     const int vb0 = first_view(slice), vb1 = first_view(slice1);
     const int nvs = vb1 - vb0;
     static_assert(ORB_PX == 2, "a thread's two orbits are packed");
@@ -568,7 +570,17 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
             tt[2 * (buf * ORB_VC + tid)] = make_float4(T.x, T.x, T.y, T.y);
             tt[2 * (buf * ORB_VC + tid) + 1] = make_float4(T.z * T.z, T.z * T.z, T.z * T.w, T.z * T.w);
         }
-        if (FORM != ORB_PLAIN) {
+        if (FORM == ORB_PLAIN4) {
+            constexpr int CH = ORB_RW / 4;   // copies per window
+            for (int k = tid; k < nv * 8 * CH; k += ORB_TH) {
+                const int q = k / CH, j = k - q * CH;
+                const int win = q & 3, row = (q >> 2) & 1, vi = q >> 3;
+                const int base = wbs[2 * (v0 - vb0 + vi) + (win >> 1)];
+                const int d = ((win & 1) ? B - ORB_RW - base : base) + 4 * j;
+                const bool ok = d >= 0 && d < B;
+                cp_async16(dst0 + (size_t)q * ORB_RW + 4 * j, ys + (size_t)(v0 + vi + row * V2) * ld + (ok ? d : 0), ok);
+            }
+        } else if (FORM != ORB_PLAIN) {
             constexpr int CH = ORB_RW / 2;   // copies per window
             for (int k = tid; k < nv * 4 * CH; k += ORB_TH) {
                 const int q = k / CH, j = k - q * CH;
@@ -627,9 +639,12 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
             const float4 Ta = tv[2 * vi], Tb = tv[2 * vi + 1];
             const float2 Tx = pk(Ta.x, Ta.y), Ty = pk(Ta.z, Ta.w), Tz = pk(Tb.x, Tb.y), Tw = pk(Tb.z, Tb.w);
             const int2 wb = *reinterpret_cast<const int2 *>(wbs + 2 * (v0 - vb0 + vi));
-            // [window][value](view v, view v + V/2)
-            const float2 *e_v = reinterpret_cast<const float2 *>(tb) + (size_t)vi * 4 * ORB_RW, *m_v = e_v + ORB_RW,
-                         *e9_v = e_v + 2 * ORB_RW, *m9_v = e_v + 3 * ORB_RW;
+            // value i of window w: (view v, view v + V/2)
+            const float *win = tb + (size_t)vi * 8 * ORB_RW;
+            auto at = [&](int w, unsigned i) {
+                if constexpr (FORM == ORB_PLAIN4) return pk(win[w * ORB_RW + i], win[(4 + w) * ORB_RW + i]);
+                else return reinterpret_cast<const float2 *>(win)[w * ORB_RW + i];
+            };
             // e - 1/2 of P and of R90 P for the thread's two orbits, (x, y) = (xq, yq) and (xq, yq + ORB_TY),
             // their windows' places and weights: packed (14 issue slots a view for 28; ct_backproject 63.8 -> 62.7 us
             // at 512^2 / 720 views, each value rounded as before)
@@ -646,8 +661,8 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
                 const float w0 = fmaxf(0.0f, (j ? a0.y : a0.x)), w1 = fmaxf(0.0f, (j ? a1.y : a1.x));
                 const float w09 = fmaxf(0.0f, (j ? a09.y : a09.x)), w19 = fmaxf(0.0f, (j ? a19.y : a19.x));
                 const unsigned km = ORB_RW - 5 + ms - k, km9 = ORB_RW - 5 + ms - k9;
-                const float2 e0 = e_v[k], e1 = e_v[k + 1], m0 = m_v[km], m1 = m_v[km + 1];
-                const float2 f0 = e9_v[k9], f1 = e9_v[k9 + 1], n0 = m9_v[km9], n1 = m9_v[km9 + 1];
+                const float2 e0 = at(0, k), e1 = at(0, k + 1), m0 = at(1, km), m1 = at(1, km + 1);
+                const float2 f0 = at(2, k9), f1 = at(2, k9 + 1), n0 = at(3, km9), n1 = at(3, km9 + 1);
                 cP = fmaf(w0, e0.x, fmaf(w1, e1.x, cP));           // P at v
                 c180 = fmaf(w1, m0.x, fmaf(w0, m1.x, c180));       // R180 P at v
                 c90 = fmaf(w0, e0.y, fmaf(w1, e1.y, c90));         // R90 P at v + V/2

@@ -5,6 +5,7 @@
 #include <cmath>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include <cooperative_groups.h>
@@ -1056,13 +1057,18 @@ void launch_pair_rows(const Geometry *g, const float *in, float *out, int batch,
 }
 
 // Whether a caller's sinogram is better read in its own rows than interleaved
-// first: where the pass and its launch (about 1.5 us) cost more than copying
-// the windows value by value, that is for little work and few views (64^2 / 90
-// views 5.1 against 6.0 us, 128^2 / 90 6.2 / 6.4, 256^2 / 32 5.8 / 6.6; but
-// 128^2 / 180 8.0 / 7.9, 64^2 / 720 17.1 / 13.1, 512^2 / 32 8.6 / 7.6).
+// first, which takes a pass, a launch and scratch (about 1.2 us in a graph, 2
+// to 4 as a call).  Rows of whole 16-byte pieces are copied so, and interleaving
+// gains 4 to 6 % of a large launch only (graph, own rows / interleaved: 64^2 /
+// 90 views 4.5 / 5.8 us, 256^2 / 90 6.4 / 7.6, 512^2 / 90 13.1 / 13.7, 512^2 /
+// 360 34.6 / 34.2, 512^2 / 720 65.0 / 62.5, 1024^2 / 720 235 / 222).  Others
+// are copied value by value: for little work and few views (64^2 / 90 4.9 /
+// 5.8 us, 128^2 / 90 5.7 / 6.4, 256^2 / 32 5.3 / 6.4; but 128^2 / 180 7.6 /
+// 7.6, 64^2 / 720 15.7 / 12.1, 512^2 / 32 7.8 / 7.0).
 bool orbit_plain_rows(const Geometry *g, int batch)
 {
-    return g->n_views <= 128 && (double)g->n * g->n * g->n_views * batch <= 2.5e6;
+    const double pixel_views = (double)g->n * g->n * g->n_views * batch;
+    return g->ld == g->n_bins ? pixel_views <= 1.2e8 : g->n_views <= 128 && pixel_views <= 2.5e6;
 }
 
 void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int mode, const float *xin,
@@ -1076,54 +1082,50 @@ void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int
     const bool al = g->ld == g->n_bins;
     const int ld = plain ? g->n_bins : g->ld;
     const size_t NN = (size_t)g->n * g->n;
-    // grid.z holds 65535: larger batches go in several launches
-    const int most = 65535 / csz;
-    for (int i0 = 0; i0 < batch; i0 += most, y += (size_t)most * g->n_views * ld, out += most * NN) {
-        const int images = std::min(most, batch - i0);
-        const dim3 grd((q + ORB_T - 1) / ORB_T, (q + ORB_T - 1) / ORB_T, csz * images);
-        const float *xi = xin ? xin + (size_t)i0 * NN : nullptr;
+    const float4 *trig = g->d_trig;
+    const dim3 th(ORB_T, ORB_TY);
+    auto launch = [&](auto form, const float *yi, float *o, const float *xi, dim3 grd) {
+        constexpr int FORM = decltype(form)::value;
         if (csz < nsl) {
-            const int views = g->n_views / 2 / csz + 1;
-            const size_t smem = orbit_smem(views, orbit_kept_sets(nsl, csz));
-            const float4 *trig = g->d_trig;
+            // fewer blocks than slices
+            const size_t smem = orbit_smem(g->n_views / 2 / csz + 1, orbit_kept_sets(nsl, csz));
             counted();
             if (csz > 1)
-                launch_kernel_cluster(plain ? k_backproject_orbit_seq<ORB_PLAIN, true>
-                                      : al  ? k_backproject_orbit_seq<ORB_PAIR4, true>
-                                            : k_backproject_orbit_seq<ORB_PAIR, true>,
-                                      grd, dim3(ORB_T, ORB_TY), smem, st, dim3(1, 1, csz), y, ld, trig, g->n,
-                                      g->n_views, g->n_bins, nsl, csz, out);
+                launch_kernel_cluster(k_backproject_orbit_seq<FORM, true>, grd, th, smem, st, dim3(1, 1, csz), yi, ld,
+                                      trig, g->n, g->n_views, g->n_bins, nsl, csz, o);
             else
-                launch_kernel(plain ? k_backproject_orbit_seq<ORB_PLAIN, false>
-                              : al  ? k_backproject_orbit_seq<ORB_PAIR4, false>
-                                    : k_backproject_orbit_seq<ORB_PAIR, false>,
-                              grd, dim3(ORB_T, ORB_TY), smem, st, y, ld, trig, g->n, g->n_views, g->n_bins, nsl, csz,
-                              out);
-            continue;
+                launch_kernel(k_backproject_orbit_seq<FORM, false>, grd, th, smem, st, yi, ld, trig, g->n, g->n_views,
+                              g->n_bins, nsl, csz, o);
+            return;
         }
         if (nsl > 1 && cl) {
             // several slices: their sums are added in a cluster of the slices' blocks
             counted();
-            launch_kernel_cluster(plain ? k_backproject_orbit_cl<ORB_PLAIN>
-                                  : al  ? k_backproject_orbit_cl<ORB_PAIR4>
-                                        : k_backproject_orbit_cl<ORB_PAIR>,
-                                  grd, dim3(ORB_T, ORB_TY), orbit_smem(), st, dim3(1, 1, nsl), y, ld,
-                                  (const float4 *)g->d_trig, g->n, g->n_views, g->n_bins, nsl, mode != 0 ? 1 : 0, out,
-                                  xi, scal);
-            continue;
+            launch_kernel_cluster(k_backproject_orbit_cl<FORM>, grd, th, orbit_smem(), st, dim3(1, 1, nsl), yi, ld, trig,
+                                  g->n, g->n_views, g->n_bins, nsl, mode != 0 ? 1 : 0, o, xi, scal);
+            return;
         }
         // one slice: the block's sums are complete and it writes the result;
         // several slices without a cluster: slice images, then k_orbit_reduce
         const int fin = nsl == 1 ? 1 + (mode != 0) : 0;
         counted(fin ? 1 : 2);
-        launch_kernel(plain ? k_backproject_orbit<ORB_PLAIN>
-                      : al  ? k_backproject_orbit<ORB_PAIR4>
-                            : k_backproject_orbit<ORB_PAIR>,
-                      grd, dim3(ORB_T, ORB_TY), orbit_smem(), st, y, ld, partial, g->d_trig, g->n, g->n_views,
-                      g->n_bins, nsl, fin, out, xi, scal);
-        if (fin) continue;
-        launch_kernel(mode == 0 ? k_orbit_reduce<0> : k_orbit_reduce<1>, dim3((unsigned)((NN + 255) / 256), images),
-                      dim3(256), 0, st, (const float *)partial, out, xi, scal, NN, nsl);
+        launch_kernel(k_backproject_orbit<FORM>, grd, th, orbit_smem(), st, yi, ld, partial, trig, g->n, g->n_views,
+                      g->n_bins, nsl, fin, o, xi, scal);
+        if (fin) return;
+        launch_kernel(mode == 0 ? k_orbit_reduce<0> : k_orbit_reduce<1>,
+                      dim3((unsigned)((NN + 255) / 256), grd.z / nsl), dim3(256), 0, st, (const float *)partial, o, xi,
+                      scal, NN, nsl);
+    };
+    // grid.z holds 65535: larger batches go in several launches
+    const int most = 65535 / csz;
+    for (int i0 = 0; i0 < batch; i0 += most) {
+        const dim3 grd((q + ORB_T - 1) / ORB_T, (q + ORB_T - 1) / ORB_T, csz * std::min(most, batch - i0));
+        const float *yi = y + (size_t)i0 * g->n_views * ld, *xi = xin ? xin + i0 * NN : nullptr;
+        float *o = out + i0 * NN;
+        if (plain && al) launch(std::integral_constant<int, ORB_PLAIN4>{}, yi, o, xi, grd);
+        else if (plain) launch(std::integral_constant<int, ORB_PLAIN>{}, yi, o, xi, grd);
+        else if (al) launch(std::integral_constant<int, ORB_PAIR4>{}, yi, o, xi, grd);
+        else launch(std::integral_constant<int, ORB_PAIR>{}, yi, o, xi, grd);
     }
 }
 
@@ -1142,15 +1144,20 @@ void kernel_attrs_joseph()
 {
     cudaFuncSetAttribute(k_project_direct, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(DIRECT_BANDS * quad_smem(2 * MR * DIRECT_BANDS) + sizeof(float4) * DIRECT_THREADS));
-    for (auto k : {k_backproject_orbit<ORB_PLAIN>, k_backproject_orbit<ORB_PAIR>, k_backproject_orbit<ORB_PAIR4>})
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
-    for (auto k : {k_backproject_orbit_cl<ORB_PLAIN>, k_backproject_orbit_cl<ORB_PAIR>, k_backproject_orbit_cl<ORB_PAIR4>})
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
-    // at most all base views with one set of kept sums, or half of them with three
-    for (auto k : {k_backproject_orbit_seq<ORB_PLAIN, true>, k_backproject_orbit_seq<ORB_PAIR, true>,
-                   k_backproject_orbit_seq<ORB_PAIR4, true>, k_backproject_orbit_seq<ORB_PLAIN, false>,
-                   k_backproject_orbit_seq<ORB_PAIR, false>, k_backproject_orbit_seq<ORB_PAIR4, false>})
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem(4 * ORB_MAXS + 1, 3));
+    auto orbit_attrs = [](auto form) {
+        constexpr int FORM = decltype(form)::value;
+        cudaFuncSetAttribute(k_backproject_orbit<FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)orbit_smem());
+        cudaFuncSetAttribute(k_backproject_orbit_cl<FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)orbit_smem());
+        // at most all base views with one set of kept sums, or half of them with three
+        const int shared = (int)orbit_smem(4 * ORB_MAXS + 1, 3);
+        cudaFuncSetAttribute(k_backproject_orbit_seq<FORM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, shared);
+        cudaFuncSetAttribute(k_backproject_orbit_seq<FORM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, shared);
+    };
+    orbit_attrs(std::integral_constant<int, ORB_PLAIN>{});
+    orbit_attrs(std::integral_constant<int, ORB_PLAIN4>{});
+    orbit_attrs(std::integral_constant<int, ORB_PAIR>{});
+    orbit_attrs(std::integral_constant<int, ORB_PAIR4>{});
     for (auto k : {k_project_quad<2>, k_project_quad<4>})
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, QUAD_SMEM_MAX);
     for (auto k : {k_project_qbal<2, false>, k_project_qbal<2, true>, k_project_qbal<4, false>, k_project_qbal<4, true>})
