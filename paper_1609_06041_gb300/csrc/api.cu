@@ -515,8 +515,8 @@ ct_status ct_geometry_create(int n, int n_views, int n_bins, const double *angle
     g->n_fft = 1;
     while (g->n_fft < 2 * n_bins) g->n_fft <<= 1;
     g->p_fft = fft_length(n_bins);
-    g->ld = (n_bins + 3) & ~3;
     g->orbit = !angles && (n_views % 2 == 0) && (n % 2 == 0);   // V <= 8192, so a slice has <= 1024 base views
+    g->ld = g->orbit ? (n_bins + 3) & ~3 : n_bins;
     cudaGetDevice(&g->device);
     g->n_sm = 0;
     if (cudaDeviceGetAttribute(&g->n_sm, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess || g->n_sm < 1) {
@@ -705,7 +705,7 @@ ct_status ct_backproject(const ct_geometry *g, const float *sino, float *img, in
     if (!img || !sino) return fail(CT_ERR_ARG, "ct_backproject: NULL pointer");
     if (!aligned16(img) || !aligned16(sino)) return fail(CT_ERR_ARG, "ct_backproject: pointers must be 16-byte aligned");
     if (!orbit_ok(g)) {
-        launch_backproject(g, sino, g->n_bins, img, 0, nullptr, nullptr, batch, S(stream));
+        launch_backproject(g, sino, img, 0, nullptr, nullptr, batch, S(stream));
         return cuda_check("ct_backproject");
     }
     // views v and v + V/2 interleaved first (stream-ordered scratch), 2 to 3 us at 512^2 / 720 views; small sinograms,
@@ -963,7 +963,7 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
     // A^T, by rotation orbits when the geometry allows
     auto backproject = [&](const float *yy, float *out, int md, const float *xin) {
         if (orbit_ok(g)) launch_backproject_orbit(g, yy, out, md, xin, scal, 1, orb, st, allow_fork);
-        else launch_backproject(g, yy, g->ld, out, md, xin, scal, 1, st);
+        else launch_backproject(g, yy, out, md, xin, scal, 1, st);
     };
     float *pbuf[2] = {(float *)(ws + L.p0), (float *)(ws + L.p1)};
     const int half = prm->precond ? g->n_bins : 1;

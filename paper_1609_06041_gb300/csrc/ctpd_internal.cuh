@@ -42,7 +42,7 @@ struct Geometry {
     int n, n_views, n_bins, device;
     int n_fft;            // P = 2^ceil(log2(2B)), the period of the taps
     int p_fft;            // transform length of D's convolution: n_fft, at least 64
-    int ld;               // row stride of the sinograms A^T reads inside the library: n_bins rounded up to 4
+    int ld;               // row stride of the sinograms A^T reads inside the library: n_bins, rounded up to 4 for orbits
     int n_row, n_col;     // views stepping along rows / columns
     float win_eps;        // candidate-window margin (bins) of the backprojector
     ViewP *d_views;       // device, n_views entries
@@ -433,8 +433,7 @@ void launch_band_reduce(const Geometry *g, const float *partial, float *out, int
 // form for solves run side by side, whose clusters would wait for a GPC's
 // SMs to free together.  The orbit form's y is laid out by at_rows(g), zeros
 // past n_bins, 16-byte aligned (launch_pair_rows copies a sinogram so), or,
-// with plain set, in rows of n_bins floats; the general form's rows are ld
-// floats apart.  slices > 0 fixes the slice count; blocks > 0 (mode 0 in the
+// with plain set, in rows of n_bins floats, as the general form's is.  slices > 0 fixes the slice count; blocks > 0 (mode 0 in the
 // cluster form; a divisor of the slices): that many blocks share a tile's
 // slices, to the same bits.
 bool orbit_ok(const Geometry *g);
@@ -447,7 +446,7 @@ bool orbit_plain_rows(const Geometry *g, int batch);
 int orbit_slices_rule(const Geometry *g, bool pow2);
 int orbit_blocks(const Geometry *g, int nsl, int images);
 void launch_pair_rows(const Geometry *g, const float *in, float *out, int batch, cudaStream_t st);
-void launch_backproject(const Geometry *g, const float *y, int ld, float *out, int mode,
+void launch_backproject(const Geometry *g, const float *y, float *out, int mode,
                         const float *xin, const double *scal, int batch, cudaStream_t st);
 
 // Sinograms that A^T reads inside the library (mu_bar, the adjoint's dL/dr)

@@ -635,7 +635,7 @@ constexpr int BWW = 32;         // staged ray pairs per view (>= 15 (|cos|+|sin|
 
 template <int MODE>
 __global__ void __launch_bounds__(BTH)
-k_backproject_tiles(const float *__restrict__ y, int ld, float *__restrict__ out,
+k_backproject_tiles(const float *__restrict__ y, float *__restrict__ out,
                     const float4 *__restrict__ trig, int N, int V, int B,
                     const float *__restrict__ xin, const double *__restrict__ scal)
 {
@@ -648,7 +648,7 @@ k_backproject_tiles(const float *__restrict__ y, int ld, float *__restrict__ out
     const int slice = tid >> 6, l = tid & 63;
     const int R0 = blockIdx.y * BT, C0 = blockIdx.x * BT;
     const int r = R0 + (l >> 2), c0 = C0 + (l & 3) * 4;
-    const float *ys = y + (size_t)blockIdx.z * V * ld;
+    const float *ys = y + (size_t)blockIdx.z * V * B;
     const float h = 0.5f * (float)(N - 1);
     const float hb_lo = 0.5f * (float)(B - 1) - 0.5f;   // e - 1/2 is rounded to find floor(e)
     const float yr = (float)r - h;
@@ -678,7 +678,7 @@ k_backproject_tiles(const float *__restrict__ y, int ld, float *__restrict__ out
         for (int k = tid; k < nv * BWW; k += BTH) {
             const int vi = k / BWW, w = k - vi * BWW;
             const int d = wbase[vi] + w;
-            const float *yv = ys + (size_t)(v0 + vi) * ld;
+            const float *yv = ys + (size_t)(v0 + vi) * B;
             const float sc = sv[vi].z;
             const float y0 = (d >= 0 && d < B) ? yv[d] : 0.0f;
             const float y1 = (d + 1 >= 0 && d + 1 < B) ? yv[d + 1] : 0.0f;
@@ -1129,15 +1129,15 @@ void launch_backproject_orbit(const Geometry *g, const float *y, float *out, int
     }
 }
 
-void launch_backproject(const Geometry *g, const float *y, int ld, float *out, int mode,
+void launch_backproject(const Geometry *g, const float *y, float *out, int mode,
                         const float *xin, const double *scal, int batch, cudaStream_t st)
 {
     dim3 grd((g->n + BT - 1) / BT, (g->n + BT - 1) / BT, batch);
     counted();
     if (mode == 0)
-        k_backproject_tiles<0><<<grd, BTH, 0, st>>>(y, ld, out, g->d_trig, g->n, g->n_views, g->n_bins, xin, scal);
+        k_backproject_tiles<0><<<grd, BTH, 0, st>>>(y, out, g->d_trig, g->n, g->n_views, g->n_bins, xin, scal);
     else
-        k_backproject_tiles<1><<<grd, BTH, 0, st>>>(y, ld, out, g->d_trig, g->n, g->n_views, g->n_bins, xin, scal);
+        k_backproject_tiles<1><<<grd, BTH, 0, st>>>(y, out, g->d_trig, g->n, g->n_views, g->n_bins, xin, scal);
 }
 
 void kernel_attrs_joseph()

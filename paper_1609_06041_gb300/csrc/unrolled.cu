@@ -76,14 +76,14 @@ struct CK {
 
 CK ck_at(char *ws, const UL &L, const Geometry *g, int S, int k)
 {
-    // x first, then mu_bar: both 16-byte aligned where the orbit backprojector serves (N even)
+    // x, p and mu_bar first: 16-byte aligned where N is even (p is read in pairs then, mu_bar by the orbit backprojector)
     const size_t J = (size_t)g->n * g->n, Ip = (size_t)g->n_views * g->ld;
     float *base = (float *)(ws + L.ck) + (size_t)k * L.ck_stride;
     CK c;
     c.x = base;
-    c.mubar = c.x + S * J;
-    c.p = c.mubar + S * Ip;
-    c.mu = c.p + S * 2 * J;
+    c.p = c.x + S * J;
+    c.mubar = c.p + S * 2 * J;
+    c.mu = c.mubar + S * Ip;
     return c;
 }
 
@@ -145,7 +145,7 @@ void backproject(const Geometry *g, const float *y, float *out, int mode, const 
     if (orbit_ok(g))
         launch_backproject_orbit(g, y, out, mode, xin, scal, S, (float *)(ws + L.orb), st, true,
                                  g->tune_orb > 0 ? 0 : 4);
-    else launch_backproject(g, y, g->ld, out, mode, xin, scal, S, st);
+    else launch_backproject(g, y, out, mode, xin, scal, S, st);
 }
 
 }  // namespace
