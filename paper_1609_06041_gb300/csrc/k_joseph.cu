@@ -867,13 +867,15 @@ int orbit_slices(const Geometry *g, bool cluster)
 // each taking `share` slices of `views` base views.  A block costs about 0.3,
 // 0.07 per slice after its first and, per base view, 0.19 alone on its SM,
 // 0.135 with another, 0.118 as one of three and 0.105 of four and more, the
-// most blocks of any SM counting; adding the blocks' sums in a cluster costs 1.
+// most blocks of any SM counting; adding the blocks' sums in a cluster costs 1
+// and 0.6 per slice after a block's first.
 static double orbit_cost(const Geometry *g, int images, int blocks, int share, double views)
 {
     static const double per[] = {0.19, 0.135, 0.118, 0.105};
     const int q = (g->n / 2 + ORB_T - 1) / ORB_T;
     const long long k = ((long long)q * q * images * blocks + g->n_sm - 1) / g->n_sm;
-    return (double)k * (share * views * per[std::min(k, 4LL) - 1] + 0.3 + 0.07 * (share - 1)) + (blocks > 1 ? 1.0 : 0.0);
+    return (double)k * (share * views * per[std::min(k, 4LL) - 1] + 0.3 + 0.07 * (share - 1)) +
+           (blocks > 1 ? 1.0 + 0.6 * (share - 1) : 0.0);
 }
 
 // The built-in count of base-view slices, which fixes the order of the sums:
@@ -901,11 +903,12 @@ int orbit_slices_rule(const Geometry *g, bool pow2)
 // Blocks that share a tile's nsl slices (a power of two) in a launch of
 // several images, by the same model: a batch that fills the device wants
 // fewer than a lone image.  The count of slices stays, so an image has the
-// same bits in any batch.  (Launches in a graph, a block per slice of a lone
-// image's eight -> the rule's blocks; with four slices always: 16 x 64^2 / 90
-// 7.4 -> 7.6, 7.9; 64 x 64^2 / 90 16.4 -> 15.2, 14.4; 256 x 64^2 / 90 51.2 ->
-// 38.2, 43.0; 64 x 128^2 / 60 42.7 -> 26.9, 32.4; 4 x 256^2 / 90 15.8 ->
-// 14.7, 13.9; 16 x 256^2 / 180 73.7 -> 63.3, 66.0 us.)
+// same bits in any batch.  (Launches in a graph, aligned rows, a block per
+// slice of a lone image's eight -> the rule's blocks; with four slices always:
+// 64 x 64^2 / 90 15.0 -> 13.9, 13.2; 256 x 64^2 / 90 48.7 -> 36.0, 41.4; 128 x
+// 48^2 / 60 22.8 -> 16.6, 16.8; 64 x 128^2 / 60 42.0 -> 26.3, 32.0; 4 x 256^2 /
+// 90 15.3 -> 14.0, 13.7; 8 x 256^2 / 90 26.8 -> 22.4, 23.0; 4 x 256^2 / 180
+// 22.0 -> 21.3, 20.7; 16 x 256^2 / 180 73.7 -> 63.7, 68.5 us.)
 int orbit_blocks(const Geometry *g, int nsl, int images)
 {
     int best = nsl;

@@ -35,7 +35,8 @@ def test_large_batches(N, V, B, slices, batch):
 # blocks of slices: 4, 2 and 1 of 8 (14 views: a slice of no base views), 2 and 1 of 4, 1 of 2
 @pytest.mark.parametrize("N,V,batch", [(34, 14, 5), (64, 90, 16), (128, 180, 5), (34, 16, 16), (100, 16, 4), (34, 14, 16),
                                        (100, 14, 3), (100, 60, 16), (256, 32, 3), (320, 60, 2), (192, 16, 2),
-                                       (256, 60, 4), (512, 60, 2)])
+                                       (256, 60, 4), (512, 60, 2), (34, 90, 64), (96, 60, 16), (192, 60, 4), (34, 180, 128),
+                                       (100, 180, 32), (384, 90, 2), (320, 90, 3)])
 @pytest.mark.parametrize("wide", [False, True])
 def test_blocks_that_share_the_slices(N, V, batch, wide):
     P = need_gpu()
