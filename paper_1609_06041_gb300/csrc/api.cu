@@ -624,8 +624,8 @@ ct_status ct_geometry_create(int n, int n_views, int n_bins, const double *angle
     g->pool = scratch_pool_acquire(g->device);
     kernel_attrs_filter();
     kernel_attrs_tv();
-    kernel_attrs_joseph();
-    kernel_attrs_fft();
+    kernel_attrs_joseph(g);
+    kernel_attrs_fft(g);
     kernel_attrs_grad();
     ct_status st = cuda_check("ct_geometry_create");
     if (st != CT_OK) {

@@ -503,7 +503,7 @@ void launch_dual_sv(const Geometry *g, const float2 *hs, const float2 *hd, const
                     cudaStream_t st);
 // s = sqrt(kappa w), kappa = scal[S_KAPPA]
 void launch_sv_scale(const float *w, const double *scal, float *s, size_t n, cudaStream_t st);
-void kernel_attrs_fft();
+void kernel_attrs_fft(const Geometry *g);
 void launch_dual_fft_batched(const Geometry *g, const float2 *hhat, const float *partial, const float *b,
                              const float *mu_in, float *mu_out, float *mu_bar, const float *winv, int lowdose,
                              const double *scal, int batch, cudaStream_t st);
@@ -622,6 +622,7 @@ void launch_lanczos_fused(float *w, const float *tp, const float *tc, size_t n, 
 size_t dot_partials_doubles();
 void kernel_attrs_filter();
 void kernel_attrs_tv();
-void kernel_attrs_joseph();
+// shared-memory limits of the kernels this geometry's calls launch (which also loads them)
+void kernel_attrs_joseph(const Geometry *g);
 
 }  // namespace ctpd

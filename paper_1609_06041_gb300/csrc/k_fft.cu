@@ -656,23 +656,23 @@ void launch_dual_bwd_fft(const Geometry *g, const float2 *hhat, const float *par
 
 bool fft_supported(const Geometry *g) { return g->n_fft <= FFT_MAX_P; }
 
-void kernel_attrs_fft()
+void kernel_attrs_fft(const Geometry *g)
 {
-    for (int p = 64; p <= FFT_MAX_P; p <<= 1)
-        with_length(p, [&](auto L) {
-            constexpr int P = decltype(L)::value;
-            const int sm = (int)block_smem(P);
-            cudaFuncSetAttribute(k_hhat<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_filter_fft<P, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_filter_fft<P, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_filter_fft<P, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_dual_fft<P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_dual_fft<P, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_dual_bwd_fft<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_filter_sv<P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_filter_sv<P, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_dual_sv<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        });
+    if (!fft_supported(g)) return;
+    with_length(g->p_fft, [&](auto L) {
+        constexpr int P = decltype(L)::value;
+        const int sm = (int)block_smem(P);
+        cudaFuncSetAttribute(k_hhat<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_filter_fft<P, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_filter_fft<P, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_filter_fft<P, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_dual_fft<P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_dual_fft<P, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_dual_bwd_fft<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_filter_sv<P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_filter_sv<P, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_dual_sv<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    });
 }
 
 }  // namespace ctpd

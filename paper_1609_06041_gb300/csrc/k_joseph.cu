@@ -1143,7 +1143,7 @@ void launch_backproject(const Geometry *g, const float *y, float *out, int mode,
         k_backproject_tiles<1><<<grd, BTH, 0, st>>>(y, out, g->d_trig, g->n, g->n_views, g->n_bins, xin, scal);
 }
 
-void kernel_attrs_joseph()
+void kernel_attrs_joseph(const Geometry *g)
 {
     cudaFuncSetAttribute(k_project_direct, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(DIRECT_BANDS * quad_smem(2 * MR * DIRECT_BANDS) + sizeof(float4) * DIRECT_THREADS));
@@ -1157,10 +1157,13 @@ void kernel_attrs_joseph()
         cudaFuncSetAttribute(k_backproject_orbit_seq<FORM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, shared);
         cudaFuncSetAttribute(k_backproject_orbit_seq<FORM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, shared);
     };
-    orbit_attrs(std::integral_constant<int, ORB_PLAIN>{});
-    orbit_attrs(std::integral_constant<int, ORB_PLAIN4>{});
-    orbit_attrs(std::integral_constant<int, ORB_PAIR>{});
-    orbit_attrs(std::integral_constant<int, ORB_PAIR4>{});
+    if (g->orbit && g->ld == g->n_bins) {
+        orbit_attrs(std::integral_constant<int, ORB_PLAIN4>{});
+        orbit_attrs(std::integral_constant<int, ORB_PAIR4>{});
+    } else if (g->orbit) {
+        orbit_attrs(std::integral_constant<int, ORB_PLAIN>{});
+        orbit_attrs(std::integral_constant<int, ORB_PAIR>{});
+    }
     for (auto k : {k_project_quad<2>, k_project_quad<4>})
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, QUAD_SMEM_MAX);
     for (auto k : {k_project_qbal<2, false>, k_project_qbal<2, true>, k_project_qbal<4, false>, k_project_qbal<4, true>})
