@@ -709,12 +709,16 @@ ct_status ct_backproject(const ct_geometry *g, const float *sino, float *img, in
         return cuda_check("ct_backproject");
     }
     // views v and v + V/2 interleaved first (stream-ordered scratch), 2 to 3 us at 512^2 / 720 views; small sinograms,
-    // and calls for which there is no scratch, are read in their own rows
+    // calls for which there is no scratch, and captured ones (allocation nodes would keep the caller's graph from being
+    // cloned, nested or instantiated twice) are read in their own rows, to the same bits
     const int slices = g->tune_orb > 0 ? g->tune_orb : g->orb_rule_op;
     const int blocks = g->tune_orb > 0 ? slices : orbit_blocks(g, slices, batch);
     const size_t bytes = sizeof(float) * (size_t)batch * g->n_views * g->ld;
     float *pairs = nullptr;
-    if (!orbit_plain_rows(g, batch) && scratch_alloc(g, &pairs, bytes, S(stream)) != cudaSuccess) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (!orbit_plain_rows(g, batch) &&
+        (cudaStreamIsCapturing(S(stream), &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+         scratch_alloc(g, &pairs, bytes, S(stream)) != cudaSuccess)) {
         cudaGetLastError();
         pairs = nullptr;
     }
