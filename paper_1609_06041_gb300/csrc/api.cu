@@ -677,7 +677,7 @@ ct_status ct_project(const ct_geometry *g, const float *img, float *sino, int ba
     launch_project_bands(g, img, partial, batch, S(stream));
     {
         PdlScope pdl(true);   // launched as the projector ends; it waits for it
-        launch_band_reduce(g, partial, sino, 0, nullptr, nullptr, nullptr, batch, S(stream));
+        launch_band_reduce(g, partial, sino, batch, S(stream));
     }
     cudaFreeAsync(partial, S(stream));
     return cuda_check("ct_project");
@@ -1061,7 +1061,7 @@ ct_status ctpd::pdtv_solve(const ct_geometry *g, const float *b, const float *w,
                 } else if (use_fft) {
                     launch_filter_fft_bands(g, hhat, band, mubar, 1, st, at_rows(g));
                 } else {
-                    launch_band_reduce(g, band, r, 0, nullptr, nullptr, nullptr, 1, st);
+                    launch_band_reduce(g, band, r, 1, st);
                     launch_filter(g, taps, half, r, mubar, at_rows(g), nullptr, nullptr, 0, nullptr, 1, st);
                 }
                 backproject(mubar, out, 0, nullptr);

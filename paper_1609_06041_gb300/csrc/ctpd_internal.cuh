@@ -421,11 +421,8 @@ void launch_project_direct(const Geometry *g, const float *x, float *out, int ba
 void *proj_plans_create();
 void proj_plans_free(void *p);
 void proj_plans_clear(Geometry *g);
-// out = scale_v * sum_b partial[b]   (mode 0), minus b and winv*mu (mode 1),
-// minus b (mode 2).
-void launch_band_reduce(const Geometry *g, const float *partial, float *out, int mode,
-                        const float *b, const float *winv, const float *mu, int batch,
-                        cudaStream_t st);
+// out = scale_v * sum_b partial[b]
+void launch_band_reduce(const Geometry *g, const float *partial, float *out, int batch, cudaStream_t st);
 // Backprojection; mode 0: out = A^T y; mode 1: out = xin - tau*A^T y with
 // tau = (float)scal[S_TAU].  The orbit form adds its base-view slices in a
 // thread-block cluster (cluster, or partial NULL), or through slice images
@@ -584,7 +581,6 @@ void launch_eps_step(const Geometry *g, const float *q, float *out, Rows ldo, fl
 // Small helpers
 void launch_fill(float *p, float v, size_t n, cudaStream_t st);
 void launch_recip(const float *w, float *winv, size_t n, cudaStream_t st);
-void launch_scale_by(const float *in, const float *s, int sqrt_s, float *out, size_t n, cudaStream_t st);
 // A solve's setup around its Lanczos runs (n = V B).  First the input checks
 // into flags, winv = 1 / w with its partial sums (w NULL: neither), sw =
 // sqrt(winv), the start vectors t_sino (n) and t_img (n_img) (each may be

@@ -527,12 +527,10 @@ void launch_project_bands(const Geometry *g, const float *x, float *partial, int
                                                      g->n_col, N, g->n_views, g->n_bins, partial);
 }
 
-// out[v][d] = scale_v * sum_b partial[b][v][d]  (+ residual epilogue)
-template <int MODE>
+// out[v][d] = scale_v * sum_b partial[b][v][d]; SCALED: times fac[0]
+template <bool SCALED>
 __global__ void k_band_reduce(const float *__restrict__ partial, float *__restrict__ out,
-                              const ViewP *__restrict__ views, int nb, int V, int B,
-                              const float *__restrict__ b, const float *__restrict__ winv,
-                              const float *__restrict__ mu)
+                              const ViewP *__restrict__ views, int nb, int V, int B, const double *__restrict__ fac)
 {
     pdl_wait();
     const int d = blockIdx.x * blockDim.x + threadIdx.x, v = blockIdx.y;
@@ -541,15 +539,12 @@ __global__ void k_band_reduce(const float *__restrict__ partial, float *__restri
     const float *p = partial + (size_t)blockIdx.z * nb * VB + (size_t)v * B + d;
     float acc = 0.0f;
     for (int k = 0; k < nb; ++k) acc += p[k * VB];
-    const size_t o = (size_t)blockIdx.z * VB + (size_t)v * B + d;
     float val = acc * views[v].scale;
-    if (MODE == 1) val = val - b[o] - winv[o] * mu[o];
-    else if (MODE == 2) val = val - b[o];
-    else if (MODE == 3) val *= (float)(*reinterpret_cast<const double *>(b));
-    out[o] = val;
+    if (SCALED) val *= (float)*fac;
+    out[(size_t)blockIdx.z * VB + (size_t)v * B + d] = val;
 }
 
-// The plain sum (mode 0) for B % 4 == 0, four bins a thread and four bands'
+// The plain sum for B % 4 == 0, four bins a thread and four bands'
 // loads together: with the projector before it, 512^2 / 720 views 70.3 -> 68.7
 // us, 1024^2 / 720 341.6 -> 329.9 (eight and sixteen bands together are slower,
 // 71.0 and 71.4 us: more rows of the partial sums open at once).
@@ -581,22 +576,21 @@ k_band_reduce4(const float4 *__restrict__ partial, float4 *__restrict__ out, con
     out[(size_t)blockIdx.y * vb4 + i] = make_float4(acc.x * s, acc.y * s, acc.z * s, acc.w * s);
 }
 
-void launch_band_reduce(const Geometry *g, const float *partial, float *out, int mode,
-                        const float *b, const float *winv, const float *mu, int batch, cudaStream_t st)
+void launch_band_reduce(const Geometry *g, const float *partial, float *out, int batch, cudaStream_t st)
 {
     dim3 grd((g->n_bins + 255) / 256, g->n_views, batch);
     const int nb = proj_bands(g->n);
     counted();
     const unsigned b4 = g->n_bins / 4, vb4 = b4 * g->n_views;
     // below 20000 rays the grid of four-bin threads is too small (256^2 / 32 views: 7.6 against 7.3 us)
-    if (mode == 0 && g->n_bins % 4 == 0 && 4 * vb4 >= 20000 &&
+    if (g->n_bins % 4 == 0 && 4 * vb4 >= 20000 &&
         (reinterpret_cast<uintptr_t>(partial) | reinterpret_cast<uintptr_t>(out)) % 16 == 0) {
         launch_kernel(k_band_reduce4, dim3((vb4 + 255) / 256, batch), dim3(256), 0, st, (const float4 *)partial,
                       (float4 *)out, g->d_views, nb, vb4, b4);
         return;
     }
-    launch_kernel(mode == 0 ? k_band_reduce<0> : mode == 1 ? k_band_reduce<1> : k_band_reduce<2>, grd, dim3(256), 0, st,
-                  partial, out, g->d_views, nb, g->n_views, g->n_bins, b, winv, mu);
+    launch_kernel(k_band_reduce<false>, grd, dim3(256), 0, st, partial, out, g->d_views, nb, g->n_views, g->n_bins,
+                  nullptr);
 }
 
 // out = fac * A x from the band partials (fac: one device double)
@@ -605,8 +599,7 @@ void launch_band_reduce_scaled(const Geometry *g, const float *partial, float *o
 {
     dim3 grd((g->n_bins + 255) / 256, g->n_views, batch);
     counted();
-    k_band_reduce<3><<<grd, 256, 0, st>>>(partial, out, g->d_views, proj_bands(g->n), g->n_views, g->n_bins,
-                                          reinterpret_cast<const float *>(fac), nullptr, nullptr);
+    k_band_reduce<true><<<grd, 256, 0, st>>>(partial, out, g->d_views, proj_bands(g->n), g->n_views, g->n_bins, fac);
 }
 
 // =====================================================================

@@ -67,19 +67,6 @@ __device__ __forceinline__ float hash_sign(size_t i)
     return (x & 1u) ? 1.0f : -1.0f;
 }
 
-// out = in * s (sqrt_s: in * sqrt(s))
-__global__ void k_scale_by(const float *in, const float *s, int sqrt_s, float *out, size_t n)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        out[i] = in[i] * (sqrt_s ? sqrtf(s[i]) : s[i]);
-}
-
-void launch_scale_by(const float *in, const float *s, int sqrt_s, float *out, size_t n, cudaStream_t st)
-{
-    counted();
-    k_scale_by<<<grid_for(n, 256), 256, 0, st>>>(in, s, sqrt_s, out, n);
-}
-
 // Deterministic reductions: a fixed grid of DOT_BLOCKS blocks; each thread
 // sums its grid-stride elements in float, warps add their lanes by a fixed
 // shuffle tree, the warp sums of a block are added in order, and the block
