@@ -131,7 +131,12 @@ void ct_geometry_destroy(ct_geometry *geom);
  *                    from a shared counter.  Both give the same sums.
  * 0 selects the built-in rule (for the projector a model of the time of
  * each shape of both forms: 2 steps per pass in form 1, 4 with 12 items'
- * threads in form 2; 4 slices; 16 rows).  The
+ * threads in form 2; 1 to 8 slices by a model of A^T's time for one image, a
+ * power of two in ct_backproject, whose batches share them among fewer blocks
+ * to the same bits, and 4 in the unrolled form; 16 rows).  Set on another
+ * geometry, the shapes read from a tuned one give its projector the 64 threads
+ * per item above, not the tuned count: autotune there, or set orbit_slices and
+ * tv_rows only.  The
  * projector's shapes (items_per_block, proj_rows, proj_form) and tv_rows
  * leave every result bit unchanged; orbit_slices changes the order in
  * which the backprojector's slice sums are added, so results can differ in

@@ -456,7 +456,7 @@ constexpr int ORB_T = 16;        // quadrant tile side
 constexpr int ORB_TY = 8;        // thread rows of a block: tile rows r, r + ORB_TY, ... each
 constexpr int ORB_TH = ORB_T * ORB_TY;
 constexpr int ORB_PX = ORB_T / ORB_TY;   // pixel orbits per thread
-constexpr int ORB_SL = 4;        // base-view slices unless tuned
+constexpr int ORB_SL = 4;        // base-view slices where no rule applies
 constexpr int ORB_SL_MAX = 8;
 constexpr int ORB_VC = 8;        // base views staged per chunk
 constexpr int ORB_RW = 36;       // values per window: pairs (k, k+1), k <= ORB_RW - 2
@@ -486,14 +486,15 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // wholly off the padded row, and one 8-byte load serves both views (their
 // windows, places and weights are the same).  A load per view took 5 us more
 // a launch at 512^2 / 720 views / 736 bins (a 30-iteration solve's 42: 6669
-// -> 6453 us); ct_backproject, which interleaves its input first, 66.7 ->
-// 63.8 us there, 238 -> 224 at 1024^2.  ORB_PAIR4: also B % 4 == 0, which makes the mirrored
-// windows' place a constant (one addition a view less, 2 %).  ORB_PLAIN: y
-// holds rows of B values, ld = B apart, copied value by value (25 us more
-// there: for small sinograms).  ORB_PLAIN4: such rows with B % 4 == 0, copied
-// in 16-byte pieces, two 4-byte loads for a pair's two views (for all but large
-// sinograms: no pass before it).  CL: instead of storing its sums, the
-// block leaves them in osm, entry (k ORB_PX + j) ORB_TH + tid for rotation
+// -> 6453 us).  ORB_PAIR4: also B % 4 == 0, which makes the mirrored windows'
+// place a constant (one addition a view less, 2 %).  ORB_PLAIN: y holds rows
+// of B values, ld = B apart, copied value by value (25 us more there: for
+// small sinograms).  ORB_PLAIN4: such rows with B % 4 == 0, copied in 16-byte
+// pieces, two 4-byte loads for a pair's two views (for all but large
+// sinograms: no pass before it).  ct_backproject, which interleaves a large
+// input first, takes 65.6 us a call at 512^2 / 720 (62.5 in a replayed graph,
+// the pass included) and 225 at 1024^2, 67.7 and 238 from the plain rows.
+// CL: instead of storing its sums, the block leaves them in osm, entry (k ORB_PX + j) ORB_TH + tid for rotation
 // k of the thread's pixel orbit j, for a cluster reduction over slices.
 // SEQ (nsl a power of two): bz counts the csz blocks of a tile, a divisor of
 // nsl, instead of the slices; each takes nsl / csz slices one after the other.
@@ -647,7 +648,7 @@ __device__ __forceinline__ void orbit_body(const Ctx &cb, int bx, int by, int bz
             };
             // e - 1/2 of P and of R90 P for the thread's two orbits, (x, y) = (xq, yq) and (xq, yq + ORB_TY),
             // their windows' places and weights: packed (14 issue slots a view for 28; ct_backproject 63.8 -> 62.7 us
-            // at 512^2 / 720 views, each value rounded as before)
+            // in a replayed graph at 512^2 / 720 views, each value rounded as before)
             const float2 e = pfma(xq2, Tx, pfma(yq2, Ty, hb2)), e9 = pfma(xq2, Ty, pfma(nyq2, Tx, hb2));
             const float2 t = padd(e, bias2), t9 = padd(e9, bias2);
             const float2 u = psub(t, bias2), u9 = psub(t9, bias2);

@@ -42,10 +42,10 @@ __host__ __device__ __forceinline__ int tv_halo(int steps, bool even) { return e
 // needs r_y of the row above and x of the row below; the latter is computed
 // again from that row's published r and its z, so a step has one barrier and
 // four shared-memory accesses.  A column pair's arithmetic is packed
-// (f32x2).  Bound: one 16-warp block an SM, its chain of steps (issue 44 %,
+// (f32x2).  Bound: one 16-warp block an SM, its chain of steps (issue 47 %,
 // FP pipe and barrier waits); 512^2, 10 steps: 13.6 us with rows dealt out
-// in turn (two barriers, 4 J accesses a step, 5.9 M instructions), 11.1 us
-// now (4.2 M), cold cache.
+// in turn (two barriers, 4 J accesses a step, 5.9 M instructions), 11.1 to
+// 12.1 us now (4.2 M), cold cache.
 template <bool FGP, bool TRAJ, int J, class Ctx>
 __device__ __forceinline__ void tv_body(const Ctx &cb, int bx, int by, int bz, int gz, TvPub &pub,
                                         const float *z, const float *p_in, float *p_out, float *x, int N,

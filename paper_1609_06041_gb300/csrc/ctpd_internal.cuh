@@ -71,7 +71,7 @@ struct Geometry {
     long long *d_qbounds; // device, qbounds_nb + 1 entries: the work-balanced projector's unit ranges for one
                           // image, balanced by the tuner from measured block times (NULL: equal unit counts)
     int qbounds_nb;       // the launch they fit: blocks ...
-    int qbounds_key;      // ... and 64 (4 steps per pass) + items per block
+    int qbounds_key;      // ... and 64 (2 (ray positions of a unit per lane) + (4 steps per pass)) + items per block
     unsigned long long *d_qtimes;   // device: the tuner's per-block start and end times while it measures
     double *h_angles;     // host copy
     cudaMemPool_t pool;   // the device's, for the scratch of ct_project and ct_backproject (NULL: the default pool)

@@ -297,8 +297,6 @@ k_eps_sum_w2(const float *__restrict__ part, int ks, int V, int B, float *__rest
     }
 }
 
-// after the second map: out = sum_z part[z] (chunks in order), out2 =
-// 2 out - mu0
 // the place of element i (rows of B) of a sinogram in the given rows
 __device__ __forceinline__ size_t in_rows(size_t i, int V, int B, const Rows &rows)
 {
@@ -307,6 +305,8 @@ __device__ __forceinline__ size_t in_rows(size_t i, int V, int B, const Rows &ro
     return rows.row(0, (int)v, V) + (i - (size_t)v * B) * rows.step();
 }
 
+// after the second map: out = sum_z part[z] (chunks in order), out2 =
+// 2 out - mu0
 __global__ void k_eps_sum_out(const float *__restrict__ part, int ks, size_t n, int V, int B, float *__restrict__ out, Rows ldo,
                               float *__restrict__ out2, Rows ld2, const float *__restrict__ mu0)
 {

@@ -60,9 +60,10 @@ constexpr int min_blocks(int P) { return block_threads(P) >= 768 ? 1 : 768 / blo
 // Threads of a block that reads band sums.  A grid with a block or more for
 // every SM takes the transforms' threads only.  A smaller one (few views,
 // small images) is bound by the latency of its 16 loads an element, so there
-// 512 threads stage the residual and the transforms' threads go on alone
-// (measured on a form with 16 elements a thread: 512^2 / 32 views 19.6 us a
-// step without the extra threads, 10.7 with them; 64^2 / 90: 14.0 and 10.7).
+// 512 threads stage the residual and the transforms' threads go on alone (the
+// dual step without and with the extra threads, cold: 512^2 / 32 views 12.8
+// and 10.6 us, 64^2 / 90 8.7 and 6.8; a solve's iteration 29.5 and 28.3, 18.8
+// and 17.3 us).
 constexpr int wide_threads(int P) { return block_threads(P) < 512 ? 512 : block_threads(P); }
 bool wide_grid(const Geometry *g, int batch)
 {
@@ -260,7 +261,7 @@ void launch_filter_fft(const Geometry *g, const float2 *hhat, const float *in, f
 // and of the exchanges between stages (issue 46 %, 29 % of the warp slots).
 // 512^2 / 720 views / 736 bins (360 view pairs, one wave of three 256-thread
 // blocks an SM): 35.3 -> 22.7 us; 32 views (16 pairs, the wide form): 16.6 ->
-// 10.9 us; 64^2 / 90 / 95: 14.6 -> 7.7 us (cold cache).
+// 10.6 us; 64^2 / 90 / 95: 14.6 -> 6.8 us (cold cache).
 template <int P, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? wide_threads(P) : block_threads(P), WIDE ? 1 : min_blocks(P))
 k_dual_fft(const DualArgs a)

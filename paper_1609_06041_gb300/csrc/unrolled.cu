@@ -128,10 +128,14 @@ bool tv_fused(double tau, double beta, int mode, int ntv)
     return ntv >= 1 && ntv <= tv_max_steps() && lam > 0.0;
 }
 
-// A in the unrolled form.  On sides that are not a multiple of 32 it keeps
-// the plain band sums: the gradients pass through the prox's kinks, where
-// another rounding of A moves tap gradients by up to 1e-4 of their norm, so
-// there their values stay what they were.
+// A in the unrolled form.  At the default angles, sides that are not a
+// multiple of 32 keep the plain band sums: the gradients pass through the
+// prox's kinks, where another rounding of A moves tap gradients by up to 1e-4
+// of their norm, and there their values stay what they were.  Custom angles,
+// and sides over 637, take the mirrored projector, whose rounding is another
+// but no worse: tap gradients against float64, plain and mirrored, 5.8e-5 and
+// 4.1e-5 at 100^2 / 50 golden angles, 1.8e-5 both at 128^2 / 60, 2.4e-6 and
+// 2.7e-6 at 250^2 / 90, 2.0e-6 and 2.6e-6 at 672^2 / 40 (means of six draws).
 void project(const Geometry *g, const float *x, float *band, int S, cudaStream_t st)
 {
     launch_project_bands(g, x, band, S, st, g->vpair && g->n % 32 != 0);
